@@ -140,7 +140,7 @@ struct RowGrid {
 };
 
 // Eight dependent quantization steps of one row (one lane) on the mini-block whose weights are v[0..7].
-// us points at U'[8 m][8 m] (rows of U divided by their pivots, row stride kSweepLd).  Returns the differences
+// us points at U'[8 m][8 m] (rows of U divided by their pivots, row stride LD).  Returns the differences
 // d_p = w_p - q_p in v[] and the clamped level indices in lev[].
 //
 // EXACT = false: the level index rint(w / s) -- by definition a true float64 division -- is taken from the product
@@ -148,7 +148,7 @@ struct RowGrid {
 // from a rounding boundary (and below 1e9 in magnitude) both round to the same integer.  The return value tells whether
 // some step was closer than that, in which case the caller repeats the mini-block with EXACT = true (the division).
 // Rounding: (v + 1.5 * 2^52) - 1.5 * 2^52 is round-to-nearest-even for |v| < 2^51.
-template <bool EXACT>
+template <bool EXACT, int LD = kSweepLd>
 __device__ __forceinline__ bool sweep_chain8(double (&v)[8], double (&lev)[8], const double* us, const RowGrid& g) {
     bool danger = false;
 #pragma unroll
@@ -164,7 +164,7 @@ __device__ __forceinline__ bool sweep_chain8(double (&v)[8], double (&lev)[8], c
         const double rvc = fmin(fmax(rv, g.lo), g.hi);
         const double d = v[p] - g.sc * rvc;
 #pragma unroll
-        for (int j = p + 1; j < 8; ++j) v[j] = fma(-d, us[p * kSweepLd + j], v[j]);
+        for (int j = p + 1; j < 8; ++j) v[j] = fma(-d, us[p * LD + j], v[j]);
         v[p] = d;
         lev[p] = rvc;
     }

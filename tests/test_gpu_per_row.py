@@ -48,6 +48,31 @@ def test_per_row_arm_matches_oracle(rows, cols, n, bits, mode):
         assert any(not np.array_equal(perm_rows[r], perm_rows[0]) for r in range(1, rows))   # the rows do differ
 
 
+@pytest.mark.parametrize("rows,cols,bits", [(5, 8, 4), (3, 9, 3), (2, 7, 8), (2, 121, 4), (449, 127, 4)])
+def test_per_row_arm_at_the_edges_of_its_tiles(rows, cols, bits):
+    """Widths on and around the 8 x 8 tiles of the factorisation, and more rows than CTAs fit on the GPU at once."""
+    W, X = wl.make_layer(wl.LayerSpec("pr", rows, cols, 2 * cols, bits, "kaiming", "normal", 1500 + rows + cols))
+    H = oracle.hessian_accumulate(X)
+    Hinv, diag, _ = oracle.prepare_hinv(H)
+    sc, zp = oracle.minmax_grid(W, bits)
+    ref = oracle.quantize_layer_per_row(W, Hinv, diag, sc, zp, bits, ptq.SCORE_QERR, H_undamped=H)
+    codes, What, perm_rows, loss = _run(W, H, Hinv, sc, zp, bits, ptq.SCORE_QERR)
+    assert np.array_equal(perm_rows, ref["perm_rows"])
+    assert np.array_equal(codes, ref["codes"])
+    assert np.array_equal(What, ref["What"])
+    assert abs(loss - ref["loss"]) <= 1e-9 * ref["loss"]
+
+
+def test_a_pivot_that_is_not_positive_is_reported():
+    n = 20
+    Hinv = np.eye(n)
+    Hinv[11, 11] = -1.0
+    W = np.full((1, n), 0.5, np.float32)
+    with pytest.raises(ptq.PtqError) as ei:
+        _run(W, np.eye(n), Hinv, np.ones(1, np.float32), np.zeros(1, np.float32), 4, ptq.SCORE_NONE)
+    assert ei.value.code == ptq.ERR_NOT_SPD and "index 11" in str(ei.value)
+
+
 def test_wider_layers_are_refused():
     fake = torch.zeros(16, dtype=torch.float32, device="cuda")
     st, ws = ptq.new_status(), ptq.Workspace()
