@@ -18,6 +18,7 @@
 // Every wait on an mbarrier is bounded; when one expires the CTA records PTQ_ERR_TIMEOUT, drains and returns.
 #pragma once
 #include "common.cuh"
+#include <utility>
 
 namespace ptq {
 
@@ -30,6 +31,7 @@ constexpr int kGramStages = 3;
 constexpr int kGramABytes = kGramTM * kGramKB;                    // 8 KB per slice
 constexpr int kGramBBytes = kGramTN * kGramKB;                    // 4 KB per slice
 constexpr int kGramStageBytes = kSlices * (kGramABytes + kGramBBytes);   // 72 KB
+static_assert(kGramABytes == 8192 && kGramBBytes == 4096 && kGramTN == 64, "tc_slice_products relies on them");
 constexpr int kGramSmemBytes = kGramStages * kGramStageBytes + 1024 /*align*/ + 256 /*barriers*/;
 constexpr int kGramThreads = 192;          // warp 0: TMA, warp 1: MMA + TMEM, warps 2..5: epilogue
 constexpr int kGramMaxChunk = 16384;       // calibration columns per launch: 6 * 2^14 * 16384 < 2^31
@@ -264,15 +266,6 @@ __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::
 __device__ __forceinline__ void tc_commit(uint32_t bar) {
     asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
 }
-__device__ __forceinline__ void tc_mma_i8(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
-                                          uint32_t accumulate) {
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "setp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::i8 [%0], %1, %2, %3, {%5, %5, %5, %5}, p;\n\t}\n"
-        ::"r"(d_tmem), "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate), "r"(0u)
-        : "memory");
-}
 __device__ __forceinline__ void tc_ld16(uint32_t taddr, uint32_t (&r)[16]) {
     asm volatile(
         "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
@@ -282,36 +275,59 @@ __device__ __forceinline__ void tc_ld16(uint32_t taddr, uint32_t (&r)[16]) {
 }
 __device__ __forceinline__ void tc_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 
-// Shared-memory matrix descriptor: K-major operand, 64-byte rows, SWIZZLE_64B; 8-row groups are 512 bytes apart.
-__device__ __forceinline__ uint64_t make_desc_sw64(uint32_t smem_addr) {
-    uint64_t d = 0;
-    d |= (uint64_t)((smem_addr >> 4) & 0x3FFF);        // start address / 16
-    d |= (uint64_t)1 << 16;                            // leading byte offset / 16 (not used by swizzled K-major)
-    d |= (uint64_t)(512 >> 4) << 32;                   // stride byte offset / 16
-    d |= (uint64_t)1 << 46;                            // descriptor version of this architecture
-    d |= (uint64_t)4 << 61;                            // SWIZZLE_64B
-    return d;
-}
-
-// The same descriptor as two 32-bit words; the address field (bits 0..13, shared-memory address / 16) is added to the
-// low word at run time: all tiles lie below 256 KB, so the sum never leaves the field.
+// Shared-memory matrix descriptor of a K-major operand with 64-byte rows, SWIZZLE_64B, 8-row groups 512 bytes apart, as
+// two 32-bit words: the low one holds the start address / 16 (bits 0..13) and a leading offset that swizzled K-major
+// operands do not use, the high one the stride / 16, the descriptor version (bit 46) and the swizzle mode (bits 61..63).
+// The address field is added to the low word at run time: all tiles lie below 256 KB, so the sum never leaves the field.
 constexpr uint32_t kDescLo = 1u << 16;
 constexpr uint32_t kDescHi = (uint32_t)(512 >> 4) | (1u << 14) | (4u << 29);
-__device__ __forceinline__ void tc_mma_i8_lohi(uint32_t d_tmem, uint32_t a_lo, uint32_t b_lo, uint32_t hi,
-                                               uint32_t idesc, uint32_t accumulate) {
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t.reg .b64 da, db;\n\t"
-        "mov.b64 da, {%1, %3};\n\t"
-        "mov.b64 db, {%2, %3};\n\t"
-        "setp.ne.b32 p, %5, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::i8 [%0], da, db, %4, {%6, %6, %6, %6}, p;\n\t}\n"
-        ::"r"(d_tmem), "r"(a_lo), "r"(b_lo), "r"(hi), "r"(idesc), "r"(accumulate), "r"(0u)
-        : "memory");
+// How an MMA treats the buffer in which the tensor core holds its A operand: KEEP loads A and keeps it, LAST multiplies by
+// the A kept, ONCE neither.
+enum { TC_A_ONCE = 0, TC_A_KEEP = 1, TC_A_LAST = 2 };
+template <int A_USE>
+__device__ __forceinline__ void tc_mma_i8_lohi(uint32_t d_tmem, uint32_t a_lo, uint32_t b_lo, uint32_t hi, uint32_t idesc,
+                                               uint32_t accumulate) {
+#define PTQ_TC_MMA_I8(QUAL)                                                                                      \
+    asm volatile("{\n\t.reg .pred p;\n\t.reg .b64 da, db;\n\t"                                                   \
+                 "mov.b64 da, {%1, %3};\n\t"                                                                     \
+                 "mov.b64 db, {%2, %3};\n\t"                                                                     \
+                 "setp.ne.b32 p, %5, 0;\n\t"                                                                     \
+                 "tcgen05.mma.cta_group::1.kind::i8" QUAL " [%0], da, db, %4, {%6, %6, %6, %6}, p;\n\t}\n"       \
+                 ::"r"(d_tmem), "r"(a_lo), "r"(b_lo), "r"(hi), "r"(idesc), "r"(accumulate), "r"(0u)              \
+                 : "memory")
+    if constexpr (A_USE == TC_A_KEEP) PTQ_TC_MMA_I8(".collector::a::fill");
+    else if constexpr (A_USE == TC_A_LAST) PTQ_TC_MMA_I8(".collector::a::lastuse");
+    else PTQ_TC_MMA_I8(".collector::a::discard");
+#undef PTQ_TC_MMA_I8
 }
 
-// Instruction descriptor: int8 x int8 -> int32, both operands K-major, M = 128, N = 64.
-constexpr uint32_t kGramIdesc = (2u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(kGramTN >> 3) << 17) |
-                                ((uint32_t)(kGramTM >> 4) << 24);
+// Instruction descriptor: int8 x int8 -> int32, both operands K-major, M = 128.
+template <int N>
+constexpr uint32_t kIdescI8 = (2u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(128 >> 4) << 24);
+// The products of slice A of the row operand with the slices 0 .. G - 1 - A of the column operand, whose results belong
+// to the accumulator groups A .. G - 1.  The 64-row tiles of consecutive column slices follow one another in shared
+// memory and the 64-column accumulators of consecutive groups in TMEM, so all of them together are ONE product with
+// N = 64 (G - A); only above 256, the largest N, it takes two, the second of which reuses the row operand the tensor core
+// still holds.
+template <int A, int G>
+__device__ __forceinline__ void tc_slice_row(uint32_t d_tmem, uint32_t a_lo, uint32_t b_lo, uint32_t first) {
+    constexpr int N = 64 * (G - A), N0 = N > 256 ? 256 : N;
+    const uint32_t acc = A > 0 ? 1u : first;
+    if constexpr (N > 256) {
+        tc_mma_i8_lohi<TC_A_KEEP>(d_tmem + A * 64, a_lo, b_lo, kDescHi, kIdescI8<N0>, acc);
+        tc_mma_i8_lohi<TC_A_LAST>(d_tmem + A * 64 + N0, a_lo, b_lo + (N0 / 64) * (4096 >> 4), kDescHi, kIdescI8<N - N0>,
+                                  acc);
+    } else {
+        tc_mma_i8_lohi<TC_A_ONCE>(d_tmem + A * 64, a_lo, b_lo, kDescHi, kIdescI8<N0>, acc);
+    }
+}
+// All slice pairs (a, b) with a + b < G of one 32-byte K step.  a_lo, b_lo: descriptor words of slice 0 of the operands,
+// whose slices are 8 KB (128 rows) and 4 KB (64 rows) apart; first = 0: the accumulators are overwritten.
+template <int G, int... As>
+__device__ __forceinline__ void tc_slice_products(uint32_t d_tmem, uint32_t a_lo, uint32_t b_lo, uint32_t first,
+                                                  std::integer_sequence<int, As...>) {
+    (tc_slice_row<As, G>(d_tmem, a_lo + As * (8192 >> 4), b_lo, first), ...);
+}
 
 // Tile t of the enumeration: row block bi (128 rows), column block bj (64 columns) with 64*bj + 63 >= 128*bi.
 __device__ __forceinline__ void gram_tile_coords(int tile, int nbj, int& bi, int& bj) {
@@ -435,20 +451,9 @@ gram_i8_kernel(const __grid_constant__ CUtensorMap tmapA, const __grid_constant_
                     const uint32_t sb = kDescLo + ((base + stage * kGramStageBytes) >> 4);
                     const uint32_t first = kb > kb0 ? 1u : 0u;    // the first product of a group overwrites
 #pragma unroll
-                    for (int t = 0; t < kGroups; ++t) {
-#pragma unroll
-                        for (int a = 0; a <= t; ++a) {
-                            const int b = t - a;
-#pragma unroll
-                            for (int ks = 0; ks < kGramKB / 32; ++ks) {
-                                const uint32_t alo = sb + (uint32_t)((a * kGramABytes) >> 4) + (uint32_t)(ks * 2);
-                                const uint32_t blo = sb + (uint32_t)((kSlices * kGramABytes + b * kGramBBytes) >> 4) +
-                                                     (uint32_t)(ks * 2);
-                                tc_mma_i8_lohi(tmem_base + t * kGramTN, alo, blo, kDescHi, kGramIdesc,
-                                               (a > 0 || ks > 0) ? 1u : first);
-                            }
-                        }
-                    }
+                    for (int ks = 0; ks < kGramKB / 32; ++ks)
+                        tc_slice_products<kGroups>(tmem_base, sb + ks * 2, sb + ks * 2 + ((kSlices * kGramABytes) >> 4),
+                                                   ks > 0 ? 1u : first, std::make_integer_sequence<int, kSlices>());
                     tc_commit(empty_bar(stage));     // the stage may be refilled once these MMAs have read it
                     if (++stage == kGramStages) { stage = 0; phase ^= 1u; }
                 }

@@ -29,6 +29,7 @@ constexpr int kXStages = 2;
 constexpr int kXABytes = kXTM * kXKB;        // 8 KB per slice
 constexpr int kXBBytes = kXTN * kXKB;        // 4 KB per slice
 constexpr int kXStageBytes = kXSlices * (kXABytes + kXBBytes);     // 84 KB
+static_assert(kXABytes == kGramABytes && kXBBytes == kGramBBytes && kXTN == kGramTN, "tc_slice_products relies on them");
 constexpr int kXEpiDoubles = 4 * 32 * 17;    // per epilogue warp: 32 rows x 16 columns (+1 padding)
 constexpr int kXSmemBytes = kXStages * kXStageBytes + 1024 /*align*/ + 256 /*barriers*/ + kXEpiDoubles * 8;
 constexpr int kXThreads = 192;               // warp 0: TMA, warp 1: MMA + TMEM, warps 2..5: epilogue
@@ -311,20 +312,9 @@ i8gemm_kernel(const __grid_constant__ CUtensorMap tmapA, const __grid_constant__
                     const uint32_t sb = kDescLo + ((base + stage * kXStageBytes) >> 4);
                     const uint32_t first = kb > kb0 ? 1u : 0u;    // the first product of a group overwrites
 #pragma unroll
-                    for (int g = 0; g < kXGroups; ++g) {
-#pragma unroll
-                        for (int a = 0; a <= g; ++a) {
-                            const int b = g - a;
-#pragma unroll
-                            for (int ks = 0; ks < kXKB / 32; ++ks) {
-                                const uint32_t alo = sb + (uint32_t)((a * kXABytes) >> 4) + (uint32_t)(ks * 2);
-                                const uint32_t blo = sb + (uint32_t)((kXSlices * kXABytes + b * kXBBytes) >> 4) +
-                                                     (uint32_t)(ks * 2);
-                                tc_mma_i8_lohi(tmem_base + g * kXTN, alo, blo, kDescHi, kGramIdesc,
-                                               (a > 0 || ks > 0) ? 1u : first);
-                            }
-                        }
-                    }
+                    for (int ks = 0; ks < kXKB / 32; ++ks)
+                        tc_slice_products<kXGroups>(tmem_base, sb + ks * 2, sb + ks * 2 + ((kXSlices * kXABytes) >> 4),
+                                                    ks > 0 ? 1u : first, std::make_integer_sequence<int, kXSlices>());
                     tc_commit(empty_bar(stage));     // the stage may be refilled once these MMAs have read it
                     if (++stage == kXStages) { stage = 0; phase ^= 1u; }
                 }
