@@ -5,6 +5,7 @@
 #pragma once
 #include "common.cuh"
 #include "dgemm.cuh"
+#include <type_traits>
 #include <utility>
 
 namespace ptq {
@@ -42,11 +43,11 @@ __global__ void damp_copy_kernel(const double* __restrict__ H, double* __restric
 }
 
 // ------------------------------------------------------------------------------------------------------------
-// Blocked upper Cholesky A = U^T U as ONE persistent cooperative kernel (one CTA per SM, 256 threads).
+// Blocked upper Cholesky A = U^T U as ONE persistent cooperative kernel (one CTA per SM, 512 threads).
 // For each 64-row block k:
-//   strip phase    every CTA that owns a 64-column panel chunk factorises the 64 x 64 diagonal block itself (all
+//   strip phase    every CTA that owns a 40-column panel chunk factorises the 64 x 64 diagonal block itself (all
 //                  CTAs do the same arithmetic on it, so no broadcast is needed) and applies the same row
-//                  operations to its chunk: the unblocked algorithm on a 64 x 128 strip, eight pivots at a time
+//                  operations to its chunk: the unblocked algorithm on a 64 x 104 strip, eight pivots at a time
 //                  (see chol_strip).  That replaces "factor the block, then solve the panel against it".
 //   trailing phase A[i][j] -= U[k][i]^T U[k][j] on the upper 64 x 64 tiles, float64 tensor-core MMA, operands
 //                  double-buffered through shared memory with cp.async.
@@ -56,9 +57,11 @@ __global__ void damp_copy_kernel(const double* __restrict__ H, double* __restric
 // PTQ_ERR_TIMEOUT, raises the abort word and leaves; the other CTAs see the abort word and leave too.
 // A non-positive or non-finite pivot is reported (PTQ_ERR_NOT_SPD, pivot index) and replaced by 1.
 // ------------------------------------------------------------------------------------------------------------
-constexpr int kCholThreads = 256;
+constexpr int kCholThreads = 512;
 constexpr int kCholLd = kNB + 4;                               // operand row stride (68 = 4 mod 16: conflict-free)
-constexpr size_t kCholSmemBytes = sizeof(double) * (2 * 2 * kNB * kCholLd) + 16;
+constexpr int kCholBlock = kNB * kCholLd;                      // doubles of a 64 x 64 operand block
+constexpr int kCholOpndDoubles = 2 /*operands*/ * 2 /*slots*/ * kCholBlock;
+constexpr size_t kCholSmemBytes = sizeof(double) * kCholOpndDoubles + 16;
 
 __device__ __forceinline__ unsigned ld_acquire_u32(const unsigned* p) {
     unsigned v;
@@ -95,21 +98,23 @@ __device__ __forceinline__ void cp_async16_cg(void* smem_dst, const void* gsrc, 
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(d), "l"(gsrc), "r"(sz) : "memory");
 }
 
+// -x by its sign bit: an arithmetic negation would queue for the float64 pipe behind the MMAs it is an operand of.
+__device__ __forceinline__ double flip_sign(double x) {
+    return __hiloint2double(__double2hiint(x) ^ (int)0x80000000, __double2loint(x));
+}
+
 // Loads the 64 x ncols block A[r0 .. r0+63][c0 .. c0+ncols-1] into dst[64][kCholLd], ncols = 1 << lg in {16, 32, 64};
-// entries beyond n are zero.  Every thread copies a fixed column (pair) of successive row groups, so a block that lies
-// inside the matrix needs one pointer increment per copy and no bounds test.
-// NT threads take part (the first NT of the CTA): all of them, or the first four warps when the other four are to
-// go on computing meanwhile.
-template <int NT = kCholThreads>
+// entries beyond n are zero.  Every one of the NT threads (tid = 0 .. NT - 1) copies a fixed column (pair) of successive row
+// groups, so a block that lies inside the matrix needs one pointer increment per copy and no bounds test.
+template <int NT>
 __device__ __forceinline__ void chol_load_block(double* dst, const double* __restrict__ A, int64_t ld, int n, int r0,
-                                                int c0, int lg, int vec16) {
-    if (NT < kCholThreads && threadIdx.x >= NT) return;
+                                                int c0, int lg, int vec16, int tid) {
     const bool interior = r0 + kNB <= n && c0 + (1 << lg) <= n;
     if (vec16) {
         const int sh = lg - 1;                           // pairs per row = 1 << sh
-        const int c = (threadIdx.x & ((1 << sh) - 1)) * 2;
+        const int c = (tid & ((1 << sh) - 1)) * 2;
         const int rstep = NT >> sh;
-        int r = threadIdx.x >> sh;
+        int r = tid >> sh;
         const double* src = A + (int64_t)(r0 + r) * ld + c0 + c;
         double* d = dst + r * kCholLd + c;
         if (interior) {
@@ -121,9 +126,9 @@ __device__ __forceinline__ void chol_load_block(double* dst, const double* __res
             }
         }
     } else {
-        const int c = threadIdx.x & ((1 << lg) - 1);
+        const int c = tid & ((1 << lg) - 1);
         const int rstep = NT >> lg;
-        int r = threadIdx.x >> lg;
+        int r = tid >> lg;
         const double* src = A + (int64_t)(r0 + r) * ld + c0 + c;
         double* d = dst + r * kCholLd + c;
         for (; r < kNB; r += rstep, src += (int64_t)rstep * ld, d += rstep * kCholLd) {
@@ -134,225 +139,270 @@ __device__ __forceinline__ void chol_load_block(double* dst, const double* __res
 }
 
 // ------------------------------------------------------------------------------------------------------------
-// Strip factorisation: the 64 x 128 strip [diagonal block | 64 panel columns] is held in registers as 8 x 8
-// MMA accumulator fragments (warp w owns strip columns 16 w .. 16 w + 15, all 64 rows).  Pivots are taken eight
-// at a time.  For pivot block b:
+// Strip factorisation: the 64 x 104 strip [diagonal block | 40 panel columns] is held in registers as 8 x 8 MMA accumulator
+// fragments, eight strip columns (one column group, all 64 rows) per warp.  Pivots are taken eight at a time.  For pivot
+// block b:
 //   1. warp 0 factorises the 8 x 8 diagonal mini-block M = U_M^T U_M (all of M in every lane, so the serial chain of
 //      eight pivots has no data exchange in it) and carries the identity along to obtain W = U_M^-T;
-//   2. the new rows U[8 b .. 8 b + 7][:] = W R come from two MMAs per fragment (R: the row panel, published before);
-//   3. they are published; every warp subtracts them from the rows of pivot block b + 1 FIRST and publishes those
-//      rows at once, so that warp 0 can start on the next mini-block,
-//   4. while the other warps subtract them from the rows further down, A[i][c] -= U[p][i] U[p][c], again by MMA.
-// Warp 0 owns the first 16 columns of the diagonal block, whose fragments below row 16 are never used: it has no
-// update work of its own in step 4 and is therefore the one that runs the chain.  Named barrier 1 hands the row panel
-// to warp 0 (the others only arrive), named barrier 2 hands W to everybody.
+//   2. it makes the next mini-block itself, M' = T - (W R)^T (W R), from what the owner of those columns has put out
+//      before: the rows R of this pivot block and T, the next diagonal tile without this pivot block's update;
+//   3. meanwhile every other warp forms the new rows U[8 b .. 8 b + 7][own columns] = W R and, when all of them are out,
+//      subtracts them from its rows further down, A[i][c] -= U[p][i] U[p][c], by MMA, and brings the rows of the next
+//      pivot block up to date with the block row above (look-ahead).
+// Named barriers, by the parity of b: 1 / 2 (owner, warp 0) hand over R and T, 3 / 4 (all) hand out W; 5 (all but warp 0)
+// makes the new rows visible.  Owners only arrive at 1 / 2 and warp 0 only arrives at 3 / 4, so warp 0 may be one pivot
+// block ahead of or behind the other warps, hence two of each.  It is never two ahead: R and T of block b + 1 leave their
+// owner after the barriers 3 / 4 and 5 of block b; nor two behind: they wait for it at 3 / 4.
+//
+// What bounds a strip is the chain, and what used to bound the chain were the MMAs of other warps: scalar float64
+// instructions queue behind the float64 MMAs of their scheduler (measured: 9 clocks per dependent FMA alone, 137 next to
+// one warp that streams MMAs on the same scheduler, 9 again when the MMAs are on the other three).  So warp 0 has its
+// scheduler to itself: warps 4, 8 and 12 take no part in a strip, and the updates are dealt to the other three schedulers,
+// which is also why a strip has 40 panel columns (twelve warps with one column group each) and not 64: 1800 MMAs over
+// three schedulers then take about as long as the eight chains with their hand-overs.  Measured per block row, from grid
+// barrier to grid barrier, on matrices whose trailing tiles do not fill the GPU: 30.0 k clocks with the chain sharing its
+// scheduler (8 warps, 64 panel columns) -> 26.5 k, of which 4 k before the first chain, 9.9 k in the chains, 6.8 k between
+// them and 4.5 k for stores and the barrier.  One factorisation: 39 -> 30 us at 128 columns, 654 -> 623 us at 2304.
 // ------------------------------------------------------------------------------------------------------------
-constexpr int kStripLd = 132;                                            // row stride of the 8-row panels
+constexpr int kStripPanel = 40;                                          // panel columns of a strip
+constexpr int kStripGroups = (kNB + kStripPanel) / 8;                    // column groups: 0 .. 7 diagonal, 8 .. 12 panel
+constexpr int kStripLd = kNB + kStripPanel + 12;                         // row stride of the 8-row panels (116 = 4 mod 16)
 constexpr int kStripCostTiles = 4;                                       // a strip takes about as long as four trailing tiles
-constexpr int kStripSmemDoubles = 2 * 8 * kStripLd + 64;
-static_assert(kStripSmemDoubles <= 2 * 2 * kNB * kCholLd, "the strip panels alias the trailing-phase operand buffers");
+constexpr int kStripThreads = 32 * kStripGroups;                         // threads of the warps that take part
+constexpr int kStripSmemDoubles = 2 * 8 * kStripLd + 64 /*M*/ + 64 /*W R*/ + 2 * 64 /*W*/ + 2 * 2 * 64 /*R, T*/;
+static_assert(kStripSmemDoubles + 2 * kCholBlock <= kCholOpndDoubles,
+              "the strip panels and the look-ahead operands alias the trailing-phase operand buffers");
 
-__device__ __forceinline__ void strip_bar_sync(int id) {
-    asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(kCholThreads) : "memory");
-}
-__device__ __forceinline__ void strip_bar_arrive(int id) {
-    asm volatile("bar.arrive %0, %1;" ::"r"(id), "r"(kCholThreads) : "memory");
-}
+template <int ID, int COUNT>
+__device__ __forceinline__ void named_bar_sync() { asm volatile("bar.sync %0, %1;" ::"n"(ID), "n"(COUNT) : "memory"); }
+template <int ID, int COUNT>
+__device__ __forceinline__ void named_bar_arrive() { asm volatile("bar.arrive %0, %1;" ::"n"(ID), "n"(COUNT) : "memory"); }
 
-// Rows of pivot block B of this warp's columns go to the row panel.
-template <int B>
-__device__ __forceinline__ void chol_strip_publish(const double (&acc)[8][2][2], double* Rbuf, int c0, int lq, int lr) {
-#pragma unroll
-    for (int cb = 0; cb < 2; ++cb)
-        *reinterpret_cast<double2*>(Rbuf + lq * kStripLd + c0 + 8 * cb + 2 * lr) =
-            make_double2(acc[B][cb][0], acc[B][cb][1]);
-}
+struct StripSmem {
+    double* R;       // [8][kStripLd] rows of the pivot block (every warp reads back its own columns only)
+    double* U;       // [8][kStripLd] new rows
+    double* M;       // [8][8] mini-block (warp 0 only)
+    double* V;       // [8][8] W R of the next eight columns (warp 0 only)
+    double* W;       // [2][8][8] by parity of the pivot block: a warp may read W late, while warp 0 is in its next chain
+    double* X;       // [2][2][8][8] by the same parity: R and T of the next eight columns
+    __device__ __forceinline__ explicit StripSmem(double* p)
+        : R(p), U(R + 8 * kStripLd), M(U + 8 * kStripLd), V(M + 64), W(V + 64), X(W + 128) {}
+};
 
 // acc[r] -= U[:, 8 r .. 8 r + 7]^T U[:, own columns] for the fragment rows R0 <= r < R1 (U: the eight rows in Ubuf).
 template <int R0, int R1>
-__device__ __forceinline__ void chol_strip_update(double (&acc)[8][2][2], const double* Ubuf, int warp, int c0, int lq,
-                                                  int lr) {
+__device__ __forceinline__ void chol_strip_update(double (&acc)[8][2], const double* Ubuf, int grp, int lq, int lr) {
     if constexpr (R0 < R1) {
-        double bf[2][2];
-#pragma unroll
-        for (int cb = 0; cb < 2; ++cb) {
-            bf[cb][0] = Ubuf[lr * kStripLd + c0 + 8 * cb + lq];
-            bf[cb][1] = Ubuf[(4 + lr) * kStripLd + c0 + 8 * cb + lq];
-        }
+        const double b0 = Ubuf[lr * kStripLd + 8 * grp + lq], b1 = Ubuf[(4 + lr) * kStripLd + 8 * grp + lq];
 #pragma unroll
         for (int r = R0; r < R1; ++r) {
-            const double n0 = -Ubuf[lr * kStripLd + 8 * r + lq];
-            const double n1 = -Ubuf[(4 + lr) * kStripLd + 8 * r + lq];
-#pragma unroll
-            for (int cb = 0; cb < 2; ++cb) {
-                if (warp < 4 && 8 * r > c0 + 8 * cb + 7) continue;       // entirely below the diagonal: never used
-                dmma_884(acc[r][cb][0], acc[r][cb][1], n0, bf[cb][0]);
-                dmma_884(acc[r][cb][0], acc[r][cb][1], n1, bf[cb][1]);
-            }
+            if (grp < 8 && r > grp) continue;                            // entirely below the diagonal: never used
+            dmma_884(acc[r][0], acc[r][1], flip_sign(Ubuf[lr * kStripLd + 8 * r + lq]), b0);
+            dmma_884(acc[r][0], acc[r][1], flip_sign(Ubuf[(4 + lr) * kStripLd + 8 * r + lq]), b1);
         }
     }
 }
 
 // Look-ahead update of fragment row RB of this warp's strip columns with the block row above (see chol_strip):
-//     acc[RB] -= ua[:, 8 RB .. 8 RB + 7]^T bsrc[:, own 16 columns]        (ua, bsrc: 64 x 64 in shared memory)
-// Applied one fragment row at a time, just before the row is needed, by the warps that wait for warp 0's chain.
+//     acc[RB] -= ua[:, 8 RB .. 8 RB + 7]^T bsrc[:, own 8 columns]        (ua, bsrc: 64 rows in shared memory)
+// Applied one fragment row at a time, shortly before the row is needed, by the warps that wait for warp 0's chain.
 template <int RB>
-__device__ __forceinline__ void chol_strip_lookahead(double (&acc)[8][2][2], const double* ua, const double* bsrc,
-                                                     bool is_diag, int sc0, int lq, int lr) {
-    double prod[2][2] = {{0.0, 0.0}, {0.0, 0.0}};
-#pragma unroll 4
-    for (int kk = 0; kk < kNB; kk += 4) {
-        const double af = ua[(kk + lr) * kCholLd + 8 * RB + lq];
-#pragma unroll
-        for (int cb = 0; cb < 2; ++cb) {
-            // fragments of the diagonal block that lie entirely below the diagonal are never used
-            if (is_diag && 8 * RB > sc0 + 8 * cb + 7) continue;
-            dmma_884(prod[cb][0], prod[cb][1], af, bsrc[(kk + lr) * kCholLd + 8 * cb + lq]);
-        }
-    }
-#pragma unroll
-    for (int cb = 0; cb < 2; ++cb) {
-        acc[RB][cb][0] -= prod[cb][0];
-        acc[RB][cb][1] -= prod[cb][1];
-    }
+__device__ __forceinline__ void chol_strip_lookahead(double (&acc)[8][2], const double* ua, const double* bsrc, int grp,
+                                                     int lq, int lr) {
+    if (grp < 8 && RB > grp) return;            // fragments that lie entirely below the diagonal are never used
+#pragma unroll 8
+    for (int kk = 0; kk < kNB; kk += 4)
+        dmma_884(acc[RB][0], acc[RB][1], flip_sign(ua[(kk + lr) * kCholLd + 8 * RB + lq]), bsrc[(kk + lr) * kCholLd + lq]);
 }
 
+// Step 1 above.  mb: the mini-block M (row-major, 8 x 8, upper part); leaves W in Wbuf.  Returns the first pivot that is not
+// positive and finite (it is replaced by 1) or -1.
+__device__ __forceinline__ int chol_chain8(const double* mb, double* Wbuf, int lane) {
+    double m[8][8];
+#pragma unroll
+    for (int p = 0; p < 8; ++p)
+#pragma unroll
+        for (int j = p; j < 8; ++j) m[p][j] = mb[p * 8 + j];
+    // lane j carries column j of the identity along, which becomes column j of W = U_M^-T
+    const int jc = lane & 7;
+    double x[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) x[i] = i == jc ? 1.0 : 0.0;
+    int bad = -1;
+#pragma unroll
+    for (int p = 0; p < 8; ++p) {
+        // A bad pivot is replaced by 1 and remembered; the report is made after the chain, so that the eight steps
+        // stay one straight line of code.
+        const double d0 = m[p][p];
+        const bool ok = d0 > 0.0 && d0 < 1.0e300;
+        bad = (!ok && bad < 0) ? p : bad;
+        const double d = ok ? d0 : 1.0;
+        // 1 / d is what the chain waits for: the hardware's approximation (about 20 bits) times the first terms of
+        // 1 / (1 - e) = 1 + e + e^2 + .., e = 1 - d y; what is left out is of order e^3, far below one ulp
+        double y, z;
+        asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(d));
+        const double e = fma(-d, y, 1.0);
+        const double inv = fma(y, fma(e, e, e), y);
+        // 1 / sqrt(d), beside the chain: z (1 + g / 2 + 3 g^2 / 8), g = 1 - d z^2, likewise
+        asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(z) : "d"(d));
+        const double g = fma(-(z * z), d, 1.0);
+        const double rs = fma(z, g * fma(0.375, g, 0.5), z);
+        const double tx = x[p] * inv;
+        x[p] *= rs;
+#pragma unroll
+        for (int i = p + 1; i < 8; ++i) {
+            const double f = m[p][i] * inv;
+#pragma unroll
+            for (int j = i; j < 8; ++j) m[i][j] = fma(-f, m[p][j], m[i][j]);
+            x[i] = fma(-m[p][i], tx, x[i]);
+        }
+    }
+    if (lane < 8) {
+#pragma unroll
+        for (int p = 0; p < 8; ++p) Wbuf[p * 8 + lane] = x[p];    // W[p][j] = (U_M^-T)[p][j]
+    }
+    return bad;
+}
+
+// Two MMAs: the 8 x 8 product W R in accumulator layout, W row-major in Wbuf, R with row stride ldr.
+__device__ __forceinline__ double2 chol_new_rows(const double* Wbuf, const double* R, int ldr, int lq, int lr) {
+    double2 v = make_double2(0.0, 0.0);
+    dmma_884(v.x, v.y, Wbuf[lq * 8 + lr], R[lr * ldr + lq]);
+    dmma_884(v.x, v.y, Wbuf[lq * 8 + 4 + lr], R[(4 + lr) * ldr + lq]);
+    return v;
+}
+
+// Warp 0: the chains of all eight pivot blocks and the mini-blocks in between.  first: the first mini-block in accumulator
+// layout (group 0's only fragment in use).  Returns the first eight rows of the factor in those columns.
+__device__ __forceinline__ double2 chol_strip_chain(double2 first, const StripSmem& sm, int lane, int k0, bool reporter,
+                                                    int32_t* status) {
+    const int lq = lane >> 2, lr = lane & 3;
+    *reinterpret_cast<double2*>(sm.M + lq * 8 + 2 * lr) = first;
+    *reinterpret_cast<double2*>(sm.R + lq * kStripLd + 2 * lr) = first;
+    __syncwarp();
+#pragma unroll 1
+    for (int b = 0; b < 8; ++b) {
+        double* Wb = sm.W + (b & 1) * 64;
+        const int bad = chol_chain8(sm.M, Wb, lane);
+        if (b & 1) named_bar_arrive<4, kStripThreads>(); else named_bar_arrive<3, kStripThreads>();
+        if (bad >= 0 && reporter) report(status, PTQ_ERR_NOT_SPD, k0 + 8 * b + bad);
+        __syncwarp();
+        if (b < 7) {
+            const double* X = sm.X + (b & 1) * 128;
+            if (b & 1) named_bar_sync<2, 64>(); else named_bar_sync<1, 64>();      // R and T of the next eight columns are out
+            const double2 v = chol_new_rows(Wb, X, 8, lq, lr);
+            *reinterpret_cast<double2*>(sm.V + lq * 8 + 2 * lr) = v;
+            double2 t = *reinterpret_cast<const double2*>(X + 64 + lq * 8 + 2 * lr);
+            __syncwarp();
+            const double u0 = sm.V[lr * 8 + lq], u1 = sm.V[(4 + lr) * 8 + lq];
+            dmma_884(t.x, t.y, flip_sign(u0), u0);
+            dmma_884(t.x, t.y, flip_sign(u1), u1);
+            *reinterpret_cast<double2*>(sm.M + lq * 8 + 2 * lr) = t;
+            __syncwarp();
+        }
+        if (b == 0) first = chol_new_rows(Wb, sm.R, kStripLd, lq, lr);
+    }
+    return first;
+}
+
+// Every other warp: pivot block B.
 template <int B>
-__device__ __forceinline__ void chol_strip_block(double (&acc)[8][2][2], double* Rbuf, double* Ubuf, double* Wbuf,
-                                                 int warp, int lane, int k0, bool reporter, int32_t* status,
+__device__ __forceinline__ void chol_strip_block(double (&acc)[8][2], const StripSmem& sm, int grp, int lane, bool update,
                                                  const double* ua, const double* bsrc) {
     const int lq = lane >> 2, lr = lane & 3;
-    const int c0 = 16 * warp;
-    if (warp == 0) {
-        // 1. the mini-block; lane j carries column j of the identity along, which becomes column j of W = U_M^-T
-        double m[8][8];
-#pragma unroll
-        for (int p = 0; p < 8; ++p)
-#pragma unroll
-            for (int j = p; j < 8; ++j) m[p][j] = Rbuf[p * kStripLd + 8 * B + j];
-        const int jc = lane & 7;
-        double x[8];
-#pragma unroll
-        for (int i = 0; i < 8; ++i) x[i] = i == jc ? 1.0 : 0.0;
-        int bad = -1;                    // first pivot of this mini-block that is not positive and finite
-#pragma unroll
-        for (int p = 0; p < 8; ++p) {
-            // A bad pivot is replaced by 1 and remembered; the report is made after the chain, so that the eight steps
-            // stay one straight line of code.
-            const double d0 = m[p][p];
-            const bool ok = d0 > 0.0 && d0 < 1.0e300;
-            bad = (!ok && bad < 0) ? p : bad;
-            const double d = ok ? d0 : 1.0;
-            // 1 / sqrt(d): the hardware's approximation (about 20 bits) refined without a branch by
-            // y (1 + e / 2 + 3 e^2 / 8), e = 1 - d y^2, which leaves an error of order e^3, far below one ulp;
-            // the library routine is three times as long a chain
-            double y;
-            asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(d));
-            const double e = fma(-(y * y), d, 1.0);
-            const double rs = fma(y, e * fma(0.375, e, 0.5), y);
-            const double inv = rs * rs;
-            const double tx = x[p] * inv;
-            x[p] *= rs;
-#pragma unroll
-            for (int i = p + 1; i < 8; ++i) {
-                const double f = m[p][i] * inv;
-                x[i] = fma(-m[p][i], tx, x[i]);
-#pragma unroll
-                for (int j = i; j < 8; ++j) m[i][j] = fma(-f, m[p][j], m[i][j]);
-            }
+    // While warp 0 is in its chain: the update by the pivot block before, and the look-ahead update of the rows of the next
+    // pivot block.  The owner of the next eight columns puts out what warp 0 is going to need first; it has brought its next
+    // diagonal fragment up to date one pivot block early, so that only the update by the pivot block before stands in between.
+    const bool owner = B < 7 && grp == B + 1;
+    if constexpr (B > 0) chol_strip_update<B, (B < 7 ? B + 2 : 8)>(acc, sm.U, grp, lq, lr);
+    if (owner) {
+        if constexpr (B == 0) {
+            if (update) chol_strip_lookahead<1>(acc, ua, bsrc, grp, lq, lr);
         }
-        if (lane < 8) {
-#pragma unroll
-            for (int p = 0; p < 8; ++p) Wbuf[p * 8 + lane] = x[p];    // W[p][j] = (U_M^-T)[p][j]
-        }
-        if (bad >= 0 && reporter) report(status, PTQ_ERR_NOT_SPD, k0 + 8 * B + bad);
-    } else {
-        // while warp 0 is in its chain: 4. (of the mini-block before) the rows further down, and the look-ahead update
-        // of the rows of the next pivot block, which are needed right after this mini-block
-        if constexpr (B > 0) chol_strip_update<B + 1, 8>(acc, Ubuf, warp, c0, lq, lr);
-        if constexpr (B < 7) {
-            if (bsrc != nullptr) chol_strip_lookahead<B + 1>(acc, ua, bsrc, warp < 4, c0, lq, lr);
-        }
+        double* X = sm.X + (B & 1) * 128 + lq * 8 + 2 * lr;
+        *reinterpret_cast<double2*>(X) = make_double2(acc[B][0], acc[B][1]);
+        if constexpr (B < 7) *reinterpret_cast<double2*>(X + 64) = make_double2(acc[B + 1][0], acc[B + 1][1]);
+        named_bar_arrive<1 + (B & 1), 64>();
     }
-    strip_bar_sync(2);       // W is there; nobody reads the previous new rows any more
-    // 2. new rows = W R
-    const double a0 = Wbuf[lq * 8 + lr], a1 = Wbuf[lq * 8 + 4 + lr];
-#pragma unroll
-    for (int cb = 0; cb < 2; ++cb) {
-        const double b0 = Rbuf[lr * kStripLd + c0 + 8 * cb + lq];
-        const double b1 = Rbuf[(4 + lr) * kStripLd + c0 + 8 * cb + lq];
-        double r0 = 0.0, r1 = 0.0;
-        dmma_884(r0, r1, a0, b0);
-        dmma_884(r0, r1, a1, b1);
-        acc[B][cb][0] = r0;
-        acc[B][cb][1] = r1;
-        *reinterpret_cast<double2*>(Ubuf + lq * kStripLd + c0 + 8 * cb + 2 * lr) = make_double2(r0, r1);
-    }
-    __syncthreads();
-    // 3. the rows of the next pivot block first, and out they go
+    if constexpr (B > 0 && B < 6) chol_strip_update<B + 2, 8>(acc, sm.U, grp, lq, lr);
     if constexpr (B < 7) {
-        chol_strip_update<B + 1, B + 2>(acc, Ubuf, warp, c0, lq, lr);
-        chol_strip_publish<B + 1>(acc, Rbuf, c0, lq, lr);
-        if (warp == 0) strip_bar_sync(1); else strip_bar_arrive(1);
+        if (update && !owner) chol_strip_lookahead<B + 1>(acc, ua, bsrc, grp, lq, lr);
     }
+    if constexpr (B < 6) {
+        if (update && grp == B + 2) chol_strip_lookahead<B + 2>(acc, ua, bsrc, grp, lq, lr);
+    }
+    // the rows of this pivot block as an MMA operand (read back by this warp only)
+    *reinterpret_cast<double2*>(sm.R + lq * kStripLd + 8 * grp + 2 * lr) = make_double2(acc[B][0], acc[B][1]);
+    named_bar_sync<3 + (B & 1), kStripThreads>();             // W is there; nobody reads the previous new rows any more
+    if (grp >= B) {
+        const double2 v = chol_new_rows(sm.W + (B & 1) * 64, sm.R + 8 * grp, kStripLd, lq, lr);
+        acc[B][0] = v.x;
+        acc[B][1] = v.y;
+        *reinterpret_cast<double2*>(sm.U + lq * kStripLd + 8 * grp + 2 * lr) = v;
+    }
+    if constexpr (B < 7) named_bar_sync<5, kStripThreads - 32>();             // the new rows are out
 }
 template <int... Bs>
-__device__ __forceinline__ void chol_strip_blocks(double (&acc)[8][2][2], double* Rbuf, double* Ubuf, double* Wbuf,
-                                                  int warp, int lane, int k0, bool reporter, int32_t* status,
-                                                  const double* ua, const double* bsrc,
-                                                  std::integer_sequence<int, Bs...>) {
-    chol_strip_publish<0>(acc, Rbuf, 16 * warp, lane >> 2, lane & 3);
-    if (warp == 0) strip_bar_sync(1); else strip_bar_arrive(1);
-    (chol_strip_block<Bs>(acc, Rbuf, Ubuf, Wbuf, warp, lane, k0, reporter, status, ua, bsrc), ...);
+__device__ __forceinline__ void chol_strip_blocks(double (&acc)[8][2], const StripSmem& sm, int grp, int lane, bool update,
+                                                  const double* ua, const double* bsrc, std::integer_sequence<int, Bs...>) {
+    (chol_strip_block<Bs>(acc, sm, grp, lane, update, ua, bsrc), ...);
 }
 
-// Factorises the diagonal block of A at k0 and applies the same row operations to 64 panel columns with it: columns
-// pc0 .. pc0 + 63 of rows k0 .. k0 + 63 of the matrix P (row stride ld), or, when `identity` is set, of the identity
-// block (whose transform is the inverse of the transposed diagonal factor).  P == nullptr: diagonal block only.
+// Factorises the diagonal block of A at k0 and applies the same row operations to 40 panel columns with it: columns
+// pc0 .. pc0 + 39 of rows k0 .. k0 + 63 of the matrix P (row stride ld); with add_identity the entries on P's diagonal are
+// taken as 1 (P = W, zero there in memory: the transform of the identity block is the inverse of the transposed diagonal
+// factor).  P == nullptr: diagonal block only.
 // Every CTA working on this block row reads the diagonal block of A, at a time of its own, so the factor of that
 // block is NOT written in place: the CTA with write_diag set stores it to D (64 x 64, row stride 64), and the kernel
 // copies all diagonal factors into A at its very end.
-// When upd_a is given, the strip is first brought up to date with the previous block row (look-ahead):
+// look_ahead: the strip is first brought up to date with the previous block row, which is final by then:
 //     strip -= upd_a^T [upd_a | upd_b],   upd_a[kk][r] = U[k0 - 64 + kk][k0 + r],  upd_b[kk][c] = P[k0 - 64 + kk][pc0 + c]
-// (both 64 x 64 in shared memory, row stride kCholLd; upd_b == nullptr: the panel part needs no update).
-__device__ __forceinline__ void chol_strip(double* __restrict__ A, int64_t ld, int n, int k0, double* __restrict__ P,
-                                           int pc0, bool identity, bool write_diag, double* __restrict__ D,
-                                           double* smem, int vec16, int32_t* status, const double* upd_a,
-                                           const double* upd_b) {
-    // "warp" below is the index of the 16-column group a warp owns, not its hardware number.  Warps w and w + 4 share a
-    // scheduler; warp 0 (group 0, the chain) is paired with the next lightest group (diagonal columns 16 .. 31, whose
-    // fragments below row 32 are unused) and the heavier groups are spread over the other schedulers:
-    // hardware warp 0 1 2 3 4 5 6 7 -> group 0 2 3 6 1 4 5 7.
-    const int lane = threadIdx.x & 31, warp = (int)((0x75416320u >> (4 * (threadIdx.x >> 5))) & 7u);
+// (64 x 64 in shared memory, row stride kCholLd; only 40 columns of upd_b are used).
+// Not inlined: the chain alone needs nearly all of the 128 registers, and what the kernel keeps across a strip is saved
+// once around the call instead of inside the chain.
+__device__ __noinline__ void chol_strip(double* __restrict__ A, int64_t ld, int n, int k0, double* __restrict__ P,
+                                        int pc0, bool add_identity, bool write_diag, double* __restrict__ D, int vec16,
+                                        int32_t* status, bool look_ahead) {
+    extern __shared__ __align__(16) unsigned char chol_smem_raw[];
+    double* smem = reinterpret_cast<double*>(chol_smem_raw);
+    // operands of the look-ahead update, beyond the strip's own panel buffers
+    double* upd_a = smem + kStripSmemDoubles;
+    double* upd_b = upd_a + kCholBlock;
+    const bool has_b = look_ahead && P != nullptr;
+    if (look_ahead) {
+        chol_load_block<kCholThreads>(upd_a, A, ld, n, k0 - kNB, k0, 6, vec16, threadIdx.x);
+        if (has_b) chol_load_block<kCholThreads>(upd_b, P, ld, n, k0 - kNB, pc0, 6, vec16, threadIdx.x);
+        cp_async_commit();
+    }
+    // Column group of every warp; 15: takes no part.  Warps w, w + 4, w + 8 and w + 12 share a scheduler: scheduler 0 holds
+    // the chain (group 0) alone, the others {8 9 5 1}, {10 11 4 3} and {12 7 6 2}, about 600 MMAs each.
+    const int lane = threadIdx.x & 31, grp = (int)((0x231F645F7B9FCA80ull >> (4 * (threadIdx.x >> 5))) & 15u);
     const int lq = lane >> 2, lr = lane & 3;
-    double* Rbuf = smem;
-    double* Ubuf = smem + 8 * kStripLd;
-    double* Wbuf = smem + 2 * 8 * kStripLd;
-    const bool is_diag = warp < 4;
-    const int gc0 = is_diag ? k0 + 16 * warp : pc0 + 16 * (warp - 4);       // first global column of this warp
-    const int sc0 = 16 * warp;                                               // first strip column
-    double acc[8][2][2];
-    // panel columns that lie inside the matrix and are not the identity: plain vector loads
-    const bool fast_panel = !is_diag && P != nullptr && !identity && vec16 && k0 + kNB <= n && pc0 + kNB <= n;
-    if (fast_panel) {
-        const double* src = P + (int64_t)(k0 + lq) * ld + gc0 + 2 * lr;
+    const StripSmem sm(smem);
+    const bool is_diag = grp < 8;
+    const int gc0 = is_diag ? k0 + 8 * grp : pc0 + 8 * (grp - 8);           // first global column of this warp
+    const int sc0 = 8 * grp;                                                 // first strip column
+    double acc[8][2];
+    if (grp < kStripGroups) {
+        // columns that lie inside the matrix: plain vector loads (of the diagonal block only the fragments from the
+        // diagonal up; what lies below the diagonal in the diagonal fragment itself is never used)
+        const bool fast = vec16 && k0 + kNB <= n && (is_diag || (P != nullptr && pc0 + kStripPanel <= n));
+        if (fast) {
+            const double* src = (is_diag ? A : P) + (int64_t)(k0 + lq) * ld + gc0 + 2 * lr;
 #pragma unroll
-        for (int rb = 0; rb < 8; ++rb)
-#pragma unroll
-            for (int cb = 0; cb < 2; ++cb) {
-                const double2 v = __ldcg(reinterpret_cast<const double2*>(src + (int64_t)(8 * rb) * ld + 8 * cb));
-                acc[rb][cb][0] = v.x;
-                acc[rb][cb][1] = v.y;
+            for (int rb = 0; rb < 8; ++rb) {
+                if (is_diag && rb > grp) { acc[rb][0] = acc[rb][1] = 0.0; continue; }
+                const double2 v = __ldcg(reinterpret_cast<const double2*>(src + (int64_t)(8 * rb) * ld));
+                acc[rb][0] = v.x;
+                acc[rb][1] = v.y;
             }
-    } else {
+        } else {
 #pragma unroll
-        for (int rb = 0; rb < 8; ++rb)
-#pragma unroll
-            for (int cb = 0; cb < 2; ++cb) {
+            for (int rb = 0; rb < 8; ++rb) {
                 const int row = 8 * rb + lq, grow = k0 + row;
 #pragma unroll
                 for (int e = 0; e < 2; ++e) {
-                    const int sc = sc0 + 8 * cb + 2 * lr + e, gc = gc0 + 8 * cb + 2 * lr + e;
+                    const int sc = sc0 + 2 * lr + e, gc = gc0 + 2 * lr + e;
                     double val = 0.0;
                     if (is_diag) {
                         if (sc >= row) {
@@ -360,144 +410,246 @@ __device__ __forceinline__ void chol_strip(double* __restrict__ A, int64_t ld, i
                             else if (sc == row) val = 1.0;                   // identity padding below n
                         }
                     } else if (P != nullptr && grow < n && gc < n) {
-                        val = identity ? (sc - kNB == row ? 1.0 : 0.0) : __ldcg(P + (int64_t)grow * ld + gc);
+                        val = __ldcg(P + (int64_t)grow * ld + gc);
                     }
-                    acc[rb][cb][e] = val;
+                    acc[rb][e] = val;
                 }
             }
-    }
-    // Look-ahead update with the block row above: only the first fragment row (and warp 0's second: warp 0 runs the
-    // chains and has no other rows in use) is brought up to date here; the others follow inside the strip, each while
-    // warp 0 works on the mini-block before it.
-    const double* bsrc = nullptr;
-    if (upd_a != nullptr) {
-        cp_async_wait<0>();
-        __syncthreads();
-        bsrc = is_diag ? upd_a + 16 * warp : (upd_b != nullptr ? upd_b + 16 * (warp - 4) : nullptr);
-        if (bsrc != nullptr) {
-            chol_strip_lookahead<0>(acc, upd_a, bsrc, is_diag, sc0, lq, lr);
-            if (warp == 0) chol_strip_lookahead<1>(acc, upd_a, bsrc, is_diag, sc0, lq, lr);
         }
-    }
-    chol_strip_blocks(acc, Rbuf, Ubuf, Wbuf, warp, lane, k0, write_diag && threadIdx.x == 0, status, upd_a, bsrc,
-                      std::make_integer_sequence<int, 8>());
-    if (is_diag) {
-        if (write_diag) {
+        if (add_identity && !is_diag) {
 #pragma unroll
             for (int rb = 0; rb < 8; ++rb)
 #pragma unroll
-                for (int cb = 0; cb < 2; ++cb) {
-                    const int row = 8 * rb + lq, sc = sc0 + 8 * cb + 2 * lr;
-                    if (sc >= row) D[row * kNB + sc] = acc[rb][cb][0];
-                    if (sc + 1 >= row) D[row * kNB + sc + 1] = acc[rb][cb][1];
-                }
+                for (int e = 0; e < 2; ++e)
+                    if (gc0 + 2 * lr + e == k0 + 8 * rb + lq) acc[rb][e] = 1.0;
+        }
+    }
+    // Look-ahead update with the block row above: only the first fragment row is brought up to date here; the others
+    // follow inside the strip, each while warp 0 works on the mini-block before it.
+    const double* bsrc = is_diag ? upd_a + 8 * grp : upd_b + 8 * (grp - 8);
+    const bool update = look_ahead && (is_diag || has_b);
+    if (look_ahead) {
+        cp_async_wait<0>();
+        __syncthreads();
+        if (update && grp < kStripGroups) chol_strip_lookahead<0>(acc, upd_a, bsrc, grp, lq, lr);
+    }
+    if (grp >= kStripGroups) return;
+    if (grp == 0) {
+        const double2 v = chol_strip_chain(make_double2(acc[0][0], acc[0][1]), sm, lane, k0, write_diag && lane == 0, status);
+        if (write_diag) {
+            if (2 * lr >= lq) D[lq * kNB + 2 * lr] = v.x;
+            if (2 * lr + 1 >= lq) D[lq * kNB + 2 * lr + 1] = v.y;
+        }
+        return;
+    }
+    chol_strip_blocks(acc, sm, grp, lane, update, upd_a, bsrc, std::make_integer_sequence<int, 8>());
+    if (is_diag) {
+        if (write_diag) {
+#pragma unroll
+            for (int rb = 0; rb < 8; ++rb) {
+                const int row = 8 * rb + lq, sc = sc0 + 2 * lr;
+                if (sc >= row) D[row * kNB + sc] = acc[rb][0];
+                if (sc + 1 >= row) D[row * kNB + sc + 1] = acc[rb][1];
+            }
         }
     } else if (P != nullptr) {
 #pragma unroll
-        for (int rb = 0; rb < 8; ++rb)
-#pragma unroll
-            for (int cb = 0; cb < 2; ++cb) {
-                const int grow = k0 + 8 * rb + lq, gc = gc0 + 8 * cb + 2 * lr;
-                if (grow >= n || gc >= n) continue;
-                double* dst = P + (int64_t)grow * ld + gc;
-                if (vec16) {
-                    __stcg(reinterpret_cast<double2*>(dst), make_double2(acc[rb][cb][0], acc[rb][cb][1]));
-                } else {
-                    __stcg(dst, acc[rb][cb][0]);
-                    if (gc + 1 < n) __stcg(dst + 1, acc[rb][cb][1]);
-                }
+        for (int rb = 0; rb < 8; ++rb) {
+            const int grow = k0 + 8 * rb + lq, gc = gc0 + 2 * lr;
+            if (grow >= n || gc >= n) continue;
+            double* dst = P + (int64_t)grow * ld + gc;
+            if (vec16) {
+                __stcg(reinterpret_cast<double2*>(dst), make_double2(acc[rb][0], acc[rb][1]));
+            } else {
+                __stcg(dst, acc[rb][0]);
+                if (gc + 1 < n) __stcg(dst + 1, acc[rb][1]);
             }
+        }
     }
 }
 
-// One H x 64 piece of a trailing tile: C[i0 .. i0 + H)[j0 .. j0 + 64) -= as^T bs with the operands in shared memory
-// (as[kk][r], bs[kk][c]); eight warps as 2 x 4, each (H / 2) x 16.  tri_off >= 0: the piece lies in a diagonal tile
-// and only entries with c >= tri_off + r are touched.
+// One H x 64 piece of a trailing tile, C[i0 .. i0 + H)[j0 .. j0 + 64); the 16 warps as 4 x 4 (H = 16: 2 x 8).
+// tri >= 0: the piece lies in a diagonal tile, tri rows below its top, and only entries with c >= tri + r are touched.
+struct CholPiece {
+    double* C;
+    const double* Bsrc;
+    int i0, j0, tri;
+};
 template <int H>
-__device__ __forceinline__ void chol_trailing_piece(double* __restrict__ C, int64_t ld, int n, const double* as,
-                                                    const double* bs, int i0, int j0, int tri_off, int vec16) {
-    constexpr int FM = H / 16, FN = 2;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int wm0 = (warp >> 2) * (H / 2), wn0 = (warp & 3) * 16;
-    const int lq = lane >> 2, lr = lane & 3;
-    // the old values of the tile are requested first and only consumed after the MMA loop, so that their latency
-    // hides behind it
-    double old[FM][FN][2], acc[FM][FN][2];
-    bool keep[FM][FN][2];
-    // a piece inside the matrix and off the diagonal needs no bounds or triangle tests at all
-    const bool plain = vec16 && tri_off < 0 && i0 + H <= n && j0 + kNB <= n;
-    if (plain) {
-        const double* src = C + (int64_t)(i0 + wm0 + lq) * ld + j0 + wn0 + 2 * lr;
-#pragma unroll
-        for (int a = 0; a < FM; ++a)
-#pragma unroll
-            for (int b = 0; b < FN; ++b) {
-                const double2 v = __ldcg(reinterpret_cast<const double2*>(src + (int64_t)(8 * a) * ld + 8 * b));
-                old[a][b][0] = v.x;
-                old[a][b][1] = v.y;
-                acc[a][b][0] = acc[a][b][1] = 0.0;
-                keep[a][b][0] = keep[a][b][1] = true;
-            }
-    } else
-#pragma unroll
-    for (int a = 0; a < FM; ++a) {
-        const int r = wm0 + a * 8 + lq;
-#pragma unroll
-        for (int b = 0; b < FN; ++b) {
-            const int c = wn0 + b * 8 + 2 * lr;
-            const bool in = i0 + r < n && j0 + c < n;
-            keep[a][b][0] = in && (tri_off < 0 || c >= tri_off + r);
-            keep[a][b][1] = in && j0 + c + 1 < n && (tri_off < 0 || c + 1 >= tri_off + r);
-            const double* src = C + (int64_t)(i0 + r) * ld + j0 + c;
-            if (vec16 && keep[a][b][0]) {             // n even: the pair is inside; keep[0] implies keep[1]
-                const double2 v = __ldcg(reinterpret_cast<const double2*>(src));
-                old[a][b][0] = v.x;
-                old[a][b][1] = v.y;
-            } else {
-                old[a][b][0] = keep[a][b][0] ? __ldcg(src) : 0.0;
-                old[a][b][1] = keep[a][b][1] ? __ldcg(src + 1) : 0.0;
-            }
-            acc[a][b][0] = acc[a][b][1] = 0.0;
+struct CholPieceShape {
+    static constexpr int WN = H == 16 ? 8 : 4;                 // warps side by side
+    static constexpr int FM = H * WN / 128, FN = 8 / WN;       // 8 x 8 fragments of a warp
+};
+__device__ __forceinline__ bool chol_piece_has(const CholPiece& pc, int n, int r, int c) {
+    return pc.i0 + r < n && pc.j0 + c < n && (pc.tri < 0 || c >= pc.tri + r);
+}
+// a piece inside the matrix and off the diagonal needs no bounds or triangle tests at all
+template <int H>
+__device__ __forceinline__ bool chol_piece_plain(const CholPiece& pc, int n, int vec16) {
+    return vec16 && pc.tri < 0 && pc.i0 + H <= n && pc.j0 + kNB <= n;
+}
+// The two entries of the piece at (r, c), (r, c + 1); zero where the piece has none.
+__device__ __forceinline__ double2 chol_pair_load(const CholPiece& pc, const double* src, int n, int r, int c, bool plain,
+                                                  int vec16) {
+    const bool k0 = plain || chol_piece_has(pc, n, r, c);
+    if (plain || (vec16 && k0)) return __ldcg(reinterpret_cast<const double2*>(src));       // n even: the pair is inside
+    return make_double2(k0 ? __ldcg(src) : 0.0, chol_piece_has(pc, n, r, c + 1) ? __ldcg(src + 1) : 0.0);
+}
+__device__ __forceinline__ void chol_pair_store(const CholPiece& pc, double* dst, int n, int r, int c, bool plain, int vec16,
+                                                double2 v) {
+    const bool k0 = plain || chol_piece_has(pc, n, r, c);
+    if (plain || (vec16 && k0)) {
+        __stcg(reinterpret_cast<double2*>(dst), v);
+    } else {
+        if (k0) __stcg(dst, v.x);
+        if (chol_piece_has(pc, n, r, c + 1)) __stcg(dst + 1, v.y);
+    }
+}
+
+// Trailing tiles of block row k restricted to the target block rows row_base <= i < row_limit.
+//   tiles of A: (i, j), row_base <= i <= j: A[i][j] -= U[k][i]^T U[k][j]
+//   tiles of W: (i, c), row_base <= i, c <= k:  W[i][c] -= U[k][i]^T W[k][c]       (row-major lists, A first)
+// In look-ahead mode the CTAs come here after `strips_b` strips of the next block row, the CTAs 0 .. n_more - 1 after
+// one more; a strip costs about as much as kStripCostTiles tiles, so they take correspondingly fewer pieces (the
+// busier CTAs from the end of the list) and all CTAs finish at about the same time.
+// Not inlined, for the sake of the registers, like chol_strip.
+__device__ __noinline__ void chol_trailing_phase(double* __restrict__ A, double* __restrict__ Wm, int n, int64_t ld, int vec16,
+                                                 int k, int row_base, int row_limit, int n_more, int strips_b) {
+    extern __shared__ __align__(16) unsigned char chol_smem_raw[];
+    const int G = gridDim.x, nb = (n + kNB - 1) / kNB;
+    const int k0 = k * kNB;
+    const int m = nb - row_base;                                        // tiles in the first target row
+    const int R = (row_limit < nb ? row_limit : nb) - row_base;         // target block rows
+    if (R <= 0) return;
+    const int TA = R * m - R * (R - 1) / 2;
+    const int TW = Wm != nullptr ? R * (k + 1) : 0;
+    const int T = TA + TW;
+    if (T <= 0) return;
+    // tiles are cut into 64 / H row pieces so that a short tile list still spreads over the grid
+    const int lgH = 4 * T <= G ? 4 : (T <= G ? 5 : 6);
+    const int lgP = 6 - lgH;
+    const int TP = T << lgP;
+    const int S = n_more < G ? n_more : G, N = G - S;
+    const int cs = kStripCostTiles << lgP;
+    const int cost_a = (strips_b + 1) * cs, cost_b = strips_b * cs;
+    int ps = 0;
+    if (S > 0) {
+        const int target = (int)((unsigned)(TP + S * cost_a + N * cost_b + G - 1) / (unsigned)G);
+        ps = target > cost_a ? target - cost_a : 0;
+        if (N == 0) ps = (int)((unsigned)(TP + S - 1) / (unsigned)S);
+    }
+    const int TPn = TP - S * ps > 0 ? TP - S * ps : 0;
+    const int pn = N > 0 ? (int)((unsigned)(TPn + N - 1) / (unsigned)N) : 0;
+    int tp_beg, tp_end;
+    if ((int)blockIdx.x >= S) {
+        tp_beg = ((int)blockIdx.x - S) * pn;
+        tp_end = tp_beg + pn < TPn ? tp_beg + pn : TPn;
+    } else {
+        tp_beg = TPn + (int)blockIdx.x * ps;
+        tp_end = tp_beg + ps < TP ? tp_beg + ps : TP;
+    }
+    if (tp_beg >= tp_end) return;
+    // pieces are asked for in ascending order, so the row of the triangular list is found by walking on from the
+    // row of the previous piece
+    int cur_r = 0, cur_start = 0;                       // row cur_r of the A list starts at tile cur_start
+    auto piece_of = [&](int tp) {
+        CholPiece pc;
+        const int t = tp >> lgP;
+        const int h0 = (tp & ((1 << lgP) - 1)) << lgH;
+        if (t < TA) {
+            while (t >= cur_start + (m - cur_r)) { cur_start += m - cur_r; ++cur_r; }
+            const int r = cur_r;
+            const int bi = row_base + r, bj = bi + (t - cur_start);
+            pc.C = A; pc.Bsrc = A; pc.i0 = bi * kNB + h0; pc.j0 = bj * kNB;
+            pc.tri = bi == bj ? h0 : -1;
+        } else {
+            const int tw = t - TA;
+            const int r = (int)((unsigned)tw / (unsigned)(k + 1)), c = tw - r * (k + 1);
+            pc.C = Wm; pc.Bsrc = Wm; pc.i0 = (row_base + r) * kNB + h0; pc.j0 = c * kNB;
+            pc.tri = -1;
         }
-    }
-#pragma unroll 4
-    for (int kk = 0; kk < kNB; kk += 4) {
-        double af[FM], bf[FN];
-#pragma unroll
-        for (int a = 0; a < FM; ++a) af[a] = as[(kk + lr) * kCholLd + wm0 + a * 8 + lq];
-#pragma unroll
-        for (int b = 0; b < FN; ++b) bf[b] = bs[(kk + lr) * kCholLd + wn0 + b * 8 + lq];
-#pragma unroll
-        for (int a = 0; a < FM; ++a)
-#pragma unroll
-            for (int b = 0; b < FN; ++b) dmma_884(acc[a][b][0], acc[a][b][1], af[a], bf[b]);
-    }
-    if (plain) {
-        double* dst = C + (int64_t)(i0 + wm0 + lq) * ld + j0 + wn0 + 2 * lr;
+        return pc;
+    };
+    // Operand blocks: a slot of abuf holds U[k][i-block] (as[kk][r]), a slot of bbuf U or W [k][j-block] (bs[kk][c]).
+    // Every CTA takes a contiguous run of the list, in which consecutive tiles mostly share their row block: the A
+    // operand then stays where it is and only B is fetched.  What the next piece needs, its operands and its old
+    // values, is requested at the start of this one, and the products go straight into the old values (one operand's
+    // sign flipped): subtractions afterwards would queue behind the other warps' MMAs.  One barrier per piece.
+    double* abuf = reinterpret_cast<double*>(chol_smem_raw);      // [2][64][kCholLd]
+    double* bbuf = abuf + 2 * kCholBlock;                         // [2][64][kCholLd]
+    auto run = [&](auto height) {
+        constexpr int H = decltype(height)::value, FM = CholPieceShape<H>::FM, FN = CholPieceShape<H>::FN;
+        constexpr int WN = CholPieceShape<H>::WN, LGH = H == 64 ? 6 : (H == 32 ? 5 : 4);
+        const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, lq = lane >> 2, lr = lane & 3;
+        const int wm0 = (warp / WN) * 8 * FM, wn0 = (warp % WN) * 8 * FN;
+        const int pr = wm0 + lq, pq = wn0 + 2 * lr;       // this lane's entries: (pr + 8 a, pq + 8 b), and one further
+        int stage = 0, a_slot = 0;
+        CholPiece cur = piece_of(tp_beg), nxt = cur;
+        chol_load_block<kCholThreads>(abuf, A, ld, n, k0, cur.i0, LGH, vec16, tid);
+        chol_load_block<kCholThreads>(bbuf, cur.Bsrc, ld, n, k0, cur.j0, 6, vec16, tid);
+        double2 acc[FM][FN], old[FM][FN];
+        bool plain = chol_piece_plain<H>(cur, n, vec16);
 #pragma unroll
         for (int a = 0; a < FM; ++a)
 #pragma unroll
             for (int b = 0; b < FN; ++b)
-                __stcg(reinterpret_cast<double2*>(dst + (int64_t)(8 * a) * ld + 8 * b),
-                       make_double2(old[a][b][0] - acc[a][b][0], old[a][b][1] - acc[a][b][1]));
-        return;
-    }
+                acc[a][b] = chol_pair_load(cur, cur.C + (int64_t)(cur.i0 + pr + 8 * a) * ld + cur.j0 + pq + 8 * b, n,
+                                           pr + 8 * a, pq + 8 * b, plain, vec16);
+        cp_async_commit();
+        for (int tp = tp_beg; tp < tp_end; ++tp) {
+            const bool more = tp + 1 < tp_end;
+            if (more) nxt = piece_of(tp + 1);
+            const bool new_a = more && nxt.i0 != cur.i0, plain_n = chol_piece_plain<H>(nxt, n, vec16);
+            const int a_next = a_slot ^ (new_a ? 1 : 0);
+            const double* as = abuf + a_slot * kCholBlock;
+            const double* bs = bbuf + stage * kCholBlock;
+            cp_async_wait<0>();
+            __syncthreads();         // this piece's operands have landed; the slots of the piece before are free
+            if (more) {
+                // half of the warps request the next operands: the copies keep the issuing warps busy for several
+                // hundred cycles, during which the others already feed the tensor pipe
+                if (warp < 8) {
+                    chol_load_block<kCholThreads / 2>(bbuf + (stage ^ 1) * kCholBlock, nxt.Bsrc, ld, n, k0, nxt.j0, 6, vec16, tid);
+                    if (new_a)
+                        chol_load_block<kCholThreads / 2>(abuf + a_next * kCholBlock, A, ld, n, k0, nxt.i0, LGH, vec16, tid);
+                }
 #pragma unroll
-    for (int a = 0; a < FM; ++a) {
-        const int r = wm0 + a * 8 + lq;
+                for (int a = 0; a < FM; ++a)
 #pragma unroll
-        for (int b = 0; b < FN; ++b) {
-            const int c = wn0 + b * 8 + 2 * lr;
-            double* dst = C + (int64_t)(i0 + r) * ld + j0 + c;
-            const double v0 = old[a][b][0] - acc[a][b][0], v1 = old[a][b][1] - acc[a][b][1];
-            if (vec16 && keep[a][b][0]) {
-                __stcg(reinterpret_cast<double2*>(dst), make_double2(v0, v1));
-            } else {
-                if (keep[a][b][0]) __stcg(dst, v0);
-                if (keep[a][b][1]) __stcg(dst + 1, v1);
+                    for (int b = 0; b < FN; ++b)
+                        old[a][b] = chol_pair_load(nxt, nxt.C + (int64_t)(nxt.i0 + pr + 8 * a) * ld + nxt.j0 + pq + 8 * b,
+                                                   n, pr + 8 * a, pq + 8 * b, plain_n, vec16);
             }
+#pragma unroll 4
+            for (int kk = lr; kk < kNB; kk += 4) {
+                double af[FM], bf[FN];
+#pragma unroll
+                for (int a = 0; a < FM; ++a) af[a] = as[kk * kCholLd + wm0 + a * 8 + lq];
+#pragma unroll
+                for (int b = 0; b < FN; ++b) bf[b] = flip_sign(bs[kk * kCholLd + wn0 + b * 8 + lq]);
+#pragma unroll
+                for (int a = 0; a < FM; ++a)
+#pragma unroll
+                    for (int b = 0; b < FN; ++b) dmma_884(acc[a][b].x, acc[a][b].y, af[a], bf[b]);
+            }
+            cp_async_commit();
+#pragma unroll
+            for (int a = 0; a < FM; ++a)
+#pragma unroll
+                for (int b = 0; b < FN; ++b) {
+                    chol_pair_store(cur, cur.C + (int64_t)(cur.i0 + pr + 8 * a) * ld + cur.j0 + pq + 8 * b, n, pr + 8 * a,
+                                    pq + 8 * b, plain, vec16, acc[a][b]);
+                    acc[a][b] = old[a][b];
+                }
+            stage ^= 1;
+            a_slot = a_next;
+            cur = nxt;
+            plain = plain_n;
         }
-    }
+    };
+    if (lgH == 6) run(std::integral_constant<int, 64>());
+    else if (lgH == 5) run(std::integral_constant<int, 32>());
+    else run(std::integral_constant<int, 16>());
 }
 
 __global__ void __launch_bounds__(kCholThreads, 1)
@@ -505,138 +657,37 @@ chol_coop_kernel(double* __restrict__ A, double* __restrict__ Wm, double* __rest
                  int vec16, unsigned* bar, int32_t* status, long long spin_limit, int k_first, int nb_stop,
                  int row_limit) {
     extern __shared__ __align__(16) unsigned char chol_smem_raw[];
-    double* opnd = reinterpret_cast<double*>(chol_smem_raw);                // [2 stages][2 operands][64][kCholLd]
-    int* s_flag = reinterpret_cast<int*>(opnd + 2 * 2 * kNB * kCholLd);     // the strip panels alias opnd
+    int* s_flag = reinterpret_cast<int*>(chol_smem_raw + sizeof(double) * kCholOpndDoubles);
     const int tid = threadIdx.x;
     const int G = gridDim.x;
     const int nb = (n + kNB - 1) / kNB;
     unsigned epoch = 0;
 
-    // strip work items of block row k: the panel chunks of A right of the block, then (with Wm) the chunks 0 .. k of
-    // row block k of W, the last of which starts as the identity
-    auto strip_items = [&](int k) { return (nb - 1 - k) + (Wm != nullptr ? k + 1 : 0); };
-    auto strip_item = [&](int k, int g, double*& P, int& pc0, bool& ident) {
-        const int chunksA = nb - 1 - k;
-        P = nullptr; pc0 = 0; ident = false;
-        if (g < chunksA) { P = A; pc0 = (k + 1 + g) * kNB; }
-        else if (g < strip_items(k)) { P = Wm; pc0 = (g - chunksA) * kNB; ident = (g - chunksA) == k; }
+    // strip work items of block row k: the 40-column chunks of A right of the block, then (with Wm) those of row block k of
+    // W up to the end of the block's own columns, which start as the identity
+    auto chunks_a = [&](int k) { const int w = n - (k + 1) * kNB; return w > 0 ? (w + kStripPanel - 1) / kStripPanel : 0; };
+    auto chunks_w = [&](int k) {
+        const int w = (k + 1) * kNB < n ? (k + 1) * kNB : n;
+        return Wm != nullptr ? (w + kStripPanel - 1) / kStripPanel : 0;
+    };
+    auto strip_items = [&](int k) { return chunks_a(k) + chunks_w(k); };
+    auto strip_item = [&](int k, int g, double*& P, int& pc0) {
+        const int ca = chunks_a(k);
+        P = nullptr; pc0 = 0;
+        if (g < ca) { P = A; pc0 = (k + 1) * kNB + g * kStripPanel; }
+        else if (g < strip_items(k)) { P = Wm; pc0 = (g - ca) * kStripPanel; }
     };
     // plain strip phase of block row k over the whole grid
     auto strip_phase = [&](int k) {
         const int items = strip_items(k);
         const int reps = items > 0 ? items : 1;                              // last block without Wm: diagonal only
         for (int g = blockIdx.x; g < reps; g += G) {
-            double* P; int pc0; bool ident;
-            strip_item(k, g, P, pc0, ident);
-            chol_strip(A, ld, n, k * kNB, P, pc0, ident, g == 0, Dbuf + (size_t)k * kNB * kNB, opnd, vec16, status, nullptr,
-                       nullptr);
+            double* P; int pc0;
+            strip_item(k, g, P, pc0);
+            chol_strip(A, ld, n, k * kNB, P, pc0, P == Wm, g == 0, Dbuf + (size_t)k * kNB * kNB, vec16, status, false);
             __syncthreads();     // the panel buffers are reused by the next repetition and by the trailing phase
         }
     };
-    // Trailing tiles of block row k restricted to the target block rows row_base <= i < row_limit.
-    //   tiles of A: (i, j), row_base <= i <= j: A[i][j] -= U[k][i]^T U[k][j]
-    //   tiles of W: (i, c), row_base <= i, c <= k:  W[i][c] -= U[k][i]^T W[k][c]       (row-major lists, A first)
-    // In look-ahead mode the CTAs come here after `strips_b` strips of the next block row, the CTAs 0 .. n_more - 1 after
-    // one more; a strip costs about as much as kStripCostTiles tiles, so they take correspondingly fewer pieces (the
-    // busier CTAs from the end of the list) and all CTAs finish at about the same time.
-    auto trailing_phase = [&](int k, int row_base, int n_more, int strips_b) {
-        const int k0 = k * kNB;
-        const int m = nb - row_base;                                        // tiles in the first target row
-        const int R = (row_limit < nb ? row_limit : nb) - row_base;         // target block rows
-        if (R <= 0) return;
-        const int TA = R * m - R * (R - 1) / 2;
-        const int TW = Wm != nullptr ? R * (k + 1) : 0;
-        const int T = TA + TW;
-        if (T <= 0) return;
-        // tiles are cut into 64 / H row pieces so that a short tile list still spreads over the grid
-        const int lgH = 4 * T <= G ? 4 : (2 * T <= G ? 5 : 6);
-        const int lgP = 6 - lgH;
-        const int TP = T << lgP;
-        const int S = n_more < G ? n_more : G, N = G - S;
-        const int cs = kStripCostTiles << lgP;
-        const int cost_a = (strips_b + 1) * cs, cost_b = strips_b * cs;
-        int ps = 0;
-        if (S > 0) {
-            const long work = (long)TP + (long)S * cost_a + (long)N * cost_b;
-            const int target = (int)((work + G - 1) / G);
-            ps = target > cost_a ? target - cost_a : 0;
-            if (N == 0) ps = (TP + S - 1) / S;
-        }
-        const int TPn = TP - S * ps > 0 ? TP - S * ps : 0;
-        const int pn = N > 0 ? (TPn + N - 1) / N : 0;
-        int tp_beg, tp_end;
-        if ((int)blockIdx.x >= S) {
-            tp_beg = ((int)blockIdx.x - S) * pn;
-            tp_end = tp_beg + pn < TPn ? tp_beg + pn : TPn;
-        } else {
-            tp_beg = TPn + (int)blockIdx.x * ps;
-            tp_end = tp_beg + ps < TP ? tp_beg + ps : TP;
-        }
-        if (tp_beg >= tp_end) return;
-        struct Piece { double* C; const double* Bsrc; int i0, j0, tri; };
-        // pieces are asked for in ascending order, so the row of the triangular list is found by walking on from the
-        // row of the previous piece
-        int cur_r = 0, cur_start = 0;                       // row cur_r of the A list starts at tile cur_start
-        auto piece_of = [&](int tp) {
-            Piece pc;
-            const int t = tp >> lgP;
-            const int h0 = (tp & ((1 << lgP) - 1)) << lgH;
-            if (t < TA) {
-                while (t >= cur_start + (m - cur_r)) { cur_start += m - cur_r; ++cur_r; }
-                const int r = cur_r;
-                const int bi = row_base + r, bj = bi + (t - cur_start);
-                pc.C = A; pc.Bsrc = A; pc.i0 = bi * kNB + h0; pc.j0 = bj * kNB;
-                pc.tri = bi == bj ? h0 : -1;
-            } else {
-                const int tw = t - TA;
-                const int r = tw / (k + 1), c = tw - r * (k + 1);
-                pc.C = Wm; pc.Bsrc = Wm; pc.i0 = (row_base + r) * kNB + h0; pc.j0 = c * kNB;
-                pc.tri = -1;
-            }
-            return pc;
-        };
-        // Operand blocks: slot s of the A half holds U[k][i-block] (as[kk][r]), slot s of the B half U or W [k][j-block].
-        // Every CTA takes a contiguous run of the list, in which consecutive tiles mostly share their row block: the A
-        // operand then stays where it is and only B is fetched.
-        double* abuf = opnd;                                  // [2][64][kCholLd]
-        double* bbuf = opnd + 2 * kNB * kCholLd;              // [2][64][kCholLd]
-        int stage = 0, a_slot = 0, a_next = 0;
-        Piece cur{}, nxt{};
-        if (tp_beg < tp_end) {
-            cur = piece_of(tp_beg);
-            chol_load_block(abuf, A, ld, n, k0, cur.i0, lgH, vec16);
-            chol_load_block(bbuf, cur.Bsrc, ld, n, k0, cur.j0, 6, vec16);
-        }
-        cp_async_commit();
-        for (int tp = tp_beg; tp < tp_end; ++tp) {
-            cp_async_wait<0>();
-            __syncthreads();         // this tile's operands have landed; the slots of the tile before are free
-            // The next tile's operands are requested by the first four warps only: the copies keep the issuing warps
-            // busy for several hundred cycles, during which the other four (one per scheduler) already feed the
-            // tensor pipe.
-            if (tp + 1 < tp_end) {
-                nxt = piece_of(tp + 1);
-                a_next = a_slot;
-                if (nxt.i0 != cur.i0) {
-                    a_next = a_slot ^ 1;
-                    chol_load_block<kCholThreads / 2>(abuf + a_next * kNB * kCholLd, A, ld, n, k0, nxt.i0, lgH, vec16);
-                }
-                chol_load_block<kCholThreads / 2>(bbuf + (stage ^ 1) * kNB * kCholLd, nxt.Bsrc, ld, n, k0, nxt.j0, 6,
-                                                  vec16);
-            }
-            cp_async_commit();
-            const double* as = abuf + a_slot * kNB * kCholLd;
-            const double* bs = bbuf + stage * kNB * kCholLd;
-            if (lgH == 6) chol_trailing_piece<64>(cur.C, ld, n, as, bs, cur.i0, cur.j0, cur.tri, vec16);
-            else if (lgH == 5) chol_trailing_piece<32>(cur.C, ld, n, as, bs, cur.i0, cur.j0, cur.tri, vec16);
-            else chol_trailing_piece<16>(cur.C, ld, n, as, bs, cur.i0, cur.j0, cur.tri, vec16);
-            stage ^= 1;
-            a_slot = a_next;
-            cur = nxt;
-        }
-        cp_async_wait<0>();
-    };
-
     // The block rows k_first .. nb_stop - 1 are factorised (block row k_first must already carry the updates of all rows
     // above it); their updates are applied to the target rows below row_limit.
     //   k_first = 0, nb_stop = nb, row_limit = nb : the whole factorisation;
@@ -652,7 +703,7 @@ chol_coop_kernel(double* __restrict__ A, double* __restrict__ Wm, double* __rest
         if (!grid_barrier(bar, epoch * (unsigned)G, s_flag, spin_limit)) break;
         // Block row k is final; the updates of block rows < k have been applied everywhere.
         if (k + 1 >= nbs) {                  // last factorised block row of a partial run: its update only
-            trailing_phase(k, k + 1, 0, 0);
+            chol_trailing_phase(A, Wm, n, ld, vec16, k, k + 1, row_limit, 0, 0);
             continue;
         }
         const int next_items = strip_items(k + 1) > 0 ? strip_items(k + 1) : 1;
@@ -660,20 +711,13 @@ chol_coop_kernel(double* __restrict__ A, double* __restrict__ Wm, double* __rest
         // strip up to date with block row k itself) and then join the trailing tiles of block row k below row k + 1 with
         // a share reduced by what their strips cost, so nobody idles and there is one grid barrier per block row.
         for (int g = blockIdx.x; g < next_items; g += G) {
-            double* P; int pc0; bool ident;
-            strip_item(k + 1, g, P, pc0, ident);
-            double* ua = opnd + 2 * kNB * kCholLd;        // beyond the strip's own panel buffers
-            double* ub = ua + kNB * kCholLd;
-            const bool need_b = P != nullptr && !ident;
+            double* P; int pc0;
+            strip_item(k + 1, g, P, pc0);
             __syncthreads();
-            chol_load_block(ua, A, ld, n, k * kNB, (k + 1) * kNB, 6, vec16);
-            if (need_b) chol_load_block(ub, P, ld, n, k * kNB, pc0, 6, vec16);
-            cp_async_commit();
-            chol_strip(A, ld, n, (k + 1) * kNB, P, pc0, ident, g == 0, Dbuf + (size_t)(k + 1) * kNB * kNB, opnd, vec16,
-                       status, ua, need_b ? ub : nullptr);
+            chol_strip(A, ld, n, (k + 1) * kNB, P, pc0, P == Wm, g == 0, Dbuf + (size_t)(k + 1) * kNB * kNB, vec16, status, true);
             __syncthreads();
         }
-        trailing_phase(k, k + 2, next_items % G, next_items / G);
+        chol_trailing_phase(A, Wm, n, ld, vec16, k, k + 2, row_limit, next_items % G, next_items / G);
     }
     cp_async_wait<0>();
     // the diagonal factors move from the side buffer into A once nobody reads the original diagonal blocks any more
@@ -721,7 +765,7 @@ inline int cholesky_upper(double* A, int n, double* Wm, double* Dbuf, unsigned* 
     // gets only as many CTAs as it ever has work items, which makes its grid barriers cheaper and leaves SMs to kernels
     // of other streams.
     const int nbr = (n + kNB - 1) / kNB;
-    const long items = (long)nbr * (nbr + 1) / 2 + (Wm != nullptr ? (long)nbr * nbr : 0);
+    const long items = 2L * ((long)nbr * (nbr + 1) / 2 + (Wm != nullptr ? (long)nbr * nbr : 0));
     const int budget = coop_cta_budget(dev);
     const int grid = items < budget ? (int)(items < 1 ? 1 : items) : budget;
     if (cudaMemsetAsync(bar, 0, 2 * sizeof(unsigned), stream) != cudaSuccess) return PTQ_ERR_CUDA;
