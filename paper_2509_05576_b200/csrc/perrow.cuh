@@ -95,13 +95,8 @@ __global__ void __launch_bounds__(kPerRowThreads, 3) per_row_kernel(const float*
     auto tile = [&](int r, int c) { return tiles + ((c * (c + 1) >> 1) + r) * 64; };       // r <= c
     const int i = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int lq = lane >> 2, lr = lane & 3;
-    RowGrid rg;
-    rg.sc = (double)scale[i];
-    rg.zp = (double)zero[i];
-    rg.rsc = 1.0 / rg.sc;
     const double maxq = (double)((1 << bits) - 1);
-    rg.lo = -rg.zp;
-    rg.hi = maxq - rg.zp;
+    const RowGrid rg = make_row_grid((double)scale[i], (double)zero[i], maxq);
 
     // 1. scores and order
     unsigned long long* key = reinterpret_cast<unsigned long long*>(dw);

@@ -268,6 +268,22 @@ def test_identity_inverse_hessian_gives_round_to_nearest():
         assert np.array_equal(What, (sc[:, None].astype(np.float64) * (v - zp[:, None])).astype(np.float32))
 
 
+@pytest.mark.parametrize("zero", [0.0, 7.0, -5.0, 300.0, 2.0e9])
+@pytest.mark.parametrize("bits", [3, 8])
+def test_rounding_step_clamps_for_any_zero_point(zero, bits):
+    """Levels below, inside and far beyond the code range, for zero-points inside and outside of it (identity: no
+    compensation, so every weight is quantized as it stands)."""
+    rng = np.random.Generator(np.random.PCG64(77))
+    W = (rng.standard_normal((33, 70)) * 3.0).astype(np.float32)
+    W[0, :6] = [1e12, -1e12, 0.5, -0.5, 1.5, 2.0e9]
+    W[1] = (np.arange(70) - 35).astype(np.float32) - np.float32(zero if abs(zero) < 1e6 else 0.0)
+    sc, zp = np.full(33, 0.25, np.float32), np.full(33, zero, np.float32)
+    sc[1] = 1.0
+    codes, _, _ = _sweep(W, np.eye(70), np.arange(70, dtype=np.int32), sc, zp, bits)
+    v = np.clip(np.rint(W.astype(np.float64) / sc[:, None].astype(np.float64)) + zp[:, None].astype(np.float64), 0, 2 ** bits - 1)
+    assert np.array_equal(codes, v.astype(np.uint8))
+
+
 def test_invalid_permutation_is_reported_not_followed():
     W, X = _layer(8, 64, 100, 601)
     Hinv, diag, _ = oracle.prepare_hinv(oracle.hessian_accumulate(X))
