@@ -227,7 +227,6 @@ size_t ptq_workspace_bytes(int call_id, int rows, int cols, int n) {
             add((size_t)rows * c * sizeof(double));         // permuted W (float64), later dW
             add((size_t)rows * c * sizeof(double));         // scaled errors E
             add((size_t)rows * c);                          // codes in permuted order
-            add(c * sizeof(int32_t));                       // flags
             add(c * sizeof(int32_t));                       // inverse permutation
             add(loss_partials_count(rows, cols) * sizeof(double));
             add(2 * sizeof(unsigned));                      // grid barrier of the factorisation kernel
@@ -334,10 +333,9 @@ int ptq_prepare_hinv(const double* H, int cols, int damp_mode, double damp, doub
     double* Dbuf = cv.take<double>(chol_scratch_doubles(n));
     void* pws = chol_panel_workspace_bytes(n) ? static_cast<void*>(cv.take<char>(chol_panel_workspace_bytes(n))) : nullptr;
     { Launch l(K_LAMBDA, stream); lambda_kernel<<<1, 256, 0, stream>>>(H, n, damp_mode, damp, lambda_out, status); }
-    { Launch l(K_DAMP_COPY, stream); damp_copy_kernel<<<dim3(grid_x_for(n, 256), n), 256, 0, stream>>>(H, R, n, lambda_out); }
+    { Launch l(K_DAMP_COPY, stream); damp_copy_kernel<<<dim3(grid_x_for(n, 256), n), 256, 0, stream>>>(H, R, V, n, lambda_out, bar); }
     // W = U^-T comes out of the factorisation sweep itself (V must start as zero)
-    if (cudaMemsetAsync(V, 0, (size_t)n * n * sizeof(double), stream) != cudaSuccess) return PTQ_ERR_CUDA;
-    int st = cholesky_upper_auto(R, n, V, Dbuf, bar, pws, status, stream);
+    int st = cholesky_upper_auto(R, n, V, Dbuf, bar, pws, status, stream, true);
     if (st) return st;
     if (n >= kSlicedMinCols && n <= kXMaxK && x_operand_bytes(n, n) <= (size_t)n * n * sizeof(double)) {
         // Hinv = W^T W on the int8 tensor path: the columns of the lower-triangular W are sliced once (into R, which is
@@ -345,15 +343,13 @@ int ptq_prepare_hinv(const double* H, int cols, int damp_mode, double damp, doub
         Carver rv(R);
         const XOperand w = x_slice_operand(rv, V, n, 1, n, n, stream);
         XGemmParams prm{};
-        prm.C = Hinv; prm.ldc = n; prm.alpha = 1.0; prm.status = status;
+        prm.C = Hinv; prm.ldc = n; prm.alpha = 1.0; prm.status = status; prm.diag = Hinv_diag;
         prm.out_mode = X_OUT_SYM; prm.k_mode = X_K_FROM_MAX;
         st = x_product(w, w, prm, stream);
     } else {
-        st = lauum_lower(V, Hinv, n, stream);
+        st = lauum_lower(V, Hinv, Hinv_diag, n, stream);
     }
-    if (st) return st;
-    { Launch l(K_EXTRACT_DIAG, stream); extract_diag_kernel<<<cdiv(n, 256), 256, 0, stream>>>(Hinv, n, Hinv_diag); }
-    return launch_status();
+    return st ? st : launch_status();
 }
 
 int ptq_minmax_grid(const float* W, int rows, int cols, int64_t ldw, int bits, float* scale, float* zero,
@@ -638,7 +634,6 @@ int ptq_quantize_layer(const float* W, int rows, int cols, int64_t ldw, const do
     double* Wp = cv.take<double>((size_t)rows * n);
     double* E = cv.take<double>((size_t)rows * n);
     uint8_t* codes_p = cv.take<uint8_t>((size_t)rows * n);
-    int32_t* flags = cv.take<int32_t>(n);
     int32_t* invperm = cv.take<int32_t>(n);
     double* partials = cv.take<double>(loss_partials_count(rows, cols));
     unsigned* bar = cv.take<unsigned>(2);
@@ -648,14 +643,14 @@ int ptq_quantize_layer(const float* W, int rows, int cols, int64_t ldw, const do
                     ? static_cast<void*>(cv.take<char>(i8gemm_workspace_bytes(rows, n, kSuperBlock))) : nullptr;
     void* pws = chol_panel_workspace_bytes(n) ? static_cast<void*>(cv.take<char>(chol_panel_workspace_bytes(n))) : nullptr;
 
-    // flags and invperm are adjacent pieces of the workspace: clear both
-    if (cudaMemsetAsync(flags, 0, (size_t)((char*)invperm - (char*)flags) + (size_t)n * sizeof(int32_t), stream) !=
-        cudaSuccess)
-        return PTQ_ERR_CUDA;
-    { Launch l(K_PERM_CHECK, stream); perm_check_kernel<<<cdiv(n, 256), 256, 0, stream>>>(perm, n, flags, invperm, status); }
-    { Launch l(K_GATHER_SYM, stream); gather_sym_kernel<<<dim3(grid_x_for(n, 256), n), 256, 0, stream>>>(Hinv, perm, n, U); }
-    { Launch l(K_GATHER_W, stream); gather_w_kernel<<<dim3(grid_x_for(n, 256), rows), 256, 0, stream>>>(W, rows, n, ldw, perm, Wp); }
-    int st = cholesky_upper_auto(U, n, nullptr, Dbuf, bar, pws, status, stream);   // blocked Eq. 12
+    const int n_flags = cdiv(rows, kSweepRows) + 1;
+    { Launch l(K_PERM_CHECK, stream); perm_check_kernel<<<cdiv(n, 256), 256, 0, stream>>>(perm, n, invperm, bar, sweep_flags, n_flags, status); }
+    {
+        Launch l(K_SWEEP_GATHER, stream);
+        const int gy = n + rows < kMaxGridY ? n + rows : kMaxGridY;
+        sweep_gather_kernel<<<dim3(grid_x_for(n, 256), gy), 256, 0, stream>>>(Hinv, W, rows, n, ldw, perm, invperm, U, Wp, E, status);
+    }
+    int st = cholesky_upper_auto(U, n, nullptr, Dbuf, bar, pws, status, stream, true);   // blocked Eq. 12
     if (st) return st;
 
     if (rows >= kSuperBlockMinRows && n >= 4 * kSuperBlock) {
@@ -666,7 +661,7 @@ int ptq_quantize_layer(const float* W, int rows, int cols, int64_t ldw, const do
         for (int off = 0; off < n; off += kSuperBlock) {
             const int sb = n - off < kSuperBlock ? n - off : kSuperBlock;
             st = sweep_launch(Wp + off, U + (size_t)off * n + off, E + off, codes_p + off, scale, zero, rows, sb, bits,
-                              sweep_flags, status, stream, n);
+                              sweep_flags, status, stream, n, true, off == 0);
             if (st) return st;
             if (off + sb < n) {
                 // W[:, later] -= E[:, sb] U[sb, later] on the int8 tensor path (i8gemm.cuh), float64-accurate
@@ -676,7 +671,7 @@ int ptq_quantize_layer(const float* W, int rows, int cols, int64_t ldw, const do
             }
         }
     } else {
-        st = sweep_launch(Wp, U, E, codes_p, scale, zero, rows, n, bits, sweep_flags, status, stream);
+        st = sweep_launch(Wp, U, E, codes_p, scale, zero, rows, n, bits, sweep_flags, status, stream, n, true, true);
         if (st) return st;
     }
 

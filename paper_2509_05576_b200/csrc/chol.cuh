@@ -32,14 +32,17 @@ __global__ void __launch_bounds__(256) lambda_kernel(const double* __restrict__ 
 }
 
 // A = H + lambda I, from each row's 64-column diagonal tile on (the factorisation reads the upper triangle only, whole
-// tiles on the diagonal); one grid row per matrix row.
-__global__ void damp_copy_kernel(const double* __restrict__ H, double* __restrict__ A, int n,
-                                 const double* __restrict__ lambda) {
+// tiles on the diagonal), and V = 0 (where the inverse of the factor will be built); one grid row per matrix row.  Also
+// clears the factorisation's grid barrier.
+__global__ void damp_copy_kernel(const double* __restrict__ H, double* __restrict__ A, double* __restrict__ V, int n,
+                                 const double* __restrict__ lambda, unsigned* __restrict__ bar) {
     const int i = blockIdx.y;
     const double lam = *lambda;
     const int64_t row = (int64_t)i * n;
-    for (int j = (i & ~(kNB - 1)) + blockIdx.x * blockDim.x + threadIdx.x; j < n; j += gridDim.x * blockDim.x)
-        A[row + j] = H[row + j] + (i == j ? lam : 0.0);
+    const int first = blockIdx.x * blockDim.x + threadIdx.x, step = gridDim.x * blockDim.x;
+    if (i == 0 && first < 2) bar[first] = 0u;
+    for (int j = (i & ~(kNB - 1)) + first; j < n; j += step) A[row + j] = H[row + j] + (j == i ? lam : 0.0);
+    for (int j = first; j < n; j += step) V[row + j] = 0.0;
 }
 
 // ------------------------------------------------------------------------------------------------------------
@@ -741,8 +744,10 @@ chol_coop_kernel(double* __restrict__ A, double* __restrict__ Wm, double* __rest
 inline size_t chol_scratch_doubles(int n) { return (size_t)((n + kNB - 1) / kNB) * kNB * kNB; }
 // nb_stop > 0: factorise the block rows k_first .. nb_stop - 1 only (see the kernel for what row_limit selects;
 // row_limit <= 0: all rows below are updated).  A partial run that updates everything below must not ask for Wm.
+// bar_ready: the caller has cleared `bar`.
 inline int cholesky_upper(double* A, int n, double* Wm, double* Dbuf, unsigned* bar, int32_t* status,
-                          cudaStream_t stream, int nb_stop = 0, int k_first = 0, int row_limit = 0) {
+                          cudaStream_t stream, int nb_stop = 0, int k_first = 0, int row_limit = 0,
+                          bool bar_ready = false) {
     const int nb_all = (n + kNB - 1) / kNB;
     if (nb_stop <= 0) nb_stop = nb_all;
     if (row_limit <= 0) row_limit = nb_all;
@@ -768,7 +773,7 @@ inline int cholesky_upper(double* A, int n, double* Wm, double* Dbuf, unsigned* 
     const long items = 2L * ((long)nbr * (nbr + 1) / 2 + (Wm != nullptr ? (long)nbr * nbr : 0));
     const int budget = coop_cta_budget(dev);
     const int grid = items < budget ? (int)(items < 1 ? 1 : items) : budget;
-    if (cudaMemsetAsync(bar, 0, 2 * sizeof(unsigned), stream) != cudaSuccess) return PTQ_ERR_CUDA;
+    if (!bar_ready && cudaMemsetAsync(bar, 0, 2 * sizeof(unsigned), stream) != cudaSuccess) return PTQ_ERR_CUDA;
     int64_t ld = n;
     int vec16 = ((n & 1) == 0 && aligned16(A) && aligned16(Wm)) ? 1 : 0;
     long long spin_limit = kSpinLimitCycles;
@@ -783,20 +788,15 @@ inline int cholesky_upper(double* A, int n, double* Wm, double* Dbuf, unsigned* 
 }
 
 // Hinv = W^T W for the lower-triangular W = U^-T: Hinv[i][j] = sum over k >= max(i, j) of W[k][i] W[k][j]; upper tiles
-// computed, mirrored below.
-inline int lauum_lower(const double* W, double* Hinv, int n, cudaStream_t stream) {
+// computed, mirrored below; its diagonal also goes to diag.
+inline int lauum_lower(const double* W, double* Hinv, double* diag, int n, cudaStream_t stream) {
     GemmParams g = gemm_defaults();
     g.A = W; g.lda = n; g.a_trans = 1;
     g.B = W; g.ldb = n; g.b_trans = 0;
-    g.C = Hinv; g.ldc = n;
+    g.C = Hinv; g.ldc = n; g.diag = diag;
     g.M = n; g.N = n; g.K = n;
     g.kbeg_mode = 1; g.upper_only = 1; g.mirror = 1;
     return launch_dgemm(K_DGEMM_LAUUM, g, 1, stream);
-}
-
-__global__ void extract_diag_kernel(const double* __restrict__ A, int n, double* __restrict__ d) {
-    const int j = blockIdx.x * blockDim.x + threadIdx.x;
-    if (j < n) d[j] = A[(int64_t)j * n + j];
 }
 
 }  // namespace ptq

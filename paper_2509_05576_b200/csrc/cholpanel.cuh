@@ -21,12 +21,12 @@ inline size_t chol_panel_workspace_bytes(int n) {
 
 // Same contract as cholesky_upper (whole factorisation); xws: chol_panel_workspace_bytes(n) bytes of scratch.
 inline int cholesky_upper_auto(double* A, int n, double* Wm, double* Dbuf, unsigned* bar, void* xws, int32_t* status,
-                               cudaStream_t stream) {
-    if (n < kPanelMinCols || xws == nullptr) return cholesky_upper(A, n, Wm, Dbuf, bar, status, stream);
+                               cudaStream_t stream, bool bar_ready) {
+    if (n < kPanelMinCols || xws == nullptr) return cholesky_upper(A, n, Wm, Dbuf, bar, status, stream, 0, 0, 0, bar_ready);
     const int nb = (n + kNB - 1) / kNB;
     for (int kf = 0; kf < nb; kf += kPanelBlocks) {
         const int pe = kf + kPanelBlocks < nb ? kf + kPanelBlocks : nb;
-        int st = cholesky_upper(A, n, Wm, Dbuf, bar, status, stream, pe, kf, pe);
+        int st = cholesky_upper(A, n, Wm, Dbuf, bar, status, stream, pe, kf, pe, bar_ready && kf == 0);
         if (st) return st;
         if (pe >= nb) break;
         const int r0 = kf * kNB, c0 = pe * kNB;               // panel rows r0 .. c0 - 1, everything from c0 on is below it

@@ -14,36 +14,49 @@
 
 namespace ptq {
 
-// flags[] must be zero on entry.  Reports out-of-range or repeated entries; invperm[perm[p]] = p.
-__global__ void perm_check_kernel(const int32_t* __restrict__ perm, int cols, int32_t* __restrict__ flags,
-                                  int32_t* __restrict__ invperm, int32_t* status) {
-    const int p = blockIdx.x * blockDim.x + threadIdx.x;
+__device__ __forceinline__ int clamp_index(int j, int n) { return j < 0 ? 0 : (j >= n ? n - 1 : j); }
+
+// invperm[perm[p]] = p; reports entries out of range.  A repeated entry shows once all of invperm is written, see
+// sweep_gather_kernel.  Also clears the counters of the kernels to come (zero: `zeros` words).
+__global__ void __launch_bounds__(256) perm_check_kernel(const int32_t* __restrict__ perm, int cols,
+                                                          int32_t* __restrict__ invperm, unsigned* __restrict__ bar,
+                                                          unsigned* __restrict__ sweep_flags, int n_flags, int32_t* status) {
+    const int p = blockIdx.x * 256 + threadIdx.x;
+    if (p < 2) bar[p] = 0u;
+    for (int f = p; f < n_flags; f += gridDim.x * 256) sweep_flags[f] = 0u;
     if (p >= cols) return;
     const int j = perm[p];
     if (j < 0 || j >= cols) { report(status, PTQ_ERR_INVALID_ARG, p, 1); return; }
-    if (atomicExch(&flags[j], 1) != 0) { report(status, PTQ_ERR_INVALID_ARG, p, 2); return; }
     invperm[j] = p;
 }
 
-__device__ __forceinline__ int clamp_index(int j, int n) { return j < 0 ? 0 : (j >= n ? n - 1 : j); }
-
-// A[a][b] = Hinv[perm[a]][perm[b]] for b from the start of row a's 64-column diagonal tile on: the factorisation and
-// everything after it read the upper triangle only (whole 64 x 64 tiles on the diagonal), the rest of A is left alone.
-__global__ void gather_sym_kernel(const double* __restrict__ Hinv, const int32_t* __restrict__ perm, int n,
-                                  double* __restrict__ A) {
-    const int a = blockIdx.y;
-    const int b_first = a & ~(kNB - 1);
-    const int64_t src = (int64_t)clamp_index(perm[a], n) * n;
-    for (int b = b_first + blockIdx.x * blockDim.x + threadIdx.x; b < n; b += gridDim.x * blockDim.x)
-        A[(int64_t)a * n + b] = Hinv[src + clamp_index(perm[b], n)];
-}
-
-// Wp[i][p] = (double) W[i][perm[p]]
-__global__ void gather_w_kernel(const float* __restrict__ W, int rows, int cols, int64_t ldw,
-                                const int32_t* __restrict__ perm, double* __restrict__ Wp) {
-    const int i = blockIdx.y;
-    for (int p = blockIdx.x * blockDim.x + threadIdx.x; p < cols; p += gridDim.x * blockDim.x)
-        Wp[(int64_t)i * cols + p] = (double)W[(int64_t)i * ldw + clamp_index(perm[p], cols)];
+// Everything the sweep starts from, one grid row per row of the matrix and then of the weights:
+//   A[a][b] = Hinv[perm[a]][perm[b]] for b from the start of row a's 64-column diagonal tile on: the factorisation and
+//   everything after it read the upper triangle only (whole 64 x 64 tiles on the diagonal), the rest of A is left alone;
+//   Wp[i][p] = (double) W[i][perm[p]];  E[i][p] = NaN, "not published yet" for the owners of the next blocks, which poll
+//   the values themselves.
+// A position whose column some other position also names (invperm points elsewhere) is reported.
+// One launch in place of three kernels' and clears' worth of them: they are short and a launch takes about as long.
+__global__ void __launch_bounds__(256) sweep_gather_kernel(const double* __restrict__ Hinv, const float* __restrict__ W, int rows,
+                                                            int n, int64_t ldw, const int32_t* __restrict__ perm,
+                                                            const int32_t* __restrict__ invperm, double* __restrict__ A,
+                                                            double* __restrict__ Wp, double* __restrict__ E, int32_t* status) {
+    const int step = gridDim.x * 256, first = blockIdx.x * 256 + threadIdx.x;
+    const int total = n + rows;
+    for (int y = blockIdx.y; y < total; y += gridDim.y) {
+        if (y < n) {
+            const int src_row = perm[y];
+            if (first == 0 && src_row >= 0 && src_row < n && invperm[src_row] != y) report(status, PTQ_ERR_INVALID_ARG, y, 2);
+            const int64_t src = (int64_t)clamp_index(src_row, n) * n;
+            for (int b = (y & ~(kNB - 1)) + first; b < n; b += step) A[(int64_t)y * n + b] = Hinv[src + clamp_index(perm[b], n)];
+        } else {
+            const int i = y - n;
+            for (int q = first; q < n; q += step) {
+                Wp[(int64_t)i * n + q] = (double)W[(int64_t)i * ldw + clamp_index(perm[q], n)];
+                E[(int64_t)i * n + q] = __longlong_as_double(-1ll);
+            }
+        }
+    }
 }
 
 // ------------------------------------------------------------------------------------------------------------
@@ -556,9 +569,10 @@ __global__ void __launch_bounds__(kSweepThreads, 1) sweep_coop_kernel(SweepParam
 // Launches the sweep: one CTA per SM, cooperative so that every CTA a waiting CTA depends on is resident.
 // n columns are swept; ld (0: n) is the row stride of Wp, U, E and codes_p, so that the first n columns of wider
 // arrays can be swept (the rows of U beyond column n are then applied by the caller).
+// e_ready, flags_ready: the caller has set E to NaN and the progress counters to zero.
 inline int sweep_launch(double* Wp, const double* U, double* E, uint8_t* codes_p, const float* scale, const float* zero,
                         int rows, int n, int bits, unsigned* flags, int32_t* status, cudaStream_t stream,
-                        int64_t ld = 0) {
+                        int64_t ld = 0, bool e_ready = false, bool flags_ready = false) {
     if (ld == 0) ld = n;
     DeviceState* dev = nullptr;
     int st = current_device_state(&dev);
@@ -581,9 +595,10 @@ inline int sweep_launch(double* Wp, const double* U, double* E, uint8_t* codes_p
         grid = groups_l * per;
     }
     const int groups = cdiv(rows, kSweepRows);
-    if (cudaMemsetAsync(flags, 0, ((size_t)groups + 1) * sizeof(unsigned), stream) != cudaSuccess) return PTQ_ERR_CUDA;
+    if (!flags_ready && cudaMemsetAsync(flags, 0, ((size_t)groups + 1) * sizeof(unsigned), stream) != cudaSuccess)
+        return PTQ_ERR_CUDA;
     // every byte 0xFF is a NaN: "not published yet" for the owner of the next block, which polls the values themselves
-    if (cudaMemset2DAsync(E, (size_t)ld * sizeof(double), 0xFF, (size_t)n * sizeof(double), (size_t)rows, stream) !=
+    if (!e_ready && cudaMemset2DAsync(E, (size_t)ld * sizeof(double), 0xFF, (size_t)n * sizeof(double), (size_t)rows, stream) !=
         cudaSuccess)
         return PTQ_ERR_CUDA;
     SweepParams prm;
@@ -609,7 +624,7 @@ __global__ void finalize_kernel(const uint8_t* __restrict__ codes_p, const int32
     const int i = blockIdx.y;
     const double sc = (double)scale[i], zp = (double)zero[i];
     for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < cols; j += gridDim.x * blockDim.x) {
-        const uint8_t c = codes_p[(int64_t)i * cols + invperm[j]];
+        const uint8_t c = codes_p[(int64_t)i * cols + clamp_index(invperm[j], cols)];
         codes[(int64_t)i * cols + j] = c;
         const float q = (float)(sc * ((double)c - zp));
         if (What) What[(int64_t)i * cols + j] = q;

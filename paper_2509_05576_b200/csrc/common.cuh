@@ -140,8 +140,8 @@ inline int ensure_smem_attr(DeviceState* d, SmemAttrSlot slot, F set) {
 // ---------------------------------------------------------------------------------------------------------
 enum KernelId {
     K_GRAM_SPLIT = 0, K_GRAM_I8, K_GRAM_FINISH, K_CONVERT_F64, K_DGEMM_GRAM, K_LAMBDA, K_DAMP_COPY, K_CHOL_COOP,
-    K_DGEMM_LAUUM, K_EXTRACT_DIAG, K_MINMAX_GRID, K_SCORE_PARTIAL,
-    K_SCORE_FINAL, K_RANK_SORT, K_PERM_CHECK, K_GATHER_SYM, K_GATHER_W, K_SWEEP_COOP, K_FINALIZE,
+    K_DGEMM_LAUUM, K_MINMAX_GRID, K_SCORE_PARTIAL,
+    K_SCORE_FINAL, K_RANK_SORT, K_PERM_CHECK, K_SWEEP_GATHER, K_SWEEP_COOP, K_FINALIZE,
     K_DGEMM_LOSS, K_SUM_PARTIALS, K_SELFTEST, K_FP64_PROBE, K_DYN_AUX, K_DYN_GATHER,
     K_DGEMM_DYN, K_PER_ROW, K_DGEMM_EQ11, K_X_SLICE, K_X_GEMM, K_COUNT
 };
@@ -149,8 +149,8 @@ enum KernelId {
 inline const char* kernel_name(int id) {
     static const char* names[K_COUNT] = {
         "gram_split", "gram_i8_tcgen05", "gram_finish", "convert_f64", "dgemm_gram_f64", "lambda", "damp_copy", "chol_coop",
-        "dgemm_lauum", "extract_diag",
-        "minmax_grid", "score_partial", "score_final", "rank_sort", "perm_check", "gather_sym", "gather_w",
+        "dgemm_lauum",
+        "minmax_grid", "score_partial", "score_final", "rank_sort", "perm_check", "sweep_gather",
         "sweep_coop", "finalize", "dgemm_loss", "sum_partials", "selftest_wait", "fp64_probe", "dyn_aux", "dyn_gather",
         "dgemm_dyn", "per_row", "dgemm_eq11", "x_slice", "i8gemm_tcgen05"};
     return (id >= 0 && id < K_COUNT) ? names[id] : "unknown";

@@ -12,6 +12,7 @@ struct GemmParams {
     const double* A;   // a_trans == 0: A[i * lda + k]   a_trans == 1: A[k * lda + i]
     const double* B;   // b_trans == 0: B[k * ldb + j]   b_trans == 1: B[j * ldb + k]
     double* C;         // C[i * ldc + j] = alpha * sum_k A B + beta * C
+    double* diag;      // not null: diag[i] = C[i][i] as well
     int64_t lda, ldb, ldc;
     int M, N, K;
     int a_trans, b_trans;
@@ -260,6 +261,7 @@ __device__ __forceinline__ void dgemm_tile(const GemmParams& p, int bx, int by, 
                 if (p.beta != 0.0) v = fma(p.beta, C[(int64_t)gi * p.ldc + gj], v);
                 C[(int64_t)gi * p.ldc + gj] = v;
                 if (do_mirror) C[(int64_t)gj * p.ldc + gi] = v;
+                if (p.diag != nullptr && gi == gj) p.diag[gi] = v;
             }
     }
 }

@@ -79,7 +79,12 @@ struct GramSource {
 // ------------------------------------------------------------------------------------------------------------
 __global__ void __launch_bounds__(256) gram_split_conv_kernel(GramSource src, int cols, int n, int cols_pad, int n_pad,
                                                                int8_t* __restrict__ Q, int32_t* __restrict__ shifts,
-                                                               int32_t* status);
+                                                               int32_t* status, ulonglong2* __restrict__ iacc, int n_iacc);
+
+// The slicing pass also clears the workspace in which the products of tiles cut along K meet (n_iacc 16-byte words).
+__device__ __forceinline__ void gram_clear_iacc(ulonglong2* __restrict__ iacc, int n_iacc) {
+    for (int i = blockIdx.x * 256 + threadIdx.x; i < n_iacc; i += gridDim.x * 256) iacc[i] = make_ulonglong2(0ull, 0ull);
+}
 
 __device__ __forceinline__ void gram_pack4(const long long (&v)[4], uint32_t (&packed)[kSlices]) {
 #pragma unroll
@@ -99,9 +104,10 @@ __device__ __forceinline__ void gram_pack4(const long long (&v)[4], uint32_t (&p
 __global__ void __launch_bounds__(256) gram_split_kernel(const float* __restrict__ X, int cols, int n, int64_t ldx,
                                                           int cols_pad, int n_pad, int vec_ok,
                                                           int8_t* __restrict__ Q, int32_t* __restrict__ shifts,
-                                                          int32_t* status) {
+                                                          int32_t* status, ulonglong2* __restrict__ iacc, int n_iacc) {
     __shared__ float smax[256];
     __shared__ int sbad;
+    gram_clear_iacc(iacc, n_iacc);
     const int row = blockIdx.x;
     const size_t plane = (size_t)cols_pad * n_pad;
     int8_t* q0 = Q + (size_t)row * n_pad;
@@ -178,9 +184,10 @@ __device__ __forceinline__ float conv_fetch(const GramSource& s, const float* __
 
 __global__ void __launch_bounds__(256) gram_split_conv_kernel(GramSource src, int cols, int n, int cols_pad, int n_pad,
                                                                int8_t* __restrict__ Q, int32_t* __restrict__ shifts,
-                                                               int32_t* status) {
+                                                               int32_t* status, ulonglong2* __restrict__ iacc, int n_iacc) {
     __shared__ float smax[256];
     __shared__ int sbad;
+    gram_clear_iacc(iacc, n_iacc);
     const int row = blockIdx.x;
     const size_t plane = (size_t)cols_pad * n_pad;
     int8_t* q0 = Q + (size_t)row * n_pad;
@@ -627,22 +634,6 @@ inline int gram_accumulate(double* H, GramSource src, int cols, int n, void* ws,
     for (int c0 = 0; c0 < n; c0 += kGramMaxChunk) {
         const int nc = n - c0 < kGramMaxChunk ? n - c0 : kGramMaxChunk;
         const int n_pad = cdiv(nc, 128) * 128;
-        {
-            Launch l(K_GRAM_SPLIT, stream);
-            if (src.conv) {
-                src.col0 = c0;
-                gram_split_conv_kernel<<<cols_pad, 256, 0, stream>>>(src, cols, nc, cols_pad, n_pad, Q, shifts, status);
-            } else {
-                const int vec_ok = (aligned16(src.base) && (src.ldx & 3) == 0) ? 1 : 0;
-                gram_split_kernel<<<cols_pad, 256, 0, stream>>>(src.base + c0, cols, nc, src.ldx, cols_pad, n_pad, vec_ok,
-                                                                Q, shifts, status);
-            }
-        }
-        CUtensorMap mapA, mapB;
-        int st = make_slice_map(&mapA, Q, cols_pad, n_pad, kGramTM);
-        if (st) return st;
-        st = make_slice_map(&mapB, Q, cols_pad, n_pad, kGramTN);
-        if (st) return st;
         // The tiles of the last, partly filled wave (all tiles of a narrow matrix) are cut along K so that every SM
         // gets a work item of about the same length.
         const int nkb = n_pad / kGramKB;
@@ -656,9 +647,25 @@ inline int gram_accumulate(double* H, GramSource src, int cols, int n, void* ws,
             if (ksplit > 1) n_full = num_tiles - rem;
         }
         const int sliced = num_tiles - n_full;
-        if (sliced > 0 &&
-            cudaMemsetAsync(iacc, 0, (size_t)sliced * kGramTileAccWords * sizeof(unsigned long long), stream) != cudaSuccess)
-            return PTQ_ERR_CUDA;
+        ulonglong2* clr = reinterpret_cast<ulonglong2*>(iacc);
+        const int n_clr = (int)((size_t)sliced * kGramTileAccWords / 2);
+        {
+            Launch l(K_GRAM_SPLIT, stream);
+            if (src.conv) {
+                src.col0 = c0;
+                gram_split_conv_kernel<<<cols_pad, 256, 0, stream>>>(src, cols, nc, cols_pad, n_pad, Q, shifts, status,
+                                                                     clr, n_clr);
+            } else {
+                const int vec_ok = (aligned16(src.base) && (src.ldx & 3) == 0) ? 1 : 0;
+                gram_split_kernel<<<cols_pad, 256, 0, stream>>>(src.base + c0, cols, nc, src.ldx, cols_pad, n_pad, vec_ok,
+                                                                Q, shifts, status, clr, n_clr);
+            }
+        }
+        CUtensorMap mapA, mapB;
+        int st = make_slice_map(&mapA, Q, cols_pad, n_pad, kGramTM);
+        if (st) return st;
+        st = make_slice_map(&mapB, Q, cols_pad, n_pad, kGramTN);
+        if (st) return st;
         const int items = n_full + sliced * ksplit;
         const int grid = items < num_sms ? items : num_sms;
         {

@@ -200,6 +200,7 @@ struct XGemmParams {
     const double* D;        // X_OUT_REDUCE: [m x n], row stride ldd
     int64_t ldd;
     double* partials;       // X_OUT_REDUCE: one per tile (0 for tiles without work)
+    double* diag;           // X_OUT_SYM: diag[i] = C[i][i] as well, unless null
 };
 
 // K blocks [kb0, kb1) of tile (bi, bj); an empty range or a tile below the diagonal (X_OUT_SYM) has no work at all.
@@ -412,6 +413,7 @@ i8gemm_kernel(const __grid_constant__ CUtensorMap tmapA, const __grid_constant__
                         if (col < prm.n) {
                             const double fj = __longlong_as_double((long long)(1023 + 24 - prm.sh_b[col]) << 52);
                             prm.C[(int64_t)col * prm.ldc + row] = (v[c] * fi) * fj;
+                            if (col == row && prm.diag != nullptr) prm.diag[row] = (v[c] * fi) * fj;
                         }
                     }
                 }

@@ -300,6 +300,21 @@ def test_invalid_permutation_is_reported_not_followed():
     assert ei.value.code == ptq.ERR_INVALID_ARG
 
 
+def test_a_repeated_column_is_reported():
+    W, X = _layer(8, 300, 400, 602)
+    Hinv, diag, _ = oracle.prepare_hinv(oracle.hessian_accumulate(X))
+    sc, zp = oracle.minmax_grid(W, 4)
+    perm = np.arange(300, dtype=np.int32)
+    perm[299] = 0                    # column 299 is missing, column 0 is named twice
+    codes = torch.empty((8, 300), dtype=torch.uint8, device="cuda")
+    st, ws = ptq.new_status(), ptq.Workspace()
+    ptq.quantize_layer(_cuda(W), _cuda(Hinv), _cuda(perm), _cuda(sc), _cuda(zp), 4, codes, None, None, None, ws, st)
+    torch.cuda.synchronize()
+    with pytest.raises(ptq.PtqError) as ei:
+        ptq.check_status(st)
+    assert ei.value.code == ptq.ERR_INVALID_ARG
+
+
 # ------------------------------------------------------------------------------------------ whole path
 @pytest.mark.parametrize("rows,cols,n,bits,xdist", [
     (64, 128, 1024, 4, "halfnormal"),
