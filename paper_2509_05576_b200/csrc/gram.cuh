@@ -86,20 +86,42 @@ __device__ __forceinline__ void gram_clear_iacc(ulonglong2* __restrict__ iacc, i
     for (int i = blockIdx.x * 256 + threadIdx.x; i < n_iacc; i += gridDim.x * 256) iacc[i] = make_ulonglong2(0ull, 0ull);
 }
 
-__device__ __forceinline__ void gram_pack4(const long long (&v)[4], uint32_t (&packed)[kSlices]) {
-#pragma unroll
-    for (int s = 0; s < kSlices; ++s) packed[s] = 0u;
+// The balanced base-256 digits of v, least significant first, as bytes: with 128 added at every digit the bytes of the sum
+// are the digits plus 128, which is what flipping each byte's top bit takes off again.  (|v| < 2^(8 N - 1).)  The slicing
+// passes were bound by cutting the digits off one by one in 64-bit arithmetic: Hessian of 2304 x 4096 252 -> 232 us, of
+// 4608 x 8192 1.24 -> 1.20 ms with this.
+template <int N>
+__device__ __forceinline__ unsigned long long balanced_digits(long long v) {
+    constexpr unsigned long long bias = 0x8080808080808080ull >> (64 - 8 * N);
+    return ((unsigned long long)v + bias) ^ bias;
+}
+// Digits of four consecutive values, one word per slice (most significant slice first).
+template <int N>
+__device__ __forceinline__ void pack_digits4(const long long (&v)[4], uint32_t (&packed)[N]) {
+    uint32_t lo[4], hi[4];
 #pragma unroll
     for (int u = 0; u < 4; ++u) {
-        long long t = v[u];
-#pragma unroll
-        for (int s = kSlices - 1; s >= 0; --s) {          // least significant digit first
-            const long long d = ((t + 128) & 255) - 128;  // balanced digit in [-128, 127]
-            t = (t - d) >> 8;
-            packed[s] |= ((uint32_t)(d & 255)) << (8 * u);
-        }
+        const unsigned long long d = balanced_digits<N>(v[u]);
+        lo[u] = (uint32_t)d;
+        hi[u] = (uint32_t)(d >> 32);
     }
+    // 4 x 4 byte transposes of the low and of the high words
+    auto transpose = [](const uint32_t (&w)[4], uint32_t (&t)[4]) {
+        const uint32_t a = __byte_perm(w[0], w[1], 0x5140), b = __byte_perm(w[2], w[3], 0x5140);
+        const uint32_t c = __byte_perm(w[0], w[1], 0x7362), e = __byte_perm(w[2], w[3], 0x7362);
+        t[0] = __byte_perm(a, b, 0x5410);
+        t[1] = __byte_perm(a, b, 0x7632);
+        t[2] = __byte_perm(c, e, 0x5410);
+        t[3] = __byte_perm(c, e, 0x7632);
+    };
+    uint32_t tl[4], th[4];
+    transpose(lo, tl);
+    transpose(hi, th);
+#pragma unroll
+    for (int s = 0; s < N; ++s) packed[N - 1 - s] = s < 4 ? tl[s & 3] : th[s & 3];
 }
+// 2^sh, |sh| <= 1000.
+__device__ __forceinline__ double power_of_two(int sh) { return __longlong_as_double((long long)(1023 + sh) << 52); }
 
 __global__ void __launch_bounds__(256) gram_split_kernel(const float* __restrict__ X, int cols, int n, int64_t ldx,
                                                           int cols_pad, int n_pad, int vec_ok,
@@ -145,16 +167,21 @@ __global__ void __launch_bounds__(256) gram_split_kernel(const float* __restrict
     int sh = 0;
     if (rowmax > 0.f && !rowbad) sh = kShiftTarget - (ilogbf(rowmax) + 1);   // |x| 2^sh < 2^46
     if (threadIdx.x == 0) shifts[row] = sh;
+    const double scale = power_of_two(sh);
     for (int k = threadIdx.x * 4; k < n_pad; k += 1024) {
         long long v[4];
+        float xv[4];
+        if (vec_ok && k + 3 < n) {
+            const float4 q = *reinterpret_cast<const float4*>(x + k);
+            xv[0] = q.x; xv[1] = q.y; xv[2] = q.z; xv[3] = q.w;
+        } else {
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            const int kk = k + u;
-            const float xv = (kk < n && !rowbad) ? x[kk] : 0.f;
-            v[u] = __double2ll_rn(scalbn((double)xv, sh));
+            for (int u = 0; u < 4; ++u) xv[u] = k + u < n ? x[k + u] : 0.f;
         }
+#pragma unroll
+        for (int u = 0; u < 4; ++u) v[u] = rowbad ? 0ll : __double2ll_rn((double)xv[u] * scale);
         uint32_t packed[kSlices];
-        gram_pack4(v, packed);
+        pack_digits4<kSlices>(v, packed);
 #pragma unroll
         for (int s = 0; s < kSlices; ++s) *reinterpret_cast<uint32_t*>(q0 + s * plane + k) = packed[s];
     }
@@ -229,6 +256,7 @@ __global__ void __launch_bounds__(256) gram_split_conv_kernel(GramSource src, in
     int sh = 0;
     if (rowmax > 0.f && !rowbad) sh = kShiftTarget - (ilogbf(rowmax) + 1);   // |x| 2^sh < 2^46
     if (threadIdx.x == 0) shifts[row] = sh;
+    const double scale = power_of_two(sh);
     for (int k = threadIdx.x * 4; k < n_pad; k += 1024) {
         long long v[4];
         ConvCursor cur;
@@ -236,11 +264,11 @@ __global__ void __launch_bounds__(256) gram_split_conv_kernel(GramSource src, in
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
             const float xv = (k + u < n && !rowbad) ? conv_fetch(src, plane0, cur, ki, kj) : 0.f;
-            v[u] = __double2ll_rn(scalbn((double)xv, sh));
+            v[u] = __double2ll_rn((double)xv * scale);
             cur.next(src);
         }
         uint32_t packed[kSlices];
-        gram_pack4(v, packed);
+        pack_digits4<kSlices>(v, packed);
 #pragma unroll
         for (int s = 0; s < kSlices; ++s) *reinterpret_cast<uint32_t*>(q0 + s * plane + k) = packed[s];
     }

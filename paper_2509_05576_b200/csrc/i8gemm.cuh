@@ -45,20 +45,6 @@ inline size_t i8gemm_workspace_bytes(int m, int n, int k) {
 }
 // Output / K-range modes and the slicing of one operand at a time: see XGemmParams, x_slice_operand, x_product below.
 
-__device__ __forceinline__ void x_pack4(const long long (&v)[4], uint32_t (&packed)[kXSlices]) {
-#pragma unroll
-    for (int s = 0; s < kXSlices; ++s) packed[s] = 0u;
-#pragma unroll
-    for (int u = 0; u < 4; ++u) {
-        long long t = v[u];
-#pragma unroll
-        for (int s = kXSlices - 1; s >= 0; --s) {         // least significant digit first
-            const long long d = ((t + 128) & 255) - 128;  // balanced digit in [-128, 127]
-            t = (t - d) >> 8;
-            packed[s] |= ((uint32_t)(d & 255)) << (8 * u);
-        }
-    }
-}
 // Shift of a row whose largest magnitude is m: |x| 2^sh < 2^54 (0 for an all-zero or non-finite row).
 __device__ __forceinline__ int x_row_shift(double m) {
     if (!(m > 0.0) || !(m < 1.0e300)) return 0;
@@ -93,15 +79,16 @@ __global__ void __launch_bounds__(256) x_slice_rows_kernel(const double* __restr
     const int sh = x_row_shift(smax[0]);
     const bool dead = sh == 0 && !(smax[0] > 0.0 && smax[0] < 1.0e300);
     if (threadIdx.x == 0) shifts[row] = sh;
+    const double scale = power_of_two(sh);
     for (int kk = threadIdx.x * 4; kk < k_pad; kk += 1024) {
         long long v[4];
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
             const double xv = (kk + u < k && !dead) ? x[kk + u] : 0.0;
-            v[u] = __double2ll_rn(scalbn(xv, sh));
+            v[u] = __double2ll_rn(xv * scale);
         }
         uint32_t packed[kXSlices];
-        x_pack4(v, packed);
+        pack_digits4<kXSlices>(v, packed);
 #pragma unroll
         for (int s = 0; s < kXSlices; ++s) *reinterpret_cast<uint32_t*>(q0 + s * plane + kk) = packed[s];
     }
@@ -150,6 +137,7 @@ __global__ void __launch_bounds__(256) x_slice_cols_kernel(const double* __restr
     const bool dead = !(mm > 0.0 && mm < 1.0e300);
     const int sh = dead ? 0 : x_row_shift(mm);
     if (blockIdx.y == 0 && wy == 0 && col < cols_pad) shifts[col] = sh;
+    const double scale = power_of_two(sh);
     const int kend = kbeg + kXColChunk < k_pad ? kbeg + kXColChunk : k_pad;
     for (int k0 = kbeg; k0 < kend; k0 += 32) {
         // thread (wy, lane): rows k0 + wy, + 8, + 16, + 24 of column `col`
@@ -157,13 +145,9 @@ __global__ void __launch_bounds__(256) x_slice_cols_kernel(const double* __restr
         for (int r = 0; r < 4; ++r) {
             const int kk = k0 + wy + 8 * r;
             const double xv = (!dead && kk < k) ? X[(int64_t)kk * ld + col] : 0.0;
-            long long t = __double2ll_rn(scalbn(xv, sh));
+            const unsigned long long d = balanced_digits<kXSlices>(__double2ll_rn(xv * scale));
 #pragma unroll
-            for (int s = kXSlices - 1; s >= 0; --s) {
-                const long long d = ((t + 128) & 255) - 128;
-                t = (t - d) >> 8;
-                dig[s][lane][wy + 8 * r] = (uint8_t)(d & 255);
-            }
+            for (int s = 0; s < kXSlices; ++s) dig[kXSlices - 1 - s][lane][wy + 8 * r] = (uint8_t)(d >> (8 * s));
         }
         __syncthreads();
         // out: for every slice and column, 32 consecutive bytes; thread -> (column = threadIdx / 8, 4 bytes = threadIdx % 8)
