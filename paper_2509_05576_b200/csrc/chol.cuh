@@ -213,9 +213,12 @@ template <int RB>
 __device__ __forceinline__ void chol_strip_lookahead(double (&acc)[8][2], const double* ua, const double* bsrc, int grp,
                                                      int lq, int lr) {
     if (grp < 8 && RB > grp) return;            // fragments that lie entirely below the diagonal are never used
+    // summed apart and subtracted once: added one by one to the old value they would be rounded to its size sixteen times
+    double p0 = 0.0, p1 = 0.0;
 #pragma unroll 8
-    for (int kk = 0; kk < kNB; kk += 4)
-        dmma_884(acc[RB][0], acc[RB][1], flip_sign(ua[(kk + lr) * kCholLd + 8 * RB + lq]), bsrc[(kk + lr) * kCholLd + lq]);
+    for (int kk = 0; kk < kNB; kk += 4) dmma_884(p0, p1, ua[(kk + lr) * kCholLd + 8 * RB + lq], bsrc[(kk + lr) * kCholLd + lq]);
+    acc[RB][0] -= p0;
+    acc[RB][1] -= p1;
 }
 
 // Step 1 above.  mb: the mini-block M (row-major, 8 x 8, upper part); leaves W in Wbuf.  Returns the first pivot that is not
@@ -575,9 +578,9 @@ __device__ __noinline__ void chol_trailing_phase(double* __restrict__ A, double*
     };
     // Operand blocks: a slot of abuf holds U[k][i-block] (as[kk][r]), a slot of bbuf U or W [k][j-block] (bs[kk][c]).
     // Every CTA takes a contiguous run of the list, in which consecutive tiles mostly share their row block: the A
-    // operand then stays where it is and only B is fetched.  What the next piece needs, its operands and its old
-    // values, is requested at the start of this one, and the products go straight into the old values (one operand's
-    // sign flipped): subtractions afterwards would queue behind the other warps' MMAs.  One barrier per piece.
+    // operand then stays where it is and only B is fetched.  The next piece's operands and this one's old values are
+    // requested at the start of the piece; the products are summed apart and subtracted from the old values once (added one
+    // by one to them they would be rounded to their size sixteen times).  One barrier per piece.
     double* abuf = reinterpret_cast<double*>(chol_smem_raw);      // [2][64][kCholLd]
     double* bbuf = abuf + 2 * kCholBlock;                         // [2][64][kCholLd]
     auto run = [&](auto height) {
@@ -590,19 +593,11 @@ __device__ __noinline__ void chol_trailing_phase(double* __restrict__ A, double*
         CholPiece cur = piece_of(tp_beg), nxt = cur;
         chol_load_block<kCholThreads>(abuf, A, ld, n, k0, cur.i0, LGH, vec16, tid);
         chol_load_block<kCholThreads>(bbuf, cur.Bsrc, ld, n, k0, cur.j0, 6, vec16, tid);
-        double2 acc[FM][FN], old[FM][FN];
-        bool plain = chol_piece_plain<H>(cur, n, vec16);
-#pragma unroll
-        for (int a = 0; a < FM; ++a)
-#pragma unroll
-            for (int b = 0; b < FN; ++b)
-                acc[a][b] = chol_pair_load(cur, cur.C + (int64_t)(cur.i0 + pr + 8 * a) * ld + cur.j0 + pq + 8 * b, n,
-                                           pr + 8 * a, pq + 8 * b, plain, vec16);
         cp_async_commit();
         for (int tp = tp_beg; tp < tp_end; ++tp) {
             const bool more = tp + 1 < tp_end;
             if (more) nxt = piece_of(tp + 1);
-            const bool new_a = more && nxt.i0 != cur.i0, plain_n = chol_piece_plain<H>(nxt, n, vec16);
+            const bool new_a = more && nxt.i0 != cur.i0, plain = chol_piece_plain<H>(cur, n, vec16);
             const int a_next = a_slot ^ (new_a ? 1 : 0);
             const double* as = abuf + a_slot * kCholBlock;
             const double* bs = bbuf + stage * kCholBlock;
@@ -616,20 +611,23 @@ __device__ __noinline__ void chol_trailing_phase(double* __restrict__ A, double*
                     if (new_a)
                         chol_load_block<kCholThreads / 2>(abuf + a_next * kCholBlock, A, ld, n, k0, nxt.i0, LGH, vec16, tid);
                 }
-#pragma unroll
-                for (int a = 0; a < FM; ++a)
-#pragma unroll
-                    for (int b = 0; b < FN; ++b)
-                        old[a][b] = chol_pair_load(nxt, nxt.C + (int64_t)(nxt.i0 + pr + 8 * a) * ld + nxt.j0 + pq + 8 * b,
-                                                   n, pr + 8 * a, pq + 8 * b, plain_n, vec16);
             }
+            double2 acc[FM][FN], old[FM][FN];
+#pragma unroll
+            for (int a = 0; a < FM; ++a)
+#pragma unroll
+                for (int b = 0; b < FN; ++b) {
+                    old[a][b] = chol_pair_load(cur, cur.C + (int64_t)(cur.i0 + pr + 8 * a) * ld + cur.j0 + pq + 8 * b, n,
+                                               pr + 8 * a, pq + 8 * b, plain, vec16);
+                    acc[a][b] = make_double2(0.0, 0.0);
+                }
 #pragma unroll 4
             for (int kk = lr; kk < kNB; kk += 4) {
                 double af[FM], bf[FN];
 #pragma unroll
                 for (int a = 0; a < FM; ++a) af[a] = as[kk * kCholLd + wm0 + a * 8 + lq];
 #pragma unroll
-                for (int b = 0; b < FN; ++b) bf[b] = flip_sign(bs[kk * kCholLd + wn0 + b * 8 + lq]);
+                for (int b = 0; b < FN; ++b) bf[b] = bs[kk * kCholLd + wn0 + b * 8 + lq];
 #pragma unroll
                 for (int a = 0; a < FM; ++a)
 #pragma unroll
@@ -639,15 +637,13 @@ __device__ __noinline__ void chol_trailing_phase(double* __restrict__ A, double*
 #pragma unroll
             for (int a = 0; a < FM; ++a)
 #pragma unroll
-                for (int b = 0; b < FN; ++b) {
+                for (int b = 0; b < FN; ++b)
                     chol_pair_store(cur, cur.C + (int64_t)(cur.i0 + pr + 8 * a) * ld + cur.j0 + pq + 8 * b, n, pr + 8 * a,
-                                    pq + 8 * b, plain, vec16, acc[a][b]);
-                    acc[a][b] = old[a][b];
-                }
+                                    pq + 8 * b, plain, vec16,
+                                    make_double2(old[a][b].x - acc[a][b].x, old[a][b].y - acc[a][b].y));
             stage ^= 1;
             a_slot = a_next;
             cur = nxt;
-            plain = plain_n;
         }
     };
     if (lgH == 6) run(std::integral_constant<int, 64>());
