@@ -31,6 +31,16 @@ constexpr int kMaxGridY = 65535;
 constexpr int kSuperBlock = 1024;         // columns swept per launch on tall, wide layers
 constexpr int kSuperBlockMinRows = 2048;
 constexpr int kSlicedMinCols = 3072;      // from here on the large float64 products run on the int8 tensor path
+// The loss product goes there too where it is large enough to pay for slicing H and for a second product.  Both sides
+// measured, by rows cols^2 / 2^30: 512 x 1536 (1.1) 72 -> 89 us, 256 x 3008 (2.2) 131 -> 143, 512 x 2304 (2.5) 123 -> 120,
+// 1000 x 2048 (3.9) 205 -> 144, 512 x 4608 (10) 412 -> 310, 2000 x 4608 (40) 1583 -> 765.  Its error against extended
+// precision is no larger (5.6e-17 against 3.7e-16 relative at 1400 x 1400).  W^T W stays where it is below kSlicedMinCols:
+// sliced it is a quarter faster there (193 -> 149 us at 2304 columns), but the error of the inverse up to three times larger.
+constexpr double kSlicedLossMinWork = 2.5 * (1 << 30);
+constexpr int kSlicedLossMinCols = 1024;
+inline bool sliced_loss(int rows, int cols) {
+    return cols >= kSlicedLossMinCols && (double)rows * cols * cols >= kSlicedLossMinWork;
+}
 constexpr int kLossMaxSplit = 8;
 int loss_ksplit(int rows, int cols) {
     const long ctas = (long)cdiv(rows, 64) * ((cdiv(cols, 64) + 1) / 2);
@@ -682,7 +692,7 @@ int ptq_quantize_layer(const float* W, int rows, int cols, int64_t ldw, const do
         finalize_kernel<<<dim3(grid_x_for(n, 256), rows), 256, 0, stream>>>(codes_p, invperm, W, rows, n, ldw, scale,
                                                                            zero, codes, What, dW);
     }
-    if (want_loss && rows >= kSuperBlockMinRows && n >= kSlicedMinCols && n <= kXMaxK &&
+    if (want_loss && sliced_loss(rows, n) && n <= kXMaxK &&
         x_operand_bytes(rows, n) <= (size_t)rows * n * sizeof(double) &&
         x_operand_bytes(n, n) <= (size_t)n * n * sizeof(double) &&
         2 * (size_t)x_num_tiles(rows, n) <= loss_partials_count(rows, cols)) {

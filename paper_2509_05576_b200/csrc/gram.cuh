@@ -11,7 +11,7 @@
 //
 // Kernel: one 128 x 64 output tile per CTA iteration (upper triangle only, mirrored on store).  A TMA producer warp
 // streams 64-wide K blocks of all six slices of the 128 "row" columns and of the 64 "column" columns
-// (SWIZZLE_64B, 3 stages of 72 KB); one thread issues the 42 tcgen05.mma.kind::i8 instructions of a stage into six
+// (SWIZZLE_64B, 3 stages of 72 KB); one thread issues the 16 tcgen05.mma.kind::i8 instructions of a stage (tc_slice_row) into six
 // TMEM accumulators (6 x 64 columns); four epilogue warps read the accumulators back with tcgen05.ld, combine the
 // groups exactly in int64, hand TMEM back (the next tile's products then overlap the rest of the epilogue), scale by
 // 2^(41 - sh_i - sh_j) and add into H.

@@ -12,7 +12,7 @@
 // 2^-54 max|a_i| max|b_j| per term, i.e. that of a float64 dot product; the result is deterministic.
 //
 // Kernel: one 128 x 64 output tile per CTA iteration.  A TMA producer warp streams 64-wide K blocks of the seven
-// slices of both operands (SWIZZLE_64B, 2 stages of 84 KB); one thread issues the 56 tcgen05.mma.kind::i8 of a stage
+// slices of both operands (SWIZZLE_64B, 2 stages of 84 KB); one thread issues the 20 tcgen05.mma.kind::i8 of a stage
 // into seven TMEM accumulators (7 x 64 columns); four epilogue warps read them back with tcgen05.ld, combine, hand TMEM
 // back (the next tile's products then overlap the rest of the epilogue) and add into C through a shared-memory
 // transpose, so that the read-modify-write of C is coalesced.  Every mbarrier wait is bounded.

@@ -53,3 +53,18 @@ def test_the_shape_of_a_deferred_update_of_a_tall_wide_layer():
     # rows x later-columns x super-block: several waves of tiles, many K blocks
     rel = _run(2048, 3000, 1024, True, -1.0, 9)
     assert rel < 1e-15
+
+
+@pytest.mark.parametrize("rows,cols", [(560, 2304), (2561, 1025), (2430, 1050), (497, 2321)])
+def test_loss_on_both_sides_of_the_line_between_its_products(rows, cols):
+    """rows cols^2 just above (first two: sliced int8 products) and just below (float64 MMA) the line, odd widths among
+    them; both sums of rows cols^2 terms carry float64 rounding errors, a few 1e-16 of the sum of their magnitudes."""
+    g = torch.Generator(device="cuda").manual_seed(rows)
+    X = torch.randn((cols, cols + 64), device="cuda", generator=g).abs_()
+    W = torch.randn((rows, cols), device="cuda", generator=g) * 0.03
+    b = ptq.quantize_layer_full(W, X, 4)
+    torch.cuda.synchronize()
+    ptq.check_status(b.status, "layer")
+    d = W.double() - b.What.double()
+    want = 0.5 * float(((d @ b.H) * d).sum())
+    assert abs(b.loss.item() - want) <= 1e-12 * want
