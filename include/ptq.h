@@ -231,6 +231,8 @@ int ptq_sort_scores(const double *S, int cols, int ascending, int32_t *perm, voi
  *   B: b_is_kn = 0: [n x k], row stride ldb;  b_is_kn = 1: the matrix is stored as [k x n] (so C += alpha A B), stride ldb
  *   k <= 16384 (PTQ_ERR_UNSUPPORTED beyond).  Rows of A / of B with wildly different magnitudes are fine (each has its
  *   own power-of-two scale); within a row, entries below 2^-54 of the row's largest magnitude are rounded away.
+ *   A NaN, an infinity or a magnitude of 2^900 and more is recorded in `status` (PTQ_ERR_NONFINITE, index = the row of A
+ *   or of B^T) and makes every entry of C that its row enters NaN.
  * Workspace: ptq_gemm_nt_sliced_workspace_bytes(m, n, k).
  */
 size_t ptq_gemm_nt_sliced_workspace_bytes(int m, int n, int k);

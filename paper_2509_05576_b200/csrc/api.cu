@@ -351,7 +351,7 @@ int ptq_prepare_hinv(const double* H, int cols, int damp_mode, double damp, doub
         // Hinv = W^T W on the int8 tensor path: the columns of the lower-triangular W are sliced once (into R, which is
         // free now) and serve as both operands; only k >= max(i, j) contributes, upper tiles computed and mirrored
         Carver rv(R);
-        const XOperand w = x_slice_operand(rv, V, n, 1, n, n, stream);
+        const XOperand w = x_slice_operand(rv, V, n, 1, n, n, status, stream);
         XGemmParams prm{};
         prm.C = Hinv; prm.ldc = n; prm.alpha = 1.0; prm.status = status; prm.diag = Hinv_diag;
         prm.out_mode = X_OUT_SYM; prm.k_mode = X_K_FROM_MAX;
@@ -701,8 +701,8 @@ int ptq_quantize_layer(const float* W, int rows, int cols, int64_t ldw, const do
         // with reduction epilogues, k before the tile's own block (weight 2 * 1/2) and k in it (weight 1/2).
         // The slices of dW go where E was, those of H where U was: both are free now.
         Carver ev(E), uv(U);
-        const XOperand a = x_slice_operand(ev, dW, n, 0, rows, n, stream);
-        const XOperand b = x_slice_operand(uv, H_undamped, n, 0, n, n, stream);
+        const XOperand a = x_slice_operand(ev, dW, n, 0, rows, n, status, stream);
+        const XOperand b = x_slice_operand(uv, H_undamped, n, 0, n, n, status, stream);
         const int tiles = x_num_tiles(rows, n);
         XGemmParams prm{};
         prm.status = status; prm.out_mode = X_OUT_REDUCE; prm.D = dW; prm.ldd = n;

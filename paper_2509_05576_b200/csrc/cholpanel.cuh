@@ -33,7 +33,7 @@ inline int cholesky_upper_auto(double* A, int n, double* Wm, double* Dbuf, unsig
         const int depth = c0 - r0, rest = n - c0;
         Carver cv(xws);
         // rows of the operand = columns c0 .. n - 1 of the panel's rows of U
-        const XOperand u = x_slice_operand(cv, A + (size_t)r0 * n + c0, n, 1, rest, depth, stream);
+        const XOperand u = x_slice_operand(cv, A + (size_t)r0 * n + c0, n, 1, rest, depth, status, stream);
         XGemmParams prm{};
         prm.C = A + (size_t)c0 * n + c0; prm.ldc = n; prm.alpha = -1.0; prm.status = status;
         prm.out_mode = X_OUT_ADD_UPPER; prm.k_mode = X_K_ALL;
@@ -41,7 +41,7 @@ inline int cholesky_upper_auto(double* A, int n, double* Wm, double* Dbuf, unsig
         if (st) return st;
         if (Wm != nullptr) {
             // rows of the operand = columns 0 .. c0 - 1 of the panel's rows of W
-            const XOperand w = x_slice_operand(cv, Wm + (size_t)r0 * n, n, 1, c0, depth, stream);
+            const XOperand w = x_slice_operand(cv, Wm + (size_t)r0 * n, n, 1, c0, depth, status, stream);
             prm.C = Wm + (size_t)c0 * n; prm.out_mode = X_OUT_ADD;
             st = x_product(u, w, prm, stream);
             if (st) return st;

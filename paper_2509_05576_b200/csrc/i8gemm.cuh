@@ -45,17 +45,25 @@ inline size_t i8gemm_workspace_bytes(int m, int n, int k) {
 }
 // Output / K-range modes and the slicing of one operand at a time: see XGemmParams, x_slice_operand, x_product below.
 
-// Shift of a row whose largest magnitude is m: |x| 2^sh < 2^54 (0 for an all-zero or non-finite row).
+// Integers have no NaN and no infinity.  A row with one (or with a magnitude of 2^900 and more, whose power of two would
+// leave the double range) is recorded in the status word, gets zero digits and this shift: the epilogue's factor
+// 2^(24 - shift) is then infinite and its sums zero, so every entry formed from the row is 0 * inf = NaN, as the float64
+// products have it.
+constexpr double kXMaxMagnitude = 8.452712498170644e270;     // 2^900
+constexpr int kXShiftBad = -1000;
+static_assert(1023 + 24 - kXShiftBad == 2047, "exponent field of an infinity");
+// Shift of a row whose largest magnitude is m: |x| 2^sh < 2^54 (0 for an all-zero row).
 __device__ __forceinline__ int x_row_shift(double m) {
-    if (!(m > 0.0) || !(m < 1.0e300)) return 0;
-    int sh = kXShiftTarget - (ilogb(m) + 1);
-    return sh < -900 ? -900 : (sh > 900 ? 900 : sh);
+    if (!(m < kXMaxMagnitude)) return kXShiftBad;
+    if (!(m > 0.0)) return 0;
+    const int sh = kXShiftTarget - (ilogb(m) + 1);
+    return sh > 900 ? 900 : sh;
 }
 
 // Slices of the rows of X [rows x k] (row stride ld): Q[s][row][kk], one CTA per (padded) row.
 __global__ void __launch_bounds__(256) x_slice_rows_kernel(const double* __restrict__ X, int rows, int k, int64_t ld,
                                                             int rows_pad, int k_pad, int8_t* __restrict__ Q,
-                                                            int32_t* __restrict__ shifts) {
+                                                            int32_t* __restrict__ shifts, int32_t* status) {
     __shared__ double smax[256];
     const int row = blockIdx.x;
     const size_t plane = (size_t)rows_pad * k_pad;
@@ -69,22 +77,29 @@ __global__ void __launch_bounds__(256) x_slice_rows_kernel(const double* __restr
     }
     const double* x = X + (int64_t)row * ld;
     double m = 0.0;
-    for (int kk = threadIdx.x; kk < k; kk += 256) m = fmax(m, fabs(x[kk]));
+    bool bad = false;
+    for (int kk = threadIdx.x; kk < k; kk += 256) {
+        const double a = fabs(x[kk]);
+        bad |= !(a < kXMaxMagnitude);                         // a maximum would drop a NaN
+        m = fmax(m, a);
+    }
     smax[threadIdx.x] = m;
-    __syncthreads();
+    bad = __syncthreads_or(bad) != 0;
     for (int w = 128; w > 0; w >>= 1) {
         if (threadIdx.x < w) smax[threadIdx.x] = fmax(smax[threadIdx.x], smax[threadIdx.x + w]);
         __syncthreads();
     }
-    const int sh = x_row_shift(smax[0]);
-    const bool dead = sh == 0 && !(smax[0] > 0.0 && smax[0] < 1.0e300);
-    if (threadIdx.x == 0) shifts[row] = sh;
-    const double scale = power_of_two(sh);
+    const int sh = bad ? kXShiftBad : x_row_shift(smax[0]);
+    if (threadIdx.x == 0) {
+        shifts[row] = sh;
+        if (bad) report(status, PTQ_ERR_NONFINITE, row, 5);
+    }
+    const double scale = power_of_two(bad ? 0 : sh);
     for (int kk = threadIdx.x * 4; kk < k_pad; kk += 1024) {
         long long v[4];
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
-            const double xv = (kk + u < k && !dead) ? x[kk + u] : 0.0;
+            const double xv = (kk + u < k && !bad) ? x[kk + u] : 0.0;
             v[u] = __double2ll_rn(xv * scale);
         }
         uint32_t packed[kXSlices];
@@ -112,7 +127,7 @@ __global__ void __launch_bounds__(256) x_colmax_kernel(const double* __restrict_
     if (col < cols)
         for (int kk = k0 + wy; kk < k1; kk += 8) {
             const double a = fabs(X[(int64_t)kk * ld + col]);
-            m = a > m || !(a == a) ? a : m;                   // a NaN sticks, so that the column is treated as dead
+            m = a > m || !(a == a) ? a : m;                   // a NaN sticks
         }
     smax[wy][lane] = m;
     __syncthreads();
@@ -127,24 +142,28 @@ __global__ void __launch_bounds__(256) x_colmax_kernel(const double* __restrict_
 __global__ void __launch_bounds__(256) x_slice_cols_kernel(const double* __restrict__ X, int k, int cols, int64_t ld,
                                                             int cols_pad, int k_pad,
                                                             const unsigned long long* __restrict__ colmax,
-                                                            int8_t* __restrict__ Q, int32_t* __restrict__ shifts) {
+                                                            int8_t* __restrict__ Q, int32_t* __restrict__ shifts,
+                                                            int32_t* status) {
     __shared__ uint8_t dig[kXSlices][32][36];          // [slice][column][kk within the tile]
     const int c0 = blockIdx.x * 32, kbeg = blockIdx.y * kXColChunk;
     const int lane = threadIdx.x & 31, wy = threadIdx.x >> 5;          // 8 row slices x 32 columns
     const size_t plane = (size_t)cols_pad * k_pad;
     const int col = c0 + lane;
     const double mm = col < cols ? __longlong_as_double((long long)colmax[col]) : 0.0;
-    const bool dead = !(mm > 0.0 && mm < 1.0e300);
-    const int sh = dead ? 0 : x_row_shift(mm);
-    if (blockIdx.y == 0 && wy == 0 && col < cols_pad) shifts[col] = sh;
-    const double scale = power_of_two(sh);
+    const int sh = x_row_shift(mm);
+    const bool bad = sh == kXShiftBad;
+    if (blockIdx.y == 0 && wy == 0 && col < cols_pad) {
+        shifts[col] = sh;
+        if (bad) report(status, PTQ_ERR_NONFINITE, col, 5);
+    }
+    const double scale = power_of_two(bad ? 0 : sh);
     const int kend = kbeg + kXColChunk < k_pad ? kbeg + kXColChunk : k_pad;
     for (int k0 = kbeg; k0 < kend; k0 += 32) {
         // thread (wy, lane): rows k0 + wy, + 8, + 16, + 24 of column `col`
 #pragma unroll
         for (int r = 0; r < 4; ++r) {
             const int kk = k0 + wy + 8 * r;
-            const double xv = (!dead && kk < k) ? X[(int64_t)kk * ld + col] : 0.0;
+            const double xv = (!bad && kk < k) ? X[(int64_t)kk * ld + col] : 0.0;
             const unsigned long long d = balanced_digits<kXSlices>(__double2ll_rn(xv * scale));
 #pragma unroll
             for (int s = 0; s < kXSlices; ++s) dig[kXSlices - 1 - s][lane][wy + 8 * r] = (uint8_t)(d >> (8 * s));
@@ -465,7 +484,7 @@ inline size_t x_operand_bytes(int rows, int k) {
            align_up((size_t)(cdiv(rows, 128) * 128) * sizeof(unsigned long long));
 }
 // X is [rows x k] (transposed = 0, row stride ld) or [k x rows] (transposed = 1: the operand's rows are X's columns).
-inline XOperand x_slice_operand(Carver& cv, const double* X, int64_t ld, int transposed, int rows, int k,
+inline XOperand x_slice_operand(Carver& cv, const double* X, int64_t ld, int transposed, int rows, int k, int32_t* status,
                                 cudaStream_t stream) {
     const int rows_pad = cdiv(rows, 128) * 128, k_pad = cdiv(k, 128) * 128;
     XOperand op;
@@ -478,9 +497,9 @@ inline XOperand x_slice_operand(Carver& cv, const double* X, int64_t ld, int tra
         cudaMemsetAsync(colmax, 0, (size_t)rows_pad * sizeof(unsigned long long), stream);
         x_colmax_kernel<<<dim3(rows_pad / 32, cdiv(k, kXColChunk)), 256, 0, stream>>>(X, k, rows, ld, colmax);
         x_slice_cols_kernel<<<dim3(rows_pad / 32, cdiv(k_pad, kXColChunk)), 256, 0, stream>>>(X, k, rows, ld, rows_pad, k_pad,
-                                                                                              colmax, op.Q, op.sh);
+                                                                                              colmax, op.Q, op.sh, status);
     } else {
-        x_slice_rows_kernel<<<rows_pad, 256, 0, stream>>>(X, rows, k, ld, rows_pad, k_pad, op.Q, op.sh);
+        x_slice_rows_kernel<<<rows_pad, 256, 0, stream>>>(X, rows, k, ld, rows_pad, k_pad, op.Q, op.sh, status);
     }
     return op;
 }
@@ -520,8 +539,8 @@ inline int i8gemm_nt(double* C, int64_t ldc, const double* A, int64_t lda, const
     if (m <= 0 || n <= 0 || k <= 0) return PTQ_OK;
     if (k > kXMaxK) return PTQ_ERR_UNSUPPORTED;
     Carver cv(ws);
-    const XOperand a = x_slice_operand(cv, A, lda, 0, m, k, stream);
-    const XOperand b = x_slice_operand(cv, B, ldb, b_is_kn, n, k, stream);
+    const XOperand a = x_slice_operand(cv, A, lda, 0, m, k, status, stream);
+    const XOperand b = x_slice_operand(cv, B, ldb, b_is_kn, n, k, status, stream);
     XGemmParams prm{};
     prm.C = C; prm.ldc = ldc; prm.alpha = alpha; prm.status = status;
     prm.out_mode = X_OUT_ADD; prm.k_mode = X_K_ALL;

@@ -68,3 +68,63 @@ def test_loss_on_both_sides_of_the_line_between_its_products(rows, cols):
     d = W.double() - b.What.double()
     want = 0.5 * float(((d @ b.H) * d).sum())
     assert abs(b.loss.item() - want) <= 1e-12 * want
+
+
+def _identity_layer(rows, cols, seed, hot):
+    """W (float32) rounded as it stands (identity inverse Hessian) and a Hessian of normal activations; `hot` scales four
+    input channels, whose weights are zero."""
+    g = torch.Generator(device="cuda").manual_seed(seed)
+    X = torch.randn((cols, cols + cols // 2), dtype=torch.float64, device="cuda", generator=g)
+    W = torch.randn((rows, cols), device="cuda", generator=g) * (2.0 / cols) ** 0.5
+    if hot != 1.0:
+        X[:4] *= hot
+        W[:, :4] = 0.0
+    H = 2.0 * (X @ X.T)
+    return W, 0.5 * (H + H.T)
+
+
+def _direct_loss(W, H):
+    """The loss of ptq_quantize_layer, dW, the status word and how often the two products of the loss were launched."""
+    rows, cols = W.shape
+    st, ws = ptq.new_status(), ptq.Workspace()
+    sc, zp = (torch.empty(rows, dtype=torch.float32, device="cuda") for _ in range(2))
+    ptq.minmax_grid(W, 4, sc, zp, st)
+    codes = torch.empty((rows, cols), dtype=torch.uint8, device="cuda")
+    What = torch.empty((rows, cols), dtype=torch.float32, device="cuda")
+    loss = torch.zeros(1, dtype=torch.float64, device="cuda")
+    names = [ptq.lib().ptq_kernel_name(k).decode() for k in range(ptq.lib().ptq_kernel_count())]
+    ids = [names.index("i8gemm_tcgen05"), names.index("dgemm_loss")]
+    before = [ptq.launch_count(k) for k in ids]
+    ptq.quantize_layer(W, torch.eye(cols, dtype=torch.float64, device="cuda"),
+                       torch.arange(cols, dtype=torch.int32, device="cuda"), sc, zp, 4, codes, What, H, loss, ws, st)
+    torch.cuda.synchronize()
+    return loss.item(), W.double() - What.double(), st.tolist(), [ptq.launch_count(k) - b for k, b in zip(ids, before)]
+
+
+@pytest.mark.parametrize("value", [float("nan"), float("inf")])
+@pytest.mark.parametrize("rows,cols", [(512, 2304), (1000, 2048)])
+def test_a_value_that_is_not_finite_in_the_hessian_shows_in_the_loss(rows, cols, value):
+    W, H = _identity_layer(rows, cols, 5, 1.0)
+    H[77, 1900] = H[1900, 77] = value
+    loss, _, status, launches = _direct_loss(W, H)
+    assert launches[0] > 0 and launches[1] == 0               # the sliced products
+    assert not np.isfinite(loss)
+    assert status[0] == ptq.ERR_NONFINITE
+
+
+@pytest.mark.parametrize("value", [float("nan"), float("-inf")])
+@pytest.mark.parametrize("b_is_kn", [False, True])
+def test_a_value_that_is_not_finite_shows_in_its_row_or_column_of_the_product(b_is_kn, value):
+    g = torch.Generator(device="cuda").manual_seed(3)
+    A = torch.randn((130, 300), dtype=torch.float64, device="cuda", generator=g)
+    B = torch.randn((300, 70) if b_is_kn else (70, 300), dtype=torch.float64, device="cuda", generator=g)
+    A[129, 299] = value
+    B[(299, 65) if b_is_kn else (65, 299)] = value
+    C = torch.zeros((130, 70), dtype=torch.float64, device="cuda")
+    st, ws = ptq.new_status(), ptq.Workspace()
+    ptq.gemm_nt_sliced(C, A, B, 1.0, ws, st, b_is_kn=b_is_kn)
+    torch.cuda.synchronize()
+    assert st.tolist()[0] == ptq.ERR_NONFINITE and st.tolist()[1] in (129, 65)
+    bad = torch.zeros_like(C, dtype=torch.bool)
+    bad[129], bad[:, 65] = True, True
+    assert torch.equal(C.isnan(), bad) and bool(C[~bad].isfinite().all())
