@@ -157,13 +157,14 @@ __global__ void __launch_bounds__(256) x_slice_cols_kernel(const double* __restr
         if (bad) report(status, PTQ_ERR_NONFINITE, col, 5);
     }
     const double scale = power_of_two(bad ? 0 : sh);
+    const int kx = mm > 0.0 && !bad ? k : 0;           // nothing is read of a column of zeros, nor beyond the last column
     const int kend = kbeg + kXColChunk < k_pad ? kbeg + kXColChunk : k_pad;
     for (int k0 = kbeg; k0 < kend; k0 += 32) {
         // thread (wy, lane): rows k0 + wy, + 8, + 16, + 24 of column `col`
 #pragma unroll
         for (int r = 0; r < 4; ++r) {
             const int kk = k0 + wy + 8 * r;
-            const double xv = (!bad && kk < k) ? X[(int64_t)kk * ld + col] : 0.0;
+            const double xv = kk < kx ? X[(int64_t)kk * ld + col] : 0.0;
             const unsigned long long d = balanced_digits<kXSlices>(__double2ll_rn(xv * scale));
 #pragma unroll
             for (int s = 0; s < kXSlices; ++s) dig[kXSlices - 1 - s][lane][wy + 8 * r] = (uint8_t)(d >> (8 * s));
