@@ -34,7 +34,10 @@ constexpr int kSlicedMinCols = 3072;      // from here on the large float64 prod
 // The loss product goes there too where it is large enough to pay for slicing H and for a second product.  Both sides
 // measured, by rows cols^2 / 2^30: 512 x 1536 (1.1) 72 -> 89 us, 256 x 3008 (2.2) 131 -> 143, 512 x 2304 (2.5) 123 -> 120,
 // 1000 x 2048 (3.9) 205 -> 144, 512 x 4608 (10) 412 -> 310, 2000 x 4608 (40) 1583 -> 765.  Its error against extended
-// precision is no larger (5.6e-17 against 3.7e-16 relative at 1400 x 1400).  W^T W stays where it is below kSlicedMinCols:
+// precision is no larger, also where the channels differ in scale (the operands are equilibrated, i8gemm.cuh).  Median and
+// largest relative error over ten kinds of activations at three calibration lengths, float64 library sums / this: 512 x 2304
+// 1.1e-16, 8.9e-13 / 9.8e-17, 2.1e-12; 1000 x 2048 1.1e-16, 2.1e-13 / 1.7e-16, 1.6e-13; 512 x 4608 1.3e-16, 6.0e-13 /
+// 1.3e-16, 2.8e-13 (the largest are those of inputs that share one component, where most of the sum cancels).  W^T W stays where it is below kSlicedMinCols:
 // sliced it is a quarter faster there (193 -> 149 us at 2304 columns), but the error of the inverse up to three times larger.
 constexpr double kSlicedLossMinWork = 2.5 * (1 << 30);
 constexpr int kSlicedLossMinCols = 1024;
@@ -687,22 +690,24 @@ int ptq_quantize_layer(const float* W, int rows, int cols, int64_t ldw, const do
 
     const bool want_loss = H_undamped && loss_out;
     double* dW = want_loss ? Wp : nullptr;
+    const bool sliced = want_loss && sliced_loss(rows, n) && n <= kXMaxK &&
+                        x_operand_bytes(rows, n) <= (size_t)rows * n * sizeof(double) &&
+                        x_operand_bytes(n, n) <= (size_t)n * n * sizeof(double) &&
+                        2 * (size_t)x_num_tiles(rows, n) <= loss_partials_count(rows, cols);
+    int8_t* kexp = sliced ? reinterpret_cast<int8_t*>(Dbuf) : nullptr;      // the factorisation is done with Dbuf
     {
         Launch l(K_FINALIZE, stream);
         finalize_kernel<<<dim3(grid_x_for(n, 256), rows), 256, 0, stream>>>(codes_p, invperm, W, rows, n, ldw, scale,
-                                                                           zero, codes, What, dW);
+                                                                           zero, codes, What, dW, H_undamped, kexp);
     }
-    if (want_loss && sliced_loss(rows, n) && n <= kXMaxK &&
-        x_operand_bytes(rows, n) <= (size_t)rows * n * sizeof(double) &&
-        x_operand_bytes(n, n) <= (size_t)n * n * sizeof(double) &&
-        2 * (size_t)x_num_tiles(rows, n) <= loss_partials_count(rows, cols)) {
+    if (sliced) {
         // 1/2 sum_ij dW_ij (dW H)_ij on the int8 tensor path.  H is symmetric: per 64-column block j the column blocks
         // k < j count twice (they stand in for the blocks k > j as well) and the block k = j once, so two products
         // with reduction epilogues, k before the tile's own block (weight 2 * 1/2) and k in it (weight 1/2).
         // The slices of dW go where E was, those of H where U was: both are free now.
         Carver ev(E), uv(U);
-        const XOperand a = x_slice_operand(ev, dW, n, 0, rows, n, status, stream);
-        const XOperand b = x_slice_operand(uv, H_undamped, n, 0, n, n, status, stream);
+        const XOperand a = x_slice_operand(ev, dW, n, 0, rows, n, status, stream, kexp, 1);
+        const XOperand b = x_slice_operand(uv, H_undamped, n, 0, n, n, status, stream, kexp, -1);
         const int tiles = x_num_tiles(rows, n);
         XGemmParams prm{};
         prm.status = status; prm.out_mode = X_OUT_REDUCE; prm.D = dW; prm.ldd = n;

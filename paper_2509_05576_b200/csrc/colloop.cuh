@@ -616,11 +616,21 @@ inline int sweep_launch(double* Wp, const double* U, double* E, uint8_t* codes_p
     return PTQ_OK;
 }
 
-// Back to the original column order: codes, What = float32(scale * (code - zero)), dW = W - What (float64).
+// Half the exponent of a diagonal entry of the Hessian: 2^-e brings the column's entries to the size of correlations
+// (i8gemm.cuh).  Held to a byte, so that a matrix that is not positive semidefinite cannot overflow by it.
+__device__ __forceinline__ int loss_exponent(double d) {
+    if (!(d > 0.0) || !isfinite(d)) return 0;
+    const int e = ilogb(d) >> 1;
+    return e < -127 ? -127 : (e > 127 ? 127 : e);
+}
+
+// Back to the original column order: codes, What = float32(scale * (code - zero)), dW = W - What (float64).  With kexp, also
+// the exponents by which the loss equilibrates its operands, from the diagonal of H.
 __global__ void finalize_kernel(const uint8_t* __restrict__ codes_p, const int32_t* __restrict__ invperm,
                                 const float* __restrict__ W, int rows, int cols, int64_t ldw,
                                 const float* __restrict__ scale, const float* __restrict__ zero,
-                                uint8_t* __restrict__ codes, float* __restrict__ What, double* __restrict__ dW) {
+                                uint8_t* __restrict__ codes, float* __restrict__ What, double* __restrict__ dW,
+                                const double* __restrict__ H, int8_t* __restrict__ kexp) {
     const int i = blockIdx.y;
     const double sc = (double)scale[i], zp = (double)zero[i];
     for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < cols; j += gridDim.x * blockDim.x) {
@@ -629,6 +639,7 @@ __global__ void finalize_kernel(const uint8_t* __restrict__ codes_p, const int32
         const float q = (float)(sc * ((double)c - zp));
         if (What) What[(int64_t)i * cols + j] = q;
         if (dW) dW[(int64_t)i * cols + j] = (double)W[(int64_t)i * ldw + j] - (double)q;
+        if (kexp && i == 0) kexp[j] = (int8_t)loss_exponent(H[(int64_t)j * cols + j]);
     }
 }
 

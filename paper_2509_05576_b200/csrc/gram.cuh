@@ -316,9 +316,9 @@ __device__ __forceinline__ void tc_wait_ld() { asm volatile("tcgen05.wait::ld.sy
 // The address field is added to the low word at run time: all tiles lie below 256 KB, so the sum never leaves the field.
 constexpr uint32_t kDescLo = 1u << 16;
 constexpr uint32_t kDescHi = (uint32_t)(512 >> 4) | (1u << 14) | (4u << 29);
-// How an MMA treats the buffer in which the tensor core holds its A operand: KEEP loads A and keeps it, LAST multiplies by
-// the A kept, ONCE neither.
-enum { TC_A_ONCE = 0, TC_A_KEEP = 1, TC_A_LAST = 2 };
+// How an MMA treats the buffer in which the tensor core holds its A operand: KEEP loads A and keeps it, AGAIN multiplies by
+// the A kept and keeps it, LAST multiplies by it for the last time, ONCE neither.
+enum { TC_A_ONCE = 0, TC_A_KEEP = 1, TC_A_LAST = 2, TC_A_AGAIN = 3 };
 template <int A_USE>
 __device__ __forceinline__ void tc_mma_i8_lohi(uint32_t d_tmem, uint32_t a_lo, uint32_t b_lo, uint32_t hi, uint32_t idesc,
                                                uint32_t accumulate) {
@@ -332,6 +332,7 @@ __device__ __forceinline__ void tc_mma_i8_lohi(uint32_t d_tmem, uint32_t a_lo, u
                  : "memory")
     if constexpr (A_USE == TC_A_KEEP) PTQ_TC_MMA_I8(".collector::a::fill");
     else if constexpr (A_USE == TC_A_LAST) PTQ_TC_MMA_I8(".collector::a::lastuse");
+    else if constexpr (A_USE == TC_A_AGAIN) PTQ_TC_MMA_I8(".collector::a::use");
     else PTQ_TC_MMA_I8(".collector::a::discard");
 #undef PTQ_TC_MMA_I8
 }
@@ -339,15 +340,28 @@ __device__ __forceinline__ void tc_mma_i8_lohi(uint32_t d_tmem, uint32_t a_lo, u
 // Instruction descriptor: int8 x int8 -> int32, both operands K-major, M = 128.
 template <int N>
 constexpr uint32_t kIdescI8 = (2u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(128 >> 4) << 24);
-// The products of slice A of the row operand with the slices 0 .. G - 1 - A of the column operand, whose results belong
-// to the accumulator groups A .. G - 1.  The 64-row tiles of consecutive column slices follow one another in shared
-// memory and the 64-column accumulators of consecutive groups in TMEM, so all of them together are ONE product with
+// The products of slice A of the row operand with the slices 0 .. G - 1 - A of the column operand (of its S slices), whose
+// results belong to the accumulator groups A .. G - 1.  The 64-row tiles of consecutive column slices follow one another in
+// shared memory and the 64-column accumulators of consecutive groups in TMEM, so all of them together are ONE product with
 // N = 64 (G - A); only above 256, the largest N, it takes two, the second of which reuses the row operand the tensor core
 // still holds.
-template <int A, int G>
+// With one group more than there are slices (G = S + 1) the last group has no product with slice 0: slice 1 opens it, and
+// where it has to overwrite (first = 0) its product there is on its own.
+template <int A, int G, int S>
 __device__ __forceinline__ void tc_slice_row(uint32_t d_tmem, uint32_t a_lo, uint32_t b_lo, uint32_t first) {
-    constexpr int N = 64 * (G - A), N0 = N > 256 ? 256 : N;
+    static_assert(G <= S + 1, "slice 1 opens the group that slice 0 has no product for");
+    constexpr int N = 64 * (G - A < S ? G - A : S), N0 = N > 256 ? 256 : N;
     const uint32_t acc = A > 0 ? 1u : first;
+    if constexpr (A == 1 && G == S + 1) {
+        static_assert(N > 320, "groups 1 .. 4, the middle ones and the last");
+        if (first == 0u) {
+            tc_mma_i8_lohi<TC_A_KEEP>(d_tmem + A * 64, a_lo, b_lo, kDescHi, kIdescI8<256>, 1u);
+            tc_mma_i8_lohi<TC_A_AGAIN>(d_tmem + A * 64 + 256, a_lo, b_lo + 4 * (4096 >> 4), kDescHi, kIdescI8<N - 320>, 1u);
+            tc_mma_i8_lohi<TC_A_LAST>(d_tmem + A * 64 + N - 64, a_lo, b_lo + (N / 64 - 1) * (4096 >> 4), kDescHi,
+                                      kIdescI8<64>, 0u);
+            return;
+        }
+    }
     if constexpr (N > 256) {
         tc_mma_i8_lohi<TC_A_KEEP>(d_tmem + A * 64, a_lo, b_lo, kDescHi, kIdescI8<N0>, acc);
         tc_mma_i8_lohi<TC_A_LAST>(d_tmem + A * 64 + N0, a_lo, b_lo + (N0 / 64) * (4096 >> 4), kDescHi, kIdescI8<N - N0>,
@@ -361,7 +375,7 @@ __device__ __forceinline__ void tc_slice_row(uint32_t d_tmem, uint32_t a_lo, uin
 template <int G, int... As>
 __device__ __forceinline__ void tc_slice_products(uint32_t d_tmem, uint32_t a_lo, uint32_t b_lo, uint32_t first,
                                                   std::integer_sequence<int, As...>) {
-    (tc_slice_row<As, G>(d_tmem, a_lo + As * (8192 >> 4), b_lo, first), ...);
+    (tc_slice_row<As, G, (int)sizeof...(As)>(d_tmem, a_lo + As * (8192 >> 4), b_lo, first), ...);
 }
 
 // Tile t of the enumeration: row block bi (128 rows), column block bj (64 columns) with 64*bj + 63 >= 128*bi.

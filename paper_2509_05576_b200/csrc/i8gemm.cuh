@@ -9,11 +9,20 @@
 // every Da_s Db_t^T is an exact int8 x int8 -> int32 tensor-core product, pairs with s + t = g share one int32 TMEM
 // accumulator, groups g <= 6 are kept (28 products; the dropped ones weigh 2^-56 and less), the groups are combined
 // exactly in int64, rounded to float64 and scaled by 2^(48 - sh_i - sh_j).  The error of an entry is of the order of
-// 2^-54 max|a_i| max|b_j| per term, i.e. that of a float64 dot product; the result is deterministic.
+// 2^-54 max|a_i| max|b_j| per term, i.e. that of a float64 dot product whose terms are of one size; the result is
+// deterministic.
+//
+// The loss 1/2 tr(dW H dW^T) is a sum of terms of very different sizes where the input channels differ in scale, and much
+// of it cancels where they are correlated.  Its operands are therefore equilibrated first, dW_ij 2^e_j and H_jk 2^-e_j with
+// e_j half the exponent of H_jj (powers of two: nothing is rounded, and dW H does not change), which makes the entries of a
+// row of H as alike as those of a correlation matrix, and group 7 is kept as well (34 products).  Relative error of the loss
+// against 80-bit sums, 128 x 1152 layers quantized by the oracle, largest of five draws (float64 MMA / these products /
+// without either measure): channel scales log-normal with sigma 2: 5e-15 / 1e-15 / 3e-14; four channels 10^4 times larger whose
+// weights are zero: 3e-16 / 4e-16 / 4e-13; one component shared by all channels: 7e-13 / 7e-13 / 6e-12.
 //
 // Kernel: one 128 x 64 output tile per CTA iteration.  A TMA producer warp streams 64-wide K blocks of the seven
 // slices of both operands (SWIZZLE_64B, 2 stages of 84 KB); one thread issues the 20 tcgen05.mma.kind::i8 of a stage
-// into seven TMEM accumulators (7 x 64 columns); four epilogue warps read them back with tcgen05.ld, combine, hand TMEM
+// into seven TMEM accumulators (7 x 64 columns; the loss: 22 into eight); four epilogue warps read them back with tcgen05.ld, combine, hand TMEM
 // back (the next tile's products then overlap the rest of the epilogue) and add into C through a shared-memory
 // transpose, so that the read-modify-write of C is coalesced.  Every mbarrier wait is bounded.
 #pragma once
@@ -24,6 +33,7 @@ namespace ptq {
 
 constexpr int kXSlices = 7;
 constexpr int kXGroups = 7;                  // groups g = s + t = 0..6
+constexpr int kXLossGroups = 8;              // and 7: all of TMEM (8 x 64 columns)
 constexpr int kXTM = 128, kXTN = 64, kXKB = 64;
 constexpr int kXStages = 2;
 constexpr int kXABytes = kXTM * kXKB;        // 8 KB per slice
@@ -52,19 +62,23 @@ inline size_t i8gemm_workspace_bytes(int m, int n, int k) {
 constexpr double kXMaxMagnitude = 8.452712498170644e270;     // 2^900
 constexpr int kXShiftBad = -1000;
 static_assert(1023 + 24 - kXShiftBad == 2047, "exponent field of an infinity");
-// Shift of a row whose largest magnitude is m: |x| 2^sh < 2^54 (0 for an all-zero row).
-__device__ __forceinline__ int x_row_shift(double m) {
+// Shift of a row whose largest magnitude is m: |x| 2^sh < 2^54 (0 for an all-zero row); at most `most`.
+__device__ __forceinline__ int x_row_shift(double m, int most = 900) {
     if (!(m < kXMaxMagnitude)) return kXShiftBad;
     if (!(m > 0.0)) return 0;
     const int sh = kXShiftTarget - (ilogb(m) + 1);
-    return sh > 900 ? 900 : sh;
+    return sh > most ? most : sh;
 }
 
-// Slices of the rows of X [rows x k] (row stride ld): Q[s][row][kk], one CTA per (padded) row.
-__global__ void __launch_bounds__(256) x_slice_rows_kernel(const double* __restrict__ X, int rows, int k, int64_t ld,
-                                                            int rows_pad, int k_pad, int8_t* __restrict__ Q,
-                                                            int32_t* __restrict__ shifts, int32_t* status) {
-    __shared__ double smax[256];
+// Slices of the rows of X [rows x k] (row stride ld): Q[s][row][kk], one CTA per (padded) row.  KEXP: the columns are
+// multiplied by 2^(ksign kexp[kk]) first; kexp is 4-byte aligned and may be read up to its next multiple of four.  (One byte
+// an exponent: what is read beside a row is an eighth of it.  4608 x 4608: 59 us without, 60 us with exponents.)
+template <bool KEXP>
+__global__ void __launch_bounds__(256, 6) x_slice_rows_kernel(const double* __restrict__ X, int rows, int k, int64_t ld,
+                                                              int rows_pad, int k_pad, int8_t* __restrict__ Q,
+                                                              int32_t* __restrict__ shifts, int32_t* status,
+                                                              const int8_t* __restrict__ kexp, int ksign) {
+    __shared__ unsigned long long smax[256];
     const int row = blockIdx.x;
     const size_t plane = (size_t)rows_pad * k_pad;
     int8_t* q0 = Q + (size_t)row * k_pad;
@@ -76,31 +90,37 @@ __global__ void __launch_bounds__(256) x_slice_rows_kernel(const double* __restr
         return;
     }
     const double* x = X + (int64_t)row * ld;
-    double m = 0.0;
-    bool bad = false;
+    // the largest magnitude by its bit pattern: non-negative doubles are ordered as integers, a NaN above all of them (a
+    // floating-point maximum would drop it)
+    unsigned long long m = 0ull;
     for (int kk = threadIdx.x; kk < k; kk += 256) {
-        const double a = fabs(x[kk]);
-        bad |= !(a < kXMaxMagnitude);                         // a maximum would drop a NaN
-        m = fmax(m, a);
+        const double v = KEXP ? x[kk] * power_of_two(ksign * (int)kexp[kk]) : x[kk];
+        const unsigned long long a = (unsigned long long)__double_as_longlong(fabs(v));
+        m = a > m ? a : m;
     }
     smax[threadIdx.x] = m;
-    bad = __syncthreads_or(bad) != 0;
+    __syncthreads();
     for (int w = 128; w > 0; w >>= 1) {
-        if (threadIdx.x < w) smax[threadIdx.x] = fmax(smax[threadIdx.x], smax[threadIdx.x + w]);
+        if (threadIdx.x < w && smax[threadIdx.x + w] > smax[threadIdx.x]) smax[threadIdx.x] = smax[threadIdx.x + w];
         __syncthreads();
     }
-    const int sh = bad ? kXShiftBad : x_row_shift(smax[0]);
+    // with an exponent on top: within power_of_two's range
+    const int sh = x_row_shift(__longlong_as_double((long long)smax[0]), KEXP ? 850 : 900);
+    const bool bad = sh == kXShiftBad;
     if (threadIdx.x == 0) {
         shifts[row] = sh;
         if (bad) report(status, PTQ_ERR_NONFINITE, row, 5);
     }
-    const double scale = power_of_two(bad ? 0 : sh);
+    const int sh0 = bad ? 0 : sh, kx = bad ? 0 : k;
     for (int kk = threadIdx.x * 4; kk < k_pad; kk += 1024) {
         long long v[4];
+        char4 e4 = make_char4(0, 0, 0, 0);
+        if (KEXP && kk < k) e4 = *reinterpret_cast<const char4*>(kexp + kk);
+        const int e[4] = {e4.x, e4.y, e4.z, e4.w};
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
-            const double xv = (kk + u < k && !bad) ? x[kk + u] : 0.0;
-            v[u] = __double2ll_rn(xv * scale);
+            const double xv = kk + u < kx ? x[kk + u] : 0.0;
+            v[u] = __double2ll_rn(xv * power_of_two(KEXP ? sh0 + ksign * e[u] : sh0));
         }
         uint32_t packed[kXSlices];
         pack_digits4<kXSlices>(v, packed);
@@ -220,6 +240,7 @@ __device__ __forceinline__ bool x_tile_range(const XGemmParams& prm, int bi, int
     return kb0 < kb1;
 }
 
+template <int GROUPS>
 __global__ void __launch_bounds__(kXThreads, 1)
 i8gemm_kernel(const __grid_constant__ CUtensorMap tmapA, const __grid_constant__ CUtensorMap tmapB, XGemmParams prm) {
     extern __shared__ unsigned char xg_smem_raw[];
@@ -318,8 +339,8 @@ i8gemm_kernel(const __grid_constant__ CUtensorMap tmapA, const __grid_constant__
                     const uint32_t first = kb > kb0 ? 1u : 0u;    // the first product of a group overwrites
 #pragma unroll
                     for (int ks = 0; ks < kXKB / 32; ++ks)
-                        tc_slice_products<kXGroups>(tmem_base, sb + ks * 2, sb + ks * 2 + ((kXSlices * kXABytes) >> 4),
-                                                    ks > 0 ? 1u : first, std::make_integer_sequence<int, kXSlices>());
+                        tc_slice_products<GROUPS>(tmem_base, sb + ks * 2, sb + ks * 2 + ((kXSlices * kXABytes) >> 4),
+                                                  ks > 0 ? 1u : first, std::make_integer_sequence<int, kXSlices>());
                     tc_commit(empty_bar(stage));     // the stage may be refilled once these MMAs have read it
                     if (++stage == kXStages) { stage = 0; phase ^= 1u; }
                 }
@@ -345,25 +366,21 @@ i8gemm_kernel(const __grid_constant__ CUtensorMap tmapA, const __grid_constant__
             if (!ok) break;
             tc_fence_after();
             const int row = bi * kXTM + r_in_tile;
-            // 1. drain: v = hi 2^32 + lo with lo = G6 + 2^8 G5 + 2^16 G4 + 2^24 G3, hi = G2 + 2^8 G1 + 2^16 G0, both exact
+            // 1. drain: v = hi 2^32 + lo with lo = 2^-8 G7 + G6 + 2^8 G5 + 2^16 G4 + 2^24 G3, hi = G2 + 2^8 G1 + 2^16 G0,
+            //    both exact (lo times 2^8 where there is a group 7: below 2^63, as |G3| < 4 2^14 kXMaxK)
             double v[kXTN];
 #pragma unroll
             for (int ch = 0; ch < kXTN / 16; ++ch) {
                 long long lo[16], hi[16];
                 uint32_t r[16];
                 const uint32_t taddr = tmem_base + ((uint32_t)(quarter * 32) << 16) + ch * 16;
-                tc_ld16(taddr + 6 * kXTN, r); tc_wait_ld();
 #pragma unroll
-                for (int c = 0; c < 16; ++c) lo[c] = (long long)(int)r[c];
-                tc_ld16(taddr + 5 * kXTN, r); tc_wait_ld();
+                for (int g = GROUPS - 1; g >= 3; --g) {
+                    tc_ld16(taddr + g * kXTN, r); tc_wait_ld();
 #pragma unroll
-                for (int c = 0; c < 16; ++c) lo[c] += (long long)(int)r[c] << 8;
-                tc_ld16(taddr + 4 * kXTN, r); tc_wait_ld();
-#pragma unroll
-                for (int c = 0; c < 16; ++c) lo[c] += (long long)(int)r[c] << 16;
-                tc_ld16(taddr + 3 * kXTN, r); tc_wait_ld();
-#pragma unroll
-                for (int c = 0; c < 16; ++c) lo[c] += (long long)(int)r[c] << 24;
+                    for (int c = 0; c < 16; ++c)
+                        lo[c] = (g == GROUPS - 1 ? 0ll : lo[c]) + ((long long)(int)r[c] << (8 * (GROUPS - 1 - g)));
+                }
                 tc_ld16(taddr + 2 * kXTN, r); tc_wait_ld();
 #pragma unroll
                 for (int c = 0; c < 16; ++c) hi[c] = (long long)(int)r[c];
@@ -374,7 +391,9 @@ i8gemm_kernel(const __grid_constant__ CUtensorMap tmapA, const __grid_constant__
 #pragma unroll
                 for (int c = 0; c < 16; ++c) hi[c] += (long long)(int)r[c] << 16;
 #pragma unroll
-                for (int c = 0; c < 16; ++c) v[ch * 16 + c] = fma((double)hi[c], 4294967296.0, (double)lo[c]);
+                for (int c = 0; c < 16; ++c) 
+                    v[ch * 16 + c] = fma((double)hi[c], 4294967296.0,
+                                         GROUPS == kXGroups ? (double)lo[c] : (double)lo[c] * 0.00390625);
             }
             tc_fence_before();
             mbar_arrive(acc_empty);
@@ -485,8 +504,9 @@ inline size_t x_operand_bytes(int rows, int k) {
            align_up((size_t)(cdiv(rows, 128) * 128) * sizeof(unsigned long long));
 }
 // X is [rows x k] (transposed = 0, row stride ld) or [k x rows] (transposed = 1: the operand's rows are X's columns).
+// kexp (with transposed = 0): column kk is multiplied by 2^(ksign kexp[kk]), see x_slice_rows_kernel.
 inline XOperand x_slice_operand(Carver& cv, const double* X, int64_t ld, int transposed, int rows, int k, int32_t* status,
-                                cudaStream_t stream) {
+                                cudaStream_t stream, const int8_t* kexp = nullptr, int ksign = 1) {
     const int rows_pad = cdiv(rows, 128) * 128, k_pad = cdiv(k, 128) * 128;
     XOperand op;
     op.Q = cv.take<int8_t>(i8gemm_plane_bytes(rows, k));
@@ -499,8 +519,10 @@ inline XOperand x_slice_operand(Carver& cv, const double* X, int64_t ld, int tra
         x_colmax_kernel<<<dim3(rows_pad / 32, cdiv(k, kXColChunk)), 256, 0, stream>>>(X, k, rows, ld, colmax);
         x_slice_cols_kernel<<<dim3(rows_pad / 32, cdiv(k_pad, kXColChunk)), 256, 0, stream>>>(X, k, rows, ld, rows_pad, k_pad,
                                                                                               colmax, op.Q, op.sh, status);
+    } else if (kexp) {
+        x_slice_rows_kernel<true><<<rows_pad, 256, 0, stream>>>(X, rows, k, ld, rows_pad, k_pad, op.Q, op.sh, status, kexp, ksign);
     } else {
-        x_slice_rows_kernel<<<rows_pad, 256, 0, stream>>>(X, rows, k, ld, rows_pad, k_pad, op.Q, op.sh, status);
+        x_slice_rows_kernel<false><<<rows_pad, 256, 0, stream>>>(X, rows, k, ld, rows_pad, k_pad, op.Q, op.sh, status, nullptr, 1);
     }
     return op;
 }
@@ -512,7 +534,9 @@ inline int x_product(const XOperand& a, const XOperand& b, XGemmParams prm, cuda
     int st = current_device_state(&dev);
     if (st) return st;
     st = ensure_smem_attr(dev, SA_XGEMM, [] {
-        return cudaFuncSetAttribute(i8gemm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kXSmemBytes);
+        const cudaError_t e = cudaFuncSetAttribute(i8gemm_kernel<kXGroups>, cudaFuncAttributeMaxDynamicSharedMemorySize, kXSmemBytes);
+        if (e != cudaSuccess) return e;
+        return cudaFuncSetAttribute(i8gemm_kernel<kXLossGroups>, cudaFuncAttributeMaxDynamicSharedMemorySize, kXSmemBytes);
     });
     if (st) return st;
     const int k_pad = cdiv(a.k, 128) * 128;
@@ -527,7 +551,8 @@ inline int x_product(const XOperand& a, const XOperand& b, XGemmParams prm, cuda
     const int grid = tiles < dev->sms ? tiles : dev->sms;
     {
         Launch l(K_X_GEMM, stream);
-        i8gemm_kernel<<<grid, kXThreads, kXSmemBytes, stream>>>(mapA, mapB, prm);
+        if (prm.out_mode == X_OUT_REDUCE) i8gemm_kernel<kXLossGroups><<<grid, kXThreads, kXSmemBytes, stream>>>(mapA, mapB, prm);
+        else i8gemm_kernel<kXGroups><<<grid, kXThreads, kXSmemBytes, stream>>>(mapA, mapB, prm);
     }
     return launch_status();
 }

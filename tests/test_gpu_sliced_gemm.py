@@ -128,3 +128,38 @@ def test_a_value_that_is_not_finite_shows_in_its_row_or_column_of_the_product(b_
     bad = torch.zeros_like(C, dtype=torch.bool)
     bad[129], bad[:, 65] = True, True
     assert torch.equal(C.isnan(), bad) and bool(C[~bad].isfinite().all())
+
+
+def _loss_in_two_doubles(D, H):
+    """1/2 sum_ij D_ij (D H)_ij with every product and every sum carried as an unevaluated pair of doubles (Dekker's
+    two-product, Knuth's two-sum): about 100 bits."""
+    def split(x):
+        t = x * 134217729.0
+        hi = t - (t - x)
+        return hi, x - hi
+    Dh, Dl = split(D)
+    Hh, Hl = split(H)
+    s, c = torch.zeros_like(D), torch.zeros_like(D)
+    for k in range(D.shape[1]):
+        a, ah, al = D[:, k:k + 1], Dh[:, k:k + 1], Dl[:, k:k + 1]
+        b, bh, bl = H[k:k + 1], Hh[k:k + 1], Hl[k:k + 1]
+        p = a * b
+        t = s + p
+        z = t - s
+        c += ((s - (t - z)) + (p - z)) + (((ah * bh - p) + ah * bl + al * bh) + al * bl)
+        s = t
+    s, c, D = (x.cpu().numpy().astype(np.longdouble) for x in (s, c, D))
+    return 0.5 * np.sum((s + c) * D)
+
+
+@pytest.mark.parametrize("rows,cols,hot", [(512, 2304, 1.0), (512, 2303, 1.0e5), (1000, 1791, 1.0e6)])
+def test_loss_with_channels_of_very_different_scale(rows, cols, hot):
+    """The bound is that of a float64 product: independent rounding errors of up to u times a partial sum, sqrt(cols) of
+    them per entry of dW H, three standard deviations of their weighted sum, and a few u for the last sums."""
+    W, H = _identity_layer(rows, cols, 6, hot)
+    loss, D, status, launches = _direct_loss(W, H)
+    assert status[0] == 0 and launches[0] > 0 and launches[1] == 0               # the sliced products
+    want = _loss_in_two_doubles(D, H)
+    u = 2.0 ** -53
+    bound = 3.0 * u * cols ** 0.5 * torch.linalg.norm(D * (D.abs() @ H.abs())).item() + 4.0 * u * float(want)
+    assert abs(float(np.longdouble(loss) - want)) <= bound, (float((np.longdouble(loss) - want) / want), bound / float(want))
