@@ -175,14 +175,27 @@ __global__ void __launch_bounds__(kPerRowThreads, 3) per_row_kernel(const float*
         double v[8], lev[8];
 #pragma unroll
         for (int p = 0; p < 8; ++p) v[p] = w[8 * b + p];
+        double my_lev = 0.0, my_code = 0.0;
         if (sweep_chain8<false, 8>(v, lev, us, rg)) {
+            // by the definition: code = clamp(rint(w / s) + z), level = code - z.  (For a zero-point that is no integer of
+            // ordinary size, code and level cannot be had from one another.)
 #pragma unroll
             for (int p = 0; p < 8; ++p) v[p] = w[8 * b + p];
-            sweep_chain8<true, 8>(v, lev, us, rg);
-        }
-        double my_lev = lev[0];
 #pragma unroll
-        for (int p = 1; p < 8; ++p) my_lev = lane == p ? lev[p] : my_lev;
+            for (int p = 0; p < 8; ++p) {
+                const double code = quant_code_d(v[p], rg.sc, rg.zp, maxq), level = code - rg.zp;
+                const double d = v[p] - rg.sc * level;
+#pragma unroll
+                for (int j = p + 1; j < 8; ++j) v[j] = fma(-d, us[p * 8 + j], v[j]);
+                v[p] = d;
+                my_lev = lane == p ? level : my_lev;
+                my_code = lane == p ? code : my_code;
+            }
+        } else {
+#pragma unroll
+            for (int p = 0; p < 8; ++p) my_lev = lane == p ? lev[p] : my_lev;
+            my_code = my_lev + rg.zp;
+        }
 #pragma unroll
         for (int p = 0; p < 8; ++p) v[p] *= dinv[8 * b + p];
         for (int c = 8 * (b + 1) + lane; c < n8; c += 32) {
@@ -194,7 +207,7 @@ __global__ void __launch_bounds__(kPerRowThreads, 3) per_row_kernel(const float*
         }
         if (lane < 8 && 8 * b + lane < n) {
             const int j = perm[8 * b + lane];
-            codes[(int64_t)i * n + j] = (uint8_t)(int)(my_lev + rg.zp);
+            codes[(int64_t)i * n + j] = (uint8_t)(int)my_code;
             const float qf = (float)(rg.sc * my_lev);
             if (What) What[(int64_t)i * n + j] = qf;
             dw[j] = (double)W[(int64_t)i * ldw + j] - (double)qf;

@@ -73,6 +73,20 @@ def test_a_pivot_that_is_not_positive_is_reported():
     assert ei.value.code == ptq.ERR_NOT_SPD and "index 11" in str(ei.value)
 
 
+@pytest.mark.parametrize("zero", [7.3, -0.5, 3.0e9, 1.0e17, -1.0e17])
+def test_per_row_codes_follow_the_definition_for_any_zero_point(zero):
+    """code = clamp(rint(w / s) + z, 0, maxq), q = s (code - z) in float64, also where z is no integer of ordinary size
+    (identity: no compensation, so every weight is quantized as it stands)."""
+    rng = np.random.Generator(np.random.PCG64(91))
+    W = (rng.standard_normal((5, 20)) * 3.0).astype(np.float32)
+    sc, zp = np.full(5, 0.25, np.float32), np.full(5, zero, np.float32)
+    codes, What, _, _ = _run(W, np.eye(20), np.eye(20), sc, zp, 4, ptq.SCORE_NONE)
+    z = zp[:, None].astype(np.float64)
+    c = np.clip(np.rint(W.astype(np.float64) / 0.25) + z, 0.0, 15.0)
+    assert np.array_equal(codes, c.astype(np.uint8))
+    assert np.array_equal(What, (0.25 * (c - z)).astype(np.float32))
+
+
 def test_wider_layers_are_refused():
     fake = torch.zeros(16, dtype=torch.float32, device="cuda")
     st, ws = ptq.new_status(), ptq.Workspace()
