@@ -39,7 +39,7 @@ typedef enum {
     PTQ_ERR_INVALID_ARG = 1,
     PTQ_ERR_ALIGNMENT = 2,
     PTQ_ERR_WORKSPACE = 3,
-    PTQ_ERR_NOT_SPD = 4,     /* status[1] = failing pivot index */
+    PTQ_ERR_NOT_SPD = 4,     /* status[1] = failing pivot index (not positive, not finite, or too small to be inverted) */
     PTQ_ERR_NONFINITE = 5,
     PTQ_ERR_TIMEOUT = 6,     /* a bounded device-side wait expired */
     PTQ_ERR_CUDA = 7,        /* a CUDA runtime call failed on the host */

@@ -58,7 +58,7 @@ __global__ void damp_copy_kernel(const double* __restrict__ H, double* __restric
 // are still applying the current one to the rows below, which takes the strip off the critical path.
 // The phases are separated by a grid-wide barrier whose wait is bounded: when it expires the CTA records
 // PTQ_ERR_TIMEOUT, raises the abort word and leaves; the other CTAs see the abort word and leave too.
-// A non-positive or non-finite pivot is reported (PTQ_ERR_NOT_SPD, pivot index) and replaced by 1.
+// A pivot that is not positive, normal and finite is reported (PTQ_ERR_NOT_SPD, pivot index) and replaced by 1.
 // ------------------------------------------------------------------------------------------------------------
 constexpr int kCholThreads = 512;
 constexpr int kCholLd = kNB + 4;                               // operand row stride (68 = 4 mod 16: conflict-free)
@@ -222,7 +222,7 @@ __device__ __forceinline__ void chol_strip_lookahead(double (&acc)[8][2], const 
 }
 
 // Step 1 above.  mb: the mini-block M (row-major, 8 x 8, upper part); leaves W in Wbuf.  Returns the first pivot that is not
-// positive and finite (it is replaced by 1) or -1.
+// accepted (it is replaced by 1) or -1.
 __device__ __forceinline__ int chol_chain8(const double* mb, double* Wbuf, int lane) {
     double m[8][8];
 #pragma unroll
@@ -240,7 +240,7 @@ __device__ __forceinline__ int chol_chain8(const double* mb, double* Wbuf, int l
         // A bad pivot is replaced by 1 and remembered; the report is made after the chain, so that the eight steps
         // stay one straight line of code.
         const double d0 = m[p][p];
-        const bool ok = d0 > 0.0 && d0 < 1.0e300;
+        const bool ok = d0 >= kMinPivot && d0 < kMaxPivot;
         bad = (!ok && bad < 0) ? p : bad;
         const double d = ok ? d0 : 1.0;
         // 1 / d is what the chain waits for: the hardware's approximation (about 20 bits) times the first terms of

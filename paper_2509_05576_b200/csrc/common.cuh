@@ -13,6 +13,10 @@ namespace ptq {
 
 constexpr int kNB = 64;  // block size of the factorisations and of the column loop
 
+// Pivots of a factorisation are accepted from the smallest normal number up to 10^300: the hardware approximations that the
+// chains refine take a subnormal for zero, and the reciprocal of what lies above is (nearly) subnormal itself.
+constexpr double kMinPivot = 2.2250738585072014e-308, kMaxPivot = 1.0e300;
+
 // First error wins; later kernels keep running on whatever numbers they find (no traps, no faults).
 __device__ __forceinline__ void report(int32_t* status, int code, int index, int aux = 0) {
     if (status && atomicCAS(status, 0, code) == 0) {

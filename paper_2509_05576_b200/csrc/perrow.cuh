@@ -21,8 +21,11 @@ inline size_t per_row_smem_bytes(int cols) {
 
 // The eight pivots of the diagonal tile `m` (row-major 8 x 8, symmetric): m = L D L^T.  All of the tile sits in every
 // lane, so the serial chain has no data exchange in it; lane j carries column j of the identity along, which becomes
-// column j of L^-1.  Leaves L^-1 in Wb and the reciprocal pivots in dinv.  A pivot that is not positive and finite is
-// replaced by 1; returns the first such pivot or -1.
+// column j of L^-1.  Leaves L^-1 in Wb and the reciprocal pivots in dinv.  A pivot that is not accepted is replaced by 1;
+// returns the first such pivot or -1.
+// DIVIDE = false accepts normal pivots only.  DIVIDE = true, for the repetition of a tile with some other pivot, divides, and
+// so takes subnormal pivots as well, down to those whose reciprocal overflows.
+template <bool DIVIDE>
 __device__ __forceinline__ int per_row_chain(const double* tile, double* Wb, double* dinv, int lane) {
     double m[8][8], x[8];
 #pragma unroll
@@ -35,7 +38,7 @@ __device__ __forceinline__ int per_row_chain(const double* tile, double* Wb, dou
 #pragma unroll
     for (int p = 0; p < 8; ++p) {
         const double d0 = m[p][p];
-        const bool ok = d0 > 0.0 && d0 < 1.0e300;
+        const bool ok = DIVIDE ? d0 > 0.0 && d0 < kMaxPivot && isfinite(1.0 / d0) : d0 >= kMinPivot && d0 < kMaxPivot;
         bad = (!ok && bad < 0) ? p : bad;
         const double d = ok ? d0 : 1.0;
         // 1 / d: the hardware's approximation (about 20 bits) times the first terms of 1 / (1 - e) = 1 + e + e^2 + ..,
@@ -43,7 +46,7 @@ __device__ __forceinline__ int per_row_chain(const double* tile, double* Wb, dou
         double y;
         asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(d));
         const double e = fma(-d, y, 1.0);
-        const double inv = fma(y, fma(e, e, e), y);
+        const double inv = DIVIDE ? 1.0 / d : fma(y, fma(e, e, e), y);
         if (lane == 0) dinv[p] = inv;
 #pragma unroll
         for (int i = p + 1; i < 8; ++i) {
@@ -218,7 +221,8 @@ __global__ void __launch_bounds__(kPerRowThreads, 3) per_row_kernel(const float*
 
     for (int b = 0; b < nf; ++b) {
         if (warp == 0) {
-            const int bad = per_row_chain(tile(b, b), Wb, dinv + 8 * b, lane);
+            int bad = per_row_chain<false>(tile(b, b), Wb, dinv + 8 * b, lane);
+            if (bad >= 0) bad = per_row_chain<true>(tile(b, b), Wb, dinv + 8 * b, lane);
             if (bad >= 0 && lane == 0) report(status, PTQ_ERR_NOT_SPD, 8 * b + bad, i);
         } else if (b > 0) {
             if (warp == 1) {

@@ -139,6 +139,19 @@ def test_inverse_absolute_damping_and_not_spd_status():
     assert ei.value.code == ptq.ERR_NOT_SPD and ei.value.index == 0
 
 
+@pytest.mark.parametrize("index", [5, 69])
+def test_a_subnormal_pivot_is_reported(index):
+    H = torch.eye(70, dtype=torch.float64, device="cuda")
+    H[index, index] = 1.0e-310
+    st, ws = ptq.new_status(), ptq.Workspace()
+    Hinv, diag, lam = torch.empty_like(H), torch.empty(70, dtype=torch.float64, device="cuda"), torch.empty(1, dtype=torch.float64, device="cuda")
+    ptq.prepare_hinv(H, 0.0, ptq.DAMP_ABS, Hinv, diag, lam, ws, st)
+    torch.cuda.synchronize()
+    with pytest.raises(ptq.PtqError) as ei:
+        ptq.check_status(st)
+    assert ei.value.code == ptq.ERR_NOT_SPD and ei.value.index == index
+
+
 # ------------------------------------------------------------------------------------------ grid, scores, order
 @pytest.mark.parametrize("bits", [2, 3, 4, 8])
 def test_grid_is_bit_exact(bits):

@@ -87,6 +87,30 @@ def test_per_row_codes_follow_the_definition_for_any_zero_point(zero):
     assert np.array_equal(What, (0.25 * (c - z)).astype(np.float32))
 
 
+@pytest.mark.parametrize("pivot", [2.0e-308, 2.3e-308])
+def test_pivots_on_either_side_of_the_normal_range(pivot):
+    """1 / pivot is finite for both; nothing couples the columns, so every weight is rounded as it stands."""
+    n = 11
+    Hinv = np.eye(n)
+    Hinv[4, 4] = pivot
+    W = np.linspace(-1.0, 1.0, n, dtype=np.float32)[None, :].copy()
+    codes, What, _, loss = _run(W, np.eye(n), Hinv, np.full(1, 0.125, np.float32), np.full(1, 8.0, np.float32), 4,
+                                ptq.SCORE_NONE)
+    c = np.clip(np.rint(W / 0.125) + 8.0, 0.0, 15.0)
+    assert np.array_equal(codes, c.astype(np.uint8))
+    assert np.isfinite(loss) and np.array_equal(What, (0.125 * (c - 8.0)).astype(np.float32))
+
+
+def test_a_pivot_without_a_reciprocal_is_reported():
+    n = 11
+    Hinv = np.eye(n)
+    Hinv[4, 4] = 1.0e-310
+    with pytest.raises(ptq.PtqError) as ei:
+        _run(np.full((1, n), 0.5, np.float32), np.eye(n), Hinv, np.ones(1, np.float32), np.zeros(1, np.float32), 4,
+             ptq.SCORE_NONE)
+    assert ei.value.code == ptq.ERR_NOT_SPD and "index 4" in str(ei.value)
+
+
 def test_wider_layers_are_refused():
     fake = torch.zeros(16, dtype=torch.float32, device="cuda")
     st, ws = ptq.new_status(), ptq.Workspace()
