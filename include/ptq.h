@@ -254,6 +254,13 @@ int ptq_selftest_wait_timeout(int which, long long limit_cycles, void *ws, size_
                               void *stream);
 
 /*
+ * Self-test of the arithmetic on pivots (instrumentation; the paper has no counterpart): rcp[i] = 1 / x[i] and
+ * rsq[i] = 1 / sqrt(x[i]) as the factorisations form them, for x[i] from the smallest normal number up to 1e300.
+ *   x, rcp, rsq [n] float64 (device)
+ */
+int ptq_selftest_reciprocal(const double *x, int n, double *rcp, double *rsq, void *stream);
+
+/*
  * Float64 throughput probe (instrumentation; the paper has no counterpart): launches one kernel of 4 CTAs x 256 threads
  * per SM in which every thread runs `iters` rounds of eight independent chains of float64 FMAs (kind 0) or of float64
  * tensor-core MMAs m8n8k4 (kind 1), and nothing else.  *flops_out (host) receives the floating-point operations of

@@ -110,6 +110,15 @@ __global__ void selftest_counter_kernel(unsigned* words, int32_t* status, long l
         report(status, PTQ_ERR_TIMEOUT, blockIdx.x, 2);
 }
 
+// What the factorisations make of a pivot, one value per thread.
+__global__ void __launch_bounds__(256) selftest_reciprocal_kernel(const double* __restrict__ x, int n, double* __restrict__ rcp,
+                                                                   double* __restrict__ rsq) {
+    const int i = blockIdx.x * 256 + threadIdx.x;
+    if (i >= n) return;
+    rcp[i] = pivot_reciprocal(x[i]);
+    rsq[i] = pivot_rsqrt(x[i]);
+}
+
 // Float64 throughput probes: eight independent chains per thread, nothing but the arithmetic instruction in the loop.
 constexpr int kProbeThreads = 256, kProbeCtasPerSm = 4, kProbeChains = 8;
 __global__ void __launch_bounds__(kProbeThreads) fp64_probe_fma_kernel(int iters, double* sink) {
@@ -609,6 +618,13 @@ int ptq_selftest_wait_timeout(int which, long long limit_cycles, void* ws, size_
         return PTQ_ERR_CUDA;
     }
     return PTQ_OK;
+}
+
+int ptq_selftest_reciprocal(const double* x, int n, double* rcp, double* rsq, void* stream_) {
+    cudaStream_t stream = static_cast<cudaStream_t>(stream_);
+    if (!x || !rcp || !rsq || n < 1) return PTQ_ERR_INVALID_ARG;
+    { Launch l(K_SELFTEST, stream); selftest_reciprocal_kernel<<<cdiv(n, 256), 256, 0, stream>>>(x, n, rcp, rsq); }
+    return launch_status();
 }
 
 int ptq_fp64_probe(int kind, int iters, double* sink, double* flops_out, void* stream_) {

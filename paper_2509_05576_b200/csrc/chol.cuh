@@ -243,16 +243,8 @@ __device__ __forceinline__ int chol_chain8(const double* mb, double* Wbuf, int l
         const bool ok = d0 >= kMinPivot && d0 < kMaxPivot;
         bad = (!ok && bad < 0) ? p : bad;
         const double d = ok ? d0 : 1.0;
-        // 1 / d is what the chain waits for: the hardware's approximation (about 20 bits) times the first terms of
-        // 1 / (1 - e) = 1 + e + e^2 + .., e = 1 - d y; what is left out is of order e^3, far below one ulp
-        double y, z;
-        asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(d));
-        const double e = fma(-d, y, 1.0);
-        const double inv = fma(y, fma(e, e, e), y);
-        // 1 / sqrt(d), beside the chain: z (1 + g / 2 + 3 g^2 / 8), g = 1 - d z^2, likewise
-        asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(z) : "d"(d));
-        const double g = fma(-(z * z), d, 1.0);
-        const double rs = fma(z, g * fma(0.375, g, 0.5), z);
+        const double inv = pivot_reciprocal(d);            // what the chain waits for
+        const double rs = pivot_rsqrt(d);                  // beside the chain
         const double tx = x[p] * inv;
         x[p] *= rs;
 #pragma unroll

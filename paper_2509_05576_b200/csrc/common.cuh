@@ -17,6 +17,26 @@ constexpr int kNB = 64;  // block size of the factorisations and of the column l
 // chains refine take a subnormal for zero, and the reciprocal of what lies above is (nearly) subnormal itself.
 constexpr double kMinPivot = 2.2250738585072014e-308, kMaxPivot = 1.0e300;
 
+// 1 / d and 1 / sqrt(d) of an accepted pivot without a branch: what a chain of eight pivots waits for.  Both take the
+// hardware's approximation (a documented instruction, about 20 bits) as the start of one step of third order:
+//   1 / d:        y (1 + e + e^2), e = 1 - d y: the hyperpower iteration of order three (M. Altman, Pacific J. Math. 10, 1960),
+//                 i.e. the geometric series of 1 / (1 - e) cut off before e^3;
+//   1 / sqrt(d):  z (1 + g / 2 + 3 g^2 / 8), g = 1 - d z^2: Newton's binomial series of (1 - g)^(-1/2) cut off before g^3.
+// What is cut off is below 2^-56.  Left are the rounding of the result and, for the root, that of z^2, whose half enters:
+// at most 0.6 and 1.1 units in the last place (ptq_selftest_reciprocal).
+__device__ __forceinline__ double pivot_reciprocal(double d) {
+    double y;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(d));
+    const double e = fma(-d, y, 1.0);
+    return fma(y, fma(e, e, e), y);
+}
+__device__ __forceinline__ double pivot_rsqrt(double d) {
+    double z;
+    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(z) : "d"(d));
+    const double g = fma(-(z * z), d, 1.0);
+    return fma(z, g * fma(0.375, g, 0.5), z);
+}
+
 // First error wins; later kernels keep running on whatever numbers they find (no traps, no faults).
 __device__ __forceinline__ void report(int32_t* status, int code, int index, int aux = 0) {
     if (status && atomicCAS(status, 0, code) == 0) {
@@ -155,7 +175,7 @@ inline const char* kernel_name(int id) {
         "gram_split", "gram_i8_tcgen05", "gram_finish", "convert_f64", "dgemm_gram_f64", "lambda", "damp_copy", "chol_coop",
         "dgemm_lauum",
         "minmax_grid", "score_partial", "score_final", "rank_sort", "perm_check", "sweep_gather",
-        "sweep_coop", "finalize", "dgemm_loss", "sum_partials", "selftest_wait", "fp64_probe", "dyn_aux", "dyn_gather",
+        "sweep_coop", "finalize", "dgemm_loss", "sum_partials", "selftest", "fp64_probe", "dyn_aux", "dyn_gather",
         "dgemm_dyn", "per_row", "dgemm_eq11", "x_slice", "i8gemm_tcgen05"};
     return (id >= 0 && id < K_COUNT) ? names[id] : "unknown";
 }

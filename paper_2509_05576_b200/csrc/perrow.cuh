@@ -41,12 +41,7 @@ __device__ __forceinline__ int per_row_chain(const double* tile, double* Wb, dou
         const bool ok = DIVIDE ? d0 > 0.0 && d0 < kMaxPivot && isfinite(1.0 / d0) : d0 >= kMinPivot && d0 < kMaxPivot;
         bad = (!ok && bad < 0) ? p : bad;
         const double d = ok ? d0 : 1.0;
-        // 1 / d: the hardware's approximation (about 20 bits) times the first terms of 1 / (1 - e) = 1 + e + e^2 + ..,
-        // e = 1 - d y; what is left out is of order e^3, below one ulp
-        double y;
-        asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(d));
-        const double e = fma(-d, y, 1.0);
-        const double inv = DIVIDE ? 1.0 / d : fma(y, fma(e, e, e), y);
+        const double inv = DIVIDE ? 1.0 / d : pivot_reciprocal(d);
         if (lane == 0) dinv[p] = inv;
 #pragma unroll
         for (int i = p + 1; i < 8; ++i) {

@@ -27,7 +27,7 @@ CALL_QUANTIZE_LAYER_PER_ROW = 6
 
 EXPORTS = ["ptq_workspace_bytes", "ptq_hessian_accumulate", "ptq_hessian_accumulate_conv", "ptq_hessian_accumulate_f64", "ptq_prepare_hinv",
            "ptq_minmax_grid", "ptq_sensitivity_order", "ptq_sensitivity_order_static", "ptq_quantize_layer", "ptq_status_string", "ptq_version",
-           "ptq_sort_scores", "ptq_gemm_nt_sliced", "ptq_gemm_nt_sliced_workspace_bytes", "ptq_quantize_layer_dynamic", "ptq_quantize_layer_per_row", "ptq_selftest_wait_timeout", "ptq_fp64_probe",
+           "ptq_sort_scores", "ptq_gemm_nt_sliced", "ptq_gemm_nt_sliced_workspace_bytes", "ptq_quantize_layer_dynamic", "ptq_quantize_layer_per_row", "ptq_selftest_wait_timeout", "ptq_selftest_reciprocal", "ptq_fp64_probe",
            "ptq_kernel_count", "ptq_kernel_name", "ptq_launch_count", "ptq_profile_enable", "ptq_profile_read",
            "ptq_set_cta_limit"]
 
@@ -77,6 +77,7 @@ def lib():
         L.ptq_quantize_layer_dynamic.argtypes = [vp, c_int, c_int, c_int64, vp, vp, vp, c_int, c_int, c_int, vp, vp,
                                                  vp, vp, vp, vp, c_size_t, vp, vp]
         L.ptq_selftest_wait_timeout.argtypes = [c_int, ctypes.c_longlong, vp, c_size_t, vp, vp]
+        L.ptq_selftest_reciprocal.argtypes = [vp, c_int, vp, vp, vp]
         L.ptq_fp64_probe.argtypes = [c_int, c_int, vp, ctypes.POINTER(c_double), vp]
         L.ptq_status_string.argtypes = [c_int]
         L.ptq_status_string.restype = ctypes.c_char_p
@@ -277,6 +278,15 @@ def selftest_wait_timeout(which, limit_cycles, ws, status, stream=None):
     buf = ws.get(256)
     _check(lib().ptq_selftest_wait_timeout(int(which), int(limit_cycles), _ptr(buf), buf.numel(), _ptr(status),
                                            _stream(stream)), "ptq_selftest_wait_timeout")
+
+
+def selftest_reciprocal(x, stream=None):
+    """(1 / x, 1 / sqrt(x)) as the factorisations form them of their pivots (float64 device tensor, 1-D)."""
+    _dev(x, torch.float64, "x")
+    rcp, rsq = torch.empty_like(x), torch.empty_like(x)
+    _check(lib().ptq_selftest_reciprocal(_ptr(x), x.numel(), _ptr(rcp), _ptr(rsq), _stream(stream)),
+           "ptq_selftest_reciprocal")
+    return rcp, rsq
 
 
 def fp64_probe(kind, iters, sink, stream=None) -> float:

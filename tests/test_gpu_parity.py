@@ -152,6 +152,24 @@ def test_a_subnormal_pivot_is_reported(index):
     assert ei.value.code == ptq.ERR_NOT_SPD and ei.value.index == index
 
 
+def test_pivot_arithmetic_against_division_and_square_root():
+    """All binades an accepted pivot can have, the powers of two with their neighbours and the ends of the range; against
+    80-bit values.  Bounds: half a unit in the last place for the rounding of the result, for the root as much again for
+    that of z^2, and a tenth for the cut-off series (see pivot_reciprocal); against CUDA's own division one unit."""
+    rng = np.random.Generator(np.random.PCG64(12))
+    p2 = np.ldexp(1.0, np.arange(-1022, 997))
+    x = np.concatenate([np.ldexp(rng.uniform(1.0, 2.0, 400000), rng.integers(-1022, 996, 400000)), p2, np.nextafter(p2, np.inf),
+                        np.nextafter(p2[1:], 0.0), [np.nextafter(1.0e300, 0.0)]])
+    xd = _cuda(x)
+    rcp, rsq = (t.cpu().numpy() for t in ptq.selftest_reciprocal(xd))
+    xl = x.astype(np.longdouble)
+    for got, want, bound in ((rcp, 1.0 / xl, 0.6), (rsq, 1.0 / np.sqrt(xl), 1.1)):
+        ulp = np.spacing(want.astype(np.float64))
+        err = np.abs((got.astype(np.longdouble) - want) / ulp)
+        assert float(err.max()) <= bound, (float(err.max()), x[int(err.argmax())])
+    assert bool(((_cuda(rcp) - 1.0 / xd).abs() <= torch.from_numpy(np.spacing(rcp)).cuda()).all())
+
+
 # ------------------------------------------------------------------------------------------ grid, scores, order
 @pytest.mark.parametrize("bits", [2, 3, 4, 8])
 def test_grid_is_bit_exact(bits):
