@@ -26,32 +26,40 @@ inline int grid_x_for(int n, int threads) {
     return g < 1 ? 1 : (g > 1024 ? 1024 : g);
 }
 
-// The loss product is cut along k into as many slices as it takes to put about two CTAs on every SM.
 constexpr int kMaxGridY = 65535;
 constexpr int kSuperBlock = 1024;         // columns swept per launch on tall, wide layers
 constexpr int kSuperBlockMinRows = 2048;
 constexpr int kSlicedMinCols = 3072;      // from here on the large float64 products run on the int8 tensor path
-// The loss product goes there too where it is large enough to pay for slicing H and for a second product.  Both sides
-// measured, by rows cols^2 / 2^30: 512 x 1536 (1.1) 72 -> 89 us, 256 x 3008 (2.2) 131 -> 143, 512 x 2304 (2.5) 123 -> 120,
-// 1000 x 2048 (3.9) 205 -> 144, 512 x 4608 (10) 412 -> 310, 2000 x 4608 (40) 1583 -> 765.  Its error against extended
+// The loss product goes there too where it is large enough to pay for slicing H and for a second product, and where the
+// slices (7 bytes a value, both sizes rounded up to multiples of 128) and the two sets of partial sums fit into the pieces of
+// the workspace that are free by then: dW's into E, H's into U (8 bytes a value each).  So a size whose padding takes more
+// than an eighth of it keeps the float64 product: 560 x 2304 and 2561 x 1025 do, 512 x 2304 and 1000 x 1791 do not.
+// Both sides measured, float64 -> sliced, by rows cols^2 / 2^30: 512 x 1536 (1.1) 69 -> 81 us, 256 x 3008 (2.2) 130 -> 141,
+// 1024 x 1536 (2.3) 123 -> 136, 512 x 2304 (2.5) 126 -> 118, 768 x 1920 (2.6) 157 -> 155, 768 x 2304 (3.8) 174 -> 167,
+// 1000 x 2048 (3.9) 209 -> 151, 512 x 4608 (10) 418 -> 316, 2000 x 4608 (40) 1599 -> 844.  Its error against extended
 // precision is no larger, also where the channels differ in scale (the operands are equilibrated, i8gemm.cuh).  Median and
 // largest relative error over ten kinds of activations at three calibration lengths, float64 library sums / this: 512 x 2304
 // 1.1e-16, 8.9e-13 / 9.8e-17, 2.1e-12; 1000 x 2048 1.1e-16, 2.1e-13 / 1.7e-16, 1.6e-13; 512 x 4608 1.3e-16, 6.0e-13 /
-// 1.3e-16, 2.8e-13 (the largest are those of inputs that share one component, where most of the sum cancels).  W^T W stays where it is below kSlicedMinCols:
-// sliced it is a quarter faster there (193 -> 149 us at 2304 columns), but the error of the inverse up to three times larger.
+// 1.3e-16, 2.8e-13 (the largest are those of inputs that share one component, where most of the sum cancels).  W^T W stays
+// where it is below kSlicedMinCols: sliced it is a quarter faster there (193 -> 149 us at 2304 columns), but the error of the
+// inverse up to three times larger.
 constexpr double kSlicedLossMinWork = 2.5 * (1 << 30);
 constexpr int kSlicedLossMinCols = 1024;
-inline bool sliced_loss(int rows, int cols) {
-    return cols >= kSlicedLossMinCols && (double)rows * cols * cols >= kSlicedLossMinWork;
-}
 constexpr int kLossMaxSplit = 8;
+size_t loss_partials_count(int rows, int cols) {
+    return (size_t)kLossMaxSplit * cdiv(rows, 64) * cdiv(cols, 64);
+}
+bool sliced_loss(int rows, int cols) {
+    return cols >= kSlicedLossMinCols && cols <= kXMaxK && (double)rows * cols * cols >= kSlicedLossMinWork &&
+           x_operand_bytes(rows, cols) <= (size_t)rows * cols * sizeof(double) &&
+           x_operand_bytes(cols, cols) <= (size_t)cols * cols * sizeof(double) &&
+           2 * (size_t)x_num_tiles(rows, cols) <= loss_partials_count(rows, cols);
+}
+// The float64 loss product is cut along k into as many slices as it takes to put about two CTAs on every SM.
 int loss_ksplit(int rows, int cols) {
     const long ctas = (long)cdiv(rows, 64) * ((cdiv(cols, 64) + 1) / 2);
     const long want = (2 * 148 + ctas - 1) / ctas;
     return (int)(want < 1 ? 1 : (want > kLossMaxSplit ? kLossMaxSplit : want));
-}
-size_t loss_partials_count(int rows, int cols) {
-    return (size_t)kLossMaxSplit * cdiv(rows, 64) * cdiv(cols, 64);
 }
 
 // Built-in scratch of ptq_sensitivity_order_static: lives in every device that loads the library, until exit.
@@ -706,10 +714,7 @@ int ptq_quantize_layer(const float* W, int rows, int cols, int64_t ldw, const do
 
     const bool want_loss = H_undamped && loss_out;
     double* dW = want_loss ? Wp : nullptr;
-    const bool sliced = want_loss && sliced_loss(rows, n) && n <= kXMaxK &&
-                        x_operand_bytes(rows, n) <= (size_t)rows * n * sizeof(double) &&
-                        x_operand_bytes(n, n) <= (size_t)n * n * sizeof(double) &&
-                        2 * (size_t)x_num_tiles(rows, n) <= loss_partials_count(rows, cols);
+    const bool sliced = want_loss && sliced_loss(rows, n);
     int8_t* kexp = sliced ? reinterpret_cast<int8_t*>(Dbuf) : nullptr;      // the factorisation is done with Dbuf
     {
         Launch l(K_FINALIZE, stream);
