@@ -170,7 +170,10 @@ __device__ __forceinline__ void chol_load_block(double* dst, const double* __res
 constexpr int kStripPanel = 40;                                          // panel columns of a strip
 constexpr int kStripGroups = (kNB + kStripPanel) / 8;                    // column groups: 0 .. 7 diagonal, 8 .. 12 panel
 constexpr int kStripLd = kNB + kStripPanel + 12;                         // row stride of the 8-row panels (116 = 4 mod 16)
-constexpr int kStripCostTiles = 4;                                       // a strip takes about as long as four trailing tiles
+// Trailing tiles that a strip counts for when the pieces are dealt (chol_trailing_phase).  Both factorisations of a layer, by
+// columns, with 3 / 4 / 5: 2048: 1030 / 1007 / 1016 us, 2304: 1273 / 1228 / 1241, 2816: 1875 / 1825 / 1864; the same up to
+// 1536, where the list is shorter than the grid.
+constexpr int kStripCostTiles = 4;
 constexpr int kStripThreads = 32 * kStripGroups;                         // threads of the warps that take part
 constexpr int kStripSmemDoubles = 2 * 8 * kStripLd + 64 /*M*/ + 64 /*W R*/ + 2 * 64 /*W*/ + 2 * 2 * 64 /*R, T*/;
 static_assert(kStripSmemDoubles + 2 * kCholBlock <= kCholOpndDoubles,
@@ -523,7 +526,9 @@ __device__ __noinline__ void chol_trailing_phase(double* __restrict__ A, double*
     const int TW = Wm != nullptr ? R * (k + 1) : 0;
     const int T = TA + TW;
     if (T <= 0) return;
-    // tiles are cut into 64 / H row pieces so that a short tile list still spreads over the grid
+    // Tiles are cut into 64 / H row pieces so that a short tile list still spreads over the grid: in two where there are no
+    // more of them than CTAs (against half as many: 2304 columns 1228.5 -> 1228.0 us, 2816: 1825.8 -> 1824.4, no difference
+    // below), in four where the pieces are still no more than CTAs.
     const int lgH = 4 * T <= G ? 4 : (T <= G ? 5 : 6);
     const int lgP = 6 - lgH;
     const int TP = T << lgP;
@@ -755,8 +760,9 @@ inline int cholesky_upper(double* A, int n, double* Wm, double* Dbuf, unsigned* 
     });
     if (st) return st;
     // One CTA per SM (the cooperative launch guarantees that all of them are resident); a matrix of a few block rows
-    // gets only as many CTAs as it ever has work items, which makes its grid barriers cheaper and leaves SMs to kernels
-    // of other streams.
+    // gets no more CTAs than it has work for, which makes its grid barriers cheaper and leaves SMs to kernels of other
+    // streams.  Twice the 64 x 64 tiles of A and W: never fewer than the strips of a block row, and with W never fewer than the
+    // pieces of its trailing tiles (without W there are up to a third more pieces than CTAs at 7 to 11 block rows).
     const int nbr = (n + kNB - 1) / kNB;
     const long items = 2L * ((long)nbr * (nbr + 1) / 2 + (Wm != nullptr ? (long)nbr * nbr : 0));
     const int budget = coop_cta_budget(dev);

@@ -17,7 +17,8 @@ namespace ptq {
 __device__ __forceinline__ int clamp_index(int j, int n) { return j < 0 ? 0 : (j >= n ? n - 1 : j); }
 
 // invperm[perm[p]] = p; reports entries out of range.  A repeated entry shows once all of invperm is written, see
-// sweep_gather_kernel.  Also clears the counters of the kernels to come (zero: `zeros` words).
+// sweep_gather_kernel.  Also clears the counters of the kernels to come: the factorisation's grid barrier (bar, two words)
+// and the sweep's progress counters (sweep_flags, n_flags words).
 __global__ void __launch_bounds__(256) perm_check_kernel(const int32_t* __restrict__ perm, int cols,
                                                           int32_t* __restrict__ invperm, unsigned* __restrict__ bar,
                                                           unsigned* __restrict__ sweep_flags, int n_flags, int32_t* status) {
