@@ -6,7 +6,9 @@ inverse, grid, column scores + order, column-synchronous quantization sweep, cod
 Workload at N = 1: the ResNet-50-shaped 3x3 convolution as a matrix (W 256 x 2304, X 2304 x 4096 with
 30 % exact zeros, 4-bit per-row asymmetric grid, damping 0.01 * mean(diag H)).
 
-`python bench.py [--gpus N] [--steps K] [--warmup W]` prints ONE JSON line (rank 0).  With N > 1 (torchrun)
+`python bench.py [--gpus N] [--steps K] [--warmup W]` prints ONE JSON line (rank 0), short enough to survive where only
+the last few kilobytes of the output are kept; `--report FILE` writes everything measured (the per-kernel and per-layer
+tables too).  With N > 1 (torchrun)
 every rank quantizes its own replica of the layer (the path is single-GPU: no collective on the data path);
 `value` is the weights quantized per second by all ranks together, timed on the device, max over ranks.
 `--impl reference` times the float64 CPU oracle on the same workload instead.
@@ -278,6 +280,35 @@ def kernel_rooflines(kernels, work, peaks):
     return out
 
 
+LINE_LIMIT = 2500          # characters
+
+
+def bench_line(report):
+    """The line to print: of the report, what identifies and qualifies the result, numbers to six digits."""
+    def short(v):
+        if isinstance(v, dict):
+            return {k: short(x) for k, x in v.items()}
+        if isinstance(v, (list, tuple)):
+            return [short(x) for x in v]
+        return float(f"{v:.6g}") if isinstance(v, float) else v
+
+    out = {k: v for k, v in report.items() if k not in ("value", "ms_per_step", "e2e", "kernels", "layer_sets", "fp64_peak",
+                                                        "context", "roofline")}
+    out = short(out)
+    out.update({k: report[k] for k in ("value", "ms_per_step", "e2e")})
+    out["roofline"] = short({k: v for k, v in report["roofline"].items() if k != "per_kernel"})
+    if report.get("layer_sets"):
+        out["layer_sets_ms"] = short({name: {"one_by_one": t["total_ms"], "graphs": t.get("graph_total_ms"),
+                                             "side_by_side": t.get("overlapped_8_streams_cta_limited_ms")}
+                                      for name, t in report["layer_sets"].items()})
+    line = json.dumps(out)
+    for key in ("layer_sets_ms", "stages_ms"):            # what a longer report may lose first
+        if len(line) > LINE_LIMIT and key in out:
+            del out[key]
+            line = json.dumps(out)
+    return line
+
+
 def run_ours(args):
     import torch
     import torch.distributed as dist
@@ -454,14 +485,18 @@ def run_ours(args):
                                   "gpu_ms_on_the_same_sample": gpu_ms}
 
     if rank == 0:
-        print(json.dumps({
+        report = {
             "metric": METRIC, "value": value, "unit": UNIT, "n_gpus": world, "steps": args.steps,
             "warmup": max(args.warmup, 3), "ms_per_step": ms_per_step, "higher_is_better": True, "scaling": "weak",
             "vs_baseline": None, "dtype": "f64",
             "data": "synthetic", "config": workload_config(spec, world), "clocks": clocks, "e2e": e2e,
             "gpu_launches": int(launches), "roofline": roofline, "cpu_baseline": cpu_baseline,
             "stages_ms": stage_ms, "kernels": kernels, "fp64_peak": peaks["fp64"], "layer_sets": layer_sets,
-            "context": "paper: ResNet-50 whole-model 80 s (FastOBQ) vs 9287 s (OBQ), hardware not stated"}))
+            "context": "paper: ResNet-50 whole-model 80 s (FastOBQ) vs 9287 s (OBQ), hardware not stated"}
+        if args.report:
+            with open(args.report, "w") as f:
+                json.dump(report, f, indent=1)
+        print(bench_line(report))
     if world > 1:
         dist.destroy_process_group()
     return 0
@@ -474,6 +509,7 @@ def main():
     ap.add_argument("--warmup", type=int, default=3)
     ap.add_argument("--impl", default="ours", choices=["ours", "reference"])
     ap.add_argument("--no-cpu-baseline", action="store_true")
+    ap.add_argument("--report", default=None, metavar="FILE", help="write everything measured as JSON (rank 0)")
     ap.add_argument("--no-sets", action="store_true", help="skip the layer-set totals (the single bench layer only)")
     args = ap.parse_args()
     if args.impl == "ours" and args.gpus > 1 and "WORLD_SIZE" not in os.environ:

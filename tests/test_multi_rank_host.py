@@ -60,3 +60,41 @@ def test_reference_arm_runs_on_rank_zero_only(monkeypatch):
         gpus, steps, warmup = 2, 1, 0
     monkeypatch.setenv("RANK", "1")
     assert bench.run_reference(Args()) == 0              # other ranks return at once, without work or output
+
+
+def test_the_bench_line_keeps_its_keys_and_stays_short():
+    """Where only the last few kilobytes of the output are kept, a line with the per-layer tables cannot be read back."""
+    import json
+    import bench
+    x = 123456.78901234567
+    kernel = {"bound": "alu", "achieved": x, "peak": x, "unit": "TFLOP/s", "frac": x, "ms_per_step": x,
+              "launches_per_step": 2, "peak_source": "p" * 140}
+    layer = {"layer": "c3.layer4.0.downsample", "ms": x, "stages_ms": {k: x for k in "abcdef"}, "roofline_frac": {"a": x}}
+    one_set = {"n_layers": 54, "weights": 25502912, "total_ms": x, "weights_per_s": x, "graph_total_ms": x,
+               "overlapped_8_streams_cta_limited_ms": x, "layers": [layer] * 54, "stage_total_ms": {k: x for k in "abcdef"}}
+    report = {
+        "metric": bench.METRIC, "value": x, "unit": bench.UNIT, "n_gpus": 8, "steps": 100, "warmup": 3, "ms_per_step": x,
+        "higher_is_better": True, "scaling": "weak", "vs_baseline": None, "dtype": "f64", "data": "synthetic",
+        "config": bench.workload_config(bench.bench_spec(), 8),
+        "clocks": {"sm_mhz": 1965.0, "sm_max_mhz": 1965.0, "reasons": ["hw_slowdown", "sw_power_cap"], "samples": 100},
+        "e2e": {"value": x, "unit": bench.UNIT, "h2d_bytes_per_step": 40108032, "d2h_bytes_per_step": 589832,
+                "ms_per_step": x},
+        "gpu_launches": 2000,
+        "roofline": dict(kernel, kernel="gram_i8_tcgen05", traffic=x, launch_ms=x, algorithmic_work_per_launch=x,
+                         sweep_ns_per_column=x, per_kernel={f"kernel{i}": kernel for i in range(8)}),
+        "cpu_baseline": {"value": x, "unit": bench.UNIT, "cores": 16, "kind": "oracle", "sample": "s" * 60,
+                         "codes_equal_to_gpu": True, "order_equal_to_gpu": True},
+        "stages_ms": {k: x for k in ("hessian", "inverse", "grid", "order", "sweep")},
+        "kernels": {f"kernel{i}": {"ms_per_step": x, "launches_per_step": 2} for i in range(20)},
+        "fp64_peak": {"dfma_tflops": x, "dmma_tflops": x, "fp64_tflops": x},
+        "layer_sets": {f"c{i}_resnet50_w4": one_set for i in range(4)}, "context": "c" * 90}
+    line = bench.bench_line(report)
+    assert len(line) <= bench.LINE_LIMIT
+    got = json.loads(line)
+    for key in ("metric", "value", "unit", "n_gpus", "steps", "warmup", "ms_per_step", "higher_is_better", "scaling",
+                "vs_baseline", "dtype", "data", "config", "clocks", "e2e", "gpu_launches", "roofline", "cpu_baseline"):
+        assert key in got, key
+    assert got["value"] == x and got["ms_per_step"] == x and got["e2e"] == report["e2e"] and got["config"] == report["config"]
+    assert "layer_sets_ms" in got and "per_kernel" not in got["roofline"]
+    report["roofline"]["peak_source"] = "p" * 500
+    assert len(bench.bench_line(report)) <= bench.LINE_LIMIT
