@@ -41,11 +41,11 @@ INT8_OVER_BF16 = 2.0                                   # nominal dense 4.5 / 2.2
 # profiles/, on the bench workload (Gram: scaled from the 16384-column capture by the calibration columns processed).
 # Each entry names the kernel sources it was taken with; when they have changed since, the traffic is reported as null.
 NCU_TRAFFIC = {
-    "chol_coop": {"bytes_per_launch": (42.38e6 + 3.67e6 + 21.73e6 + 0.44e6) / 2, "sources": ["chol.cuh", "dgemm.cuh"],
-                  "sha256_16": "26deddccb8d33464"},
-    "sweep_coop": {"bytes_per_launch": 29.93e6 + 0.05e6, "sources": ["colloop.cuh"], "sha256_16": "dcc1e793b218823f"},
-    "gram_i8_tcgen05": {"bytes_per_launch": (508.4e6 + 31.9e6) * 4096 / 16384, "sources": ["gram.cuh"],
-                        "sha256_16": "67013082159ad65c"},
+    "chol_coop": {"bytes_per_launch": (45.38e6 + 5.53e6 + 21.63e6 + 0.19e6) / 2, "sources": ["chol.cuh", "dgemm.cuh"],
+                  "sha256_16": "e59387afe85874df"},
+    "sweep_coop": {"bytes_per_launch": 28.71e6 + 0.02e6, "sources": ["colloop.cuh"], "sha256_16": "712ec88ea0625c06"},
+    "gram_i8_tcgen05": {"bytes_per_launch": (507.5e6 + 27.5e6) * 4096 / 16384, "sources": ["gram.cuh"],
+                        "sha256_16": "fcdf7052c8ea150e"},
 }
 
 
