@@ -72,13 +72,20 @@ __device__ __forceinline__ unsigned ld_acquire_u32(const unsigned* p) {
     return v;
 }
 
+__device__ __forceinline__ void red_release_add_u32(unsigned* p, unsigned v) {
+    asm volatile("red.release.gpu.global.add.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
+}
+
 // bar[0]: arrival counter (monotonic, zero at launch), bar[1]: abort word.  Returns false when the CTA must leave.
 // spin_limit: SM clock cycles after which the wait gives up.
+// One thread arrives with a release and waits with an acquire; with the block's own barriers on both sides they order what
+// every thread of the grid wrote before against what every thread reads after.  Full fences around a plain atomic instead
+// cost about 600 clocks per barrier: both factorisations at 1152 columns 248 + 242 -> 242 + 236 us, at 2304 662 + 535 ->
+// 648 + 523.
 __device__ __forceinline__ bool grid_barrier(unsigned* bar, unsigned target, int* s_flag, long long spin_limit) {
     __syncthreads();
     if (threadIdx.x == 0) {
-        __threadfence();
-        atomicAdd(&bar[0], 1u);
+        red_release_add_u32(&bar[0], 1u);
         const long long t0 = clock64();
         int ok = 1;
         unsigned it = 0;
@@ -88,7 +95,6 @@ __device__ __forceinline__ bool grid_barrier(unsigned* bar, unsigned target, int
                 if (clock64() - t0 > spin_limit) { atomicExch(&bar[1], 1u); ok = 0; break; }
             }
         }
-        __threadfence();
         *s_flag = ok;
     }
     __syncthreads();
