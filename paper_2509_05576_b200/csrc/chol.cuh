@@ -48,9 +48,9 @@ __global__ void damp_copy_kernel(const double* __restrict__ H, double* __restric
 // ------------------------------------------------------------------------------------------------------------
 // Blocked upper Cholesky A = U^T U as ONE persistent cooperative kernel (one CTA per SM, 512 threads).
 // For each 64-row block k:
-//   strip phase    every CTA that owns a 40-column panel chunk factorises the 64 x 64 diagonal block itself (all
+//   strip phase    every CTA that owns a panel chunk of 8 to 40 columns factorises the 64 x 64 diagonal block itself (all
 //                  CTAs do the same arithmetic on it, so no broadcast is needed) and applies the same row
-//                  operations to its chunk: the unblocked algorithm on a 64 x 104 strip, eight pivots at a time
+//                  operations to its chunk: the unblocked algorithm on a strip of 64 rows, eight pivots at a time
 //                  (see chol_strip).  That replaces "factor the block, then solve the panel against it".
 //   trailing phase A[i][j] -= U[k][i]^T U[k][j] on the upper 64 x 64 tiles, float64 tensor-core MMA, operands
 //                  double-buffered through shared memory with cp.async.
@@ -64,7 +64,9 @@ constexpr int kCholThreads = 512;
 constexpr int kCholLd = kNB + 4;                               // operand row stride (68 = 4 mod 16: conflict-free)
 constexpr int kCholBlock = kNB * kCholLd;                      // doubles of a 64 x 64 operand block
 constexpr int kCholOpndDoubles = 2 /*operands*/ * 2 /*slots*/ * kCholBlock;
-constexpr size_t kCholSmemBytes = sizeof(double) * kCholOpndDoubles + 16;
+constexpr int kCholMaxBlockRows = 1024;                         // 65535 columns
+constexpr unsigned kStripsOnly = 8u;
+constexpr size_t kCholSmemBytes = sizeof(double) * kCholOpndDoubles + 16 + kCholMaxBlockRows * sizeof(unsigned);
 
 __device__ __forceinline__ unsigned ld_acquire_u32(const unsigned* p) {
     unsigned v;
@@ -148,8 +150,8 @@ __device__ __forceinline__ void chol_load_block(double* dst, const double* __res
 }
 
 // ------------------------------------------------------------------------------------------------------------
-// Strip factorisation: the 64 x 104 strip [diagonal block | 40 panel columns] is held in registers as 8 x 8 MMA accumulator
-// fragments, eight strip columns (one column group, all 64 rows) per warp.  Pivots are taken eight at a time.  For pivot
+// Strip factorisation: the strip [diagonal block | 8 pg panel columns], pg = 1, 2, 3 or 5, is held in registers as 8 x 8 MMA
+// accumulator fragments, eight strip columns (one column group, all 64 rows) per warp.  Pivots are taken eight at a time.  For pivot
 // block b:
 //   1. warp 0 factorises the 8 x 8 diagonal mini-block M = U_M^T U_M (all of M in every lane, so the serial chain of
 //      eight pivots has no data exchange in it) and carries the identity along to obtain W = U_M^-T;
@@ -163,32 +165,37 @@ __device__ __forceinline__ void chol_load_block(double* dst, const double* __res
 // block ahead of or behind the other warps, hence two of each.  It is never two ahead: R and T of block b + 1 leave their
 // owner after the barriers 3 / 4 and 5 of block b; nor two behind: they wait for it at 3 / 4.
 //
-// What bounds a strip is the chain, and what used to bound the chain were the MMAs of other warps: scalar float64
-// instructions queue behind the float64 MMAs of their scheduler (measured: 9 clocks per dependent FMA alone, 137 next to
-// one warp that streams MMAs on the same scheduler, 9 again when the MMAs are on the other three).  So warp 0 has its
-// scheduler to itself: warps 4, 8 and 12 take no part in a strip, and the updates are dealt to the other three schedulers,
-// which is also why a strip has 40 panel columns (twelve warps with one column group each) and not 64: 1800 MMAs over
-// three schedulers then take about as long as the eight chains with their hand-overs.  Measured per block row, from grid
-// barrier to grid barrier, on matrices whose trailing tiles do not fill the GPU: 30.0 k clocks with the chain sharing its
-// scheduler (8 warps, 64 panel columns) -> 26.5 k, of which 4 k before the first chain, 9.9 k in the chains, 6.8 k between
-// them and 4.5 k for stores and the barrier.  One factorisation: 39 -> 30 us at 128 columns, 654 -> 623 us at 2304.
+// What bounds a strip: scalar float64 instructions queue behind the float64 MMAs of their scheduler (measured: 9 clocks per
+// dependent FMA alone, 137 next to one warp that streams MMAs on the same scheduler, 9 again when the MMAs are on the other
+// three).  So warp 0 has its scheduler to itself: warps 4, 8 and 12 take no part in a strip, and the updates are dealt to the
+// other three schedulers.  With 40 panel columns (twelve warps with one column group each) they have 1800 MMAs, 9.8 k clocks at
+// the full rate, and between two hand-outs of W their own sequence (new rows, barrier, update, look-ahead) takes longer than
+// warp 0's.  Narrower strips have fewer (1400 with 24 columns, 1200 with 16, 1000 with 8), but more CTAs factorise the
+// diagonal block, so the width is chosen per block row, by how much trailing work waits (chol_coop_kernel).
 // ------------------------------------------------------------------------------------------------------------
-constexpr int kStripPanel = 40;                                          // panel columns of a strip
-constexpr int kStripGroups = (kNB + kStripPanel) / 8;                    // column groups: 0 .. 7 diagonal, 8 .. 12 panel
-constexpr int kStripLd = kNB + kStripPanel + 12;                         // row stride of the 8-row panels (116 = 4 mod 16)
-// Trailing tiles that a strip counts for when the pieces are dealt (chol_trailing_phase).  Both factorisations of a layer, by
-// columns, with 3 / 4 / 5: 2048: 1030 / 1007 / 1016 us, 2304: 1273 / 1228 / 1241, 2816: 1875 / 1825 / 1864; the same up to
-// 1536, where the list is shorter than the grid.
-constexpr int kStripCostTiles = 4;
-constexpr int kStripThreads = 32 * kStripGroups;                         // threads of the warps that take part
+constexpr int kStripMaxPanel = 40;                                       // most panel columns of a strip
+constexpr int kStripLd = kNB + kStripMaxPanel + 12;                      // row stride of the 8-row panels (116 = 4 mod 16)
+// Column groups (0 .. 7 diagonal, from 8 on panel; 15: the warp takes no part) of the sixteen warps, four bits a warp.  Warps
+// w, w + 4, w + 8 and w + 12 share a scheduler: scheduler 0 holds the chain (group 0) alone, the others about equal shares of
+// the MMAs (a panel group 200, a diagonal group g 38 to 200).
+__device__ __forceinline__ unsigned long long strip_warps(int pg) {
+    return pg == 5 ? 0x231F645F7B9FCA80ull : (pg == 3 ? 0xAFFF142F398F5670ull : (pg == 2 ? 0x2FFF31FF498F5670ull : 0x1FFF2FFF345F6780ull));
+}
+// What a strip counts for when the trailing tiles are dealt, in eighths of a tile: with 40 panel columns, with fewer.  (Both
+// factorisations of a layer with 24 / 32 / 40 for the former: 2048 columns 1030 / 1007 / 1016 us, 2304 1273 / 1228 / 1241.)
+constexpr int kStripCost = 32, kNarrowStripCost = 28;
+// Narrow strips are taken where the trailing tiles are at most this many eighths of a tile for every CTA without a strip.
+// Both factorisations with 12 / 20 / 28: 1600 columns 328 + 307 / 323 + 304 / 344 + 310 us, 2304 663 + 506 / 661 + 503 /
+// 666 + 508, no difference up to 1152.
+constexpr int kNarrowStripWork = 20;
 constexpr int kStripSmemDoubles = 2 * 8 * kStripLd + 64 /*M*/ + 64 /*W R*/ + 2 * 64 /*W*/ + 2 * 2 * 64 /*R, T*/;
 static_assert(kStripSmemDoubles + 2 * kCholBlock <= kCholOpndDoubles,
               "the strip panels and the look-ahead operands alias the trailing-phase operand buffers");
 
-template <int ID, int COUNT>
-__device__ __forceinline__ void named_bar_sync() { asm volatile("bar.sync %0, %1;" ::"n"(ID), "n"(COUNT) : "memory"); }
-template <int ID, int COUNT>
-__device__ __forceinline__ void named_bar_arrive() { asm volatile("bar.arrive %0, %1;" ::"n"(ID), "n"(COUNT) : "memory"); }
+template <int ID>
+__device__ __forceinline__ void named_bar_sync(int count) { asm volatile("bar.sync %0, %1;" ::"n"(ID), "r"(count) : "memory"); }
+template <int ID>
+__device__ __forceinline__ void named_bar_arrive(int count) { asm volatile("bar.arrive %0, %1;" ::"n"(ID), "r"(count) : "memory"); }
 
 struct StripSmem {
     double* R;       // [8][kStripLd] rows of the pivot block (every warp reads back its own columns only)
@@ -222,12 +229,17 @@ template <int RB>
 __device__ __forceinline__ void chol_strip_lookahead(double (&acc)[8][2], const double* ua, const double* bsrc, int grp,
                                                      int lq, int lr) {
     if (grp < 8 && RB > grp) return;            // fragments that lie entirely below the diagonal are never used
-    // summed apart and subtracted once: added one by one to the old value they would be rounded to its size sixteen times
-    double p0 = 0.0, p1 = 0.0;
-#pragma unroll 8
-    for (int kk = 0; kk < kNB; kk += 4) dmma_884(p0, p1, ua[(kk + lr) * kCholLd + 8 * RB + lq], bsrc[(kk + lr) * kCholLd + lq]);
-    acc[RB][0] -= p0;
-    acc[RB][1] -= p1;
+    // summed apart and subtracted once: added one by one to the old value they would be rounded to its size sixteen times.
+    // Two sums, because an MMA waits for the one before on the same accumulator (both factorisations at 1152 columns: 228 +
+    // 217 -> 220 + 209 us; the error of the inverse becomes 1 to 8 % smaller).
+    double p0 = 0.0, p1 = 0.0, q0 = 0.0, q1 = 0.0;
+#pragma unroll 4
+    for (int kk = 0; kk < kNB; kk += 8) {
+        dmma_884(p0, p1, ua[(kk + lr) * kCholLd + 8 * RB + lq], bsrc[(kk + lr) * kCholLd + lq]);
+        dmma_884(q0, q1, ua[(kk + 4 + lr) * kCholLd + 8 * RB + lq], bsrc[(kk + 4 + lr) * kCholLd + lq]);
+    }
+    acc[RB][0] -= p0 + q0;
+    acc[RB][1] -= p1 + q1;
 }
 
 // Step 1 above.  mb: the mini-block M (row-major, 8 x 8, upper part); leaves W in Wbuf.  Returns the first pivot that is not
@@ -282,7 +294,7 @@ __device__ __forceinline__ double2 chol_new_rows(const double* Wbuf, const doubl
 // Warp 0: the chains of all eight pivot blocks and the mini-blocks in between.  first: the first mini-block in accumulator
 // layout (group 0's only fragment in use).  Returns the first eight rows of the factor in those columns.
 __device__ __forceinline__ double2 chol_strip_chain(double2 first, const StripSmem& sm, int lane, int k0, bool reporter,
-                                                    int32_t* status) {
+                                                    int32_t* status, int threads) {
     const int lq = lane >> 2, lr = lane & 3;
     *reinterpret_cast<double2*>(sm.M + lq * 8 + 2 * lr) = first;
     *reinterpret_cast<double2*>(sm.R + lq * kStripLd + 2 * lr) = first;
@@ -291,12 +303,12 @@ __device__ __forceinline__ double2 chol_strip_chain(double2 first, const StripSm
     for (int b = 0; b < 8; ++b) {
         double* Wb = sm.W + (b & 1) * 64;
         const int bad = chol_chain8(sm.M, Wb, lane);
-        if (b & 1) named_bar_arrive<4, kStripThreads>(); else named_bar_arrive<3, kStripThreads>();
+        if (b & 1) named_bar_arrive<4>(threads); else named_bar_arrive<3>(threads);
         if (bad >= 0 && reporter) report(status, PTQ_ERR_NOT_SPD, k0 + 8 * b + bad);
         __syncwarp();
         if (b < 7) {
             const double* X = sm.X + (b & 1) * 128;
-            if (b & 1) named_bar_sync<2, 64>(); else named_bar_sync<1, 64>();      // R and T of the next eight columns are out
+            if (b & 1) named_bar_sync<2>(64); else named_bar_sync<1>(64);      // R and T of the next eight columns are out
             const double2 v = chol_new_rows(Wb, X, 8, lq, lr);
             *reinterpret_cast<double2*>(sm.V + lq * 8 + 2 * lr) = v;
             double2 t = *reinterpret_cast<const double2*>(X + 64 + lq * 8 + 2 * lr);
@@ -315,7 +327,7 @@ __device__ __forceinline__ double2 chol_strip_chain(double2 first, const StripSm
 // Every other warp: pivot block B.
 template <int B>
 __device__ __forceinline__ void chol_strip_block(double (&acc)[8][2], const StripSmem& sm, int grp, int lane, bool update,
-                                                 const double* ua, const double* bsrc) {
+                                                 const double* ua, const double* bsrc, int threads) {
     const int lq = lane >> 2, lr = lane & 3;
     // While warp 0 is in its chain: the update by the pivot block before, and the look-ahead update of the rows of the next
     // pivot block.  The owner of the next eight columns puts out what warp 0 is going to need first; it has brought its next
@@ -329,7 +341,7 @@ __device__ __forceinline__ void chol_strip_block(double (&acc)[8][2], const Stri
         double* X = sm.X + (B & 1) * 128 + lq * 8 + 2 * lr;
         *reinterpret_cast<double2*>(X) = make_double2(acc[B][0], acc[B][1]);
         if constexpr (B < 7) *reinterpret_cast<double2*>(X + 64) = make_double2(acc[B + 1][0], acc[B + 1][1]);
-        named_bar_arrive<1 + (B & 1), 64>();
+        named_bar_arrive<1 + (B & 1)>(64);
     }
     if constexpr (B > 0 && B < 6) chol_strip_update<B + 2, 8>(acc, sm.U, grp, lq, lr);
     if constexpr (B < 7) {
@@ -340,23 +352,23 @@ __device__ __forceinline__ void chol_strip_block(double (&acc)[8][2], const Stri
     }
     // the rows of this pivot block as an MMA operand (read back by this warp only)
     *reinterpret_cast<double2*>(sm.R + lq * kStripLd + 8 * grp + 2 * lr) = make_double2(acc[B][0], acc[B][1]);
-    named_bar_sync<3 + (B & 1), kStripThreads>();             // W is there; nobody reads the previous new rows any more
+    named_bar_sync<3 + (B & 1)>(threads);             // W is there; nobody reads the previous new rows any more
     if (grp >= B) {
         const double2 v = chol_new_rows(sm.W + (B & 1) * 64, sm.R + 8 * grp, kStripLd, lq, lr);
         acc[B][0] = v.x;
         acc[B][1] = v.y;
         *reinterpret_cast<double2*>(sm.U + lq * kStripLd + 8 * grp + 2 * lr) = v;
     }
-    if constexpr (B < 7) named_bar_sync<5, kStripThreads - 32>();             // the new rows are out
+    if constexpr (B < 7) named_bar_sync<5>(threads - 32);             // the new rows are out
 }
 template <int... Bs>
 __device__ __forceinline__ void chol_strip_blocks(double (&acc)[8][2], const StripSmem& sm, int grp, int lane, bool update,
-                                                  const double* ua, const double* bsrc, std::integer_sequence<int, Bs...>) {
-    (chol_strip_block<Bs>(acc, sm, grp, lane, update, ua, bsrc), ...);
+                                                  const double* ua, const double* bsrc, int threads, std::integer_sequence<int, Bs...>) {
+    (chol_strip_block<Bs>(acc, sm, grp, lane, update, ua, bsrc, threads), ...);
 }
 
-// Factorises the diagonal block of A at k0 and applies the same row operations to 40 panel columns with it: columns
-// pc0 .. pc0 + 39 of rows k0 .. k0 + 63 of the matrix P (row stride ld); with add_identity the entries on P's diagonal are
+// Factorises the diagonal block of A at k0 and applies the same row operations to 8 pg panel columns with it: columns
+// pc0 .. pc0 + 8 pg - 1 of rows k0 .. k0 + 63 of the matrix P (row stride ld); with add_identity the entries on P's diagonal are
 // taken as 1 (P = W, zero there in memory: the transform of the identity block is the inverse of the transposed diagonal
 // factor).  P == nullptr: diagonal block only.
 // Every CTA working on this block row reads the diagonal block of A, at a time of its own, so the factor of that
@@ -364,11 +376,11 @@ __device__ __forceinline__ void chol_strip_blocks(double (&acc)[8][2], const Str
 // copies all diagonal factors into A at its very end.
 // look_ahead: the strip is first brought up to date with the previous block row, which is final by then:
 //     strip -= upd_a^T [upd_a | upd_b],   upd_a[kk][r] = U[k0 - 64 + kk][k0 + r],  upd_b[kk][c] = P[k0 - 64 + kk][pc0 + c]
-// (64 x 64 in shared memory, row stride kCholLd; only 40 columns of upd_b are used).
+// (64 rows in shared memory, row stride kCholLd).
 // Not inlined: the chain alone needs nearly all of the 128 registers, and what the kernel keeps across a strip is saved
 // once around the call instead of inside the chain.
 __device__ __noinline__ void chol_strip(double* __restrict__ A, int64_t ld, int n, int k0, double* __restrict__ P,
-                                        int pc0, bool add_identity, bool write_diag, double* __restrict__ D, int vec16,
+                                        int pc0, int pg, bool add_identity, bool write_diag, double* __restrict__ D, int vec16,
                                         int32_t* status, bool look_ahead) {
     extern __shared__ __align__(16) unsigned char chol_smem_raw[];
     double* smem = reinterpret_cast<double*>(chol_smem_raw);
@@ -378,22 +390,21 @@ __device__ __noinline__ void chol_strip(double* __restrict__ A, int64_t ld, int 
     const bool has_b = look_ahead && P != nullptr;
     if (look_ahead) {
         chol_load_block<kCholThreads>(upd_a, A, ld, n, k0 - kNB, k0, 6, vec16, threadIdx.x);
-        if (has_b) chol_load_block<kCholThreads>(upd_b, P, ld, n, k0 - kNB, pc0, 6, vec16, threadIdx.x);
+        if (has_b) chol_load_block<kCholThreads>(upd_b, P, ld, n, k0 - kNB, pc0, pg == 5 ? 6 : (pg == 3 ? 5 : 4), vec16, threadIdx.x);
         cp_async_commit();
     }
-    // Column group of every warp; 15: takes no part.  Warps w, w + 4, w + 8 and w + 12 share a scheduler: scheduler 0 holds
-    // the chain (group 0) alone, the others {8 9 5 1}, {10 11 4 3} and {12 7 6 2}, about 600 MMAs each.
-    const int lane = threadIdx.x & 31, grp = (int)((0x231F645F7B9FCA80ull >> (4 * (threadIdx.x >> 5))) & 15u);
+    const int lane = threadIdx.x & 31, grp = (int)((strip_warps(pg) >> (4 * (threadIdx.x >> 5))) & 15u);
+    const int threads = 32 * (8 + pg);                                       // of the warps that take part
     const int lq = lane >> 2, lr = lane & 3;
     const StripSmem sm(smem);
     const bool is_diag = grp < 8;
     const int gc0 = is_diag ? k0 + 8 * grp : pc0 + 8 * (grp - 8);           // first global column of this warp
     const int sc0 = 8 * grp;                                                 // first strip column
     double acc[8][2];
-    if (grp < kStripGroups) {
+    if (grp < 15) {
         // columns that lie inside the matrix: plain vector loads (of the diagonal block only the fragments from the
         // diagonal up; what lies below the diagonal in the diagonal fragment itself is never used)
-        const bool fast = vec16 && k0 + kNB <= n && (is_diag || (P != nullptr && pc0 + kStripPanel <= n));
+        const bool fast = vec16 && k0 + kNB <= n && (is_diag || (P != nullptr && pc0 + 8 * pg <= n));
         if (fast) {
             const double* src = (is_diag ? A : P) + (int64_t)(k0 + lq) * ld + gc0 + 2 * lr;
 #pragma unroll
@@ -438,18 +449,18 @@ __device__ __noinline__ void chol_strip(double* __restrict__ A, int64_t ld, int 
     if (look_ahead) {
         cp_async_wait<0>();
         __syncthreads();
-        if (update && grp < kStripGroups) chol_strip_lookahead<0>(acc, upd_a, bsrc, grp, lq, lr);
+        if (update && grp < 15) chol_strip_lookahead<0>(acc, upd_a, bsrc, grp, lq, lr);
     }
-    if (grp >= kStripGroups) return;
+    if (grp == 15) return;
     if (grp == 0) {
-        const double2 v = chol_strip_chain(make_double2(acc[0][0], acc[0][1]), sm, lane, k0, write_diag && lane == 0, status);
+        const double2 v = chol_strip_chain(make_double2(acc[0][0], acc[0][1]), sm, lane, k0, write_diag && lane == 0, status, threads);
         if (write_diag) {
             if (2 * lr >= lq) D[lq * kNB + 2 * lr] = v.x;
             if (2 * lr + 1 >= lq) D[lq * kNB + 2 * lr + 1] = v.y;
         }
         return;
     }
-    chol_strip_blocks(acc, sm, grp, lane, update, upd_a, bsrc, std::make_integer_sequence<int, 8>());
+    chol_strip_blocks(acc, sm, grp, lane, update, upd_a, bsrc, threads, std::make_integer_sequence<int, 8>());
     if (is_diag) {
         if (write_diag) {
 #pragma unroll
@@ -517,11 +528,11 @@ __device__ __forceinline__ void chol_pair_store(const CholPiece& pc, double* dst
 //   tiles of A: (i, j), row_base <= i <= j: A[i][j] -= U[k][i]^T U[k][j]
 //   tiles of W: (i, c), row_base <= i, c <= k:  W[i][c] -= U[k][i]^T W[k][c]       (row-major lists, A first)
 // In look-ahead mode the CTAs come here after `strips_b` strips of the next block row, the CTAs 0 .. n_more - 1 after
-// one more; a strip costs about as much as kStripCostTiles tiles, so they take correspondingly fewer pieces (the
-// busier CTAs from the end of the list) and all CTAs finish at about the same time.
+// one more; a strip costs strip_cost eighths of a tile, so they take correspondingly fewer pieces (the busier CTAs from the
+// end of the list) and all CTAs finish at about the same time.
 // Not inlined, for the sake of the registers, like chol_strip.
 __device__ __noinline__ void chol_trailing_phase(double* __restrict__ A, double* __restrict__ Wm, int n, int64_t ld, int vec16,
-                                                 int k, int row_base, int row_limit, int n_more, int strips_b) {
+                                                 int k, int row_base, int row_limit, int n_more, int strips_b, int strip_cost) {
     extern __shared__ __align__(16) unsigned char chol_smem_raw[];
     const int G = gridDim.x, nb = (n + kNB - 1) / kNB;
     const int k0 = k * kNB;
@@ -539,12 +550,13 @@ __device__ __noinline__ void chol_trailing_phase(double* __restrict__ A, double*
     const int lgP = 6 - lgH;
     const int TP = T << lgP;
     const int S = n_more < G ? n_more : G, N = G - S;
-    const int cs = kStripCostTiles << lgP;
+    const int cs = strip_cost << lgP;                                   // in eighths of a piece
     const int cost_a = (strips_b + 1) * cs, cost_b = strips_b * cs;
+    const int all = 8 * TP + S * cost_a + N * cost_b;
     int ps = 0;
     if (S > 0) {
-        const int target = (int)((unsigned)(TP + S * cost_a + N * cost_b + G - 1) / (unsigned)G);
-        ps = target > cost_a ? target - cost_a : 0;
+        // what a strip CTA is short of the average, in whole pieces
+        ps = all > G * cost_a ? (int)((unsigned)(all - G * cost_a + 8 * G - 1) / (unsigned)(8 * G)) : 0;
         if (N == 0) ps = (int)((unsigned)(TP + S - 1) / (unsigned)S);
     }
     const int TPn = TP - S * ps > 0 ? TP - S * ps : 0;
@@ -663,34 +675,47 @@ chol_coop_kernel(double* __restrict__ A, double* __restrict__ Wm, double* __rest
                  int row_limit) {
     extern __shared__ __align__(16) unsigned char chol_smem_raw[];
     int* s_flag = reinterpret_cast<int*>(chol_smem_raw + sizeof(double) * kCholOpndDoubles);
+    unsigned* s_plan = reinterpret_cast<unsigned*>(s_flag + 4);                    // [block rows], see below
     const int tid = threadIdx.x;
     const int G = gridDim.x;
-    const int nb = (n + kNB - 1) / kNB;
+    const int nb = (n + kNB - 1) / kNB, nbs = nb_stop < nb ? nb_stop : nb;
     unsigned epoch = 0;
 
-    // strip work items of block row k: the 40-column chunks of A right of the block, then (with Wm) those of row block k of
-    // W up to the end of the block's own columns, which start as the identity
-    auto chunks_a = [&](int k) { const int w = n - (k + 1) * kNB; return w > 0 ? (w + kStripPanel - 1) / kStripPanel : 0; };
-    auto chunks_w = [&](int k) {
-        const int w = (k + 1) * kNB < n ? (k + 1) * kNB : n;
-        return Wm != nullptr ? (w + kStripPanel - 1) / kStripPanel : 0;
+    // Strip work items of block row k: the chunks of 8 pg columns of A right of the block, then (with Wm) those of row block k
+    // of W up to the end of the block's own columns, which start as the identity.
+    auto chunks = [&](int k, int pg, int& ca, int& all) {
+        const int wa = n - (k + 1) * kNB, ww = Wm != nullptr ? ((k + 1) * kNB < n ? (k + 1) * kNB : n) : 0;
+        ca = wa > 0 ? (int)((unsigned)(wa + 8 * pg - 1) / (unsigned)(8 * pg)) : 0;
+        all = ca + (int)((unsigned)(ww + 8 * pg - 1) / (unsigned)(8 * pg));
+        if (all < 1) all = 1;                                                // last block without Wm: diagonal only
     };
-    auto strip_items = [&](int k) { return chunks_a(k) + chunks_w(k); };
-    auto strip_item = [&](int k, int g, double*& P, int& pc0) {
-        const int ca = chunks_a(k);
-        P = nullptr; pc0 = 0;
-        if (g < ca) { P = A; pc0 = (k + 1) * kNB + g * kStripPanel; }
-        else if (g < strip_items(k)) { P = Wm; pc0 = (g - ca) * kStripPanel; }
-    };
-    // plain strip phase of block row k over the whole grid
-    auto strip_phase = [&](int k) {
-        const int items = strip_items(k);
-        const int reps = items > 0 ? items : 1;                              // last block without Wm: diagonal only
-        for (int g = blockIdx.x; g < reps; g += G) {
-            double* P; int pc0;
-            strip_item(k, g, P, pc0);
-            chol_strip(A, ld, n, k * kNB, P, pc0, P == Wm, g == 0, Dbuf + (size_t)k * kNB * kNB, vec16, status, false);
-            __syncthreads();     // the panel buffers are reused by the next repetition and by the trailing phase
+    // The strips of every block row, worked out once per launch by a thread per block row: a few integer divisions on the way
+    // from one grid barrier to the next cost as much as the whole barrier (both factorisations at 1152 columns: 222 + 209
+    // -> 209 + 195 us without them).  Packed: panel groups, chunks of A << 4, chunks << 17, and whether the strips are all that
+    // their CTAs are due (kStripsOnly).
+    for (int k = k_first + tid; k < nbs; k += kCholThreads) {
+        const int R = (row_limit < nb ? row_limit : nb) - (k + 1), m = nb - (k + 1);
+        const int T = k > k_first && R > 0 ? R * m - R * (R - 1) / 2 + (Wm != nullptr ? R * k : 0) : 0;
+        int pg = 5, ca, all;
+        chunks(k, 5, ca, all);
+        for (int c = 1; c < 5; c += c == 3 ? 2 : 1) {
+            int ca_c, all_c;
+            chunks(k, c, ca_c, all_c);
+            if (all_c <= G && 8 * T <= (G - all_c) * kNarrowStripWork) { pg = c; ca = ca_c; all = all_c; break; }
+        }
+        const bool only = all < G && 8 * T <= (G - all) * (pg == 5 ? kStripCost : kNarrowStripCost);
+        s_plan[k - k_first] = (unsigned)pg | (only ? kStripsOnly : 0u) | (unsigned)ca << 4 | (unsigned)all << 17;
+    }
+    __syncthreads();
+    auto strips = [&](int k, int pg, int ca, int all, bool look_ahead) {
+        for (int g = blockIdx.x; g < all; g += G) {
+            double* P = nullptr;
+            int pc0 = 0;
+            if (g < ca) { P = A; pc0 = (k + 1) * kNB + g * 8 * pg; }
+            else if (Wm != nullptr) { P = Wm; pc0 = (g - ca) * 8 * pg; }
+            __syncthreads();     // the panel buffers are those of the repetition before and of the trailing phase
+            chol_strip(A, ld, n, k * kNB, P, pc0, pg, P == Wm, g == 0, Dbuf + (size_t)k * kNB * kNB, vec16, status, look_ahead);
+            __syncthreads();
         }
     };
     // The block rows k_first .. nb_stop - 1 are factorised (block row k_first must already carry the updates of all rows
@@ -700,29 +725,28 @@ chol_coop_kernel(double* __restrict__ A, double* __restrict__ Wm, double* __rest
     //       the upper triangle of A[64 nb_stop :, 64 nb_stop :] (what Eq. 12 leaves after that many columns);
     //   row_limit = nb_stop : a panel -- only its own block rows are touched; the caller applies the panel to the rows
     //       below it in one product of depth 64 (nb_stop - k_first).
-    const int nbs = nb_stop < nb ? nb_stop : nb;
     const int steps = nbs < nb ? (row_limit > nbs ? nbs : nbs - 1) : nb - 1;
-    strip_phase(k_first);
+    {
+        const unsigned plan = s_plan[0];
+        strips(k_first, (int)(plan & 7u), (int)(plan >> 4 & 0x1fffu), (int)(plan >> 17), false);
+    }
     for (int k = k_first; k < steps; ++k) {
         ++epoch;
         if (!grid_barrier(bar, epoch * (unsigned)G, s_flag, spin_limit)) break;
         // Block row k is final; the updates of block rows < k have been applied everywhere.
         if (k + 1 >= nbs) {                  // last factorised block row of a partial run: its update only
-            chol_trailing_phase(A, Wm, n, ld, vec16, k, k + 1, row_limit, 0, 0);
+            chol_trailing_phase(A, Wm, n, ld, vec16, k, k + 1, row_limit, 0, 0, 0);
             continue;
         }
-        const int next_items = strip_items(k + 1) > 0 ? strip_items(k + 1) : 1;
         // Look-ahead: the CTAs factorise the strips of block row k + 1 first (item g by CTA g mod G; each brings its
         // strip up to date with block row k itself) and then join the trailing tiles of block row k below row k + 1 with
         // a share reduced by what their strips cost, so nobody idles and there is one grid barrier per block row.
-        for (int g = blockIdx.x; g < next_items; g += G) {
-            double* P; int pc0;
-            strip_item(k + 1, g, P, pc0);
-            __syncthreads();
-            chol_strip(A, ld, n, (k + 1) * kNB, P, pc0, P == Wm, g == 0, Dbuf + (size_t)(k + 1) * kNB * kNB, vec16, status, true);
-            __syncthreads();
-        }
-        chol_trailing_phase(A, Wm, n, ld, vec16, k, k + 2, row_limit, next_items % G, next_items / G);
+        const unsigned plan = s_plan[k + 1 - k_first];
+        const int pg = (int)(plan & 7u), all = (int)(plan >> 17);
+        strips(k + 1, pg, (int)(plan >> 4 & 0x1fffu), all, true);
+        if (!(plan & kStripsOnly) || (int)blockIdx.x >= all)
+            chol_trailing_phase(A, Wm, n, ld, vec16, k, k + 2, row_limit, all < G ? all : all % G, all < G ? 0 : all / G,
+                                pg == 5 ? kStripCost : kNarrowStripCost);
     }
     cp_async_wait<0>();
     // the diagonal factors move from the side buffer into A once nobody reads the original diagonal blocks any more
@@ -770,10 +794,12 @@ inline int cholesky_upper(double* A, int n, double* Wm, double* Dbuf, unsigned* 
     if (st) return st;
     // One CTA per SM (the cooperative launch guarantees that all of them are resident); a matrix of a few block rows
     // gets no more CTAs than it has work for, which makes its grid barriers cheaper and leaves SMs to kernels of other
-    // streams.  Twice the 64 x 64 tiles of A and W: never fewer than the strips of a block row, and with W never fewer than the
-    // pieces of its trailing tiles (without W there are up to a third more pieces than CTAs at 7 to 11 block rows).
+    // streams.  Twice the 64 x 64 tiles of A and W, and at least a CTA per eight columns: never fewer than the narrowest strips
+    // of a block row, and with W never fewer than the pieces of its trailing tiles (without W there are up to a third more
+    // pieces than CTAs at 7 to 11 block rows).
     const int nbr = (n + kNB - 1) / kNB;
-    const long items = 2L * ((long)nbr * (nbr + 1) / 2 + (Wm != nullptr ? (long)nbr * nbr : 0));
+    const long tiles2 = 2L * ((long)nbr * (nbr + 1) / 2 + (Wm != nullptr ? (long)nbr * nbr : 0));
+    const long items = tiles2 > (n + 7) / 8 ? tiles2 : (n + 7) / 8;
     const int budget = coop_cta_budget(dev);
     const int grid = items < budget ? (int)(items < 1 ? 1 : items) : budget;
     if (!bar_ready && cudaMemsetAsync(bar, 0, 2 * sizeof(unsigned), stream) != cudaSuccess) return PTQ_ERR_CUDA;

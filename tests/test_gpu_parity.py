@@ -473,6 +473,31 @@ def test_cta_limit_changes_the_grids_not_the_results(rows, cols, limit):
         ptq.set_cta_limit(-1)
 
 
+@pytest.mark.parametrize("cols", [8, 65, 72, 200, 333, 592, 1184])
+def test_widths_of_the_factorisation_strips(cols):
+    """The strips of a block row have 8, 16, 24 or 40 panel columns, the narrowest for which there are CTAs enough (and more
+    than one strip per CTA where even 40 are too few).  CTA limits that force every width, odd sizes and ragged last strips:
+    the inverse is the same bit for bit, and the inverse."""
+    _, X = _layer(4, cols, max(64, 2 * cols), 900 + cols)
+    H = torch.from_numpy(oracle.hessian_accumulate(X)).cuda()
+    out = []
+    for limit in (0, cols // 8 + 1, cols // 16 + 2, cols // 24 + 2, cols // 40 + 2, 3):
+        Hinv, diag, lam = torch.empty_like(H), torch.empty(cols, dtype=torch.float64, device="cuda"), torch.empty(1, dtype=torch.float64, device="cuda")
+        st, ws = ptq.new_status(), ptq.Workspace()
+        ptq.set_cta_limit(limit)
+        try:
+            ptq.prepare_hinv(H, 0.01, ptq.DAMP_REL_MEAN_DIAG, Hinv, diag, lam, ws, st)
+        finally:
+            ptq.set_cta_limit(0)
+        ptq.check_status(st)
+        out.append(Hinv.cpu().numpy())
+    for h in out[1:]:
+        assert np.array_equal(h, out[0])
+    A = H.cpu().numpy() + lam.item() * np.eye(cols)
+    ref = np.linalg.inv(A)
+    assert np.max(np.abs(out[0] - ref)) <= 20 * np.finfo(float).eps * np.linalg.cond(A) * np.max(np.abs(ref))
+
+
 @pytest.mark.gpu
 def test_layer_set_on_several_streams_equals_the_layers_one_by_one():
     """ptq.LayerSet: independent layers side by side on three streams with limited cooperative grids; every layer's
