@@ -457,6 +457,11 @@ int ptq_quantize_layer_dynamic(const float* W, int rows, int cols, int64_t ldw, 
     unsigned* sweep_flags = cv.take<unsigned>((size_t)cdiv(rows, kSweepRows) + 1);
     double* Dbuf = cv.take<double>(chol_scratch_doubles(cols));
     const bool want_loss = H_undamped && loss_out;
+    DeviceState* dev = nullptr;
+    {
+        const int dst = current_device_state(&dev);
+        if (dst) return dst;
+    }
 
     { Launch l(K_DYN_AUX, stream); iota_kernel<<<cdiv(cols, 256), 256, 0, stream>>>(obuf[0], cols); }
     const int32_t* ocur = obuf[0];           // original column index of every current position
@@ -493,9 +498,16 @@ int ptq_quantize_layer_dynamic(const float* W, int rows, int cols, int64_t ldw, 
                 gather_cols_kernel<float><<<dim3(grid_x_for(m, 256), gr), 256, 0, stream>>>(W, ldw, rows, m, ordr, Wn);
             gather_index_kernel<<<cdiv(m, 256), 256, 0, stream>>>(ocur, ordr, m, b, onew, order_out + done);
         }
-        int st = cholesky_upper(An, m, nullptr, Dbuf, bar, status, stream, b < m ? b / kNB : 0);
-        if (st) return st;
-        st = sweep_launch(Wn, An, E, codes_p, scale, zero, rows, b, bits, sweep_flags, status, stream, m);
+        int st = PTQ_OK;
+        const int budget = coop_cta_budget(dev), behind = sweep_ctas_behind(rows, b, m, b < m ? b / kNB : 0, budget);
+        if (behind > 0) {
+            st = factor_sweep_launch(An, m, b < m ? b / kNB : 0, Dbuf, bar, behind, Wn, E, codes_p, scale, zero, rows, b, bits, sweep_flags,
+                                     status, stream, budget, false);
+        } else {
+            st = cholesky_upper(An, m, nullptr, Dbuf, bar, status, stream, b < m ? b / kNB : 0);
+            if (st) return st;
+            st = sweep_launch(Wn, An, E, codes_p, scale, zero, rows, b, bits, sweep_flags, status, stream, m);
+        }
         if (st) return st;
         if (b < m) {
             // Eq. 11 for the columns still to come, all b columns at once: Wn[:, b:] -= E[:, :b] U[:b, b:]
@@ -687,10 +699,18 @@ int ptq_quantize_layer(const float* W, int rows, int cols, int64_t ldw, const do
         const int gy = n + rows < kMaxGridY ? n + rows : kMaxGridY;
         sweep_gather_kernel<<<dim3(grid_x_for(n, 256), gy), 256, 0, stream>>>(Hinv, W, rows, n, ldw, perm, invperm, U, Wp, E, status);
     }
-    int st = cholesky_upper_auto(U, n, nullptr, Dbuf, bar, pws, status, stream, true);   // blocked Eq. 12
+    DeviceState* dev = nullptr;
+    int st = current_device_state(&dev);
+    if (st) return st;
+    // blocked Eq. 12, and the sweep behind it
+    const int budget = coop_cta_budget(dev), behind = pws == nullptr ? sweep_ctas_behind(rows, n, n, 0, budget) : 0;
+    if (behind > 0) st = factor_sweep_launch(U, n, 0, Dbuf, bar, behind, Wp, E, codes_p, scale, zero, rows, n, bits, sweep_flags, status, stream, budget, true);
+    else st = cholesky_upper_auto(U, n, nullptr, Dbuf, bar, pws, status, stream, true);
     if (st) return st;
 
-    if (rows >= kSuperBlockMinRows && n >= 4 * kSuperBlock) {
+    if (behind > 0) {
+        // done
+    } else if (rows >= kSuperBlockMinRows && n >= 4 * kSuperBlock) {
         // Tall and wide layers: the deferred part of Eq. 11 dominates (rows cols^2 / 2 multiply-adds), and inside the sweep
         // kernel it runs as 32 x 64 x 64 tiles.  The columns are therefore swept in super-blocks of 1024; what a
         // super-block owes to all later columns is applied by one large product, W[:, later] -= E[:, sb] U[sb, later],

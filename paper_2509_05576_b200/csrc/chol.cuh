@@ -581,9 +581,9 @@ __device__ __forceinline__ void chol_pair_store(const CholPiece& pc, double* dst
 // end of the list) and all CTAs finish at about the same time.
 // Not inlined, for the sake of the registers, like chol_strip.
 __device__ __noinline__ void chol_trailing_phase(double* __restrict__ A, double* __restrict__ Wm, int n, int64_t ld, int vec16,
-                                                 int k, int row_base, int row_limit, int n_more, int strips_b, int strip_cost) {
+                                                 int G, int k, int row_base, int row_limit, int n_more, int strips_b, int strip_cost) {
     extern __shared__ __align__(16) unsigned char chol_smem_raw[];
-    const int G = gridDim.x, nb = (n + kNB - 1) / kNB;
+    const int nb = (n + kNB - 1) / kNB;
     const int k0 = k * kNB;
     const int m = nb - row_base;                                        // tiles in the first target row
     const int R = (row_limit < nb ? row_limit : nb) - row_base;         // target block rows
@@ -718,15 +718,14 @@ __device__ __noinline__ void chol_trailing_phase(double* __restrict__ A, double*
     else run(std::integral_constant<int, 16>());
 }
 
-__global__ void __launch_bounds__(kCholThreads, 1)
-chol_coop_kernel(double* __restrict__ A, double* __restrict__ Wm, double* __restrict__ Dbuf, int n, int64_t ld,
-                 int vec16, unsigned* bar, int32_t* status, long long spin_limit, int k_first, int nb_stop,
-                 int row_limit) {
+// The whole of it, by the CTAs 0 .. G - 1 of the grid.
+__device__ __forceinline__ void chol_factorise(double* __restrict__ A, double* __restrict__ Wm, double* __restrict__ Dbuf, int n,
+                                               int64_t ld, int vec16, unsigned* bar, int32_t* status, long long spin_limit,
+                                               int k_first, int nb_stop, int row_limit, const int G) {
     extern __shared__ __align__(16) unsigned char chol_smem_raw[];
     int* s_flag = reinterpret_cast<int*>(chol_smem_raw + sizeof(double) * kCholOpndDoubles);
     unsigned* s_plan = reinterpret_cast<unsigned*>(s_flag + 4);                    // [block rows], see below
     const int tid = threadIdx.x;
-    const int G = gridDim.x;
     const int nb = (n + kNB - 1) / kNB, nbs = nb_stop < nb ? nb_stop : nb;
     unsigned epoch = 0;
 
@@ -784,7 +783,7 @@ chol_coop_kernel(double* __restrict__ A, double* __restrict__ Wm, double* __rest
         if (!grid_barrier(bar, epoch * (unsigned)G, s_flag, spin_limit)) break;
         // Block row k is final; the updates of block rows < k have been applied everywhere.
         if (k + 1 >= nbs) {                  // last factorised block row of a partial run: its update only
-            chol_trailing_phase(A, Wm, n, ld, vec16, k, k + 1, row_limit, 0, 0, 0);
+            chol_trailing_phase(A, Wm, n, ld, vec16, G, k, k + 1, row_limit, 0, 0, 0);
             continue;
         }
         // Look-ahead: the CTAs factorise the strips of block row k + 1 first (item g by CTA g mod G; each brings its
@@ -794,7 +793,7 @@ chol_coop_kernel(double* __restrict__ A, double* __restrict__ Wm, double* __rest
         const int pg = (int)(plan & 7u), all = (int)(plan >> 17);
         strips(k + 1, pg, (int)(plan >> 4 & 0x1fffu), all, true);
         if (!(plan & kStripsOnly) || (int)blockIdx.x >= all)
-            chol_trailing_phase(A, Wm, n, ld, vec16, k, k + 2, row_limit, all < G ? all : all % G, all < G ? 0 : all / G,
+            chol_trailing_phase(A, Wm, n, ld, vec16, G, k, k + 2, row_limit, all < G ? all : all % G, all < G ? 0 : all / G,
                                 pg == 5 ? kStripCost : kNarrowStripCost);
     }
     cp_async_wait<0>();
@@ -811,12 +810,30 @@ chol_coop_kernel(double* __restrict__ A, double* __restrict__ Wm, double* __rest
     if (tid == 0 && ld_acquire_u32(&bar[1]) != 0u) report(status, PTQ_ERR_TIMEOUT, blockIdx.x, 1);
 }
 
+__global__ void __launch_bounds__(kCholThreads, 1)
+chol_coop_kernel(double* __restrict__ A, double* __restrict__ Wm, double* __restrict__ Dbuf, int n, int64_t ld,
+                 int vec16, unsigned* bar, int32_t* status, long long spin_limit, int k_first, int nb_stop,
+                 int row_limit) {
+    chol_factorise(A, Wm, Dbuf, n, ld, vec16, bar, status, spin_limit, k_first, nb_stop, row_limit, gridDim.x);
+}
+
 // In-place blocked upper Cholesky A = U^T U of the n x n matrix A (row stride n).  Only the upper triangle is read or
 // written.  With Wm (n x n, zero on entry) the same sweep also leaves W = U^-T there (lower triangular): the row
 // operations of the factorisation are applied to the identity, which gives the inverse of the Cholesky factor that
 // Sec. 5 item 1 asks for.
 // `bar` is 2 x uint32 of device scratch, Dbuf holds chol_scratch_doubles(n) doubles (the diagonal factors on their way).
 inline size_t chol_scratch_doubles(int n) { return (size_t)((n + kNB - 1) / kNB) * kNB * kNB; }
+// One CTA per SM (the cooperative launch guarantees that all of them are resident); a matrix of a few block rows
+// gets no more CTAs than it has work for, which makes its grid barriers cheaper and leaves SMs to kernels of other
+// streams.  Twice the 64 x 64 tiles of A and W, and at least a CTA per eight columns: never fewer than the narrowest strips
+// of a block row, and with W never fewer than the pieces of its trailing tiles (without W there are up to a third more
+// pieces than CTAs at 7 to 11 block rows).
+inline int chol_grid(int n, bool with_w, int budget) {
+    const int nbr = cdiv(n, kNB);
+    const long tiles2 = 2L * ((long)nbr * (nbr + 1) / 2 + (with_w ? (long)nbr * nbr : 0));
+    const long items = tiles2 > (n + 7) / 8 ? tiles2 : (n + 7) / 8;
+    return items < budget ? (int)(items < 1 ? 1 : items) : budget;
+}
 // nb_stop > 0: factorise the block rows k_first .. nb_stop - 1 only (see the kernel for what row_limit selects;
 // row_limit <= 0: all rows below are updated).  A partial run that updates everything below must not ask for Wm.
 // bar_ready: the caller has cleared `bar`.
@@ -841,16 +858,7 @@ inline int cholesky_upper(double* A, int n, double* Wm, double* Dbuf, unsigned* 
         return (e == cudaSuccess && per_sm < 1) ? cudaErrorLaunchOutOfResources : e;
     });
     if (st) return st;
-    // One CTA per SM (the cooperative launch guarantees that all of them are resident); a matrix of a few block rows
-    // gets no more CTAs than it has work for, which makes its grid barriers cheaper and leaves SMs to kernels of other
-    // streams.  Twice the 64 x 64 tiles of A and W, and at least a CTA per eight columns: never fewer than the narrowest strips
-    // of a block row, and with W never fewer than the pieces of its trailing tiles (without W there are up to a third more
-    // pieces than CTAs at 7 to 11 block rows).
-    const int nbr = (n + kNB - 1) / kNB;
-    const long tiles2 = 2L * ((long)nbr * (nbr + 1) / 2 + (Wm != nullptr ? (long)nbr * nbr : 0));
-    const long items = tiles2 > (n + 7) / 8 ? tiles2 : (n + 7) / 8;
-    const int budget = coop_cta_budget(dev);
-    const int grid = items < budget ? (int)(items < 1 ? 1 : items) : budget;
+    const int grid = chol_grid(n, Wm != nullptr, coop_cta_budget(dev));
     if (!bar_ready && cudaMemsetAsync(bar, 0, 2 * sizeof(unsigned), stream) != cudaSuccess) return PTQ_ERR_CUDA;
     int64_t ld = n;
     int vec16 = ((n & 1) == 0 && aligned16(A) && aligned16(Wm)) ? 1 : 0;

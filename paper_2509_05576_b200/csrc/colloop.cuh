@@ -10,6 +10,7 @@
 #include "dgemm.cuh"
 #include "order.cuh"
 #include "chol.cuh"
+#include <cmath>
 #include <utility>
 
 namespace ptq {
@@ -104,6 +105,9 @@ struct SweepParams {
     unsigned* flags;        // [groups] published 8-column pieces of E per group, then [1] abort word; zero at launch
     int32_t* status;
     long long spin_limit;   // SM clock cycles after which a wait on another CTA gives up
+    const double* diag;             // behind a factorisation: the diagonal blocks of the factor, 64 x 64 each,
+    unsigned* rows_done;            // its barrier (arrivals, abort word)
+    unsigned row_arrivals;          // and the arrivals per block row
 };
 
 // Waits (one thread) until *counter >= target.  Gives up when the abort word is raised or after spin_limit cycles, in
@@ -196,7 +200,18 @@ __device__ __forceinline__ bool sweep_chain8(double (&v)[8], double (&lev)[8], c
     return danger;
 }
 
-__global__ void __launch_bounds__(kSweepThreads, 1) sweep_coop_kernel(SweepParams prm) {
+// The sweep by the CTAs `first_cta` .. of the grid, kSweepThreads threads each (barrier 8: with BEHIND the block has more).
+// BEHIND: the factor is being made by the CTAs before them (factor_sweep_kernel).  Block row b of it is final once all of them have
+// arrived at their grid barrier b + 1 times; its diagonal block is then in prm.diag.
+__device__ __forceinline__ void sweep_sync() { asm volatile("bar.sync 8, %0;" ::"n"(kSweepThreads) : "memory"); }
+__device__ __forceinline__ bool sweep_sync_or(bool p) {
+    int r;
+    asm volatile("{\n\t.reg .pred p, q;\n\tsetp.ne.s32 p, %1, 0;\n\tbar.red.or.pred q, 8, %2, p;\n\tselp.s32 %0, 1, 0, q;\n\t}"
+                 : "=r"(r) : "r"((int)p), "n"(kSweepThreads) : "memory");
+    return r != 0;
+}
+template <bool BEHIND>
+__device__ __forceinline__ void sweep_columns(const SweepParams& prm, const int cta, const int G) {
     extern __shared__ __align__(16) unsigned char sweep_smem[];
     double* Us = reinterpret_cast<double*>(sweep_smem);                // [64][68] diagonal block of U, rows / pivot
     double* rdiag = Us + kNB * kSweepLd;                               // [64] 1 / U_pp
@@ -213,19 +228,18 @@ __global__ void __launch_bounds__(kSweepThreads, 1) sweep_coop_kernel(SweepParam
     const int64_t ld = prm.ld;
     const int nb = (n + kNB - 1) / kNB;
     const int groups = (rows + kSweepRows - 1) / kSweepRows;
-    const int G = gridDim.x;
     unsigned* abort_word = prm.flags + groups;
     const double maxq = (double)((1 << prm.bits) - 1);
     const int lq = lane >> 2, lr = lane & 3;
     // far-update MMA tile coordinates: 8 warps as 2 x 4, each 16 x 16
     const int wm0 = (warp >> 2) * 16, wn0 = (warp & 3) * 16;
 
-    int cpg = 1, g_first = blockIdx.x, g_step = G, ci = 0;
+    int cpg = 1, g_first = cta, g_step = G, ci = 0;
     if (groups < G) {
         const int per = G / groups;                // CTAs reserved per group; only the first cpg of them work
         cpg = per < nb ? per : nb;
-        g_first = blockIdx.x / per;
-        ci = blockIdx.x - g_first * per;
+        g_first = cta / per;
+        ci = cta - g_first * per;
         g_step = groups;                           // one group per CTA
         if (g_first >= groups || ci >= cpg) return;
     }
@@ -237,13 +251,27 @@ __global__ void __launch_bounds__(kSweepThreads, 1) sweep_coop_kernel(SweepParam
         for (int idx = tid; idx < kNB * kNB; idx += kSweepThreads) {
             const int r = idx >> 6, c = idx & 63;
             double v = (r == c) ? 1.0 : 0.0;
-            if (r < kb && c < kb && c >= r) v = __ldcg(prm.U + (int64_t)(p0 + r) * ld + p0 + c);
+            if (r < kb && c < kb && c >= r)
+                v = BEHIND ? __ldcg(prm.diag + (int64_t)b * kNB * kNB + idx) : __ldcg(prm.U + (int64_t)(p0 + r) * ld + p0 + c);
             Us[r * kSweepLd + c] = v;
         }
-        __syncthreads();
+        sweep_sync();
         if (tid < kNB) rdiag[tid] = 1.0 / Us[tid * kSweepLd + tid];
-        __syncthreads();
+        sweep_sync();
         for (int idx = tid; idx < kNB * kNB; idx += kSweepThreads) Us[(idx >> 6) * kSweepLd + (idx & 63)] *= rdiag[idx >> 6];
+    };
+
+    // block row b of the factor is there (known_rows: as many as are known to be)
+    int known_rows = 0;
+    auto wait_row = [&](int b) {
+        if (!BEHIND || b < known_rows) return true;
+        if (tid == 0) *s_flag = bounded_counter_wait(prm.rows_done, (unsigned)(b + 1) * prm.row_arrivals, prm.rows_done + 1, prm.spin_limit) ? 1 : 0;
+        sweep_sync();
+        const bool ok = *s_flag != 0;
+        sweep_sync();
+        known_rows = b + 1;
+        if (!ok && tid == 0) report(prm.status, PTQ_ERR_TIMEOUT, blockIdx.x, 6);
+        return ok;
     };
 
     for (int g = g_first; g < groups; g += g_step) {
@@ -266,15 +294,16 @@ __global__ void __launch_bounds__(kSweepThreads, 1) sweep_coop_kernel(SweepParam
             // is still being quantized, just as the owner of block b + 1 does: the deferred update of a block by the two
             // blocks before it then never waits for the group's counter, which is what used to delay its owner.
             const bool next2_mine = cpg >= 4 && b + 2 < nb && ((b + 2) % cpg) == ci;
+            if ((next2_mine || next_mine || mine) && !wait_row(next2_mine ? b + 2 : (next_mine ? b + 1 : b))) return;
             if (next2_mine) {
-                __syncthreads();
+                sweep_sync();
                 sweep_load_tile(Bb, kSweepLd, prm.U, ld, p0, p0 + 2 * kNB, kNB, kNB, n, n, prm.vec16);
                 cp_async_commit();
                 load_diag(b + 2);            // nothing of it depends on E: out of the way two blocks early
             }
             if (next_mine) {
                 // block b + 1 is quantized here next: what does not depend on E[:, b] is fetched before waiting for it
-                __syncthreads();
+                sweep_sync();
                 sweep_load_tile(Bb, kSweepLd, prm.U, ld, p0, p0 + kNB, kNB, kNB, n, n, prm.vec16);
                 cp_async_commit();
                 if (!ahead) load_diag(b + 1);
@@ -282,7 +311,7 @@ __global__ void __launch_bounds__(kSweepThreads, 1) sweep_coop_kernel(SweepParam
             if (mine) {
                 // ------------------------------------------------------------ quantize block b
                 if (!prepared) {
-                    __syncthreads();
+                    sweep_sync();
                     load_diag(b);
 #pragma unroll
                     for (int a = 0; a < 4; ++a)
@@ -292,7 +321,7 @@ __global__ void __launch_bounds__(kSweepThreads, 1) sweep_coop_kernel(SweepParam
                             blk[a][e] = (r < rows && c < n) ? __ldcg(prm.Wp + (int64_t)r * ld + c) : 0.0;
                         }
                 }
-                __syncthreads();
+                sweep_sync();
 #pragma unroll
                 for (int m = 0; m < 8; ++m) {
                     double* dm = Dm + (m & 1) * kSweepRows * kSweepDLd;
@@ -377,7 +406,7 @@ __global__ void __launch_bounds__(kSweepThreads, 1) sweep_coop_kernel(SweepParam
                         }
                     }
                 }
-                __syncthreads();
+                sweep_sync();
                 for (int idx = tid; idx < kSweepRows * kNB; idx += kSweepThreads) {
                     const int r = idx >> 6, c = idx & 63;
                     if (r0 + r < rows && c < kb) prm.codes_p[(int64_t)(r0 + r) * ld + p0 + c] = Cs[r * (kNB + 4) + c];
@@ -391,7 +420,8 @@ __global__ void __launch_bounds__(kSweepThreads, 1) sweep_coop_kernel(SweepParam
                     __threadfence();
                     *s_flag = ok;
                 }
-                __syncthreads();
+                sweep_sync();
+                if (BEHIND) known_rows = b + 1;          // its owner had it
                 if (*s_flag == 0) {
                     cp_async_wait<0>();
                     if (tid == 0) report(prm.status, PTQ_ERR_TIMEOUT, blockIdx.x, 2);
@@ -418,7 +448,7 @@ __global__ void __launch_bounds__(kSweepThreads, 1) sweep_coop_kernel(SweepParam
                 sweep_load_tile(Ea, kSweepLd, prm.E, ld, r0, p0, kSweepRows, kNB, rows, n, prm.vec16);
                 cp_async_commit();
                 cp_async_wait<0>();
-                __syncthreads();             // U[b, b + 1] (or U[b, b + 2]) is in Bb, the snapshot of E[:, b] in Ea
+                sweep_sync();             // U[b, b + 1] (or U[b, b + 2]) is in Bb, the snapshot of E[:, b] in Ea
                 // E[:, b] arrives eight columns at a time.  Every warp polls the group's counter for itself (bounded),
                 // requests the operand of piece m straight from global memory as soon as it is out, and meanwhile
                 // multiplies piece m - 1, whose operand was requested one piece earlier.
@@ -473,7 +503,7 @@ __global__ void __launch_bounds__(kSweepThreads, 1) sweep_coop_kernel(SweepParam
                         }
                     }
                 }
-                if (__syncthreads_or(ok ? 0 : 1)) {
+                if (sweep_sync_or(!ok)) {
                     if (tid == 0) report(prm.status, PTQ_ERR_TIMEOUT, blockIdx.x, 3);
                     return;
                 }
@@ -486,13 +516,14 @@ __global__ void __launch_bounds__(kSweepThreads, 1) sweep_coop_kernel(SweepParam
                 ahead = !next_mine;
                 continue;
             }
+            if (!wait_row(b)) return;
             const int b_first = b + 1 + (((ci - (b + 1)) % cpg) + cpg) % cpg;     // first owned block beyond b
             if (b_first >= nb) break;                                               // nothing left for this CTA
             const int e_lo = lazy;
             lazy = b + 1;
             for (int e = e_lo; e <= b; ++e) {
                 // operand A: E[r0 .. r0+31][64 e .. 64 e + 63]
-                __syncthreads();
+                sweep_sync();
                 sweep_load_tile(Ea, kSweepLd, prm.E, ld, r0, e * kNB, kSweepRows, kNB, rows, n, prm.vec16);
                 int stage = 0;
                 sweep_load_tile(Bb, kSweepLd, prm.U, ld, e * kNB, b_first * kNB, kNB, kNB, n, n, prm.vec16);
@@ -527,7 +558,7 @@ __global__ void __launch_bounds__(kSweepThreads, 1) sweep_coop_kernel(SweepParam
                         }
                     }
                     cp_async_wait<1>();
-                    __syncthreads();
+                    sweep_sync();
                     const double* bs = Bb + stage * kNB * kSweepLd;
 #pragma unroll 4
                     for (int kk = 0; kk < kNB; kk += 4) {
@@ -557,13 +588,34 @@ __global__ void __launch_bounds__(kSweepThreads, 1) sweep_coop_kernel(SweepParam
                             }
                         }
                     }
-                    __syncthreads();     // all warps are done with this stage before it is refilled
+                    sweep_sync();     // all warps are done with this stage before it is refilled
                     stage ^= 1;
                 }
                 cp_async_wait<0>();
             }
-            __syncthreads();             // the updated blocks are read back through global memory later
+            sweep_sync();             // the updated blocks are read back through global memory later
         }
+    }
+}
+
+__global__ void __launch_bounds__(kSweepThreads, 1) sweep_coop_kernel(SweepParams prm) {
+    sweep_columns<false>(prm, blockIdx.x, gridDim.x);
+}
+
+struct FactorArgs {
+    double* A;
+    double* Dbuf;
+    int n, vec16, nb_stop, row_limit, ctas;
+    int64_t ld;
+    unsigned* bar;
+    int32_t* status;
+    long long spin_limit;
+};
+__global__ void __launch_bounds__(kCholThreads, 1) factor_sweep_kernel(FactorArgs f, SweepParams prm) {
+    if ((int)blockIdx.x < f.ctas) {
+        chol_factorise(f.A, nullptr, f.Dbuf, f.n, f.ld, f.vec16, f.bar, f.status, f.spin_limit, 0, f.nb_stop, f.row_limit, f.ctas);
+    } else if (threadIdx.x < kSweepThreads) {
+        sweep_columns<true>(prm, blockIdx.x - f.ctas, gridDim.x - f.ctas);
     }
 }
 
@@ -607,10 +659,84 @@ inline int sweep_launch(double* Wp, const double* U, double* E, uint8_t* codes_p
     prm.rows = rows; prm.n = n; prm.bits = bits; prm.ld = ld;
     prm.vec16 = ((n & 1) == 0 && (ld & 1) == 0 && aligned16(Wp) && aligned16(U) && aligned16(E)) ? 1 : 0;
     prm.flags = flags; prm.status = status; prm.spin_limit = kSpinLimitCycles;
+    prm.diag = nullptr; prm.rows_done = nullptr; prm.row_arrivals = 0;
     void* args[] = {&prm};
     Launch l(K_SWEEP_COOP, stream);
     if (cudaLaunchCooperativeKernel((const void*)sweep_coop_kernel, dim3(grid), dim3(kSweepThreads), args,
                                     kSweepSmemBytes, stream) != cudaSuccess) {
+        cudaGetLastError();
+        return PTQ_ERR_CUDA;
+    }
+    return PTQ_OK;
+}
+
+// How many of `budget` CTAs the sweep of the first sweep_n columns gets when it runs behind the factorisation (of the block rows
+// below nb_stop of n columns) in one launch, or 0: one after the other.  From a model of both, in microseconds, fitted to
+// their measured times (within about 10 % of them from 64 to 2900 columns, 16 to 3000 rows and 18 to 148 CTAs):
+//   factorisation  sqrt(chain^2 + (work / CTAs)^2), 11.5 per block row in the chain, 3.6 per trailing tile, 12.8 per block
+//                  row and remaining block for the strips;
+//   sweep          0.11 per column in the chain, 2.6e-4 per column pair and row group for the deferred updates, which the
+//                  CTAs of a group share.
+// Behind one another they take the longer of the two; a tenth is asked of them to be worth it.  Measured, one after the
+// other -> one launch: 64 x 128 50 -> 36 us, 128 x 576 175 -> 115, 128 x 1152 334 -> 220, 1000 x 1152 372 -> 260, 256 x 2304
+// 742 -> 568, 1000 x 2048 811 -> 711, 1000 x 2900 1490 -> 1441, 2000 x 1152 478 -> 402; not taken: 2000 x 2048 1107 -> 1318.
+inline int sweep_ctas_behind(int rows, int sweep_n, int n, int nb_stop, int budget) {
+    const int groups = cdiv(rows, kSweepRows), nb = cdiv(n, kNB), nbs = nb_stop > 0 && nb_stop < nb ? nb_stop : nb;
+    if (groups >= budget) return 0;
+    double work = 0.0;
+    for (int k = 0; k < nbs; ++k) work += (1.8 * (nb - k) + 12.8) * (nb - k);
+    const double chain = 11.5 * nbs, update = 2.6e-4 * (double)sweep_n * sweep_n, steps = 0.11 * sweep_n;
+    auto factor = [&](int ctas) { return std::sqrt(chain * chain + (work / ctas) * (work / ctas)); };
+    const int most = budget / groups < cdiv(sweep_n, kNB) ? budget / groups : cdiv(sweep_n, kNB);
+    const double apart = factor(budget) + update / most + steps;
+    int best = 0;
+    double t_best = 0.9 * apart;
+    for (int per = 1; per <= most && groups * per < budget; ++per) {
+        const double f = factor(budget - groups * per), w = update / per + steps, t = f > w ? f : w;
+        if (t < t_best) { t_best = t; best = groups * per; }
+    }
+    return best;
+}
+
+// The factorisation of U (n x n, row stride n; block rows below nb_stop, 0: all) and the sweep of its first `sweep_n` columns
+// in one launch.
+inline int factor_sweep_launch(double* U, int n, int nb_stop, double* Dbuf, unsigned* bar, int sweep_ctas, double* Wp, double* E,
+                               uint8_t* codes_p, const float* scale, const float* zero, int rows, int sweep_n, int bits,
+                               unsigned* flags, int32_t* status, cudaStream_t stream, int budget, bool ready) {
+    DeviceState* dev = nullptr;
+    int st = current_device_state(&dev);
+    if (st) return st;
+    if (!dev->coop) return PTQ_ERR_UNSUPPORTED;
+    constexpr size_t smem = kCholSmemBytes > kSweepSmemBytes ? kCholSmemBytes : kSweepSmemBytes;
+    st = ensure_smem_attr(dev, SA_FACTOR_SWEEP, [] {
+        cudaError_t e = cudaFuncSetAttribute(factor_sweep_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        int per_sm = 0;
+        if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, factor_sweep_kernel, kCholThreads, smem);
+        return (e == cudaSuccess && per_sm < 1) ? cudaErrorLaunchOutOfResources : e;
+    });
+    if (st) return st;
+    const int groups = cdiv(rows, kSweepRows), nb = cdiv(n, kNB);
+    if (!ready) {
+        if (cudaMemsetAsync(bar, 0, 2 * sizeof(unsigned), stream) != cudaSuccess ||
+            cudaMemsetAsync(flags, 0, ((size_t)groups + 1) * sizeof(unsigned), stream) != cudaSuccess ||
+            cudaMemset2DAsync(E, (size_t)n * sizeof(double), 0xFF, (size_t)sweep_n * sizeof(double), (size_t)rows, stream) != cudaSuccess)
+            return PTQ_ERR_CUDA;
+    }
+    FactorArgs f;
+    f.A = U; f.Dbuf = Dbuf; f.n = n; f.ld = n; f.nb_stop = nb_stop > 0 ? nb_stop : nb; f.row_limit = nb;
+    f.vec16 = ((n & 1) == 0 && aligned16(U)) ? 1 : 0;
+    f.ctas = chol_grid(n, false, budget - sweep_ctas);
+    f.bar = bar; f.status = status; f.spin_limit = kSpinLimitCycles;
+    SweepParams prm;
+    prm.Wp = Wp; prm.U = U; prm.E = E; prm.codes_p = codes_p; prm.scale = scale; prm.zero = zero;
+    prm.rows = rows; prm.n = sweep_n; prm.bits = bits; prm.ld = n;
+    prm.vec16 = (f.vec16 && (sweep_n & 1) == 0 && aligned16(Wp) && aligned16(E)) ? 1 : 0;
+    prm.flags = flags; prm.status = status; prm.spin_limit = kSpinLimitCycles;
+    prm.diag = Dbuf; prm.rows_done = bar; prm.row_arrivals = (unsigned)f.ctas;
+    void* args[] = {&f, &prm};
+    Launch l(K_FACTOR_SWEEP, stream);
+    if (cudaLaunchCooperativeKernel((const void*)factor_sweep_kernel, dim3(f.ctas + sweep_ctas), dim3(kCholThreads), args, smem,
+                                    stream) != cudaSuccess) {
         cudaGetLastError();
         return PTQ_ERR_CUDA;
     }

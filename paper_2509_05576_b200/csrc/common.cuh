@@ -116,7 +116,7 @@ constexpr long long kSpinLimitCycles = 4000000000LL;
 // (cudaFuncSetAttribute is per device).  One table, one mutex; looked up with the caller's device current.
 // ---------------------------------------------------------------------------------------------------------
 constexpr int kMaxDevices = 64;
-enum SmemAttrSlot { SA_CHOL = 0, SA_SWEEP, SA_GRAM, SA_DGEMM, SA_SMALL, SA_XGEMM, SA_COUNT };
+enum SmemAttrSlot { SA_CHOL = 0, SA_SWEEP, SA_GRAM, SA_DGEMM, SA_SMALL, SA_XGEMM, SA_FACTOR_SWEEP, SA_COUNT };
 struct DeviceState {
     int sms = 0;
     int coop = 0;
@@ -167,7 +167,7 @@ enum KernelId {
     K_DGEMM_LAUUM, K_MINMAX_GRID, K_SCORE_PARTIAL,
     K_SCORE_FINAL, K_RANK_SORT, K_PERM_CHECK, K_SWEEP_GATHER, K_SWEEP_COOP, K_FINALIZE,
     K_DGEMM_LOSS, K_SUM_PARTIALS, K_SELFTEST, K_FP64_PROBE, K_DYN_AUX, K_DYN_GATHER,
-    K_DGEMM_DYN, K_PER_ROW, K_DGEMM_EQ11, K_X_SLICE, K_X_GEMM, K_COUNT
+    K_DGEMM_DYN, K_PER_ROW, K_DGEMM_EQ11, K_X_SLICE, K_X_GEMM, K_FACTOR_SWEEP, K_COUNT
 };
 
 inline const char* kernel_name(int id) {
@@ -176,7 +176,7 @@ inline const char* kernel_name(int id) {
         "dgemm_lauum",
         "minmax_grid", "score_partial", "score_final", "rank_sort", "perm_check", "sweep_gather",
         "sweep_coop", "finalize", "dgemm_loss", "sum_partials", "selftest", "fp64_probe", "dyn_aux", "dyn_gather",
-        "dgemm_dyn", "per_row", "dgemm_eq11", "x_slice", "i8gemm_tcgen05"};
+        "dgemm_dyn", "per_row", "dgemm_eq11", "x_slice", "i8gemm_tcgen05", "factor_sweep"};
     return (id >= 0 && id < K_COUNT) ? names[id] : "unknown";
 }
 

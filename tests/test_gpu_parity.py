@@ -473,6 +473,27 @@ def test_cta_limit_changes_the_grids_not_the_results(rows, cols, limit):
         ptq.set_cta_limit(-1)
 
 
+@pytest.mark.parametrize("rows,cols", [(1, 64), (33, 65), (40, 130), (100, 577), (300, 640), (129, 1153)])
+def test_sweep_behind_the_factorisation_equals_one_after_the_other(rows, cols):
+    """Where it pays, the factorisation of the permuted inverse and the sweep run in one launch, the sweep a few block rows
+    behind.  With no more CTAs than row groups they run one after the other: same arrays, bit for bit.  One block row, odd
+    sizes, ragged last blocks and row groups."""
+    W, X = _layer(rows, cols, 256, 77 + cols)
+    names = [ptq.lib().ptq_kernel_name(k).decode() for k in range(ptq.lib().ptq_kernel_count())]
+    fs = names.index("factor_sweep")
+    before = ptq.launch_count(fs)
+    g = gpu_layer(W, X, 4)
+    assert ptq.launch_count(fs) == before + 1
+    ptq.set_cta_limit((rows + 31) // 32)
+    try:
+        h = gpu_layer(W, X, 4)
+    finally:
+        ptq.set_cta_limit(0)
+    assert ptq.launch_count(fs) == before + 1
+    for k in ("perm", "codes", "What", "loss"):
+        assert np.array_equal(h[k], g[k]), k
+
+
 @pytest.mark.parametrize("cols", [8, 65, 72, 200, 333, 592, 1184])
 def test_widths_of_the_factorisation_strips(cols):
     """The strips of a block row have 8, 16, 24 or 40 panel columns, the narrowest for which there are CTAs enough (and more
