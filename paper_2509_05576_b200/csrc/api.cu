@@ -87,11 +87,14 @@ int order_launch(const float* W, int rows, int cols, int64_t ldw, const double* 
     if (chunks > 65535) return PTQ_ERR_UNSUPPORTED;
     if (mode != PTQ_SCORE_NONE) {
         Launch l(K_SCORE_PARTIAL, stream);
-        score_partial_kernel<float><<<dim3(cdiv(cols, kScoreCols), chunks), 256, 0, stream>>>(W, rows, cols, ldw, scale,
+        launch_chained(score_partial_kernel<float>, dim3(cdiv(cols, kScoreCols), chunks), 256, 0, stream, W, rows, cols, ldw,
+                       scale,
                                                                                             zero, bits, mode, partial);
     }
-    { Launch l(K_SCORE_FINAL, stream); score_final_kernel<<<cdiv(cols, 128), 128, 0, stream>>>(partial, chunks, cols, Hinv_diag, mode, S, status); }
-    { Launch l(K_RANK_SORT, stream); rank_sort_kernel<<<cdiv(cols, kRankCols), 256, 0, stream>>>(S, cols, ascending, perm); }
+    { Launch l(K_SCORE_FINAL, stream); launch_chained(score_final_kernel, cdiv(cols, 128), 128, 0, stream, partial, chunks,
+                                                      cols, Hinv_diag, mode, S, status); }
+    { Launch l(K_RANK_SORT, stream); launch_chained(rank_sort_kernel, cdiv(cols, kRankCols), 256, 0, stream, S, cols,
+                                                    ascending, perm, nullptr); }
     return launch_status();
 }
 
@@ -362,8 +365,9 @@ int ptq_prepare_hinv(const double* H, int cols, int damp_mode, double damp, doub
     unsigned* bar = cv.take<unsigned>(2);
     double* Dbuf = cv.take<double>(chol_scratch_doubles(n));
     void* pws = chol_panel_workspace_bytes(n) ? static_cast<void*>(cv.take<char>(chol_panel_workspace_bytes(n))) : nullptr;
-    { Launch l(K_LAMBDA, stream); lambda_kernel<<<1, 256, 0, stream>>>(H, n, damp_mode, damp, lambda_out, status); }
-    { Launch l(K_DAMP_COPY, stream); damp_copy_kernel<<<dim3(grid_x_for(n, 256), n), 256, 0, stream>>>(H, R, V, n, lambda_out, bar); }
+    { Launch l(K_LAMBDA, stream); launch_chained(lambda_kernel, 1, 256, 0, stream, H, n, damp_mode, damp, lambda_out, status); }
+    { Launch l(K_DAMP_COPY, stream); launch_chained(damp_copy_kernel, dim3(grid_x_for(n, 256), n), 256, 0, stream, H, R, V,
+                                                    n, lambda_out, bar); }
     // W = U^-T comes out of the factorisation sweep itself (V must start as zero)
     int st = cholesky_upper_auto(R, n, V, Dbuf, bar, pws, status, stream, true);
     if (st) return st;
@@ -387,7 +391,8 @@ int ptq_minmax_grid(const float* W, int rows, int cols, int64_t ldw, int bits, f
     cudaStream_t stream = static_cast<cudaStream_t>(stream_);
     if (!W || !scale || !zero || rows < 1 || cols < 1 || ldw < cols || bits < 2 || bits > 8)
         return PTQ_ERR_INVALID_ARG;
-    { Launch l(K_MINMAX_GRID, stream); minmax_grid_kernel<<<rows, 256, 0, stream>>>(W, rows, cols, ldw, bits, scale, zero, status); }
+    { Launch l(K_MINMAX_GRID, stream); launch_chained(minmax_grid_kernel, rows, 256, 0, stream, W, rows, cols, ldw, bits,
+                                                      scale, zero, status); }
     return launch_status();
 }
 
@@ -463,7 +468,7 @@ int ptq_quantize_layer_dynamic(const float* W, int rows, int cols, int64_t ldw, 
         if (dst) return dst;
     }
 
-    { Launch l(K_DYN_AUX, stream); iota_kernel<<<cdiv(cols, 256), 256, 0, stream>>>(obuf[0], cols); }
+    { Launch l(K_DYN_AUX, stream); launch_chained(iota_kernel, cdiv(cols, 256), 256, 0, stream, obuf[0], cols); }
     const int32_t* ocur = obuf[0];           // original column index of every current position
     // current state: the m columns still to do, their matrix (upper triangle valid) and their weights
     const double* Acur = Hinv;
@@ -473,30 +478,37 @@ int ptq_quantize_layer_dynamic(const float* W, int rows, int cols, int64_t ldw, 
     int m = cols, done = 0, cur = 0;
     while (m > 0) {
         const int b = block < m ? block : m;
-        { Launch l(K_DYN_AUX, stream); extract_diag_ld_kernel<<<cdiv(m, 256), 256, 0, stream>>>(Acur, lda, m, diag); }
+        { Launch l(K_DYN_AUX, stream); launch_chained(extract_diag_ld_kernel, cdiv(m, 256), 256, 0, stream, Acur, lda, m,
+                                                      diag); }
         if (mode != PTQ_SCORE_NONE) {
             Launch l(K_SCORE_PARTIAL, stream);
             if (Wcur)
-                score_partial_kernel<double><<<dim3(cdiv(m, kScoreCols), chunks), 256, 0, stream>>>(Wcur, rows, m, ldc, scale,
+                launch_chained(score_partial_kernel<double>, dim3(cdiv(m, kScoreCols), chunks), 256, 0, stream, Wcur, rows,
+                               m, ldc, scale,
                                                                                                 zero, bits, mode, partial);
             else
-                score_partial_kernel<float><<<dim3(cdiv(m, kScoreCols), chunks), 256, 0, stream>>>(W, rows, m, ldw, scale,
+                launch_chained(score_partial_kernel<float>, dim3(cdiv(m, kScoreCols), chunks), 256, 0, stream, W, rows, m,
+                               ldw, scale,
                                                                                                zero, bits, mode, partial);
         }
-        { Launch l(K_SCORE_FINAL, stream); score_final_kernel<<<cdiv(m, 128), 128, 0, stream>>>(partial, chunks, m, diag, mode, S, status); }
-        { Launch l(K_RANK_SORT, stream); rank_sort_kernel<<<cdiv(m, kRankCols), 256, 0, stream>>>(S, m, ascending, ordr, ocur); }
+        { Launch l(K_SCORE_FINAL, stream); launch_chained(score_final_kernel, cdiv(m, 128), 128, 0, stream, partial, chunks,
+                                                          m, diag, mode, S, status); }
+        { Launch l(K_RANK_SORT, stream); launch_chained(rank_sort_kernel, cdiv(m, kRankCols), 256, 0, stream, S, m,
+                                                        ascending, ordr, ocur); }
         double* An = Abuf[cur];
         double* Wn = Wbuf[cur];
         int32_t* onew = obuf[cur ^ 1];
         {
             Launch l(K_DYN_GATHER, stream);
             const int gy = m < 4096 ? m : 4096, gr = rows < 4096 ? rows : 4096;
-            gather_upper_kernel<<<dim3(grid_x_for(m, 256), gy), 256, 0, stream>>>(Acur, lda, ordr, m, An);
+            launch_chained(gather_upper_kernel, dim3(grid_x_for(m, 256), gy), 256, 0, stream, Acur, lda, ordr, m, An);
             if (Wcur)
-                gather_cols_kernel<double><<<dim3(grid_x_for(m, 256), gr), 256, 0, stream>>>(Wcur, ldc, rows, m, ordr, Wn);
+                launch_chained(gather_cols_kernel<double>, dim3(grid_x_for(m, 256), gr), 256, 0, stream, Wcur, ldc, rows, m,
+                               ordr, Wn);
             else
-                gather_cols_kernel<float><<<dim3(grid_x_for(m, 256), gr), 256, 0, stream>>>(W, ldw, rows, m, ordr, Wn);
-            gather_index_kernel<<<cdiv(m, 256), 256, 0, stream>>>(ocur, ordr, m, b, onew, order_out + done);
+                launch_chained(gather_cols_kernel<float>, dim3(grid_x_for(m, 256), gr), 256, 0, stream, W, ldw, rows, m,
+                               ordr, Wn);
+            launch_chained(gather_index_kernel, cdiv(m, 256), 256, 0, stream, ocur, ordr, m, b, onew, order_out + done);
         }
         int st = PTQ_OK;
         const int budget = coop_cta_budget(dev), behind = sweep_ctas_behind(rows, b, m, b < m ? b / kNB : 0, budget);
@@ -523,7 +535,8 @@ int ptq_quantize_layer_dynamic(const float* W, int rows, int cols, int64_t ldw, 
         {
             Launch l(K_DYN_AUX, stream);
             const int gr = rows < 4096 ? rows : 4096;
-            emit_block_kernel<<<dim3(grid_x_for(b, 256), gr), 256, 0, stream>>>(codes_p, m, onew, b, W, rows, cols, ldw,
+            launch_chained(emit_block_kernel, dim3(grid_x_for(b, 256), gr), 256, 0, stream, codes_p, m, onew, b, W, rows,
+                           cols, ldw,
                                                                             scale, zero, codes, What,
                                                                             want_loss ? dW : nullptr);
         }
@@ -546,7 +559,8 @@ int ptq_quantize_layer_dynamic(const float* W, int rows, int cols, int64_t ldw, 
         dim3 grid;
         const int st = launch_dgemm(K_DGEMM_LOSS, g, 1, stream, 64, &grid);
         if (st) return st;
-        { Launch l(K_SUM_PARTIALS, stream); sum_partials_kernel<<<1, 256, 0, stream>>>(partials, (int)(grid.x * grid.y * grid.z), 0.5, loss_out); }
+        { Launch l(K_SUM_PARTIALS, stream); launch_chained(sum_partials_kernel, 1, 256, 0, stream, partials,
+                                                           (int)(grid.x * grid.y * grid.z), 0.5, loss_out); }
     }
     return launch_status();
 }
@@ -578,13 +592,13 @@ int ptq_quantize_layer_per_row(const float* W, int rows, int cols, int64_t ldw, 
     const bool want_loss = H_undamped && loss_out;
     {
         Launch l(K_PER_ROW, stream);
-        per_row_kernel<<<rows, kPerRowThreads, per_row_smem_bytes(cols), stream>>>(
-            W, rows, cols, ldw, Hinv, scale, zero, bits, mode, ascending, codes, What, perm_rows,
+        launch_chained(per_row_kernel, rows, kPerRowThreads, per_row_smem_bytes(cols), stream, W, rows, cols, ldw, Hinv,
+                       scale, zero, bits, mode, ascending, codes, What, perm_rows,
             want_loss ? H_undamped : nullptr, want_loss ? row_loss : nullptr, status);
     }
     if (want_loss) {
         Launch l(K_SUM_PARTIALS, stream);
-        sum_partials_kernel<<<1, 256, 0, stream>>>(row_loss, rows, 1.0, loss_out);
+        launch_chained(sum_partials_kernel, 1, 256, 0, stream, row_loss, rows, 1.0, loss_out);
     }
     return launch_status();
 }
@@ -608,7 +622,8 @@ int ptq_gemm_nt_sliced(double* C, int64_t ldc, const double* A, int64_t lda, con
 int ptq_sort_scores(const double* S, int cols, int ascending, int32_t* perm, void* stream_) {
     cudaStream_t stream = static_cast<cudaStream_t>(stream_);
     if (!S || !perm || cols < 1) return PTQ_ERR_INVALID_ARG;
-    { Launch l(K_RANK_SORT, stream); rank_sort_kernel<<<cdiv(cols, kRankCols), 256, 0, stream>>>(S, cols, ascending ? 1 : 0, perm); }
+    { Launch l(K_RANK_SORT, stream); launch_chained(rank_sort_kernel, cdiv(cols, kRankCols), 256, 0, stream, S, cols,
+                                                    ascending ? 1 : 0, perm, nullptr); }
     return launch_status();
 }
 
@@ -693,11 +708,13 @@ int ptq_quantize_layer(const float* W, int rows, int cols, int64_t ldw, const do
     void* pws = chol_panel_workspace_bytes(n) ? static_cast<void*>(cv.take<char>(chol_panel_workspace_bytes(n))) : nullptr;
 
     const int n_flags = cdiv(rows, kSweepRows) + 1;
-    { Launch l(K_PERM_CHECK, stream); perm_check_kernel<<<cdiv(n, 256), 256, 0, stream>>>(perm, n, invperm, bar, sweep_flags, n_flags, status); }
+    { Launch l(K_PERM_CHECK, stream); launch_chained(perm_check_kernel, cdiv(n, 256), 256, 0, stream, perm, n, invperm, bar,
+                                                     sweep_flags, n_flags, status); }
     {
         Launch l(K_SWEEP_GATHER, stream);
         const int gy = n + rows < kMaxGridY ? n + rows : kMaxGridY;
-        sweep_gather_kernel<<<dim3(grid_x_for(n, 256), gy), 256, 0, stream>>>(Hinv, W, rows, n, ldw, perm, invperm, U, Wp, E, status);
+        launch_chained(sweep_gather_kernel, dim3(grid_x_for(n, 256), gy), 256, 0, stream, Hinv, W, rows, n, ldw, perm,
+                       invperm, U, Wp, E, status);
     }
     DeviceState* dev = nullptr;
     int st = current_device_state(&dev);
@@ -738,7 +755,8 @@ int ptq_quantize_layer(const float* W, int rows, int cols, int64_t ldw, const do
     int8_t* kexp = sliced ? reinterpret_cast<int8_t*>(Dbuf) : nullptr;      // the factorisation is done with Dbuf
     {
         Launch l(K_FINALIZE, stream);
-        finalize_kernel<<<dim3(grid_x_for(n, 256), rows), 256, 0, stream>>>(codes_p, invperm, W, rows, n, ldw, scale,
+        launch_chained(finalize_kernel, dim3(grid_x_for(n, 256), rows), 256, 0, stream, codes_p, invperm, W, rows, n, ldw,
+                       scale,
                                                                            zero, codes, What, dW, H_undamped, kexp);
     }
     if (sliced) {
@@ -758,7 +776,8 @@ int ptq_quantize_layer(const float* W, int rows, int cols, int64_t ldw, const do
         prm.k_mode = X_K_OWN_J; prm.alpha = 0.5; prm.partials = partials + tiles;
         st = x_product(a, b, prm, stream);
         if (st) return st;
-        { Launch l(K_SUM_PARTIALS, stream); sum_partials_kernel<<<1, 256, 0, stream>>>(partials, 2 * tiles, 1.0, loss_out); }
+        { Launch l(K_SUM_PARTIALS, stream); launch_chained(sum_partials_kernel, 1, 256, 0, stream, partials, 2 * tiles, 1.0,
+                                                           loss_out); }
     } else if (want_loss) {
         // sum_ic dW_ic (dW H)_ic; H is symmetric, so for the 64-column block of c only k up to the end of that block is
         // summed and the blocks before it are doubled
@@ -772,7 +791,8 @@ int ptq_quantize_layer(const float* W, int rows, int cols, int64_t ldw, const do
         dim3 grid;
         st = launch_dgemm(K_DGEMM_LOSS, g, 1, stream, 64, &grid);
         if (st) return st;
-        { Launch l(K_SUM_PARTIALS, stream); sum_partials_kernel<<<1, 256, 0, stream>>>(partials, (int)(grid.x * grid.y * grid.z), 0.5, loss_out); }
+        { Launch l(K_SUM_PARTIALS, stream); launch_chained(sum_partials_kernel, 1, 256, 0, stream, partials,
+                                                           (int)(grid.x * grid.y * grid.z), 0.5, loss_out); }
     }
     return launch_status();
 }

@@ -13,6 +13,7 @@ namespace ptq {
 // lambda = damp * mean(diag H) or damp; one CTA, fixed summation order.  Flags non-finite diagonals.
 __global__ void __launch_bounds__(256) lambda_kernel(const double* __restrict__ H, int n, int mode, double damp,
                                                       double* __restrict__ lambda_out, int32_t* status) {
+    chained_begin();
     __shared__ double red[256];
     double s = 0.0;
     bool bad = false;
@@ -36,6 +37,7 @@ __global__ void __launch_bounds__(256) lambda_kernel(const double* __restrict__ 
 // clears the factorisation's grid barrier.
 __global__ void damp_copy_kernel(const double* __restrict__ H, double* __restrict__ A, double* __restrict__ V, int n,
                                  const double* __restrict__ lambda, unsigned* __restrict__ bar) {
+    chained_begin();
     const int i = blockIdx.y;
     const double lam = *lambda;
     const int64_t row = (int64_t)i * n;

@@ -23,6 +23,7 @@ __device__ __forceinline__ int clamp_index(int j, int n) { return j < 0 ? 0 : (j
 __global__ void __launch_bounds__(256) perm_check_kernel(const int32_t* __restrict__ perm, int cols,
                                                           int32_t* __restrict__ invperm, unsigned* __restrict__ bar,
                                                           unsigned* __restrict__ sweep_flags, int n_flags, int32_t* status) {
+    chained_begin();
     const int p = blockIdx.x * 256 + threadIdx.x;
     if (p < 2) bar[p] = 0u;
     for (int f = p; f < n_flags; f += gridDim.x * 256) sweep_flags[f] = 0u;
@@ -43,6 +44,7 @@ __global__ void __launch_bounds__(256) sweep_gather_kernel(const double* __restr
                                                             int n, int64_t ldw, const int32_t* __restrict__ perm,
                                                             const int32_t* __restrict__ invperm, double* __restrict__ A,
                                                             double* __restrict__ Wp, double* __restrict__ E, int32_t* status) {
+    chained_begin();
     const int step = gridDim.x * 256, first = blockIdx.x * 256 + threadIdx.x;
     const int total = n + rows;
     for (int y = blockIdx.y; y < total; y += gridDim.y) {
@@ -758,6 +760,7 @@ __global__ void finalize_kernel(const uint8_t* __restrict__ codes_p, const int32
                                 const float* __restrict__ scale, const float* __restrict__ zero,
                                 uint8_t* __restrict__ codes, float* __restrict__ What, double* __restrict__ dW,
                                 const double* __restrict__ H, int8_t* __restrict__ kexp) {
+    chained_begin();
     const int i = blockIdx.y;
     const double sc = (double)scale[i], zp = (double)zero[i];
     for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < cols; j += gridDim.x * blockDim.x) {
@@ -773,6 +776,7 @@ __global__ void finalize_kernel(const uint8_t* __restrict__ codes_p, const int32
 // out = factor * (sum of partials in a fixed order)
 __global__ void __launch_bounds__(256) sum_partials_kernel(const double* __restrict__ partials, int count,
                                                             double factor, double* __restrict__ out) {
+    chained_begin();
     __shared__ double red[256];
     double s = 0.0;
     for (int k = threadIdx.x; k < count; k += 256) s += partials[k];

@@ -270,6 +270,7 @@ __device__ __forceinline__ void dgemm_tile(const GemmParams& p, int bx, int by, 
 // (64 (x + 1) and 64 (nbx - x)) add up to the same length for every CTA.
 template <int BT>
 __global__ void __launch_bounds__(kGemmThreads, BT == 64 ? 2 : 1) dgemm_kernel(GemmParams p) {
+    chained_wait();
     if (p.sym_double) {
         const int nbx = (p.N + BT - 1) / BT;
         const int bx = blockIdx.x, bx2 = nbx - 1 - bx;
@@ -316,9 +317,9 @@ inline int launch_dgemm(int kernel_id, const GemmParams& p, int batches, cudaStr
     if (p.sym_double) grid.x = (grid.x + 1) / 2;
     Launch scope(kernel_id, stream);
     if (bt == 128)
-        dgemm_kernel<128><<<grid, kGemmThreads, gemm_smem_bytes<128>(), stream>>>(p);
+        launch_chained(dgemm_kernel<128>, grid, kGemmThreads, gemm_smem_bytes<128>(), stream, p);
     else
-        dgemm_kernel<64><<<grid, kGemmThreads, gemm_smem_bytes<64>(), stream>>>(p);
+        launch_chained(dgemm_kernel<64>, grid, kGemmThreads, gemm_smem_bytes<64>(), stream, p);
     return launch_status();
 }
 

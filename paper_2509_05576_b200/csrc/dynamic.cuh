@@ -14,11 +14,13 @@
 namespace ptq {
 
 __global__ void iota_kernel(int32_t* __restrict__ a, int n) {
+    chained_begin();
     const int j = blockIdx.x * blockDim.x + threadIdx.x;
     if (j < n) a[j] = j;
 }
 
 __global__ void extract_diag_ld_kernel(const double* __restrict__ A, int64_t ld, int m, double* __restrict__ d) {
+    chained_begin();
     const int j = blockIdx.x * blockDim.x + threadIdx.x;
     if (j < m) d[j] = A[(int64_t)j * ld + j];
 }
@@ -26,6 +28,7 @@ __global__ void extract_diag_ld_kernel(const double* __restrict__ A, int64_t ld,
 // Anew[a][c] = A[lo][hi] with {lo, hi} = {ordr[a], ordr[c]} sorted: reads the upper triangle of A only.  One CTA row per a.
 __global__ void gather_upper_kernel(const double* __restrict__ A, int64_t ld, const int32_t* __restrict__ ordr, int m,
                                     double* __restrict__ Anew) {
+    chained_begin();
     for (int a = blockIdx.y; a < m; a += gridDim.y) {
         const int oa = ordr[a];
         for (int c = blockIdx.x * blockDim.x + threadIdx.x; c < m; c += gridDim.x * blockDim.x) {
@@ -40,6 +43,7 @@ __global__ void gather_upper_kernel(const double* __restrict__ A, int64_t ld, co
 template <typename T>
 __global__ void gather_cols_kernel(const T* __restrict__ Wc, int64_t ld, int rows, int m,
                                    const int32_t* __restrict__ ordr, double* __restrict__ Wnew) {
+    chained_begin();
     for (int i = blockIdx.y; i < rows; i += gridDim.y)
         for (int p = blockIdx.x * blockDim.x + threadIdx.x; p < m; p += gridDim.x * blockDim.x)
             Wnew[(int64_t)i * m + p] = (double)Wc[(int64_t)i * ld + ordr[p]];
@@ -48,6 +52,7 @@ __global__ void gather_cols_kernel(const T* __restrict__ Wc, int64_t ld, int row
 // orig_new[p] = orig[ordr[p]]: original column index of the column now at position p; the first b go to order_out.
 __global__ void gather_index_kernel(const int32_t* __restrict__ orig, const int32_t* __restrict__ ordr, int m, int b,
                                     int32_t* __restrict__ orig_new, int32_t* __restrict__ order_out) {
+    chained_begin();
     const int p = blockIdx.x * blockDim.x + threadIdx.x;
     if (p >= m) return;
     const int o = orig[ordr[p]];
@@ -60,6 +65,7 @@ __global__ void emit_block_kernel(const uint8_t* __restrict__ codes_p, int64_t l
                                   const float* __restrict__ W, int rows, int cols, int64_t ldw,
                                   const float* __restrict__ scale, const float* __restrict__ zero,
                                   uint8_t* __restrict__ codes, float* __restrict__ What, double* __restrict__ dW) {
+    chained_begin();
     for (int i = blockIdx.y; i < rows; i += gridDim.y) {
         const double sc = (double)scale[i], zp = (double)zero[i];
         for (int p = blockIdx.x * blockDim.x + threadIdx.x; p < b; p += gridDim.x * blockDim.x) {

@@ -127,6 +127,7 @@ __global__ void __launch_bounds__(256) gram_split_kernel(const float* __restrict
                                                           int cols_pad, int n_pad, int vec_ok,
                                                           int8_t* __restrict__ Q, int32_t* __restrict__ shifts,
                                                           int32_t* status, ulonglong2* __restrict__ iacc, int n_iacc) {
+    chained_begin();
     __shared__ float smax[256];
     __shared__ int sbad;
     gram_clear_iacc(iacc, n_iacc);
@@ -212,6 +213,7 @@ __device__ __forceinline__ float conv_fetch(const GramSource& s, const float* __
 __global__ void __launch_bounds__(256) gram_split_conv_kernel(GramSource src, int cols, int n, int cols_pad, int n_pad,
                                                                int8_t* __restrict__ Q, int32_t* __restrict__ shifts,
                                                                int32_t* status, ulonglong2* __restrict__ iacc, int n_iacc) {
+    chained_begin();
     __shared__ float smax[256];
     __shared__ int sbad;
     gram_clear_iacc(iacc, n_iacc);
@@ -396,6 +398,7 @@ gram_i8_kernel(const __grid_constant__ CUtensorMap tmapA, const __grid_constant_
                double* __restrict__ H, int cols, int n_pad,
                const int32_t* __restrict__ shifts, int num_tiles, int nbj, int32_t* status, int n_full, int ksplit,
                unsigned long long* __restrict__ iacc) {
+    chained_wait();
     extern __shared__ unsigned char gram_smem_raw[];
     const uint32_t raw = smem_u32(gram_smem_raw);
     const uint32_t base = (raw + 1023u) & ~1023u;
@@ -610,6 +613,7 @@ gram_i8_kernel(const __grid_constant__ CUtensorMap tmapA, const __grid_constant_
 __global__ void __launch_bounds__(kGramTM) gram_finish_kernel(const unsigned long long* __restrict__ iacc,
                                                                double* __restrict__ H, int cols, int n_full, int nbj,
                                                                const int32_t* __restrict__ shifts) {
+    chained_begin();
     const int tile = n_full + blockIdx.x;
     int bi, bj;
     gram_tile_coords(tile, nbj, bi, bj);
@@ -695,11 +699,13 @@ inline int gram_accumulate(double* H, GramSource src, int cols, int n, void* ws,
             Launch l(K_GRAM_SPLIT, stream);
             if (src.conv) {
                 src.col0 = c0;
-                gram_split_conv_kernel<<<cols_pad, 256, 0, stream>>>(src, cols, nc, cols_pad, n_pad, Q, shifts, status,
+                launch_chained(gram_split_conv_kernel, cols_pad, 256, 0, stream, src, cols, nc, cols_pad, n_pad, Q, shifts,
+                               status,
                                                                      clr, n_clr);
             } else {
                 const int vec_ok = (aligned16(src.base) && (src.ldx & 3) == 0) ? 1 : 0;
-                gram_split_kernel<<<cols_pad, 256, 0, stream>>>(src.base + c0, cols, nc, src.ldx, cols_pad, n_pad, vec_ok,
+                launch_chained(gram_split_kernel, cols_pad, 256, 0, stream, src.base + c0, cols, nc, src.ldx, cols_pad,
+                               n_pad, vec_ok,
                                                                 Q, shifts, status, clr, n_clr);
             }
         }
@@ -712,12 +718,13 @@ inline int gram_accumulate(double* H, GramSource src, int cols, int n, void* ws,
         const int grid = items < num_sms ? items : num_sms;
         {
             Launch l(K_GRAM_I8, stream);
-            gram_i8_kernel<<<grid, kGramThreads, kGramSmemBytes, stream>>>(mapA, mapB, H, cols, n_pad, shifts,
+            launch_chained(gram_i8_kernel, grid, kGramThreads, kGramSmemBytes, stream, mapA, mapB, H, cols, n_pad, shifts,
                                                                          num_tiles, nbj, status, n_full, ksplit, iacc);
         }
         if (sliced > 0) {
             Launch l(K_GRAM_FINISH, stream);
-            gram_finish_kernel<<<dim3(sliced, kGramTN / 16), kGramTM, 0, stream>>>(iacc, H, cols, n_full, nbj, shifts);
+            launch_chained(gram_finish_kernel, dim3(sliced, kGramTN / 16), kGramTM, 0, stream, iacc, H, cols, n_full, nbj,
+                           shifts);
         }
         if (cudaGetLastError() != cudaSuccess) return PTQ_ERR_CUDA;
     }

@@ -78,6 +78,7 @@ __global__ void __launch_bounds__(256, 6) x_slice_rows_kernel(const double* __re
                                                               int rows_pad, int k_pad, int8_t* __restrict__ Q,
                                                               int32_t* __restrict__ shifts, int32_t* status,
                                                               const int8_t* __restrict__ kexp, int ksign) {
+    chained_begin();
     __shared__ unsigned long long smax[256];
     const int row = blockIdx.x;
     const size_t plane = (size_t)rows_pad * k_pad;
@@ -138,6 +139,7 @@ __global__ void __launch_bounds__(256, 6) x_slice_rows_kernel(const double* __re
 constexpr int kXColChunk = 256;
 __global__ void __launch_bounds__(256) x_colmax_kernel(const double* __restrict__ X, int k, int cols, int64_t ld,
                                                         unsigned long long* __restrict__ colmax) {
+    chained_begin();
     __shared__ double smax[8][33];
     const int c0 = blockIdx.x * 32, k0 = blockIdx.y * kXColChunk;
     const int lane = threadIdx.x & 31, wy = threadIdx.x >> 5;
@@ -164,6 +166,7 @@ __global__ void __launch_bounds__(256) x_slice_cols_kernel(const double* __restr
                                                             const unsigned long long* __restrict__ colmax,
                                                             int8_t* __restrict__ Q, int32_t* __restrict__ shifts,
                                                             int32_t* status) {
+    chained_begin();
     __shared__ uint8_t dig[kXSlices][32][36];          // [slice][column][kk within the tile]
     const int c0 = blockIdx.x * 32, kbeg = blockIdx.y * kXColChunk;
     const int lane = threadIdx.x & 31, wy = threadIdx.x >> 5;          // 8 row slices x 32 columns
@@ -243,6 +246,7 @@ __device__ __forceinline__ bool x_tile_range(const XGemmParams& prm, int bi, int
 template <int GROUPS>
 __global__ void __launch_bounds__(kXThreads, 1)
 i8gemm_kernel(const __grid_constant__ CUtensorMap tmapA, const __grid_constant__ CUtensorMap tmapB, XGemmParams prm) {
+    chained_wait();
     extern __shared__ unsigned char xg_smem_raw[];
     const uint32_t raw = smem_u32(xg_smem_raw);
     const uint32_t base = (raw + 1023u) & ~1023u;
@@ -516,13 +520,16 @@ inline XOperand x_slice_operand(Carver& cv, const double* X, int64_t ld, int tra
     Launch l(K_X_SLICE, stream);
     if (transposed) {
         cudaMemsetAsync(colmax, 0, (size_t)rows_pad * sizeof(unsigned long long), stream);
-        x_colmax_kernel<<<dim3(rows_pad / 32, cdiv(k, kXColChunk)), 256, 0, stream>>>(X, k, rows, ld, colmax);
-        x_slice_cols_kernel<<<dim3(rows_pad / 32, cdiv(k_pad, kXColChunk)), 256, 0, stream>>>(X, k, rows, ld, rows_pad, k_pad,
+        launch_chained(x_colmax_kernel, dim3(rows_pad / 32, cdiv(k, kXColChunk)), 256, 0, stream, X, k, rows, ld, colmax);
+        launch_chained(x_slice_cols_kernel, dim3(rows_pad / 32, cdiv(k_pad, kXColChunk)), 256, 0, stream, X, k, rows, ld,
+                       rows_pad, k_pad,
                                                                                               colmax, op.Q, op.sh, status);
     } else if (kexp) {
-        x_slice_rows_kernel<true><<<rows_pad, 256, 0, stream>>>(X, rows, k, ld, rows_pad, k_pad, op.Q, op.sh, status, kexp, ksign);
+        launch_chained(x_slice_rows_kernel<true>, rows_pad, 256, 0, stream, X, rows, k, ld, rows_pad, k_pad, op.Q, op.sh,
+                       status, kexp, ksign);
     } else {
-        x_slice_rows_kernel<false><<<rows_pad, 256, 0, stream>>>(X, rows, k, ld, rows_pad, k_pad, op.Q, op.sh, status, nullptr, 1);
+        launch_chained(x_slice_rows_kernel<false>, rows_pad, 256, 0, stream, X, rows, k, ld, rows_pad, k_pad, op.Q, op.sh,
+                       status, nullptr, 1);
     }
     return op;
 }
@@ -551,8 +558,9 @@ inline int x_product(const XOperand& a, const XOperand& b, XGemmParams prm, cuda
     const int grid = tiles < dev->sms ? tiles : dev->sms;
     {
         Launch l(K_X_GEMM, stream);
-        if (prm.out_mode == X_OUT_REDUCE) i8gemm_kernel<kXLossGroups><<<grid, kXThreads, kXSmemBytes, stream>>>(mapA, mapB, prm);
-        else i8gemm_kernel<kXGroups><<<grid, kXThreads, kXSmemBytes, stream>>>(mapA, mapB, prm);
+        if (prm.out_mode == X_OUT_REDUCE) launch_chained(i8gemm_kernel<kXLossGroups>, grid, kXThreads, kXSmemBytes, stream,
+                                                         mapA, mapB, prm);
+        else launch_chained(i8gemm_kernel<kXGroups>, grid, kXThreads, kXSmemBytes, stream, mapA, mapB, prm);
     }
     return launch_status();
 }

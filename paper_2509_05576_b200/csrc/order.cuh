@@ -16,6 +16,7 @@ __device__ __forceinline__ double quant_code_d(double w, double sc, double zp, d
 __global__ void __launch_bounds__(256) minmax_grid_kernel(const float* __restrict__ W, int rows, int cols, int64_t ldw,
                                                            int bits, float* __restrict__ scale,
                                                            float* __restrict__ zero, int32_t* status) {
+    chained_begin();
     __shared__ float slo[256], shi[256];
     __shared__ int sbad;
     const int i = blockIdx.x;
@@ -67,6 +68,7 @@ __global__ void __launch_bounds__(256) score_partial_kernel(const T* __restrict_
                                                              int64_t ldw, const float* __restrict__ scale,
                                                              const float* __restrict__ zero, int bits, int mode,
                                                              double* __restrict__ partial) {
+    chained_begin();
     __shared__ double sub[8][kScoreCols + 1];
     const int c = threadIdx.x & (kScoreCols - 1), g = threadIdx.x / kScoreCols;
     const int j = blockIdx.x * kScoreCols + c;
@@ -106,6 +108,7 @@ __global__ void __launch_bounds__(256) score_partial_kernel(const T* __restrict_
 __global__ void __launch_bounds__(128) score_final_kernel(const double* __restrict__ partial, int chunks, int cols,
                                                            const double* __restrict__ hinv_diag, int mode,
                                                            double* __restrict__ S, int32_t* status) {
+    chained_begin();
     const int j = blockIdx.x * 128 + threadIdx.x;
     if (j >= cols) return;
     double s = 0.0;
@@ -133,7 +136,8 @@ constexpr int kRankChunk = 2048;
 // tie != nullptr: equal scores are ordered by tie[] (distinct values) instead of by position.
 __global__ void __launch_bounds__(256) rank_sort_kernel(const double* __restrict__ S, int cols, int ascending,
                                                          int32_t* __restrict__ perm,
-                                                         const int32_t* __restrict__ tie = nullptr) {
+                                                         const int32_t* __restrict__ tie) {
+    chained_begin();
     __shared__ unsigned long long keys[kRankChunk];
     __shared__ int32_t ties[kRankChunk];
     const int j = blockIdx.x * kRankCols + (threadIdx.x >> 4);

@@ -79,6 +79,7 @@ __global__ void __launch_bounds__(kPerRowThreads, 3) per_row_kernel(const float*
                                                                  float* __restrict__ What, int32_t* __restrict__ perm_rows,
                                                                  const double* __restrict__ H, double* __restrict__ row_loss,
                                                                  int32_t* status) {
+    chained_begin();
     extern __shared__ __align__(16) unsigned char per_row_smem[];
     __shared__ double red[kPerRowWarps];
     const int n = cols, nf = (n + 7) >> 3, n8 = 8 * nf;
