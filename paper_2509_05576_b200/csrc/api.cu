@@ -27,8 +27,6 @@ inline int grid_x_for(int n, int threads) {
 }
 
 constexpr int kMaxGridY = 65535;
-constexpr int kSuperBlock = 1024;         // columns swept per launch on tall, wide layers
-constexpr int kSuperBlockMinRows = 2048;
 constexpr int kSlicedMinCols = 3072;      // from here on the large float64 products run on the int8 tensor path
 // The loss product goes there too where it is large enough to pay for slicing H and for a second product, and where the
 // slices (7 bytes a value, both sizes rounded up to multiples of 128) and the two sets of partial sums fit into the pieces of
@@ -265,9 +263,8 @@ size_t ptq_workspace_bytes(int call_id, int rows, int cols, int n) {
             add(2 * sizeof(unsigned));                      // grid barrier of the factorisation kernel
             add(((size_t)cdiv(rows, kSweepRows) + 1) * sizeof(unsigned));   // per-row-group progress counters of the sweep
             add(chol_scratch_doubles(cols) * sizeof(double));
-            if (rows >= kSuperBlockMinRows && cols >= 4 * kSuperBlock)
-                add(i8gemm_workspace_bytes(rows, cols, kSuperBlock));   // slices of E[:, sb] and U[sb, later]
             add(chol_panel_workspace_bytes(cols));
+            if (cols >= kPanelMinCols) add(x_operand_bytes(rows, kPanelBlocks * kNB));   // slices of E[:, panel]
             break;
         case PTQ_CALL_QUANTIZE_LAYER_PER_ROW:
             if (rows < 1) return 0;
@@ -511,10 +508,11 @@ int ptq_quantize_layer_dynamic(const float* W, int rows, int cols, int64_t ldw, 
             launch_chained(gather_index_kernel, cdiv(m, 256), 256, 0, stream, ocur, ordr, m, b, onew, order_out + done);
         }
         int st = PTQ_OK;
-        const int budget = coop_cta_budget(dev), behind = sweep_ctas_behind(rows, b, m, b < m ? b / kNB : 0, budget);
+        const CholRange range = {0, b < m ? b / kNB : cdiv(m, kNB), cdiv(m, kNB)};
+        const int budget = coop_cta_budget(dev), behind = sweep_ctas_behind(rows, b, m, range, budget);
         if (behind > 0) {
-            st = factor_sweep_launch(An, m, b < m ? b / kNB : 0, Dbuf, bar, behind, Wn, E, codes_p, scale, zero, rows, b, bits, sweep_flags,
-                                     status, stream, budget, false);
+            st = factor_sweep_launch(An, m, range, Dbuf, bar, behind, Wn, E, codes_p, scale, zero, rows, b, bits, sweep_flags, status,
+                                     stream, budget, false, false);
         } else {
             st = cholesky_upper(An, m, nullptr, Dbuf, bar, status, stream, b < m ? b / kNB : 0);
             if (st) return st;
@@ -703,9 +701,8 @@ int ptq_quantize_layer(const float* W, int rows, int cols, int64_t ldw, const do
     unsigned* bar = cv.take<unsigned>(2);
     unsigned* sweep_flags = cv.take<unsigned>((size_t)cdiv(rows, kSweepRows) + 1);
     double* Dbuf = cv.take<double>(chol_scratch_doubles(n));
-    void* xws = (rows >= kSuperBlockMinRows && n >= 4 * kSuperBlock)
-                    ? static_cast<void*>(cv.take<char>(i8gemm_workspace_bytes(rows, n, kSuperBlock))) : nullptr;
-    void* pws = chol_panel_workspace_bytes(n) ? static_cast<void*>(cv.take<char>(chol_panel_workspace_bytes(n))) : nullptr;
+    void* pws = n >= kPanelMinCols ? static_cast<void*>(cv.take<char>(chol_panel_workspace_bytes(n))) : nullptr;
+    void* ews = n >= kPanelMinCols ? static_cast<void*>(cv.take<char>(x_operand_bytes(rows, kPanelBlocks * kNB))) : nullptr;
 
     const int n_flags = cdiv(rows, kSweepRows) + 1;
     { Launch l(K_PERM_CHECK, stream); launch_chained(perm_check_kernel, cdiv(n, 256), 256, 0, stream, perm, n, invperm, bar,
@@ -719,34 +716,38 @@ int ptq_quantize_layer(const float* W, int rows, int cols, int64_t ldw, const do
     DeviceState* dev = nullptr;
     int st = current_device_state(&dev);
     if (st) return st;
-    // blocked Eq. 12, and the sweep behind it
-    const int budget = coop_cta_budget(dev), behind = pws == nullptr ? sweep_ctas_behind(rows, n, n, 0, budget) : 0;
-    if (behind > 0) st = factor_sweep_launch(U, n, 0, Dbuf, bar, behind, Wp, E, codes_p, scale, zero, rows, n, bits, sweep_flags, status, stream, budget, true);
-    else st = cholesky_upper_auto(U, n, nullptr, Dbuf, bar, pws, status, stream, true);
-    if (st) return st;
-
-    if (behind > 0) {
-        // done
-    } else if (rows >= kSuperBlockMinRows && n >= 4 * kSuperBlock) {
-        // Tall and wide layers: the deferred part of Eq. 11 dominates (rows cols^2 / 2 multiply-adds), and inside the sweep
-        // kernel it runs as 32 x 64 x 64 tiles.  The columns are therefore swept in super-blocks of 1024; what a
-        // super-block owes to all later columns is applied by one large product, W[:, later] -= E[:, sb] U[sb, later],
-        // with k = 1024.
-        for (int off = 0; off < n; off += kSuperBlock) {
-            const int sb = n - off < kSuperBlock ? n - off : kSuperBlock;
-            st = sweep_launch(Wp + off, U + (size_t)off * n + off, E + off, codes_p + off, scale, zero, rows, sb, bits,
-                              sweep_flags, status, stream, n, true, off == 0);
+    // Blocked Eq. 12 and the sweep: of everything at once, or, on wide layers, panel by panel (cholpanel.cuh).  There the part of
+    // Eq. 11 that a panel's columns owe to all later ones, W[:, later] -= E[:, panel] U[panel, later], is one large product on
+    // the int8 tensor path, as the panel's share of Eq. 12 is; both take the same slices of U.  (4096 x 11008 with the
+    // updates inside the sweep kernel instead, 32 x 64 x 64 tiles: 30 ms in place of 11.)
+    const int budget = coop_cta_budget(dev), panel = n >= kPanelMinCols ? kPanelBlocks : cdiv(n, kNB);
+    for (int kf = 0; kf < cdiv(n, kNB); kf += panel) {
+        const int off = kf * kNB, cols_now = n - off < panel * kNB ? n - off : panel * kNB, rest = n - off - cols_now;
+        const CholRange range = {kf, kf + cdiv(cols_now, kNB), kf + cdiv(cols_now, kNB)};
+        const int behind = sweep_ctas_behind(rows, cols_now, n, range, budget);
+        if (behind > 0) {
+            st = factor_sweep_launch(U, n, range, Dbuf, bar, behind, Wp + off, E + off, codes_p + off, scale, zero, rows, cols_now, bits,
+                                     sweep_flags, status, stream, budget, kf == 0, true);
+        } else {
+            st = cholesky_upper(U, n, nullptr, Dbuf, bar, status, stream, range.stop, range.first, range.row_limit, kf == 0);
             if (st) return st;
-            if (off + sb < n) {
-                // W[:, later] -= E[:, sb] U[sb, later] on the int8 tensor path (i8gemm.cuh), float64-accurate
-                st = i8gemm_nt(Wp + off + sb, n, E + off, n, U + (size_t)off * n + off + sb, n, 1, rows, n - off - sb, sb,
-                               -1.0, xws, status, stream);
-                if (st) return st;
-            }
+            st = sweep_launch(Wp + off, U + (size_t)off * (n + 1), E + off, codes_p + off, scale, zero, rows, cols_now, bits, sweep_flags,
+                              status, stream, n, true, kf == 0);
         }
-    } else {
-        st = sweep_launch(Wp, U, E, codes_p, scale, zero, rows, n, bits, sweep_flags, status, stream, n, true, true);
         if (st) return st;
+        if (rest > 0) {
+            Carver pv(pws), ev(ews);
+            double* below = U + (size_t)off * n + off + cols_now;                 // U[panel, later]
+            const XOperand u = x_slice_operand(pv, below, n, 1, rest, cols_now, status, stream);
+            st = chol_apply_panel(U, n, off + cols_now, u, status, stream);
+            if (st) return st;
+            const XOperand e = x_slice_operand(ev, E + off, n, 0, rows, cols_now, status, stream);
+            XGemmParams prm{};
+            prm.C = Wp + off + cols_now; prm.ldc = n; prm.alpha = -1.0; prm.status = status;
+            prm.out_mode = X_OUT_ADD; prm.k_mode = X_K_ALL;
+            st = x_product(e, u, prm, stream);
+            if (st) return st;
+        }
     }
 
     const bool want_loss = H_undamped && loss_out;

@@ -836,6 +836,11 @@ inline int chol_grid(int n, bool with_w, int budget) {
     const long items = tiles2 > (n + 7) / 8 ? tiles2 : (n + 7) / 8;
     return items < budget ? (int)(items < 1 ? 1 : items) : budget;
 }
+// Which block rows of a factorisation: first .. stop - 1, their updates applied to the rows below row_limit (chol_factorise).
+struct CholRange {
+    int first, stop, row_limit;
+};
+inline CholRange chol_all_rows(int n) { return {0, cdiv(n, kNB), cdiv(n, kNB)}; }
 // nb_stop > 0: factorise the block rows k_first .. nb_stop - 1 only (see the kernel for what row_limit selects;
 // row_limit <= 0: all rows below are updated).  A partial run that updates everything below must not ask for Wm.
 // bar_ready: the caller has cleared `bar`.

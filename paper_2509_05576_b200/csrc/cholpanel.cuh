@@ -19,6 +19,15 @@ inline size_t chol_panel_workspace_bytes(int n) {
     return 2 * x_operand_bytes(n, kPanelBlocks * kNB);
 }
 
+// What a panel owes to the matrix below and right of it: A[c0 :, c0 :] -= U[panel, c0 :]^T U[panel, c0 :] (upper tiles), from
+// the slices of the columns c0 .. n - 1 of the panel's rows.
+inline int chol_apply_panel(double* A, int n, int c0, const XOperand& u, int32_t* status, cudaStream_t stream) {
+    XGemmParams prm{};
+    prm.C = A + (size_t)c0 * n + c0; prm.ldc = n; prm.alpha = -1.0; prm.status = status;
+    prm.out_mode = X_OUT_ADD_UPPER; prm.k_mode = X_K_ALL;
+    return x_product(u, u, prm, stream);
+}
+
 // Same contract as cholesky_upper (whole factorisation); xws: chol_panel_workspace_bytes(n) bytes of scratch.
 inline int cholesky_upper_auto(double* A, int n, double* Wm, double* Dbuf, unsigned* bar, void* xws, int32_t* status,
                                cudaStream_t stream, bool bar_ready) {
@@ -34,12 +43,11 @@ inline int cholesky_upper_auto(double* A, int n, double* Wm, double* Dbuf, unsig
         Carver cv(xws);
         // rows of the operand = columns c0 .. n - 1 of the panel's rows of U
         const XOperand u = x_slice_operand(cv, A + (size_t)r0 * n + c0, n, 1, rest, depth, status, stream);
-        XGemmParams prm{};
-        prm.C = A + (size_t)c0 * n + c0; prm.ldc = n; prm.alpha = -1.0; prm.status = status;
-        prm.out_mode = X_OUT_ADD_UPPER; prm.k_mode = X_K_ALL;
-        st = x_product(u, u, prm, stream);
+        st = chol_apply_panel(A, n, c0, u, status, stream);
         if (st) return st;
         if (Wm != nullptr) {
+            XGemmParams prm{};
+            prm.ldc = n; prm.alpha = -1.0; prm.status = status; prm.k_mode = X_K_ALL;
             // rows of the operand = columns 0 .. c0 - 1 of the panel's rows of W
             const XOperand w = x_slice_operand(cv, Wm + (size_t)r0 * n, n, 1, c0, depth, status, stream);
             prm.C = Wm + (size_t)c0 * n; prm.out_mode = X_OUT_ADD;

@@ -607,7 +607,8 @@ __global__ void __launch_bounds__(kSweepThreads, 1) sweep_coop_kernel(SweepParam
 struct FactorArgs {
     double* A;
     double* Dbuf;
-    int n, vec16, nb_stop, row_limit, ctas;
+    int n, vec16, ctas;
+    CholRange range;
     int64_t ld;
     unsigned* bar;
     int32_t* status;
@@ -615,7 +616,8 @@ struct FactorArgs {
 };
 __global__ void __launch_bounds__(kCholThreads, 1) factor_sweep_kernel(FactorArgs f, SweepParams prm) {
     if ((int)blockIdx.x < f.ctas) {
-        chol_factorise(f.A, nullptr, f.Dbuf, f.n, f.ld, f.vec16, f.bar, f.status, f.spin_limit, 0, f.nb_stop, f.row_limit, f.ctas);
+        chol_factorise(f.A, nullptr, f.Dbuf, f.n, f.ld, f.vec16, f.bar, f.status, f.spin_limit, f.range.first, f.range.stop,
+                       f.range.row_limit, f.ctas);
     } else if (threadIdx.x < kSweepThreads) {
         sweep_columns<true>(prm, blockIdx.x - f.ctas, gridDim.x - f.ctas);
     }
@@ -672,8 +674,8 @@ inline int sweep_launch(double* Wp, const double* U, double* E, uint8_t* codes_p
     return PTQ_OK;
 }
 
-// How many of `budget` CTAs the sweep of the first sweep_n columns gets when it runs behind the factorisation (of the block rows
-// below nb_stop of n columns) in one launch, or 0: one after the other.  From a model of both, in microseconds, fitted to
+// How many of `budget` CTAs the sweep of sweep_n columns gets when it runs behind the factorisation of their block rows (a range
+// of those of n columns) in one launch, or 0: one after the other.  From a model of both, in microseconds, fitted to
 // their measured times (within about 10 % of them from 64 to 2900 columns, 16 to 3000 rows and 18 to 148 CTAs):
 //   factorisation  sqrt(chain^2 + (work / CTAs)^2), 11.5 per block row in the chain, 3.6 per trailing tile, 12.8 per block
 //                  row and remaining block for the strips;
@@ -682,12 +684,15 @@ inline int sweep_launch(double* Wp, const double* U, double* E, uint8_t* codes_p
 // Behind one another they take the longer of the two; a tenth is asked of them to be worth it.  Measured, one after the
 // other -> one launch: 64 x 128 50 -> 36 us, 128 x 576 175 -> 115, 128 x 1152 334 -> 220, 1000 x 1152 372 -> 260, 256 x 2304
 // 742 -> 568, 1000 x 2048 811 -> 711, 1000 x 2900 1490 -> 1441, 2000 x 1152 478 -> 402; not taken: 2000 x 2048 1107 -> 1318.
-inline int sweep_ctas_behind(int rows, int sweep_n, int n, int nb_stop, int budget) {
-    const int groups = cdiv(rows, kSweepRows), nb = cdiv(n, kNB), nbs = nb_stop > 0 && nb_stop < nb ? nb_stop : nb;
+inline int sweep_ctas_behind(int rows, int sweep_n, int n, const CholRange& range, int budget) {
+    const int groups = cdiv(rows, kSweepRows), nb = cdiv(n, kNB);
     if (groups >= budget) return 0;
     double work = 0.0;
-    for (int k = 0; k < nbs; ++k) work += (1.8 * (nb - k) + 12.8) * (nb - k);
-    const double chain = 11.5 * nbs, update = 2.6e-4 * (double)sweep_n * sweep_n, steps = 0.11 * sweep_n;
+    for (int k = range.first; k < range.stop; ++k) {
+        const double m = nb - k - 1, r = range.row_limit - k - 1;
+        work += 3.6 * (r * m - 0.5 * r * (r - 1.0)) + 12.8 * (nb - k);
+    }
+    const double chain = 11.5 * (range.stop - range.first), update = 2.6e-4 * (double)sweep_n * sweep_n, steps = 0.11 * sweep_n;
     auto factor = [&](int ctas) { return std::sqrt(chain * chain + (work / ctas) * (work / ctas)); };
     const int most = budget / groups < cdiv(sweep_n, kNB) ? budget / groups : cdiv(sweep_n, kNB);
     const double apart = factor(budget) + update / most + steps;
@@ -700,11 +705,12 @@ inline int sweep_ctas_behind(int rows, int sweep_n, int n, int nb_stop, int budg
     return best;
 }
 
-// The factorisation of U (n x n, row stride n; block rows below nb_stop, 0: all) and the sweep of its first `sweep_n` columns
-// in one launch.
-inline int factor_sweep_launch(double* U, int n, int nb_stop, double* Dbuf, unsigned* bar, int sweep_ctas, double* Wp, double* E,
-                               uint8_t* codes_p, const float* scale, const float* zero, int rows, int sweep_n, int bits,
-                               unsigned* flags, int32_t* status, cudaStream_t stream, int budget, bool ready) {
+// The factorisation of a range of block rows of U (n x n, row stride n) and the sweep of the first sweep_n columns of that range
+// in one launch.  Wp, E, codes_p: from the column of the first block row on, row stride n.  ready: the caller has set the
+// counters and flags to zero and E to NaN.
+inline int factor_sweep_launch(double* U, int n, const CholRange& range, double* Dbuf, unsigned* bar, int sweep_ctas, double* Wp,
+                               double* E, uint8_t* codes_p, const float* scale, const float* zero, int rows, int sweep_n, int bits,
+                               unsigned* flags, int32_t* status, cudaStream_t stream, int budget, bool counters_ready, bool e_ready) {
     DeviceState* dev = nullptr;
     int st = current_device_state(&dev);
     if (st) return st;
@@ -717,24 +723,24 @@ inline int factor_sweep_launch(double* U, int n, int nb_stop, double* Dbuf, unsi
         return (e == cudaSuccess && per_sm < 1) ? cudaErrorLaunchOutOfResources : e;
     });
     if (st) return st;
-    const int groups = cdiv(rows, kSweepRows), nb = cdiv(n, kNB);
-    if (!ready) {
-        if (cudaMemsetAsync(bar, 0, 2 * sizeof(unsigned), stream) != cudaSuccess ||
-            cudaMemsetAsync(flags, 0, ((size_t)groups + 1) * sizeof(unsigned), stream) != cudaSuccess ||
-            cudaMemset2DAsync(E, (size_t)n * sizeof(double), 0xFF, (size_t)sweep_n * sizeof(double), (size_t)rows, stream) != cudaSuccess)
-            return PTQ_ERR_CUDA;
-    }
+    const int groups = cdiv(rows, kSweepRows);
+    if (!counters_ready && (cudaMemsetAsync(bar, 0, 2 * sizeof(unsigned), stream) != cudaSuccess ||
+                            cudaMemsetAsync(flags, 0, ((size_t)groups + 1) * sizeof(unsigned), stream) != cudaSuccess))
+        return PTQ_ERR_CUDA;
+    if (!e_ready && cudaMemset2DAsync(E, (size_t)n * sizeof(double), 0xFF, (size_t)sweep_n * sizeof(double), (size_t)rows, stream) !=
+        cudaSuccess)
+        return PTQ_ERR_CUDA;
     FactorArgs f;
-    f.A = U; f.Dbuf = Dbuf; f.n = n; f.ld = n; f.nb_stop = nb_stop > 0 ? nb_stop : nb; f.row_limit = nb;
+    f.A = U; f.Dbuf = Dbuf; f.n = n; f.ld = n; f.range = range;
     f.vec16 = ((n & 1) == 0 && aligned16(U)) ? 1 : 0;
     f.ctas = chol_grid(n, false, budget - sweep_ctas);
     f.bar = bar; f.status = status; f.spin_limit = kSpinLimitCycles;
     SweepParams prm;
-    prm.Wp = Wp; prm.U = U; prm.E = E; prm.codes_p = codes_p; prm.scale = scale; prm.zero = zero;
-    prm.rows = rows; prm.n = sweep_n; prm.bits = bits; prm.ld = n;
+    prm.Wp = Wp; prm.U = U + (size_t)range.first * kNB * (n + 1); prm.E = E; prm.codes_p = codes_p; prm.scale = scale;
+    prm.zero = zero; prm.rows = rows; prm.n = sweep_n; prm.bits = bits; prm.ld = n;
     prm.vec16 = (f.vec16 && (sweep_n & 1) == 0 && aligned16(Wp) && aligned16(E)) ? 1 : 0;
     prm.flags = flags; prm.status = status; prm.spin_limit = kSpinLimitCycles;
-    prm.diag = Dbuf; prm.rows_done = bar; prm.row_arrivals = (unsigned)f.ctas;
+    prm.diag = Dbuf + (size_t)range.first * kNB * kNB; prm.rows_done = bar; prm.row_arrivals = (unsigned)f.ctas;
     void* args[] = {&f, &prm};
     Launch l(K_FACTOR_SWEEP, stream);
     if (cudaLaunchCooperativeKernel((const void*)factor_sweep_kernel, dim3(f.ctas + sweep_ctas), dim3(kCholThreads), args, smem,
