@@ -15,7 +15,7 @@ struct GemmParams {
     double* diag;      // not null: diag[i] = C[i][i] as well
     int64_t lda, ldb, ldc;
     int M, N, K;
-    int a_trans, b_trans;
+    int a_trans, b_trans;  // template parameters of the kernel: a runtime stride would cost an addition per operand load
     double alpha, beta;
     int kbeg_mode;     // 0: k from 0;  1: from max(i0, j0);  2: from i0   (operands are zero before that)
     int kend_mode;     // 0: k to K;    1: to min(K, j0 + BN)              (B is zero after that)
@@ -38,7 +38,6 @@ struct GemmParams {
 
 constexpr int kGemmBK = 32;
 constexpr int kGemmStages = 3;
-constexpr int kGemmThreads = 256;
 constexpr int kGemmLdk = kGemmBK + 4;   // row stride of a k-contiguous operand tile (20 = 4 mod 16: conflict-free)
 
 template <int BT>
@@ -65,16 +64,17 @@ __device__ __forceinline__ void dmma_884(double& c0, double& c1, double a, doubl
                  : "d"(a), "d"(b));
 }
 
-// BT x BT output tile (bx, by) of batch z, 256 threads = 8 warps as 2 x 4; each warp owns (BT/2) x (BT/4) outputs as
+// BT x BT output tile (bx, by) of batch z, TH threads: 8 warps as 2 x 4 or 16 as 4 x 4, each with its share of the outputs as
 // 8 x 8 fragments.  nbx = number of column tiles (indexes the partials).
-template <int BT>
+template <int BT, int TH, int a_trans, int b_trans>
 __device__ __forceinline__ void dgemm_tile(const GemmParams& p, int bx, int by, int z, int nbx, int nby) {
     constexpr int BK = kGemmBK;
     constexpr int LDM = BT + 4;            // row stride of an m-contiguous operand tile
     constexpr int TILE = BT * kGemmLdk;
-    constexpr int WTM = BT / 2, WTN = BT / 4;
+    constexpr int WM = TH == 512 ? 4 : 2;                     // warps as WM x 4
+    constexpr int WTM = BT / WM, WTN = BT / 4;
     constexpr int FM = WTM / 8, FN = WTN / 8;
-    constexpr int EPT = BT * BK / kGemmThreads;
+    constexpr int EPT = BT * BK / TH;
     extern __shared__ __align__(16) double smem[];
 
     int N = p.N, K = p.K;
@@ -112,7 +112,6 @@ __device__ __forceinline__ void dgemm_tile(const GemmParams& p, int bx, int by, 
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int wm0 = (warp >> 2) * WTM, wn0 = (warp & 3) * WTN;
     const int lq = lane >> 2, lr = lane & 3;
-    const int a_trans = p.a_trans, b_trans = p.b_trans;
 
     double acc[FM][FN][2];
 #pragma unroll
@@ -130,7 +129,7 @@ __device__ __forceinline__ void dgemm_tile(const GemmParams& p, int bx, int by, 
         if (a_vec && kfull) {
 #pragma unroll
             for (int r = 0; r < EPT / 2; ++r) {
-                const int idx = tid + r * kGemmThreads;          // pair index
+                const int idx = tid + r * TH;          // pair index
                 if (a_trans == 0) {
                     const int k = (idx % (BK / 2)) * 2, m = idx / (BK / 2);
                     cp_async16(as + m * kGemmLdk + k, A + (int64_t)(i0 + m) * p.lda + k0 + k);
@@ -142,7 +141,7 @@ __device__ __forceinline__ void dgemm_tile(const GemmParams& p, int bx, int by, 
         } else {
 #pragma unroll
         for (int r = 0; r < EPT; ++r) {
-            const int idx = tid + r * kGemmThreads;
+            const int idx = tid + r * TH;
             int m, k, off;
             if (a_trans == 0) { k = idx % BK; m = idx / BK; off = m * kGemmLdk + k; }
             else { m = idx % BT; k = idx / BT; off = k * LDM + m; }
@@ -155,7 +154,7 @@ __device__ __forceinline__ void dgemm_tile(const GemmParams& p, int bx, int by, 
         if (b_vec && kfull) {
 #pragma unroll
             for (int r = 0; r < EPT / 2; ++r) {
-                const int idx = tid + r * kGemmThreads;
+                const int idx = tid + r * TH;
                 if (b_trans == 1) {
                     const int k = (idx % (BK / 2)) * 2, nn = idx / (BK / 2);
                     cp_async16(bs + nn * kGemmLdk + k, B + (int64_t)(j0 + nn) * p.ldb + k0 + k);
@@ -168,7 +167,7 @@ __device__ __forceinline__ void dgemm_tile(const GemmParams& p, int bx, int by, 
         }
 #pragma unroll
         for (int r = 0; r < EPT; ++r) {
-            const int idx = tid + r * kGemmThreads;
+            const int idx = tid + r * TH;
             int n, k, off;
             if (b_trans == 1) { k = idx % BK; n = idx / BK; off = n * kGemmLdk + k; }
             else { n = idx % BT; k = idx / BT; off = k * LDM + n; }
@@ -181,8 +180,8 @@ __device__ __forceinline__ void dgemm_tile(const GemmParams& p, int bx, int by, 
 
     const int nkt = kbeg < kend ? (kend - kbeg + BK - 1) / BK : 0;
     // element (m, k) of the A tile and (k, n) of the B tile, in doubles
-    const int a_sm = a_trans == 0 ? kGemmLdk : 1, a_sk = a_trans == 0 ? 1 : LDM;
-    const int b_sn = b_trans == 1 ? kGemmLdk : 1, b_sk = b_trans == 1 ? 1 : LDM;
+    constexpr int a_sm = a_trans == 0 ? kGemmLdk : 1, a_sk = a_trans == 0 ? 1 : LDM;
+    constexpr int b_sn = b_trans == 1 ? kGemmLdk : 1, b_sk = b_trans == 1 ? 1 : LDM;
     const int a_lane = (wm0 + lq) * a_sm + lr * a_sk;
     const int b_lane = (wn0 + lq) * b_sn + lr * b_sk;
 
@@ -236,7 +235,7 @@ __device__ __forceinline__ void dgemm_tile(const GemmParams& p, int bx, int by, 
         double* red = smem;
         red[tid] = s;
         __syncthreads();
-        for (int w = kGemmThreads / 2; w > 0; w >>= 1) {
+        for (int w = TH / 2; w > 0; w >>= 1) {
             if (tid < w) red[tid] += red[tid + w];
             __syncthreads();
         }
@@ -268,20 +267,28 @@ __device__ __forceinline__ void dgemm_tile(const GemmParams& p, int bx, int by, 
 
 // With sym_double the grid has half as many column tiles: CTA x handles column tiles x and nbx - 1 - x, whose k ranges
 // (64 (x + 1) and 64 (nbx - x)) add up to the same length for every CTA.
-template <int BT>
-__global__ void __launch_bounds__(kGemmThreads, BT == 64 ? 2 : 1) dgemm_kernel(GemmParams p) {
+template <int BT, int TH, int AT, int BTR>
+__global__ void __launch_bounds__(TH, BT == 64 && TH == 256 ? 2 : 1) dgemm_kernel(GemmParams p) {
     chained_wait();
     if (p.sym_double) {
         const int nbx = (p.N + BT - 1) / BT;
         const int bx = blockIdx.x, bx2 = nbx - 1 - bx;
-        dgemm_tile<BT>(p, bx, blockIdx.y, blockIdx.z, nbx, gridDim.y);
+        dgemm_tile<BT, TH, AT, BTR>(p, bx, blockIdx.y, blockIdx.z, nbx, gridDim.y);
         if (bx2 > bx) {
             __syncthreads();
-            dgemm_tile<BT>(p, bx2, blockIdx.y, blockIdx.z, nbx, gridDim.y);
+            dgemm_tile<BT, TH, AT, BTR>(p, bx2, blockIdx.y, blockIdx.z, nbx, gridDim.y);
         }
         return;
     }
-    dgemm_tile<BT>(p, blockIdx.x, blockIdx.y, blockIdx.z, gridDim.x, gridDim.y);
+    if (p.upper_only) {
+        // upper tiles only, column by column: with a triangular k range (kbeg_mode 1) the longest first
+        int bx = (int)((sqrtf(8.0f * (float)blockIdx.x + 1.0f) - 1.0f) * 0.5f);
+        while ((bx + 1) * (bx + 2) / 2 <= (int)blockIdx.x) ++bx;
+        while (bx * (bx + 1) / 2 > (int)blockIdx.x) --bx;
+        dgemm_tile<BT, TH, AT, BTR>(p, bx, blockIdx.x - bx * (bx + 1) / 2, blockIdx.z, 0, 0);
+        return;
+    }
+    dgemm_tile<BT, TH, AT, BTR>(p, blockIdx.x, blockIdx.y, blockIdx.z, gridDim.x, gridDim.y);
 }
 
 inline GemmParams gemm_defaults() {
@@ -291,6 +298,32 @@ inline GemmParams gemm_defaults() {
     return p;
 }
 
+// The kernel for one pair of operand layouts: 128 x 128 tiles, 64 x 64 tiles with two CTAs per SM, or with one of 16 warps.
+template <int AT, int BTR>
+inline cudaError_t dgemm_attributes() {
+    cudaError_t e = cudaFuncSetAttribute(dgemm_kernel<128, 256, AT, BTR>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)gemm_smem_bytes<128>());
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(dgemm_kernel<64, 256, AT, BTR>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)gemm_smem_bytes<64>());
+    if constexpr (AT == 1)
+        if (e == cudaSuccess)
+            e = cudaFuncSetAttribute(dgemm_kernel<64, 512, AT, BTR>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                     (int)gemm_smem_bytes<64>());
+    return e;
+}
+template <int AT, int BTR>
+inline void dgemm_launch(const GemmParams& p, int bt, int threads, dim3 grid, cudaStream_t stream) {
+    if constexpr (AT == 1) {
+        if (bt == 64 && threads == 512) {
+            launch_chained(dgemm_kernel<64, 512, AT, BTR>, grid, 512, gemm_smem_bytes<64>(), stream, p);
+            return;
+        }
+    }
+    if (bt == 128) launch_chained(dgemm_kernel<128, 256, AT, BTR>, grid, 256, gemm_smem_bytes<128>(), stream, p);
+    else launch_chained(dgemm_kernel<64, 256, AT, BTR>, grid, 256, gemm_smem_bytes<64>(), stream, p);
+}
+
 // Launches with 128x128 tiles when that still fills the GPU, else 64x64.  Also reports the grid used.
 inline int launch_dgemm(int kernel_id, const GemmParams& p, int batches, cudaStream_t stream, int force_bt = 0,
                         dim3* grid_out = nullptr) {
@@ -298,28 +331,29 @@ inline int launch_dgemm(int kernel_id, const GemmParams& p, int batches, cudaStr
     int dst = current_device_state(&dev);
     if (dst) return dst;
     dst = ensure_smem_attr(dev, SA_DGEMM, [] {
-        cudaError_t e = cudaFuncSetAttribute(dgemm_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             (int)gemm_smem_bytes<128>());
-        if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(dgemm_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     (int)gemm_smem_bytes<64>());
-        return e;
+        cudaError_t e = dgemm_attributes<0, 0>();
+        if (e == cudaSuccess) e = dgemm_attributes<0, 1>();
+        return e == cudaSuccess ? dgemm_attributes<1, 0>() : e;
     });
     if (dst) return dst;
     if (p.M <= 0 || p.N <= 0 || batches <= 0) return PTQ_OK;
-    int bt = force_bt;
-    if (bt == 0) {
-        const long tiles128 = (long)cdiv(p.M, 128) * cdiv(p.N, 128) * batches / (p.upper_only ? 2 : 1);
-        bt = tiles128 >= 2 * dev->sms ? 128 : 64;
-    }
+    if (p.a_trans && p.b_trans) return PTQ_ERR_UNSUPPORTED;
+    const long tiles = (long)cdiv(p.M, 64) * cdiv(p.N, 64) * batches / (p.upper_only ? 2 : 1);
+    const long tiles128 = (long)cdiv(p.M, 128) * cdiv(p.N, 128) * batches / (p.upper_only ? 2 : 1);
+    const int bt = force_bt ? force_bt : (tiles128 >= 2 * dev->sms ? 128 : 64);
+    // Sixteen warps finish a tile in half the time but read more of their operands per product: for the triangular product,
+    // whose longest tile is as long as the matrix, while there are few tiles.  With eight / sixteen:
+    // 1152 columns 72 / 64 us, 1600 111 / 86, 2048 150 / 150, 2304 179 / 203 (with the layouts known when compiled 60 at 1152,
+    // 80 at 1600, 136 at 2048, 166 at 2304; in row order of the tiles and with the layouts as arguments 68, 120, 152, 195).
+    const int threads = bt == 64 && p.kbeg_mode == 1 && tiles < 3 * dev->sms ? 512 : 256;
     dim3 grid(cdiv(p.N, bt), cdiv(p.M, bt), p.ksplit > 1 ? p.ksplit : batches);
     if (grid_out) *grid_out = grid;          // the tile grid (what the partials are indexed by)
     if (p.sym_double) grid.x = (grid.x + 1) / 2;
+    if (p.upper_only) grid = dim3(cdiv(p.N, bt) * (cdiv(p.N, bt) + 1) / 2, 1, grid.z);      // M = N
     Launch scope(kernel_id, stream);
-    if (bt == 128)
-        launch_chained(dgemm_kernel<128>, grid, kGemmThreads, gemm_smem_bytes<128>(), stream, p);
-    else
-        launch_chained(dgemm_kernel<64>, grid, kGemmThreads, gemm_smem_bytes<64>(), stream, p);
+    if (p.a_trans) dgemm_launch<1, 0>(p, bt, threads, grid, stream);
+    else if (p.b_trans) dgemm_launch<0, 1>(p, bt, threads, grid, stream);
+    else dgemm_launch<0, 0>(p, bt, threads, grid, stream);
     return launch_status();
 }
 
