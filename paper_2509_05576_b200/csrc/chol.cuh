@@ -669,28 +669,13 @@ __device__ __noinline__ void chol_trailing_phase(double* __restrict__ A, double*
             const double* bs = bbuf + stage * kCholBlock;
             cp_async_wait<0>();
             __syncthreads();         // this piece's operands have landed; the slots of the piece before are free
-            if (more) {
-                // half of the warps request the next operands: the copies keep the issuing warps busy for several
-                // hundred cycles, during which the others already feed the tensor pipe
-                if (warp < 8) {
-                    chol_load_block<kCholThreads / 2>(bbuf + (stage ^ 1) * kCholBlock, nxt.Bsrc, ld, n, k0, nxt.j0, 6, vec16, tid);
-                    if (new_a)
-                        chol_load_block<kCholThreads / 2>(abuf + a_next * kCholBlock, A, ld, n, k0, nxt.i0, LGH, vec16, tid);
-                }
-            }
             double2 acc[FM][FN], old[FM][FN];
 #pragma unroll
             for (int a = 0; a < FM; ++a)
 #pragma unroll
-                for (int b = 0; b < FN; ++b) {
-                    old[a][b] = chol_pair_load(cur, cur.C + (int64_t)(cur.i0 + pr + 8 * a) * ld + cur.j0 + pq + 8 * b, n,
-                                               pr + 8 * a, pq + 8 * b, plain, vec16);
-                    acc[a][b] = make_double2(0.0, 0.0);
-                }
-            // all of it unrolled, addresses as constants: four k steps at a time, both factorisations took 683 + 555 us at 2304
-            // columns, 258 + 253 at 1152 and 1679 + 1243 at 4608; now 662 + 535, 248 + 242 and 1645 + 1198
-#pragma unroll
-            for (int k4 = 0; k4 < kNB / 4; ++k4) {
+                for (int b = 0; b < FN; ++b) acc[a][b] = make_double2(0.0, 0.0);
+            // all k steps unrolled, addresses as constants (four at a time: 3 % slower)
+            auto k_step = [&](int k4) {
                 const int kk = 4 * k4 + lr;
                 double af[FM], bf[FN];
 #pragma unroll
@@ -701,7 +686,33 @@ __device__ __noinline__ void chol_trailing_phase(double* __restrict__ A, double*
                 for (int a = 0; a < FM; ++a)
 #pragma unroll
                     for (int b = 0; b < FN; ++b) dmma_884(acc[a][b].x, acc[a][b].y, af[a], bf[b]);
+            };
+            // The loads of a warp queue in order, so the products go first: the next operands are requested after two k steps, the
+            // old values in the middle.  With both in front, both factorisations took 636 + 520 us at 2304 columns (the second
+            // with the sweep behind it) and 1590 + 1241 at 4608; with the operands alone in front 601 + 508 and 1530 + 1213;
+            // now 591 + 507 and 1509 + 1207.
+            k_step(0);
+            k_step(1);
+            if (more) {
+                // half of the warps request the next operands: the copies keep the issuing warps busy for several
+                // hundred cycles, during which the others already feed the tensor pipe
+                if (warp < 8) {
+                    chol_load_block<kCholThreads / 2>(bbuf + (stage ^ 1) * kCholBlock, nxt.Bsrc, ld, n, k0, nxt.j0, 6, vec16, tid);
+                    if (new_a)
+                        chol_load_block<kCholThreads / 2>(abuf + a_next * kCholBlock, A, ld, n, k0, nxt.i0, LGH, vec16, tid);
+                }
             }
+#pragma unroll
+            for (int k4 = 2; k4 < 8; ++k4) k_step(k4);
+            // the old values
+#pragma unroll
+            for (int a = 0; a < FM; ++a)
+#pragma unroll
+                for (int b = 0; b < FN; ++b)
+                    old[a][b] = chol_pair_load(cur, cur.C + (int64_t)(cur.i0 + pr + 8 * a) * ld + cur.j0 + pq + 8 * b, n,
+                                               pr + 8 * a, pq + 8 * b, plain, vec16);
+#pragma unroll
+            for (int k4 = 8; k4 < kNB / 4; ++k4) k_step(k4);
             cp_async_commit();
 #pragma unroll
             for (int a = 0; a < FM; ++a)
