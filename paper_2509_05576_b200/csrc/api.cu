@@ -90,7 +90,7 @@ int order_launch(const float* W, int rows, int cols, int64_t ldw, const double* 
                                                                                             zero, bits, mode, partial);
     }
     { Launch l(K_SCORE_FINAL, stream); launch_chained(score_final_kernel, cdiv(cols, 128), 128, 0, stream, partial, chunks,
-                                                      cols, Hinv_diag, mode, S, status); }
+                                                      cols, Hinv_diag, (int64_t)1, mode, S, status); }
     { Launch l(K_RANK_SORT, stream); launch_chained(rank_sort_kernel, cdiv(cols, kRankCols), 256, 0, stream, S, cols,
                                                     ascending, perm, nullptr); }
     return launch_status();
@@ -280,7 +280,6 @@ size_t ptq_workspace_bytes(int call_id, int rows, int cols, int n) {
             add((size_t)rows * c * sizeof(double));         // dW
             add((size_t)rows * c);                          // codes of the block being swept
             add(c * sizeof(double));                        // scores
-            add(c * sizeof(double));                        // diagonal
             add((size_t)cdiv(rows, kScoreRowChunk) * c * sizeof(double));
             add(c * sizeof(int32_t));                       // order of the round
             add(c * sizeof(int32_t));                       // original column of every position (ping-pong)
@@ -448,7 +447,6 @@ int ptq_quantize_layer_dynamic(const float* W, int rows, int cols, int64_t ldw, 
     double* dW = cv.take<double>((size_t)rows * c);
     uint8_t* codes_p = cv.take<uint8_t>((size_t)rows * c);
     double* S = cv.take<double>(c);
-    double* diag = cv.take<double>(c);
     const int chunks = cdiv(rows, kScoreRowChunk);
     double* partial = cv.take<double>((size_t)chunks * c);
     int32_t* ordr = cv.take<int32_t>(c);
@@ -465,8 +463,7 @@ int ptq_quantize_layer_dynamic(const float* W, int rows, int cols, int64_t ldw, 
         if (dst) return dst;
     }
 
-    { Launch l(K_DYN_AUX, stream); launch_chained(iota_kernel, cdiv(cols, 256), 256, 0, stream, obuf[0], cols); }
-    const int32_t* ocur = obuf[0];           // original column index of every current position
+    const int32_t* ocur = nullptr;           // original column index of every current position; none yet: itself
     // current state: the m columns still to do, their matrix (upper triangle valid) and their weights
     const double* Acur = Hinv;
     int64_t lda = cols;
@@ -475,8 +472,6 @@ int ptq_quantize_layer_dynamic(const float* W, int rows, int cols, int64_t ldw, 
     int m = cols, done = 0, cur = 0;
     while (m > 0) {
         const int b = block < m ? block : m;
-        { Launch l(K_DYN_AUX, stream); launch_chained(extract_diag_ld_kernel, cdiv(m, 256), 256, 0, stream, Acur, lda, m,
-                                                      diag); }
         if (mode != PTQ_SCORE_NONE) {
             Launch l(K_SCORE_PARTIAL, stream);
             if (Wcur)
@@ -488,8 +483,10 @@ int ptq_quantize_layer_dynamic(const float* W, int rows, int cols, int64_t ldw, 
                                ldw, scale,
                                                                                                zero, bits, mode, partial);
         }
-        { Launch l(K_SCORE_FINAL, stream); launch_chained(score_final_kernel, cdiv(m, 128), 128, 0, stream, partial, chunks,
-                                                          m, diag, mode, S, status); }
+        {
+            Launch l(K_SCORE_FINAL, stream);
+            launch_chained(score_final_kernel, cdiv(m, 128), 128, 0, stream, partial, chunks, m, Acur, lda + 1, mode, S, status);
+        }
         { Launch l(K_RANK_SORT, stream); launch_chained(rank_sort_kernel, cdiv(m, kRankCols), 256, 0, stream, S, m,
                                                         ascending, ordr, ocur); }
         double* An = Abuf[cur];
@@ -497,26 +494,25 @@ int ptq_quantize_layer_dynamic(const float* W, int rows, int cols, int64_t ldw, 
         int32_t* onew = obuf[cur ^ 1];
         {
             Launch l(K_DYN_GATHER, stream);
-            const int gy = m < 4096 ? m : 4096, gr = rows < 4096 ? rows : 4096;
-            launch_chained(gather_upper_kernel, dim3(grid_x_for(m, 256), gy), 256, 0, stream, Acur, lda, ordr, m, An);
+            const dim3 grid(grid_x_for(m, 256), m + rows < 8192 ? m + rows : 8192);
+            const int n_flags = cdiv(rows, kSweepRows) + 1;
             if (Wcur)
-                launch_chained(gather_cols_kernel<double>, dim3(grid_x_for(m, 256), gr), 256, 0, stream, Wcur, ldc, rows, m,
-                               ordr, Wn);
+                launch_chained(round_gather_kernel<double>, grid, 256, 0, stream, Acur, lda, Wcur, ldc, rows, ordr, ocur, m, b, An, Wn, E,
+                               onew, order_out + done, bar, sweep_flags, n_flags);
             else
-                launch_chained(gather_cols_kernel<float>, dim3(grid_x_for(m, 256), gr), 256, 0, stream, W, ldw, rows, m,
-                               ordr, Wn);
-            launch_chained(gather_index_kernel, cdiv(m, 256), 256, 0, stream, ocur, ordr, m, b, onew, order_out + done);
+                launch_chained(round_gather_kernel<float>, grid, 256, 0, stream, Acur, lda, W, ldw, rows, ordr, ocur, m, b, An, Wn, E,
+                               onew, order_out + done, bar, sweep_flags, n_flags);
         }
         int st = PTQ_OK;
         const CholRange range = {0, b < m ? b / kNB : cdiv(m, kNB), cdiv(m, kNB)};
         const int budget = coop_cta_budget(dev), behind = sweep_ctas_behind(rows, b, m, range, budget);
         if (behind > 0) {
             st = factor_sweep_launch(An, m, range, Dbuf, bar, behind, Wn, E, codes_p, scale, zero, rows, b, bits, sweep_flags, status,
-                                     stream, budget, false, false);
+                                     stream, budget, true);
         } else {
-            st = cholesky_upper(An, m, nullptr, Dbuf, bar, status, stream, b < m ? b / kNB : 0);
+            st = cholesky_upper(An, m, nullptr, Dbuf, bar, status, stream, range.stop, 0, 0, true);
             if (st) return st;
-            st = sweep_launch(Wn, An, E, codes_p, scale, zero, rows, b, bits, sweep_flags, status, stream, m);
+            st = sweep_launch(Wn, An, E, codes_p, scale, zero, rows, b, bits, sweep_flags, status, stream, m, true);
         }
         if (st) return st;
         if (b < m) {
@@ -727,12 +723,12 @@ int ptq_quantize_layer(const float* W, int rows, int cols, int64_t ldw, const do
         const int behind = sweep_ctas_behind(rows, cols_now, n, range, budget);
         if (behind > 0) {
             st = factor_sweep_launch(U, n, range, Dbuf, bar, behind, Wp + off, E + off, codes_p + off, scale, zero, rows, cols_now, bits,
-                                     sweep_flags, status, stream, budget, kf == 0, true);
+                                     sweep_flags, status, stream, budget, kf == 0);
         } else {
             st = cholesky_upper(U, n, nullptr, Dbuf, bar, status, stream, range.stop, range.first, range.row_limit, kf == 0);
             if (st) return st;
             st = sweep_launch(Wp + off, U + (size_t)off * (n + 1), E + off, codes_p + off, scale, zero, rows, cols_now, bits, sweep_flags,
-                              status, stream, n, true, kf == 0);
+                              status, stream, n, kf == 0);
         }
         if (st) return st;
         if (rest > 0) {

@@ -633,13 +633,12 @@ __global__ void __launch_bounds__(kCholThreads, 1) factor_sweep_kernel(FactorArg
 }
 
 // Launches the sweep: one CTA per SM, cooperative so that every CTA a waiting CTA depends on is resident.
-// n columns are swept; ld (0: n) is the row stride of Wp, U, E and codes_p, so that the first n columns of wider
+// n columns are swept; ld is the row stride of Wp, U, E and codes_p, so that the first n columns of wider
 // arrays can be swept (the rows of U beyond column n are then applied by the caller).
-// e_ready, flags_ready: the caller has set E to NaN and the progress counters to zero.
+// The caller has set E to NaN and, with flags_ready, the progress counters to zero.
 inline int sweep_launch(double* Wp, const double* U, double* E, uint8_t* codes_p, const float* scale, const float* zero,
                         int rows, int n, int bits, unsigned* flags, int32_t* status, cudaStream_t stream,
-                        int64_t ld = 0, bool e_ready = false, bool flags_ready = false) {
-    if (ld == 0) ld = n;
+                        int64_t ld, bool flags_ready) {
     DeviceState* dev = nullptr;
     int st = current_device_state(&dev);
     if (st) return st;
@@ -662,10 +661,6 @@ inline int sweep_launch(double* Wp, const double* U, double* E, uint8_t* codes_p
     }
     const int groups = cdiv(rows, kSweepRows);
     if (!flags_ready && cudaMemsetAsync(flags, 0, ((size_t)groups + 1) * sizeof(unsigned), stream) != cudaSuccess)
-        return PTQ_ERR_CUDA;
-    // every byte 0xFF is a NaN: "not published yet" for the owner of the next block, which polls the values themselves
-    if (!e_ready && cudaMemset2DAsync(E, (size_t)ld * sizeof(double), 0xFF, (size_t)n * sizeof(double), (size_t)rows, stream) !=
-        cudaSuccess)
         return PTQ_ERR_CUDA;
     SweepParams prm;
     prm.Wp = Wp; prm.U = U; prm.E = E; prm.codes_p = codes_p; prm.scale = scale; prm.zero = zero;
@@ -715,11 +710,11 @@ inline int sweep_ctas_behind(int rows, int sweep_n, int n, const CholRange& rang
 }
 
 // The factorisation of a range of block rows of U (n x n, row stride n) and the sweep of the first sweep_n columns of that range
-// in one launch.  Wp, E, codes_p: from the column of the first block row on, row stride n.  ready: the caller has set the
-// counters and flags to zero and E to NaN.
+// in one launch.  Wp, E, codes_p: from the column of the first block row on, row stride n.  The caller has set E to
+// NaN and, with counters_ready, the counters and flags to zero.
 inline int factor_sweep_launch(double* U, int n, const CholRange& range, double* Dbuf, unsigned* bar, int sweep_ctas, double* Wp,
                                double* E, uint8_t* codes_p, const float* scale, const float* zero, int rows, int sweep_n, int bits,
-                               unsigned* flags, int32_t* status, cudaStream_t stream, int budget, bool counters_ready, bool e_ready) {
+                               unsigned* flags, int32_t* status, cudaStream_t stream, int budget, bool counters_ready) {
     DeviceState* dev = nullptr;
     int st = current_device_state(&dev);
     if (st) return st;
@@ -735,9 +730,6 @@ inline int factor_sweep_launch(double* U, int n, const CholRange& range, double*
     const int groups = cdiv(rows, kSweepRows);
     if (!counters_ready && (cudaMemsetAsync(bar, 0, 2 * sizeof(unsigned), stream) != cudaSuccess ||
                             cudaMemsetAsync(flags, 0, ((size_t)groups + 1) * sizeof(unsigned), stream) != cudaSuccess))
-        return PTQ_ERR_CUDA;
-    if (!e_ready && cudaMemset2DAsync(E, (size_t)n * sizeof(double), 0xFF, (size_t)sweep_n * sizeof(double), (size_t)rows, stream) !=
-        cudaSuccess)
         return PTQ_ERR_CUDA;
     FactorArgs f;
     f.A = U; f.Dbuf = Dbuf; f.n = n; f.ld = n; f.range = range;

@@ -104,9 +104,9 @@ __global__ void __launch_bounds__(256) score_partial_kernel(const T* __restrict_
     }
 }
 
-// S_j = (sum of the chunk partials, ascending) / (2 [Hinv]_jj)  for the sensitivity modes.
+// S_j = (sum of the chunk partials, ascending) / (2 [Hinv]_jj)  for the sensitivity modes; hinv_diag[j diag_step] is [Hinv]_jj.
 __global__ void __launch_bounds__(128) score_final_kernel(const double* __restrict__ partial, int chunks, int cols,
-                                                           const double* __restrict__ hinv_diag, int mode,
+                                                           const double* __restrict__ hinv_diag, int64_t diag_step, int mode,
                                                            double* __restrict__ S, int32_t* status) {
     chained_begin();
     const int j = blockIdx.x * 128 + threadIdx.x;
@@ -114,7 +114,7 @@ __global__ void __launch_bounds__(128) score_final_kernel(const double* __restri
     double s = 0.0;
     if (mode != PTQ_SCORE_NONE) {
         for (int ch = 0; ch < chunks; ++ch) s += partial[(int64_t)ch * cols + j];
-        if (mode == PTQ_SCORE_QERR || mode == PTQ_SCORE_PRUNE) s = s / (2.0 * hinv_diag[j]);
+        if (mode == PTQ_SCORE_QERR || mode == PTQ_SCORE_PRUNE) s = s / (2.0 * hinv_diag[j * diag_step]);
     }
     if (!isfinite(s)) report(status, PTQ_ERR_NONFINITE, j);
     S[j] = s;
