@@ -362,7 +362,7 @@ int ptq_prepare_hinv(const double* H, int cols, int damp_mode, double damp, doub
     double* Dbuf = cv.take<double>(chol_scratch_doubles(n));
     void* pws = chol_panel_workspace_bytes(n) ? static_cast<void*>(cv.take<char>(chol_panel_workspace_bytes(n))) : nullptr;
     { Launch l(K_LAMBDA, stream); launch_chained(lambda_kernel, 1, 256, 0, stream, H, n, damp_mode, damp, lambda_out, status); }
-    { Launch l(K_DAMP_COPY, stream); launch_chained(damp_copy_kernel, dim3(grid_x_for(n, 256), n), 256, 0, stream, H, R, V,
+    { Launch l(K_DAMP_COPY, stream); launch_chained(damp_copy_kernel, dim3(cdiv(n, 1024), n), 256, 0, stream, H, R, V,
                                                     n, lambda_out, bar); }
     // W = U^-T comes out of the factorisation sweep itself (V must start as zero)
     int st = cholesky_upper_auto(R, n, V, Dbuf, bar, pws, status, stream, true);
@@ -700,18 +700,26 @@ int ptq_quantize_layer(const float* W, int rows, int cols, int64_t ldw, const do
     void* pws = n >= kPanelMinCols ? static_cast<void*>(cv.take<char>(chol_panel_workspace_bytes(n))) : nullptr;
     void* ews = n >= kPanelMinCols ? static_cast<void*>(cv.take<char>(x_operand_bytes(rows, kPanelBlocks * kNB))) : nullptr;
 
+    DeviceState* dev = nullptr;
+    int st = current_device_state(&dev);
+    if (st) return st;
+    st = ensure_smem_attr(dev, SA_GATHER, [] {
+        return cudaFuncSetAttribute(sweep_gather_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                    kGatherMaxCols * (int)sizeof(double));
+    });
+    if (st) return st;
     const int n_flags = cdiv(rows, kSweepRows) + 1;
     { Launch l(K_PERM_CHECK, stream); launch_chained(perm_check_kernel, cdiv(n, 256), 256, 0, stream, perm, n, invperm, bar,
                                                      sweep_flags, n_flags, status); }
     {
         Launch l(K_SWEEP_GATHER, stream);
-        const int gy = n + rows < kMaxGridY ? n + rows : kMaxGridY;
-        launch_chained(sweep_gather_kernel, dim3(grid_x_for(n, 256), gy), 256, 0, stream, Hinv, W, rows, n, ldw, perm,
-                       invperm, U, Wp, E, status);
+        if (n <= kGatherMaxCols)
+            launch_chained(sweep_gather_kernel<true>, n + rows, kGatherThreads, (size_t)n * sizeof(double), stream, Hinv, W, rows, n, ldw,
+                           perm, invperm, U, Wp, E, status);
+        else
+            launch_chained(sweep_gather_kernel<false>, n + rows, kGatherThreads, 0, stream, Hinv, W, rows, n, ldw, perm, invperm, U, Wp, E,
+                           status);
     }
-    DeviceState* dev = nullptr;
-    int st = current_device_state(&dev);
-    if (st) return st;
     // Blocked Eq. 12 and the sweep: of everything at once, or, on wide layers, panel by panel (cholpanel.cuh).  There the part of
     // Eq. 11 that a panel's columns owe to all later ones, W[:, later] -= E[:, panel] U[panel, later], is one large product on
     // the int8 tensor path, as the panel's share of Eq. 12 is; both take the same slices of U.  (4096 x 11008 with the
@@ -752,7 +760,7 @@ int ptq_quantize_layer(const float* W, int rows, int cols, int64_t ldw, const do
     int8_t* kexp = sliced ? reinterpret_cast<int8_t*>(Dbuf) : nullptr;      // the factorisation is done with Dbuf
     {
         Launch l(K_FINALIZE, stream);
-        launch_chained(finalize_kernel, dim3(grid_x_for(n, 256), rows), 256, 0, stream, codes_p, invperm, W, rows, n, ldw,
+        launch_chained(finalize_kernel, dim3(cdiv(n, 1024), rows), 256, 0, stream, codes_p, invperm, W, rows, n, ldw,
                        scale,
                                                                            zero, codes, What, dW, H_undamped, kexp);
     }

@@ -33,32 +33,52 @@ __global__ void __launch_bounds__(256) perm_check_kernel(const int32_t* __restri
     invperm[j] = p;
 }
 
-// Everything the sweep starts from, one grid row per row of the matrix and then of the weights:
+// Everything the sweep starts from, one CTA per row of the matrix and then of the weights:
 //   A[a][b] = Hinv[perm[a]][perm[b]] for b from the start of row a's 64-column diagonal tile on: the factorisation and
 //   everything after it read the upper triangle only (whole 64 x 64 tiles on the diagonal), the rest of A is left alone;
 //   Wp[i][p] = (double) W[i][perm[p]];  E[i][p] = NaN, "not published yet" for the owners of the next blocks, which poll
 //   the values themselves.
 // A position whose column some other position also names (invperm points elsewhere) is reported.
 // One launch in place of three kernels' and clears' worth of them: they are short and a launch takes about as long.
-__global__ void __launch_bounds__(256) sweep_gather_kernel(const double* __restrict__ Hinv, const float* __restrict__ W, int rows,
-                                                            int n, int64_t ldw, const int32_t* __restrict__ perm,
-                                                            const int32_t* __restrict__ invperm, double* __restrict__ A,
-                                                            double* __restrict__ Wp, double* __restrict__ E, int32_t* status) {
+// STAGED: the row comes as it lies into shared memory and is picked apart there; out of memory every value would move a
+// sector of four.  For rows of up to kGatherMaxCols columns; wider ones are read in place.  31 -> 17 us at 256 x 2304, 110 -> 55 at
+// 512 x 4608, 913 -> 429 at 4096 x 11008.
+constexpr int kGatherThreads = 512, kGatherMaxCols = 25600;
+template <bool STAGED>
+__global__ void __launch_bounds__(kGatherThreads) sweep_gather_kernel(const double* __restrict__ Hinv, const float* __restrict__ W,
+                                                                      int rows, int n, int64_t ldw, const int32_t* __restrict__ perm,
+                                                                      const int32_t* __restrict__ invperm, double* __restrict__ A,
+                                                                      double* __restrict__ Wp, double* __restrict__ E, int32_t* status) {
     chained_begin();
-    const int step = gridDim.x * 256, first = blockIdx.x * 256 + threadIdx.x;
-    const int total = n + rows;
-    for (int y = blockIdx.y; y < total; y += gridDim.y) {
-        if (y < n) {
-            const int src_row = perm[y];
-            if (first == 0 && src_row >= 0 && src_row < n && invperm[src_row] != y) report(status, PTQ_ERR_INVALID_ARG, y, 2);
-            const int64_t src = (int64_t)clamp_index(src_row, n) * n;
-            for (int b = (y & ~(kNB - 1)) + first; b < n; b += step) A[(int64_t)y * n + b] = Hinv[src + clamp_index(perm[b], n)];
-        } else {
-            const int i = y - n;
-            for (int q = first; q < n; q += step) {
-                Wp[(int64_t)i * n + q] = (double)W[(int64_t)i * ldw + clamp_index(perm[q], n)];
-                E[(int64_t)i * n + q] = __longlong_as_double(-1ll);
-            }
+    extern __shared__ __align__(16) unsigned char gather_row[];
+    const int y = blockIdx.x, tid = threadIdx.x;
+    if (y < n) {
+        const int src_row = perm[y];
+        if (tid == 0 && src_row >= 0 && src_row < n && invperm[src_row] != y) report(status, PTQ_ERR_INVALID_ARG, y, 2);
+        const double* src = Hinv + (int64_t)clamp_index(src_row, n) * n;
+        double* row = reinterpret_cast<double*>(gather_row);
+        if (STAGED) {
+            for (int j = tid; j < n; j += kGatherThreads) cp_async8(row + j, src + j, true);
+            cp_async_commit();
+            cp_async_wait<0>();
+            __syncthreads();
+        }
+        for (int b = (y & ~(kNB - 1)) + tid; b < n; b += kGatherThreads) {
+            const int j = clamp_index(perm[b], n);
+            A[(int64_t)y * n + b] = STAGED ? row[j] : src[j];
+        }
+    } else {
+        const int i = y - n;
+        const float* src = W + (int64_t)i * ldw;
+        float* row = reinterpret_cast<float*>(gather_row);
+        if (STAGED) {
+            for (int j = tid; j < n; j += kGatherThreads) row[j] = src[j];
+            __syncthreads();
+        }
+        for (int q = tid; q < n; q += kGatherThreads) {
+            const int j = clamp_index(perm[q], n);
+            Wp[(int64_t)i * n + q] = (double)(STAGED ? row[j] : src[j]);
+            E[(int64_t)i * n + q] = __longlong_as_double(-1ll);
         }
     }
 }
@@ -761,7 +781,8 @@ __device__ __forceinline__ int loss_exponent(double d) {
 }
 
 // Back to the original column order: codes, What = float32(scale * (code - zero)), dW = W - What (float64).  With kexp, also
-// the exponents by which the loss equilibrates its operands, from the diagonal of H.
+// the exponents by which the loss equilibrates its operands, from the diagonal of H.  Up to four columns a thread (4096 x 11008
+// 292 -> 206 us).
 __global__ void finalize_kernel(const uint8_t* __restrict__ codes_p, const int32_t* __restrict__ invperm,
                                 const float* __restrict__ W, int rows, int cols, int64_t ldw,
                                 const float* __restrict__ scale, const float* __restrict__ zero,

@@ -141,7 +141,7 @@ constexpr long long kSpinLimitCycles = 4000000000LL;
 // (cudaFuncSetAttribute is per device).  One table, one mutex; looked up with the caller's device current.
 // ---------------------------------------------------------------------------------------------------------
 constexpr int kMaxDevices = 64;
-enum SmemAttrSlot { SA_CHOL = 0, SA_SWEEP, SA_GRAM, SA_DGEMM, SA_SMALL, SA_XGEMM, SA_FACTOR_SWEEP, SA_COUNT };
+enum SmemAttrSlot { SA_CHOL = 0, SA_SWEEP, SA_GRAM, SA_DGEMM, SA_SMALL, SA_XGEMM, SA_FACTOR_SWEEP, SA_GATHER, SA_COUNT };
 struct DeviceState {
     int sms = 0;
     int coop = 0;

@@ -68,6 +68,26 @@ def _loss_bound(D, H, loss):
     return 3.0 * u * D.shape[1] ** 0.5 * torch.linalg.norm(D * (D.abs() @ H.abs())).item() + 4.0 * u * abs(float(loss))
 
 
+@pytest.mark.parametrize("n,k", [(8, 1024), (65, 1024), (333, 1000), (40, 7)])
+def test_columns_are_sliced_alike_in_one_pass_and_in_two(n, k):
+    """Columns of up to 1024 values are cut into digits in one pass, longer ones in two.  With zeros below, the same columns
+    go the other way: the product is the same bit for bit."""
+    g = torch.Generator(device="cuda").manual_seed(n + k)
+    A = torch.randn((70, k), dtype=torch.float64, device="cuda", generator=g)
+    B = torch.randn((k, n + 3), dtype=torch.float64, device="cuda", generator=g)[:, :n]
+    B *= torch.exp(3.0 * torch.randn(n, dtype=torch.float64, device="cuda", generator=g))
+    out = []
+    for rows in (k, 1025 + k):
+        a, b = torch.zeros((70, rows), dtype=torch.float64, device="cuda"), torch.zeros((rows, n), dtype=torch.float64, device="cuda")
+        a[:, :k], b[:k] = A, B
+        C, st = torch.zeros((70, n), dtype=torch.float64, device="cuda"), ptq.new_status()
+        ptq.gemm_nt_sliced(C, a, b, 1.0, ptq.Workspace(), st, b_is_kn=True)
+        ptq.check_status(st)
+        out.append(C)
+    assert torch.equal(out[0], out[1])
+    assert torch.allclose(out[0], A @ B, rtol=0.0, atol=1e-15 * float((A.abs() @ B.abs()).max()))
+
+
 @pytest.mark.parametrize("rows,cols,sliced", [
     (512, 2304, True), (1000, 1791, True), (1400, 1400, True), (2600, 1024, True),     # above the line, the slices fit
     (560, 2304, False), (2561, 1025, False),                                           # above the line, they do not
