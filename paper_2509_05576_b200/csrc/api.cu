@@ -53,6 +53,12 @@ bool sliced_loss(int rows, int cols) {
            x_operand_bytes(cols, cols) <= (size_t)cols * cols * sizeof(double) &&
            2 * (size_t)x_num_tiles(rows, cols) <= loss_partials_count(rows, cols);
 }
+// Digits of E and U in the deferred part of Eq. 11 of layers that are swept panel by panel.  With eight the product is more
+// exact than the float64 MMA steps of the sweep for every kind of input measured, with seven it is less exact where the input
+// channels differ in scale (i8gemm.cuh).  Layers this tall and wide have never had float64 steps and keep seven: eight
+// would take 7.19 -> 7.32 ms at 4096 x 4096 and 53.6 -> 54.8 at 4096 x 11008.  Below, seven -> eight: 512 x 4608 6.18 -> 6.22 ms,
+// 2000 x 4608 7.63 -> 7.73, 512 x 8192 19.2 -> 19.3, 2000 x 8000 21.7 -> 22.1.
+inline int deferred_digits(int rows, int cols) { return rows >= 2048 && cols >= 4096 ? kXSlices : kXMoreSlices; }
 // The float64 loss product is cut along k into as many slices as it takes to put about two CTAs on every SM.
 int loss_ksplit(int rows, int cols) {
     const long ctas = (long)cdiv(rows, 64) * ((cdiv(cols, 64) + 1) / 2);
@@ -264,7 +270,8 @@ size_t ptq_workspace_bytes(int call_id, int rows, int cols, int n) {
             add(((size_t)cdiv(rows, kSweepRows) + 1) * sizeof(unsigned));   // per-row-group progress counters of the sweep
             add(chol_scratch_doubles(cols) * sizeof(double));
             add(chol_panel_workspace_bytes(cols));
-            if (cols >= kPanelMinCols) add(x_operand_bytes(rows, kPanelBlocks * kNB));   // slices of E[:, panel]
+            if (cols >= kPanelMinCols)                      // slices of E[:, panel]
+                add(x_operand_bytes(rows, kPanelBlocks * kNB, deferred_digits(rows, cols)));
             break;
         case PTQ_CALL_QUANTIZE_LAYER_PER_ROW:
             if (rows < 1) return 0;
@@ -698,7 +705,8 @@ int ptq_quantize_layer(const float* W, int rows, int cols, int64_t ldw, const do
     unsigned* sweep_flags = cv.take<unsigned>((size_t)cdiv(rows, kSweepRows) + 1);
     double* Dbuf = cv.take<double>(chol_scratch_doubles(n));
     void* pws = n >= kPanelMinCols ? static_cast<void*>(cv.take<char>(chol_panel_workspace_bytes(n))) : nullptr;
-    void* ews = n >= kPanelMinCols ? static_cast<void*>(cv.take<char>(x_operand_bytes(rows, kPanelBlocks * kNB))) : nullptr;
+    const int digits = deferred_digits(rows, n);
+    void* ews = n >= kPanelMinCols ? static_cast<void*>(cv.take<char>(x_operand_bytes(rows, kPanelBlocks * kNB, digits))) : nullptr;
 
     DeviceState* dev = nullptr;
     int st = current_device_state(&dev);
@@ -742,14 +750,14 @@ int ptq_quantize_layer(const float* W, int rows, int cols, int64_t ldw, const do
         if (rest > 0) {
             Carver pv(pws), ev(ews);
             double* below = U + (size_t)off * n + off + cols_now;                 // U[panel, later]
-            const XOperand u = x_slice_operand(pv, below, n, 1, rest, cols_now, status, stream);
+            const XOperand u = x_slice_operand(pv, below, n, 1, rest, cols_now, status, stream, nullptr, 1, digits);
             st = chol_apply_panel(U, n, off + cols_now, u, status, stream);
             if (st) return st;
-            const XOperand e = x_slice_operand(ev, E + off, n, 0, rows, cols_now, status, stream);
+            const XOperand e = x_slice_operand(ev, E + off, n, 0, rows, cols_now, status, stream, nullptr, 1, digits);
             XGemmParams prm{};
             prm.C = Wp + off + cols_now; prm.ldc = n; prm.alpha = -1.0; prm.status = status;
             prm.out_mode = X_OUT_ADD; prm.k_mode = X_K_ALL;
-            st = x_product(e, u, prm, stream);
+            st = x_product(e, u, prm, stream, digits);
             if (st) return st;
         }
     }

@@ -20,9 +20,17 @@
 // without either measure): channel scales log-normal with sigma 2: 5e-15 / 1e-15 / 3e-14; four channels 10^4 times larger whose
 // weights are zero: 3e-16 / 4e-16 / 4e-13; one component shared by all channels: 7e-13 / 7e-13 / 6e-12.
 //
-// Kernel: one 128 x 64 output tile per CTA iteration.  A TMA producer warp streams 64-wide K blocks of the seven
-// slices of both operands (SWIZZLE_64B, 2 stages of 84 KB); one thread issues the 20 tcgen05.mma.kind::i8 of a stage
-// into seven TMEM accumulators (7 x 64 columns; the loss: 22 into eight); four epilogue warps read them back with tcgen05.ld, combine, hand TMEM
+// The deferred part of Eq. 11 adds terms E_ir U_rj to weights of any size, and where the input channels differ in scale
+// neither a row of E nor a column of U is of one size.  Where it stands in for float64 MMA steps of 64 columns (deferred_digits
+// in api.cu) its operands have eight digits (|x| 2^sh < 2^62) and the groups up to 7 are kept (36 products).  Error of the updated
+// weights against extended precision over that of the float64 steps, root mean square / worst column of 2048, behind 1024
+// of 3072 columns (eight digits / seven digits / seven digits with group 7): channels of one scale 0.25 / 0.8, 0.4 / 1.7,
+// 0.26 / 0.8; channel scales log-normal with sigma 2 0.25 / 0.8, 7.2 / 41, 0.5 / 2.6; those with a small absolute damping
+// 0.19 / 0.7, 17 / 88, 1.25 / 4.3; four channels 10^4 times larger, the same damping 0.12 / 0.6, 15 / 66, 0.9 / 3.9.
+//
+// Kernel: one 128 x 64 output tile per CTA iteration.  A TMA producer warp streams 64-wide K blocks of the seven (eight)
+// slices of both operands (SWIZZLE_64B, 2 stages of 84 (96) KB); one thread issues the 20 tcgen05.mma.kind::i8 of a stage
+// into seven TMEM accumulators (7 x 64 columns; the loss: 22 into eight; eight digits: 24 into eight); four epilogue warps read them back with tcgen05.ld, combine, hand TMEM
 // back (the next tile's products then overlap the rest of the epilogue) and add into C through a shared-memory
 // transpose, so that the read-modify-write of C is coalesced.  Every mbarrier wait is bounded.
 #pragma once
@@ -33,22 +41,25 @@
 namespace ptq {
 
 constexpr int kXSlices = 7;
+constexpr int kXMoreSlices = 8;              // the digits of the seven, and one below them
 constexpr int kXGroups = 7;                  // groups g = s + t = 0..6
-constexpr int kXLossGroups = 8;              // and 7: all of TMEM (8 x 64 columns)
+constexpr int kXMoreGroups = 8;              // and 7: all of TMEM (8 x 64 columns)
 constexpr int kXTM = 128, kXTN = 64, kXKB = 64;
 constexpr int kXStages = 2;
 constexpr int kXABytes = kXTM * kXKB;        // 8 KB per slice
 constexpr int kXBBytes = kXTN * kXKB;        // 4 KB per slice
-constexpr int kXStageBytes = kXSlices * (kXABytes + kXBBytes);     // 84 KB
+__host__ __device__ constexpr int x_stage_bytes(int slices) { return slices * (kXABytes + kXBBytes); }     // 84 KB, 96 KB
 static_assert(kXABytes == kGramABytes && kXBBytes == kGramBBytes && kXTN == kGramTN, "tc_slice_products relies on them");
 constexpr int kXEpiDoubles = 4 * 32 * 17;    // per epilogue warp: 32 rows x 16 columns (+1 padding)
-constexpr int kXSmemBytes = kXStages * kXStageBytes + 1024 /*align*/ + 256 /*barriers*/ + kXEpiDoubles * 8;
+constexpr int x_smem_bytes(int slices) { return kXStages * x_stage_bytes(slices) + 1024 /*align*/ + 256 /*barriers*/ + kXEpiDoubles * 8; }
+static_assert(x_smem_bytes(kXMoreSlices) <= 227 * 1024, "shared memory of a CTA");
 constexpr int kXThreads = 192;               // warp 0: TMA, warp 1: MMA + TMEM, warps 2..5: epilogue
 constexpr int kXShiftTarget = 54;
 constexpr int kXMaxK = 16384;                // 7 * 2^14 * 16384 < 2^31
+constexpr int kXMoreMaxK = 8192;             // 8 * 2^14 * 8192 < 2^31
 
-inline size_t i8gemm_plane_bytes(int rows, int k) {
-    return (size_t)kXSlices * (size_t)(cdiv(rows, 128) * 128) * (size_t)(cdiv(k, 128) * 128);
+inline size_t i8gemm_plane_bytes(int rows, int k, int slices = kXSlices) {
+    return (size_t)slices * (size_t)(cdiv(rows, 128) * 128) * (size_t)(cdiv(k, 128) * 128);
 }
 inline size_t i8gemm_workspace_bytes(int m, int n, int k) {
     return align_up(i8gemm_plane_bytes(m, k)) + align_up(i8gemm_plane_bytes(n, k)) +
@@ -63,7 +74,8 @@ inline size_t i8gemm_workspace_bytes(int m, int n, int k) {
 constexpr double kXMaxMagnitude = 8.452712498170644e270;     // 2^900
 constexpr int kXShiftBad = -1000;
 static_assert(1023 + 24 - kXShiftBad == 2047, "exponent field of an infinity");
-// Shift of a row whose largest magnitude is m: |x| 2^sh < 2^54 (0 for an all-zero row); at most `most`.
+// Shift of a row whose largest magnitude is m: |x| 2^sh < 2^54 (0 for an all-zero row); at most `most`.  With eight digits the
+// integer is x 2^(sh + 8) and its first seven digits stand for x 2^sh, so the shift is the same for both.
 __device__ __forceinline__ int x_row_shift(double m, int most = 900) {
     if (!(m < kXMaxMagnitude)) return kXShiftBad;
     if (!(m > 0.0)) return 0;
@@ -74,8 +86,8 @@ __device__ __forceinline__ int x_row_shift(double m, int most = 900) {
 // Slices of the rows of X [rows x k] (row stride ld): Q[s][row][kk], one CTA per (padded) row.  KEXP: the columns are
 // multiplied by 2^(ksign kexp[kk]) first; kexp is 4-byte aligned and may be read up to its next multiple of four.  (One byte
 // an exponent: what is read beside a row is an eighth of it.  4608 x 4608: 59 us without, 60 us with exponents.)
-template <bool KEXP>
-__global__ void __launch_bounds__(256, 6) x_slice_rows_kernel(const double* __restrict__ X, int rows, int k, int64_t ld,
+template <bool KEXP, int SLICES>
+__global__ void __launch_bounds__(256, SLICES == kXSlices ? 6 : 5) x_slice_rows_kernel(const double* __restrict__ X, int rows, int k, int64_t ld,
                                                               int rows_pad, int k_pad, int8_t* __restrict__ Q,
                                                               int32_t* __restrict__ shifts, int32_t* status,
                                                               const int8_t* __restrict__ kexp, int ksign) {
@@ -87,7 +99,7 @@ __global__ void __launch_bounds__(256, 6) x_slice_rows_kernel(const double* __re
     if (row >= rows) {
         for (int kk = threadIdx.x * 4; kk < k_pad; kk += 1024)
 #pragma unroll
-            for (int s = 0; s < kXSlices; ++s) *reinterpret_cast<uint32_t*>(q0 + s * plane + kk) = 0u;
+            for (int s = 0; s < SLICES; ++s) *reinterpret_cast<uint32_t*>(q0 + s * plane + kk) = 0u;
         if (threadIdx.x == 0) shifts[row] = 0;
         return;
     }
@@ -122,12 +134,12 @@ __global__ void __launch_bounds__(256, 6) x_slice_rows_kernel(const double* __re
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
             const double xv = kk + u < kx ? x[kk + u] : 0.0;
-            v[u] = __double2ll_rn(xv * power_of_two(KEXP ? sh0 + ksign * e[u] : sh0));
+            v[u] = __double2ll_rn(xv * power_of_two((KEXP ? sh0 + ksign * e[u] : sh0) + 8 * (SLICES - kXSlices)));
         }
-        uint32_t packed[kXSlices];
-        pack_digits4<kXSlices>(v, packed);
+        uint32_t packed[SLICES];
+        pack_digits4<SLICES>(v, packed);
 #pragma unroll
-        for (int s = 0; s < kXSlices; ++s) *reinterpret_cast<uint32_t*>(q0 + s * plane + kk) = packed[s];
+        for (int s = 0; s < SLICES; ++s) *reinterpret_cast<uint32_t*>(q0 + s * plane + kk) = packed[s];
     }
 }
 
@@ -212,6 +224,7 @@ __global__ void __launch_bounds__(256) x_slice_cols_kernel(const double* __restr
 // columns 34 -> 26 us; 512 x 4608 6967 -> 6843 us, 4096 x 4096 7892 -> 7798.
 constexpr int kXOnceMaxK = 1024, kXOnceCols = 8, kXOnceLd = kXOnceCols + 1;       // odd: four rows on are eight banks on
 inline size_t x_once_smem_bytes(int k_pad) { return (size_t)k_pad * kXOnceLd * sizeof(double); }
+template <int SLICES>
 __global__ void __launch_bounds__(256, 3) x_slice_cols_once_kernel(const double* __restrict__ X, int k, int cols, int64_t ld, int cols_pad,
                                                                    int k_pad, int8_t* __restrict__ Q, int32_t* __restrict__ shifts,
                                                                    int32_t* status) {
@@ -249,16 +262,16 @@ __global__ void __launch_bounds__(256, 3) x_slice_cols_once_kernel(const double*
     const int lane = tid & 31, warp = tid >> 5, oc = (warp & 1) * 4 + (lane & 3);
     const int sh = x_row_shift(__longlong_as_double((long long)smax[0][oc]));
     const bool bad = sh == kXShiftBad;
-    const double scale = power_of_two(bad ? 0 : sh);
+    const double scale = power_of_two(bad ? 0 : sh + 8 * (SLICES - kXSlices));
     int8_t* q = Q + (size_t)(c0 + oc) * k_pad;
     for (int k0 = (warp >> 1) * 32 + (lane >> 2) * 4; k0 < k_pad; k0 += 128) {
         long long v[4];
 #pragma unroll
         for (int u = 0; u < 4; ++u) v[u] = bad ? 0ll : __double2ll_rn(x_once_tile[(k0 + u) * kXOnceLd + oc] * scale);
-        uint32_t packed[kXSlices];
-        pack_digits4<kXSlices>(v, packed);
+        uint32_t packed[SLICES];
+        pack_digits4<SLICES>(v, packed);
 #pragma unroll
-        for (int s = 0; s < kXSlices; ++s) *reinterpret_cast<uint32_t*>(q + s * plane + k0) = packed[s];
+        for (int s = 0; s < SLICES; ++s) *reinterpret_cast<uint32_t*>(q + s * plane + k0) = packed[s];
     }
 }
 
@@ -300,23 +313,24 @@ __device__ __forceinline__ bool x_tile_range(const XGemmParams& prm, int bi, int
     return kb0 < kb1;
 }
 
-template <int GROUPS>
+template <int GROUPS, int SLICES>
 __global__ void __launch_bounds__(kXThreads, 1)
 i8gemm_kernel(const __grid_constant__ CUtensorMap tmapA, const __grid_constant__ CUtensorMap tmapB, XGemmParams prm) {
     chained_wait();
+    constexpr int kStageBytes = x_stage_bytes(SLICES);
     extern __shared__ unsigned char xg_smem_raw[];
     const uint32_t raw = smem_u32(xg_smem_raw);
     const uint32_t base = (raw + 1023u) & ~1023u;
     unsigned char* base_ptr = xg_smem_raw + (base - raw);
-    uint64_t* bars = reinterpret_cast<uint64_t*>(base_ptr + kXStages * kXStageBytes);
-    const uint32_t bar0 = base + kXStages * kXStageBytes;
+    uint64_t* bars = reinterpret_cast<uint64_t*>(base_ptr + kXStages * kStageBytes);
+    const uint32_t bar0 = base + kXStages * kStageBytes;
     auto full_bar = [&](int s) { return bar0 + 8u * s; };
     auto empty_bar = [&](int s) { return bar0 + 8u * (kXStages + s); };
     const uint32_t acc_full = bar0 + 8u * (2 * kXStages);
     const uint32_t acc_empty = bar0 + 8u * (2 * kXStages + 1);
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * kXStages + 2);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
-    double* epi = reinterpret_cast<double*>(base_ptr + kXStages * kXStageBytes + 256);
+    double* epi = reinterpret_cast<double*>(base_ptr + kXStages * kStageBytes + 256);
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int nkb = prm.k_pad / kXKB;
@@ -358,13 +372,13 @@ i8gemm_kernel(const __grid_constant__ CUtensorMap tmapA, const __grid_constant__
                 for (int kb = kb0; kb < kb1 && ok; ++kb) {
                     ok = mbar_wait_bounded(empty_bar(stage), phase ^ 1u, abort_flag);
                     if (!ok) break;
-                    const uint32_t sbase = base + stage * kXStageBytes;
-                    mbar_arrive_expect_tx(full_bar(stage), kXStageBytes);
+                    const uint32_t sbase = base + stage * kStageBytes;
+                    mbar_arrive_expect_tx(full_bar(stage), kStageBytes);
                     armed[stage] = (int)phase;
 #pragma unroll
-                    for (int s = 0; s < kXSlices; ++s) {
+                    for (int s = 0; s < SLICES; ++s) {
                         tma_load_3d(sbase + s * kXABytes, &tmapA, kb * kXKB, bi * kXTM, s, full_bar(stage));
-                        tma_load_3d(sbase + kXSlices * kXABytes + s * kXBBytes, &tmapB, kb * kXKB, bj * kXTN, s,
+                        tma_load_3d(sbase + SLICES * kXABytes + s * kXBBytes, &tmapB, kb * kXKB, bj * kXTN, s,
                                     full_bar(stage));
                     }
                     if (++stage == kXStages) { stage = 0; phase ^= 1u; }
@@ -396,12 +410,12 @@ i8gemm_kernel(const __grid_constant__ CUtensorMap tmapA, const __grid_constant__
                     ok = mbar_wait_bounded(full_bar(stage), phase, abort_flag);
                     if (!ok) break;
                     tc_fence_after();
-                    const uint32_t sb = kDescLo + ((base + stage * kXStageBytes) >> 4);
+                    const uint32_t sb = kDescLo + ((base + stage * kStageBytes) >> 4);
                     const uint32_t first = kb > kb0 ? 1u : 0u;    // the first product of a group overwrites
 #pragma unroll
                     for (int ks = 0; ks < kXKB / 32; ++ks)
-                        tc_slice_products<GROUPS>(tmem_base, sb + ks * 2, sb + ks * 2 + ((kXSlices * kXABytes) >> 4),
-                                                  ks > 0 ? 1u : first, std::make_integer_sequence<int, kXSlices>());
+                        tc_slice_products<GROUPS>(tmem_base, sb + ks * 2, sb + ks * 2 + ((SLICES * kXABytes) >> 4),
+                                                  ks > 0 ? 1u : first, std::make_integer_sequence<int, SLICES>());
                     tc_commit(empty_bar(stage));     // the stage may be refilled once these MMAs have read it
                     if (++stage == kXStages) { stage = 0; phase ^= 1u; }
                 }
@@ -541,10 +555,10 @@ i8gemm_kernel(const __grid_constant__ CUtensorMap tmapA, const __grid_constant__
 // ------------------------------------------------------------------------------------------------------------
 // Host side
 // ------------------------------------------------------------------------------------------------------------
-inline int x_make_map(CUtensorMap* m, int8_t* Q, int rows_pad, int k_pad, int box_rows) {
+inline int x_make_map(CUtensorMap* m, int8_t* Q, int rows_pad, int k_pad, int slices, int box_rows) {
     EncodeTiledFn enc = get_encode_tiled();
     if (!enc) return PTQ_ERR_CUDA;
-    const cuuint64_t dims[3] = {(cuuint64_t)k_pad, (cuuint64_t)rows_pad, (cuuint64_t)kXSlices};
+    const cuuint64_t dims[3] = {(cuuint64_t)k_pad, (cuuint64_t)rows_pad, (cuuint64_t)slices};
     const cuuint64_t strides[2] = {(cuuint64_t)k_pad, (cuuint64_t)rows_pad * (cuuint64_t)k_pad};
     const cuuint32_t box[3] = {(cuuint32_t)kXKB, (cuuint32_t)box_rows, 1u};
     const cuuint32_t estr[3] = {1u, 1u, 1u};
@@ -554,62 +568,70 @@ inline int x_make_map(CUtensorMap* m, int8_t* Q, int rows_pad, int k_pad, int bo
     return r == CUDA_SUCCESS ? PTQ_OK : PTQ_ERR_CUDA;
 }
 
-// Slices of one operand in the workspace: planes [7][rows_pad][k_pad] and the per-row shifts.
+// Slices of one operand in the workspace: planes [slices][rows_pad][k_pad] and the per-row shifts.
 struct XOperand {
     int8_t* Q;
     int32_t* sh;
-    int rows, k;
+    int rows, k, slices;
 };
-inline size_t x_operand_bytes(int rows, int k) {
-    return align_up(i8gemm_plane_bytes(rows, k)) + align_up((size_t)(cdiv(rows, 128) * 128) * sizeof(int32_t)) +
+inline size_t x_operand_bytes(int rows, int k, int slices = kXSlices) {
+    return align_up(i8gemm_plane_bytes(rows, k, slices)) + align_up((size_t)(cdiv(rows, 128) * 128) * sizeof(int32_t)) +
            align_up((size_t)(cdiv(rows, 128) * 128) * sizeof(unsigned long long));
 }
-// X is [rows x k] (transposed = 0, row stride ld) or [k x rows] (transposed = 1: the operand's rows are X's columns).
-// kexp (with transposed = 0): column kk is multiplied by 2^(ksign kexp[kk]), see x_slice_rows_kernel.
 inline int x_attributes(DeviceState* dev) {
     return ensure_smem_attr(dev, SA_XGEMM, [] {
-        cudaError_t e = cudaFuncSetAttribute(i8gemm_kernel<kXGroups>, cudaFuncAttributeMaxDynamicSharedMemorySize, kXSmemBytes);
-        if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(i8gemm_kernel<kXLossGroups>, cudaFuncAttributeMaxDynamicSharedMemorySize, kXSmemBytes);
-        if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(x_slice_cols_once_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     (int)x_once_smem_bytes(kXOnceMaxK));
+        cudaError_t e = cudaSuccess;
+        auto smem = [&](const void* kernel, size_t bytes) {
+            if (e == cudaSuccess) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+        };
+        smem((const void*)i8gemm_kernel<kXGroups, kXSlices>, x_smem_bytes(kXSlices));
+        smem((const void*)i8gemm_kernel<kXMoreGroups, kXSlices>, x_smem_bytes(kXSlices));
+        smem((const void*)i8gemm_kernel<kXMoreGroups, kXMoreSlices>, x_smem_bytes(kXMoreSlices));
+        smem((const void*)x_slice_cols_once_kernel<kXSlices>, x_once_smem_bytes(kXOnceMaxK));
+        smem((const void*)x_slice_cols_once_kernel<kXMoreSlices>, x_once_smem_bytes(kXOnceMaxK));
         return e;
     });
 }
+// X is [rows x k] (transposed = 0, row stride ld) or [k x rows] (transposed = 1: the operand's rows are X's columns).
+// kexp (with transposed = 0): column kk is multiplied by 2^(ksign kexp[kk]), see x_slice_rows_kernel.  slices: digits per value,
+// seven, or eight without kexp and with at most kXOnceMaxK columns' length where transposed (x_product refuses what is neither).
 inline XOperand x_slice_operand(Carver& cv, const double* X, int64_t ld, int transposed, int rows, int k, int32_t* status,
-                                cudaStream_t stream, const int8_t* kexp = nullptr, int ksign = 1) {
+                                cudaStream_t stream, const int8_t* kexp = nullptr, int ksign = 1, int slices = kXSlices) {
     const int rows_pad = cdiv(rows, 128) * 128, k_pad = cdiv(k, 128) * 128;
     XOperand op;
-    op.Q = cv.take<int8_t>(i8gemm_plane_bytes(rows, k));
+    op.Q = cv.take<int8_t>(i8gemm_plane_bytes(rows, k, slices));
     op.sh = cv.take<int32_t>(rows_pad);
     unsigned long long* colmax = cv.take<unsigned long long>(rows_pad);
-    op.rows = rows; op.k = k;
+    op.rows = rows; op.k = k; op.slices = slices;
     DeviceState* dev = nullptr;
     if (current_device_state(&dev) == PTQ_OK) x_attributes(dev);          // an error shows at the launch
     Launch l(K_X_SLICE, stream);
     if (transposed && k <= kXOnceMaxK) {
-        launch_chained(x_slice_cols_once_kernel, rows_pad / kXOnceCols, 256, x_once_smem_bytes(k_pad), stream, X, k, rows, ld, rows_pad,
-                       k_pad, op.Q, op.sh, status);
-    } else if (transposed) {
+        launch_chained(slices == kXMoreSlices ? x_slice_cols_once_kernel<kXMoreSlices> : x_slice_cols_once_kernel<kXSlices>,
+                       rows_pad / kXOnceCols, 256, x_once_smem_bytes(k_pad), stream, X, k, rows, ld, rows_pad, k_pad, op.Q,
+                       op.sh, status);
+    } else if (transposed && slices == kXSlices) {
         cudaMemsetAsync(colmax, 0, (size_t)rows_pad * sizeof(unsigned long long), stream);
         launch_chained(x_colmax_kernel, dim3(rows_pad / 32, cdiv(k, kXColChunk)), 256, 0, stream, X, k, rows, ld, colmax);
         launch_chained(x_slice_cols_kernel, dim3(rows_pad / 32, cdiv(k_pad, kXColChunk)), 256, 0, stream, X, k, rows, ld,
-                       rows_pad, k_pad,
-                                                                                              colmax, op.Q, op.sh, status);
-    } else if (kexp) {
-        launch_chained(x_slice_rows_kernel<true>, rows_pad, 256, 0, stream, X, rows, k, ld, rows_pad, k_pad, op.Q, op.sh,
-                       status, kexp, ksign);
+                       rows_pad, k_pad, colmax, op.Q, op.sh, status);
+    } else if (!transposed && kexp && slices == kXSlices) {
+        launch_chained(x_slice_rows_kernel<true, kXSlices>, rows_pad, 256, 0, stream, X, rows, k, ld, rows_pad, k_pad, op.Q,
+                       op.sh, status, kexp, ksign);
+    } else if (!transposed && !kexp) {
+        launch_chained(slices == kXMoreSlices ? x_slice_rows_kernel<false, kXMoreSlices> : x_slice_rows_kernel<false, kXSlices>,
+                       rows_pad, 256, 0, stream, X, rows, k, ld, rows_pad, k_pad, op.Q, op.sh, status, nullptr, 1);
     } else {
-        launch_chained(x_slice_rows_kernel<false>, rows_pad, 256, 0, stream, X, rows, k, ld, rows_pad, k_pad, op.Q, op.sh,
-                       status, nullptr, 1);
+        op.slices = 0;
     }
     return op;
 }
 
-// The product of two sliced operands (A: m rows, B: n rows, same k <= kXMaxK) in the given output / K-range modes.
-inline int x_product(const XOperand& a, const XOperand& b, XGemmParams prm, cudaStream_t stream) {
-    if (a.k != b.k || a.k > kXMaxK) return PTQ_ERR_UNSUPPORTED;
+// The product of two sliced operands (A: m rows, B: n rows, same k <= kXMaxK) in the given output / K-range modes, of the first
+// `digits` digits of both: seven (X_OUT_REDUCE: with group 7), or eight (k <= kXMoreMaxK).
+inline int x_product(const XOperand& a, const XOperand& b, XGemmParams prm, cudaStream_t stream, int digits = kXSlices) {
+    if (a.k != b.k || a.k > kXMaxK || digits > a.slices || digits > b.slices) return PTQ_ERR_UNSUPPORTED;
+    if (digits == kXMoreSlices && (a.k > kXMoreMaxK || prm.out_mode == X_OUT_REDUCE)) return PTQ_ERR_UNSUPPORTED;
     DeviceState* dev = nullptr;
     int st = current_device_state(&dev);
     if (st) return st;
@@ -617,9 +639,9 @@ inline int x_product(const XOperand& a, const XOperand& b, XGemmParams prm, cuda
     if (st) return st;
     const int k_pad = cdiv(a.k, 128) * 128;
     CUtensorMap mapA, mapB;
-    st = x_make_map(&mapA, a.Q, cdiv(a.rows, 128) * 128, k_pad, kXTM);
+    st = x_make_map(&mapA, a.Q, cdiv(a.rows, 128) * 128, k_pad, a.slices, kXTM);
     if (st) return st;
-    st = x_make_map(&mapB, b.Q, cdiv(b.rows, 128) * 128, k_pad, kXTN);
+    st = x_make_map(&mapB, b.Q, cdiv(b.rows, 128) * 128, k_pad, b.slices, kXTN);
     if (st) return st;
     prm.m = a.rows; prm.n = b.rows; prm.k_pad = k_pad;
     prm.sh_a = a.sh; prm.sh_b = b.sh;
@@ -627,9 +649,10 @@ inline int x_product(const XOperand& a, const XOperand& b, XGemmParams prm, cuda
     const int grid = tiles < dev->sms ? tiles : dev->sms;
     {
         Launch l(K_X_GEMM, stream);
-        if (prm.out_mode == X_OUT_REDUCE) launch_chained(i8gemm_kernel<kXLossGroups>, grid, kXThreads, kXSmemBytes, stream,
-                                                         mapA, mapB, prm);
-        else launch_chained(i8gemm_kernel<kXGroups>, grid, kXThreads, kXSmemBytes, stream, mapA, mapB, prm);
+        auto kernel = digits == kXMoreSlices ? i8gemm_kernel<kXMoreGroups, kXMoreSlices>
+                                             : (prm.out_mode == X_OUT_REDUCE ? i8gemm_kernel<kXMoreGroups, kXSlices>
+                                                                             : i8gemm_kernel<kXGroups, kXSlices>);
+        launch_chained(kernel, grid, kXThreads, (size_t)x_smem_bytes(digits), stream, mapA, mapB, prm);
     }
     return launch_status();
 }

@@ -196,3 +196,61 @@ def test_loss_with_channels_of_very_different_scale(rows, cols, hot):
     want = _loss_in_two_doubles(D, H)
     bound = _loss_bound(D, H, want)
     assert abs(float(np.longdouble(loss) - want)) <= bound, (float((np.longdouble(loss) - want) / want), bound / float(want))
+
+
+def _swept(rows, cols, channel_scale, damp, damp_mode, seed):
+    """A layer whose input channels are scaled by `channel_scale`, through the sweep: its weights in the order of the sweep, and
+    from the workspace, where they are the first arrays, the factor U, the weights as they were updated and the errors E."""
+    g = torch.Generator(device="cuda").manual_seed(seed)
+    X = torch.randn((cols, cols + 512), device="cuda", generator=g) * channel_scale(cols, g)[:, None]
+    W = torch.randn((rows, cols), device="cuda", generator=g) * (2.0 / cols) ** 0.5
+    b, st, ws = ptq.LayerBuffers(rows, cols), ptq.new_status(), ptq.Workspace()
+    ptq.hessian_accumulate(b.H.zero_(), X, ws, st)
+    ptq.prepare_hinv(b.H, damp, damp_mode, b.Hinv, b.Hinv_diag, b.lam, ws, st)
+    ptq.minmax_grid(W, 4, b.scale, b.zero, st)
+    ptq.sensitivity_order(W, b.Hinv_diag, b.scale, b.zero, 4, ptq.SCORE_QERR, b.S, b.perm, ws, st)
+    ws = ptq.Workspace()
+    ptq.quantize_layer(W, b.Hinv, b.perm, b.scale, b.zero, 4, b.codes, b.What, None, None, ws, st)
+    torch.cuda.synchronize()
+    ptq.check_status(st)
+    out, at = [], 0
+    for m in (cols, rows, rows):
+        out.append(ws.buf[at:at + 8 * m * cols].view(torch.float64).view(m, cols).cpu().numpy())
+        at += (8 * m * cols + 255) // 256 * 256
+    return W.double()[:, b.perm.long()].cpu().numpy(), *out
+
+
+def _one_scale(cols, g):
+    return torch.ones(cols, device="cuda")
+
+
+def _log_normal(cols, g):
+    return torch.exp(2.0 * torch.randn(cols, device="cuda", generator=g))
+
+
+def _four_hot(cols, g):
+    s = torch.ones(cols, device="cuda")
+    s[torch.randperm(cols, device="cuda", generator=g)[:4]] = 1.0e4
+    return s
+
+
+@pytest.mark.parametrize("rows,cols", [(64, 3137), (33, 3200)])
+@pytest.mark.parametrize("scale", [_one_scale, _log_normal, _four_hot])
+@pytest.mark.parametrize("damp_mode,damp", [(ptq.DAMP_REL_MEAN_DIAG, 0.01), (ptq.DAMP_ABS, 0.01)])
+def test_deferred_updates_are_as_exact_as_float64_steps(rows, cols, scale, damp_mode, damp):
+    """W[:, later] -= E[:, panel] U[panel, later] of layers that are swept in panels of 1024 columns.  The first block of every
+    later panel stays in memory as these products have left it: its error against extended precision, as root mean square of
+    all and of each column, is no larger than that of float64 products of 64 columns each, subtracted one after the
+    other (each rounds the weights once, and a panel's product once for all)."""
+    W0, U, Wp, E = _swept(rows, cols, scale, damp, damp_mode, 40 + cols)
+    for c0 in range(1024, cols, 1024):
+        c1 = min(c0 + 64, cols)
+        e, u = E[:, :c0], U[:c0, c0:c1]
+        want = W0[:, c0:c1].astype(np.longdouble) - e.astype(np.longdouble) @ u.astype(np.longdouble)
+        steps = W0[:, c0:c1].copy()
+        for k in range(0, c0, 64):
+            steps -= e[:, k:k + 64] @ u[k:k + 64]
+        got, ref = ((a - want).astype(np.float64) ** 2 for a in (Wp[:, c0:c1], steps))
+        assert got.mean() <= ref.mean(), (c0, (got.mean() / ref.mean()) ** 0.5)
+        worst = (got.mean(axis=0) / ref.mean(axis=0)).max() ** 0.5
+        assert worst <= 1.0, (c0, worst)
