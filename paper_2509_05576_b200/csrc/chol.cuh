@@ -332,6 +332,7 @@ __device__ __forceinline__ int chol_chain8(const double* mb, double* Wbuf, int l
     w[8] = x1 * pivot_rsqrt(d1);
     const bool ok = d0 >= kMinPivot && d0 < kMaxPivot && d1 >= kMinPivot && d1 < kMaxPivot;
     if (__all_sync(0xffffffffu, ok)) return -1;
+    __syncwarp();                                          // a vote orders no memory: what W holds by now is written again
     return chol_chain8_general(mb, Wbuf, lane);
 }
 

@@ -152,6 +152,25 @@ def test_a_subnormal_pivot_is_reported(index):
     assert ei.value.code == ptq.ERR_NOT_SPD and ei.value.index == index
 
 
+@pytest.mark.parametrize("index", [0, 3, 4, 7, 66, 69])
+def test_a_rejected_pivot_counts_as_one(index):
+    """A pivot that is not accepted sends its 8 x 8 block through the general form, which writes all rows of that block's inverse
+    factor again: with a diagonal matrix the result is the inverse of the diagonal with a one at the rejected pivot (two
+    rounded factors of 1.1 units in the last place each, their product and the quotient: 4 units), and nothing of the first attempt is left in it."""
+    d = torch.linspace(0.3, 7.0, 70, dtype=torch.float64, device="cuda")
+    d[index] = -2.0
+    st, ws = ptq.new_status(), ptq.Workspace()
+    H = torch.diag(d)
+    Hinv, diag, lam = torch.empty_like(H), torch.empty_like(d), torch.empty(1, dtype=torch.float64, device="cuda")
+    ptq.prepare_hinv(H, 0.0, ptq.DAMP_ABS, Hinv, diag, lam, ws, st)
+    torch.cuda.synchronize()
+    with pytest.raises(ptq.PtqError) as ei:
+        ptq.check_status(st)
+    assert ei.value.code == ptq.ERR_NOT_SPD and ei.value.index == index
+    d[index] = 1.0
+    assert torch.allclose(Hinv, torch.diag(1.0 / d), rtol=4 * 2.0 ** -52, atol=0.0)
+
+
 def test_pivot_arithmetic_against_division_and_square_root():
     """All binades an accepted pivot can have, the powers of two with their neighbours and the ends of the range; against
     80-bit values.  Bounds: half a unit in the last place for the rounding of the result, for the root as much again for
