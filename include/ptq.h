@@ -254,6 +254,17 @@ int ptq_selftest_wait_timeout(int which, long long limit_cycles, void *ws, size_
                               void *stream);
 
 /*
+ * Self-test of what the sweep does when the factorisation it runs behind gives up (instrumentation; the paper has no
+ * counterpart).  Runs both on a unit layer of 64 x 64 in one launch, with the sweep waiting, for limit_cycles SM clock cycles,
+ * for one arrival more than the factorisation makes.  The CTAs of the sweep must record {PTQ_ERR_TIMEOUT, CTA index, 6} in
+ * `status`, raise the abort word that the rest of the sweep polls, and return.  abort_word: int32 (device), receives that word.
+ * ws: PTQ_ABANDONED_SWEEP_BYTES of device scratch.  limit_cycles in [1, 4e9].
+ */
+#define PTQ_ABANDONED_SWEEP_BYTES 262144
+int ptq_selftest_abandoned_sweep(long long limit_cycles, void *ws, size_t ws_bytes, int32_t *abort_word, int32_t *status,
+                                 void *stream);
+
+/*
  * Self-test of the arithmetic on pivots (instrumentation; the paper has no counterpart): rcp[i] = 1 / x[i] and
  * rsq[i] = 1 / sqrt(x[i]) as the factorisations form them, for x[i] from the smallest normal number up to 1e300.
  *   x, rcp, rsq [n] float64 (device)

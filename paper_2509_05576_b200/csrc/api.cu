@@ -125,6 +125,18 @@ __global__ void selftest_counter_kernel(unsigned* words, int32_t* status, long l
         report(status, PTQ_ERR_TIMEOUT, blockIdx.x, 2);
 }
 
+// What ptq_selftest_abandoned_sweep starts from: one block row, two row groups.
+constexpr int kAbandonedRows = 2 * kSweepRows;
+static_assert(kAbandonedRows == kNB, "one launch fills the matrix and the rows");
+__global__ void __launch_bounds__(kNB) selftest_unit_layer_kernel(double* __restrict__ U, double* __restrict__ Wp, double* __restrict__ E,
+                                                                   float* __restrict__ scale, float* __restrict__ zero) {
+    const int i = blockIdx.x, j = threadIdx.x;
+    U[i * kNB + j] = i == j ? 1.0 : 0.0;
+    Wp[i * kNB + j] = 0.0;
+    E[i * kNB + j] = __longlong_as_double(-1ll);
+    if (j == 0) { scale[i] = 1.0f; zero[i] = 0.0f; }
+}
+
 // What the factorisations make of a pivot, one value per thread.
 __global__ void __launch_bounds__(256) selftest_reciprocal_kernel(const double* __restrict__ x, int n, double* __restrict__ rcp,
                                                                    double* __restrict__ rsq) {
@@ -654,6 +666,34 @@ int ptq_selftest_wait_timeout(int which, long long limit_cycles, void* ws, size_
         return PTQ_ERR_CUDA;
     }
     return PTQ_OK;
+}
+
+int ptq_selftest_abandoned_sweep(long long limit_cycles, void* ws, size_t ws_bytes, int32_t* abort_word, int32_t* status,
+                                 void* stream_) {
+    cudaStream_t stream = static_cast<cudaStream_t>(stream_);
+    if (limit_cycles < 1 || limit_cycles > kSpinLimitCycles || !abort_word || !status) return PTQ_ERR_INVALID_ARG;
+    if (!ws || ws_bytes < PTQ_ABANDONED_SWEEP_BYTES) return PTQ_ERR_WORKSPACE;
+    if (!aligned16(ws)) return PTQ_ERR_ALIGNMENT;
+    constexpr int groups = kAbandonedRows / kSweepRows;
+    Carver cv(ws);
+    double* U = cv.take<double>(kNB * kNB);
+    double* Wp = cv.take<double>(kAbandonedRows * kNB);
+    double* E = cv.take<double>(kAbandonedRows * kNB);
+    double* Dbuf = cv.take<double>(chol_scratch_doubles(kNB));
+    float* scale = cv.take<float>(kAbandonedRows);
+    float* zero = cv.take<float>(kAbandonedRows);
+    uint8_t* codes = cv.take<uint8_t>(kAbandonedRows * kNB);
+    unsigned* bar = cv.take<unsigned>(2);
+    unsigned* flags = cv.take<unsigned>(groups + 1);
+    static_assert(4 * kNB * kNB * 8 + 2 * kNB * 4 + kNB * kNB + 2 * 256 <= PTQ_ABANDONED_SWEEP_BYTES, "the pieces above");
+    { Launch l(K_SELFTEST, stream); selftest_unit_layer_kernel<<<kNB, kNB, 0, stream>>>(U, Wp, E, scale, zero); }
+    // one CTA per row group, so that nothing but the wait for the factorisation can raise the sweep's abort word
+    const int st = factor_sweep_launch(U, kNB, chol_all_rows(kNB), Dbuf, bar, groups, Wp, E, codes, scale, zero, kAbandonedRows, kNB, 4,
+                                       flags, status, stream, groups + 1, false, limit_cycles, 1u);
+    if (st) return st;
+    if (cudaMemcpyAsync(abort_word, flags + groups, sizeof(int32_t), cudaMemcpyDeviceToDevice, stream) != cudaSuccess)
+        return PTQ_ERR_CUDA;
+    return launch_status();
 }
 
 int ptq_selftest_reciprocal(const double* x, int n, double* rcp, double* rsq, void* stream_) {

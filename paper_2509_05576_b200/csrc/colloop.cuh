@@ -292,7 +292,10 @@ __device__ __forceinline__ void sweep_columns(const SweepParams& prm, const int 
         const bool ok = *s_flag != 0;
         sweep_sync();
         known_rows = b + 1;
-        if (!ok && tid == 0) report(prm.status, PTQ_ERR_TIMEOUT, blockIdx.x, 6);
+        if (!ok && tid == 0) {
+            atomicExch(abort_word, 1u);          // the other CTAs of the sweep poll this one
+            report(prm.status, PTQ_ERR_TIMEOUT, blockIdx.x, 6);
+        }
         return ok;
     };
 
@@ -731,10 +734,12 @@ inline int sweep_ctas_behind(int rows, int sweep_n, int n, const CholRange& rang
 
 // The factorisation of a range of block rows of U (n x n, row stride n) and the sweep of the first sweep_n columns of that range
 // in one launch.  Wp, E, codes_p: from the column of the first block row on, row stride n.  The caller has set E to
-// NaN and, with counters_ready, the counters and flags to zero.
+// NaN and, with counters_ready, the counters and flags to zero.  sweep_spin_limit, extra_arrivals: for the self-test, which has
+// the sweep wait for more arrivals than there will be.
 inline int factor_sweep_launch(double* U, int n, const CholRange& range, double* Dbuf, unsigned* bar, int sweep_ctas, double* Wp,
                                double* E, uint8_t* codes_p, const float* scale, const float* zero, int rows, int sweep_n, int bits,
-                               unsigned* flags, int32_t* status, cudaStream_t stream, int budget, bool counters_ready) {
+                               unsigned* flags, int32_t* status, cudaStream_t stream, int budget, bool counters_ready,
+                               long long sweep_spin_limit = kSpinLimitCycles, unsigned extra_arrivals = 0) {
     DeviceState* dev = nullptr;
     int st = current_device_state(&dev);
     if (st) return st;
@@ -760,8 +765,8 @@ inline int factor_sweep_launch(double* U, int n, const CholRange& range, double*
     prm.Wp = Wp; prm.U = U + (size_t)range.first * kNB * (n + 1); prm.E = E; prm.codes_p = codes_p; prm.scale = scale;
     prm.zero = zero; prm.rows = rows; prm.n = sweep_n; prm.bits = bits; prm.ld = n;
     prm.vec16 = (f.vec16 && (sweep_n & 1) == 0 && aligned16(Wp) && aligned16(E)) ? 1 : 0;
-    prm.flags = flags; prm.status = status; prm.spin_limit = kSpinLimitCycles;
-    prm.diag = Dbuf + (size_t)range.first * kNB * kNB; prm.rows_done = bar; prm.row_arrivals = (unsigned)f.ctas;
+    prm.flags = flags; prm.status = status; prm.spin_limit = sweep_spin_limit;
+    prm.diag = Dbuf + (size_t)range.first * kNB * kNB; prm.rows_done = bar; prm.row_arrivals = (unsigned)f.ctas + extra_arrivals;
     void* args[] = {&f, &prm};
     Launch l(K_FACTOR_SWEEP, stream);
     if (cudaLaunchCooperativeKernel((const void*)factor_sweep_kernel, dim3(f.ctas + sweep_ctas), dim3(kCholThreads), args, smem,

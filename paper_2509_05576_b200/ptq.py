@@ -18,6 +18,7 @@ LIB_PATH = os.path.join(_HERE, "libptq.so")
 OK, ERR_INVALID_ARG, ERR_ALIGNMENT, ERR_WORKSPACE, ERR_NOT_SPD, ERR_NONFINITE, ERR_TIMEOUT, ERR_CUDA, ERR_UNSUPPORTED = range(9)
 ERR_STATIC_SCRATCH = 9
 STATIC_SCRATCH_BYTES = 6 << 20
+ABANDONED_SWEEP_BYTES = 262144
 DAMP_REL_MEAN_DIAG, DAMP_ABS = 0, 1
 SCORE_QERR, SCORE_PRUNE, SCORE_ERR, SCORE_W, SCORE_NONE = 0, 1, 2, 3, 4
 SCORE_ASCENDING = 16          # added to a score mode: sort by S ascending
@@ -27,7 +28,8 @@ CALL_QUANTIZE_LAYER_PER_ROW = 6
 
 EXPORTS = ["ptq_workspace_bytes", "ptq_hessian_accumulate", "ptq_hessian_accumulate_conv", "ptq_hessian_accumulate_f64", "ptq_prepare_hinv",
            "ptq_minmax_grid", "ptq_sensitivity_order", "ptq_sensitivity_order_static", "ptq_quantize_layer", "ptq_status_string", "ptq_version",
-           "ptq_sort_scores", "ptq_gemm_nt_sliced", "ptq_gemm_nt_sliced_workspace_bytes", "ptq_quantize_layer_dynamic", "ptq_quantize_layer_per_row", "ptq_selftest_wait_timeout", "ptq_selftest_reciprocal", "ptq_fp64_probe",
+           "ptq_sort_scores", "ptq_gemm_nt_sliced", "ptq_gemm_nt_sliced_workspace_bytes", "ptq_quantize_layer_dynamic", "ptq_quantize_layer_per_row", "ptq_selftest_wait_timeout", "ptq_selftest_abandoned_sweep",
+           "ptq_selftest_reciprocal", "ptq_fp64_probe",
            "ptq_kernel_count", "ptq_kernel_name", "ptq_launch_count", "ptq_profile_enable", "ptq_profile_read",
            "ptq_set_cta_limit"]
 
@@ -77,6 +79,7 @@ def lib():
         L.ptq_quantize_layer_dynamic.argtypes = [vp, c_int, c_int, c_int64, vp, vp, vp, c_int, c_int, c_int, vp, vp,
                                                  vp, vp, vp, vp, c_size_t, vp, vp]
         L.ptq_selftest_wait_timeout.argtypes = [c_int, ctypes.c_longlong, vp, c_size_t, vp, vp]
+        L.ptq_selftest_abandoned_sweep.argtypes = [ctypes.c_longlong, vp, c_size_t, vp, vp, vp]
         L.ptq_selftest_reciprocal.argtypes = [vp, c_int, vp, vp, vp]
         L.ptq_fp64_probe.argtypes = [c_int, c_int, vp, ctypes.POINTER(c_double), vp]
         L.ptq_status_string.argtypes = [c_int]
@@ -278,6 +281,14 @@ def selftest_wait_timeout(which, limit_cycles, ws, status, stream=None):
     buf = ws.get(256)
     _check(lib().ptq_selftest_wait_timeout(int(which), int(limit_cycles), _ptr(buf), buf.numel(), _ptr(status),
                                            _stream(stream)), "ptq_selftest_wait_timeout")
+
+
+def selftest_abandoned_sweep(limit_cycles, ws, status, stream=None):
+    """Has the sweep wait for a factorisation that never finishes; the sweep's abort word afterwards (device scalar)."""
+    buf, word = ws.get(ABANDONED_SWEEP_BYTES), torch.zeros(1, dtype=torch.int32, device=status.device)
+    _check(lib().ptq_selftest_abandoned_sweep(int(limit_cycles), _ptr(buf), buf.numel(), _ptr(word), _ptr(status),
+                                              _stream(stream)), "ptq_selftest_abandoned_sweep")
+    return word
 
 
 def selftest_reciprocal(x, stream=None):

@@ -89,6 +89,10 @@ def test_new_entry_points_check_their_arguments_on_the_host(lib):
     assert lib.ptq_selftest_wait_timeout(0, 10 ** 12, fake, 64, fake, None) == ptq.ERR_INVALID_ARG   # beyond the library's own limit
     assert lib.ptq_selftest_wait_timeout(0, 1000, fake, 8, fake, None) == ptq.ERR_WORKSPACE
     flops = ctypes.c_double(0.0)
+    assert lib.ptq_selftest_abandoned_sweep(0, fake, 1 << 20, fake, fake, None) == ptq.ERR_INVALID_ARG
+    assert lib.ptq_selftest_abandoned_sweep(1000, fake, 1 << 20, None, fake, None) == ptq.ERR_INVALID_ARG
+    assert lib.ptq_selftest_abandoned_sweep(1000, fake, 1000, fake, fake, None) == ptq.ERR_WORKSPACE
+    assert lib.ptq_selftest_abandoned_sweep(1000, vp(4100), 1 << 20, fake, fake, None) == ptq.ERR_ALIGNMENT
     assert lib.ptq_selftest_reciprocal(fake, 0, fake, fake, None) == ptq.ERR_INVALID_ARG
     assert lib.ptq_fp64_probe(2, 10, fake, ctypes.byref(flops), None) == ptq.ERR_INVALID_ARG
     assert lib.ptq_fp64_probe(0, 0, fake, ctypes.byref(flops), None) == ptq.ERR_INVALID_ARG

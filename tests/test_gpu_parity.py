@@ -276,6 +276,21 @@ def test_bounded_wait_runs_out_and_the_context_stays_usable(which):
         assert np.array_equal(before[k], after[k]), k
 
 
+def test_sweep_behind_a_factorisation_that_gives_up():
+    """The sweep runs behind the factorisation in one launch and waits for its block rows.  When that wait runs out it reports so
+    and raises the abort word that every other CTA of the sweep polls, and a layer made afterwards is what it was before."""
+    W, X = _layer(64, 128, 256, 90)
+    before = gpu_layer(W, X, 4)
+    st, ws = ptq.new_status(), ptq.Workspace()
+    word = ptq.selftest_abandoned_sweep(5000, ws, st)
+    torch.cuda.synchronize()
+    assert st.cpu().tolist()[0] == ptq.ERR_TIMEOUT and st.cpu().tolist()[2] == 6
+    assert word.item() == 1
+    after = gpu_layer(W, X, 4)
+    for k in ("H", "Hinv", "S", "perm", "codes", "What", "loss"):
+        assert np.array_equal(before[k], after[k]), k
+
+
 # ------------------------------------------------------------------------------------------ column sweep
 def _sweep(W, Hinv, perm, sc, zp, bits, H=None):
     rows, cols = W.shape
