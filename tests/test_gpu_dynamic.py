@@ -110,3 +110,41 @@ def test_whole_path_with_dynamic_reranking_on_a_resnet_shaped_layer():
     assert num <= WHAT_RTOL * np.linalg.norm(ref["What"].astype(np.float64))
     assert abs(float(loss.item()) - ref["loss"]) <= LOSS_RTOL * ref["loss"]
     assert nm == 0
+
+
+@pytest.mark.parametrize("rows,cols,block", [(48, 200, 64), (130, 321, 128), (70, 640, 192), (33, 1153, 256)])
+def test_rounds_with_the_sweep_behind_the_factorisation_equal_those_one_after_the_other(rows, cols, block):
+    """A round factorises part of the remaining matrix, updates the rest and sweeps the columns of that part, in one launch where
+    that pays.  With no more CTAs than row groups the sweep comes after the factorisation: the same arrays bit for bit,
+    the scaled errors in the workspace (behind two matrices and two sets of weights) included."""
+    W, H, Hinv, _, sc, zp = _inputs(rows, cols, 300, 4, 1500 + cols)
+    Wd, Hd, Hi, scd, zpd = (_cuda(a) for a in (W, H, Hinv, sc, zp))
+    names = [ptq.lib().ptq_kernel_name(k).decode() for k in range(ptq.lib().ptq_kernel_count())]
+    fs = names.index("factor_sweep")
+
+    def run(limit):
+        ws, st = ptq.Workspace(), ptq.new_status()
+        ws.get(ptq.workspace_bytes(ptq.CALL_QUANTIZE_LAYER_DYNAMIC, rows, cols, 0)).zero_()
+        codes = torch.empty((rows, cols), dtype=torch.uint8, device="cuda")
+        What = torch.empty((rows, cols), dtype=torch.float32, device="cuda")
+        order = torch.empty(cols, dtype=torch.int32, device="cuda")
+        loss = torch.zeros(1, dtype=torch.float64, device="cuda")
+        before = ptq.launch_count(fs)
+        ptq.set_cta_limit(limit)
+        try:
+            ptq.quantize_layer_dynamic(Wd, Hi, scd, zpd, 4, ptq.SCORE_QERR, block, codes, What, order, Hd, loss, ws, st)
+        finally:
+            ptq.set_cta_limit(0)
+        torch.cuda.synchronize()
+        ptq.check_status(st)
+        at = 2 * ((8 * cols * cols + 255) // 256 * 256) + 2 * ((8 * rows * cols + 255) // 256 * 256)
+        E = ws.buf[at:at + 8 * rows * cols].view(torch.int64)
+        return ptq.launch_count(fs) - before, (codes, What, order, loss, E)
+
+    launches, apart = run((rows + 31) // 32)
+    assert launches == 0
+    launches, _ = run(0)
+    assert launches > 0
+    for limit in (0, 0, 30, 60):
+        for a, b in zip(apart, run(limit)[1]):
+            assert torch.equal(a, b), limit

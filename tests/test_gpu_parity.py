@@ -529,6 +529,43 @@ def test_sweep_behind_the_factorisation_equals_one_after_the_other(rows, cols):
         assert np.array_equal(h[k], g[k]), k
 
 
+@pytest.mark.parametrize("rows,cols", [(1, 64), (33, 65), (40, 130), (100, 577), (300, 640), (129, 1153), (70, 3137)])
+def test_what_the_sweep_reads_behind_the_factorisation_is_final(rows, cols):
+    """The scaled errors E and the factor U, which the workspace begins with (U, the weights, E), from the factorisation with
+    the sweep behind it: as from one after the other, bit for bit, three times for each of several CTA limits, which change
+    how many CTAs factorise, how many sweep a row group and by how much the sweep is behind."""
+    W, X = _layer(rows, cols, 256, 77 + cols)
+    Wd = _cuda(W)
+    b, st, ws = ptq.quantize_layer_full(Wd, _cuda(X), 4), ptq.new_status(), ptq.Workspace()
+    names = [ptq.lib().ptq_kernel_name(k).decode() for k in range(ptq.lib().ptq_kernel_count())]
+    fs = names.index("factor_sweep")
+
+    def factor_and_errors(limit):
+        before = ptq.launch_count(fs)
+        ptq.set_cta_limit(limit)
+        try:
+            ptq.quantize_layer(Wd, b.Hinv, b.perm, b.scale, b.zero, 4, b.codes, b.What, None, None, ws, st)
+        finally:
+            ptq.set_cta_limit(0)
+        f64 = ws.buf[:ws.buf.numel() // 8 * 8].view(torch.float64)
+        at = sum((m * cols + 31) // 32 * 32 for m in (cols, rows))
+        U = torch.triu(f64[:cols * cols].view(cols, cols))
+        return ptq.launch_count(fs) - before, U, f64[at:at + rows * cols].clone()
+
+    groups = (rows + 31) // 32
+    launches, U, E = factor_and_errors(groups)
+    assert launches == 0 and not bool(E.isnan().any())
+    together = 0
+    for limit in (0, groups + 2, 2 * groups + 3, 3 * groups + 6, 40, 75):
+        for _ in range(3):
+            launches, U2, E2 = factor_and_errors(limit)
+            together += launches
+            assert torch.equal(U2, U) and torch.equal(E2, E), limit
+    torch.cuda.synchronize()
+    ptq.check_status(st)
+    assert together >= 3 * (1 if cols < 3072 else 4)
+
+
 @pytest.mark.parametrize("cols", [8, 65, 72, 200, 333, 592, 1184])
 def test_widths_of_the_factorisation_strips(cols):
     """The strips of a block row have 8, 16, 24 or 40 panel columns, the narrowest for which there are CTAs enough (and more
