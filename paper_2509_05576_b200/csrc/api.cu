@@ -281,9 +281,10 @@ size_t ptq_workspace_bytes(int call_id, int rows, int cols, int n) {
             add(2 * sizeof(unsigned));                      // grid barrier of the factorisation kernel
             add(((size_t)cdiv(rows, kSweepRows) + 1) * sizeof(unsigned));   // per-row-group progress counters of the sweep
             add(chol_scratch_doubles(cols) * sizeof(double));
-            add(chol_panel_workspace_bytes(cols));
-            if (cols >= kPanelMinCols)                      // slices of E[:, panel]
+            if (cols >= kPanelMinCols) {                    // slices of U[panel, later] and of E[:, panel]
+                add(x_operand_bytes(cols, kPanelBlocks * kNB, deferred_digits(rows, cols)));
                 add(x_operand_bytes(rows, kPanelBlocks * kNB, deferred_digits(rows, cols)));
+            }
             break;
         case PTQ_CALL_QUANTIZE_LAYER_PER_ROW:
             if (rows < 1) return 0;
@@ -384,7 +385,7 @@ int ptq_prepare_hinv(const double* H, int cols, int damp_mode, double damp, doub
     { Launch l(K_DAMP_COPY, stream); launch_chained(damp_copy_kernel, dim3(cdiv(n, 1024), n), 256, 0, stream, H, R, V,
                                                     n, lambda_out, bar); }
     // W = U^-T comes out of the factorisation sweep itself (V must start as zero)
-    int st = cholesky_upper_auto(R, n, V, Dbuf, bar, pws, status, stream, true);
+    int st = cholesky_inverse_upper(R, n, V, Dbuf, bar, pws, status, stream);
     if (st) return st;
     if (n >= kSlicedMinCols && n <= kXMaxK && x_operand_bytes(n, n) <= (size_t)n * n * sizeof(double)) {
         // Hinv = W^T W on the int8 tensor path: the columns of the lower-triangular W are sliced once (into R, which is
@@ -744,9 +745,12 @@ int ptq_quantize_layer(const float* W, int rows, int cols, int64_t ldw, const do
     unsigned* bar = cv.take<unsigned>(2);
     unsigned* sweep_flags = cv.take<unsigned>((size_t)cdiv(rows, kSweepRows) + 1);
     double* Dbuf = cv.take<double>(chol_scratch_doubles(n));
-    void* pws = n >= kPanelMinCols ? static_cast<void*>(cv.take<char>(chol_panel_workspace_bytes(n))) : nullptr;
     const int digits = deferred_digits(rows, n);
-    void* ews = n >= kPanelMinCols ? static_cast<void*>(cv.take<char>(x_operand_bytes(rows, kPanelBlocks * kNB, digits))) : nullptr;
+    auto panel_operand = [&](int r) {
+        return n >= kPanelMinCols ? static_cast<void*>(cv.take<char>(x_operand_bytes(r, kPanelBlocks * kNB, digits))) : nullptr;
+    };
+    void* uws = panel_operand(n);
+    void* ews = panel_operand(rows);
 
     DeviceState* dev = nullptr;
     int st = current_device_state(&dev);
@@ -788,9 +792,9 @@ int ptq_quantize_layer(const float* W, int rows, int cols, int64_t ldw, const do
         }
         if (st) return st;
         if (rest > 0) {
-            Carver pv(pws), ev(ews);
+            Carver uv(uws), ev(ews);
             double* below = U + (size_t)off * n + off + cols_now;                 // U[panel, later]
-            const XOperand u = x_slice_operand(pv, below, n, 1, rest, cols_now, status, stream, nullptr, 1, digits);
+            const XOperand u = x_slice_operand(uv, below, n, 1, rest, cols_now, status, stream, nullptr, 1, digits);
             st = chol_apply_panel(U, n, off + cols_now, u, status, stream);
             if (st) return st;
             const XOperand e = x_slice_operand(ev, E + off, n, 0, rows, cols_now, status, stream, nullptr, 1, digits);

@@ -28,14 +28,15 @@ inline int chol_apply_panel(double* A, int n, int c0, const XOperand& u, int32_t
     return x_product(u, u, prm, stream);
 }
 
-// Same contract as cholesky_upper (whole factorisation); xws: chol_panel_workspace_bytes(n) bytes of scratch.
-inline int cholesky_upper_auto(double* A, int n, double* Wm, double* Dbuf, unsigned* bar, void* xws, int32_t* status,
-                               cudaStream_t stream, bool bar_ready) {
-    if (n < kPanelMinCols || xws == nullptr) return cholesky_upper(A, n, Wm, Dbuf, bar, status, stream, 0, 0, 0, bar_ready);
+// The whole factorisation of A with W = U^-T (cholesky_upper; the caller has cleared `bar`); xws: chol_panel_workspace_bytes(n)
+// bytes of scratch.
+inline int cholesky_inverse_upper(double* A, int n, double* Wm, double* Dbuf, unsigned* bar, void* xws, int32_t* status,
+                                  cudaStream_t stream) {
+    if (n < kPanelMinCols) return cholesky_upper(A, n, Wm, Dbuf, bar, status, stream, 0, 0, 0, true);
     const int nb = (n + kNB - 1) / kNB;
     for (int kf = 0; kf < nb; kf += kPanelBlocks) {
         const int pe = kf + kPanelBlocks < nb ? kf + kPanelBlocks : nb;
-        int st = cholesky_upper(A, n, Wm, Dbuf, bar, status, stream, pe, kf, pe, bar_ready && kf == 0);
+        int st = cholesky_upper(A, n, Wm, Dbuf, bar, status, stream, pe, kf, pe, kf == 0);
         if (st) return st;
         if (pe >= nb) break;
         const int r0 = kf * kNB, c0 = pe * kNB;               // panel rows r0 .. c0 - 1, everything from c0 on is below it
@@ -45,15 +46,13 @@ inline int cholesky_upper_auto(double* A, int n, double* Wm, double* Dbuf, unsig
         const XOperand u = x_slice_operand(cv, A + (size_t)r0 * n + c0, n, 1, rest, depth, status, stream);
         st = chol_apply_panel(A, n, c0, u, status, stream);
         if (st) return st;
-        if (Wm != nullptr) {
-            XGemmParams prm{};
-            prm.ldc = n; prm.alpha = -1.0; prm.status = status; prm.k_mode = X_K_ALL;
-            // rows of the operand = columns 0 .. c0 - 1 of the panel's rows of W
-            const XOperand w = x_slice_operand(cv, Wm + (size_t)r0 * n, n, 1, c0, depth, status, stream);
-            prm.C = Wm + (size_t)c0 * n; prm.out_mode = X_OUT_ADD;
-            st = x_product(u, w, prm, stream);
-            if (st) return st;
-        }
+        // rows of the operand = columns 0 .. c0 - 1 of the panel's rows of W
+        const XOperand w = x_slice_operand(cv, Wm + (size_t)r0 * n, n, 1, c0, depth, status, stream);
+        XGemmParams prm{};
+        prm.C = Wm + (size_t)c0 * n; prm.ldc = n; prm.alpha = -1.0; prm.status = status;
+        prm.out_mode = X_OUT_ADD; prm.k_mode = X_K_ALL;
+        st = x_product(u, w, prm, stream);
+        if (st) return st;
     }
     return PTQ_OK;
 }

@@ -222,7 +222,7 @@ __device__ __forceinline__ bool sweep_chain8(double (&v)[8], double (&lev)[8], c
     return danger;
 }
 
-// The sweep by the CTAs `first_cta` .. of the grid, kSweepThreads threads each (barrier 8: with BEHIND the block has more).
+// The sweep by G CTAs, of which this is number `cta`, kSweepThreads threads each (barrier 8: with BEHIND the block has more).
 // BEHIND: the factor is being made by the CTAs before them (factor_sweep_kernel).  Block row b of it is final once all of them have
 // arrived at their grid barrier b + 1 times; its diagonal block is then in prm.diag.
 __device__ __forceinline__ void sweep_sync() { asm volatile("bar.sync 8, %0;" ::"n"(kSweepThreads) : "memory"); }
@@ -541,7 +541,6 @@ __device__ __forceinline__ void sweep_columns(const SweepParams& prm, const int 
                 ahead = !next_mine;
                 continue;
             }
-            if (!wait_row(b)) return;
             const int b_first = b + 1 + (((ci - (b + 1)) % cpg) + cpg) % cpg;     // first owned block beyond b
             if (b_first >= nb) break;                                               // nothing left for this CTA
             const int e_lo = lazy;
