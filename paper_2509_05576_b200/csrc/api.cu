@@ -92,13 +92,17 @@ int order_launch(const float* W, int rows, int cols, int64_t ldw, const double* 
     if (mode != PTQ_SCORE_NONE) {
         Launch l(K_SCORE_PARTIAL, stream);
         launch_chained(score_partial_kernel<float>, dim3(cdiv(cols, kScoreCols), chunks), 256, 0, stream, W, rows, cols, ldw,
-                       scale,
-                                                                                            zero, bits, mode, partial);
+                       scale, zero, bits, mode, partial);
     }
-    { Launch l(K_SCORE_FINAL, stream); launch_chained(score_final_kernel, cdiv(cols, 128), 128, 0, stream, partial, chunks,
-                                                      cols, Hinv_diag, (int64_t)1, mode, S, status); }
-    { Launch l(K_RANK_SORT, stream); launch_chained(rank_sort_kernel, cdiv(cols, kRankCols), 256, 0, stream, S, cols,
-                                                    ascending, perm, nullptr); }
+    {
+        Launch l(K_SCORE_FINAL, stream);
+        launch_chained(score_final_kernel, cdiv(cols, 128), 128, 0, stream, partial, chunks, cols, Hinv_diag, (int64_t)1,
+                       mode, S, status);
+    }
+    {
+        Launch l(K_RANK_SORT, stream);
+        launch_chained(rank_sort_kernel, cdiv(cols, kRankCols), 256, 0, stream, S, cols, ascending, perm, nullptr);
+    }
     return launch_status();
 }
 
@@ -381,9 +385,14 @@ int ptq_prepare_hinv(const double* H, int cols, int damp_mode, double damp, doub
     unsigned* bar = cv.take<unsigned>(2);
     double* Dbuf = cv.take<double>(chol_scratch_doubles(n));
     void* pws = chol_panel_workspace_bytes(n) ? static_cast<void*>(cv.take<char>(chol_panel_workspace_bytes(n))) : nullptr;
-    { Launch l(K_LAMBDA, stream); launch_chained(lambda_kernel, 1, 256, 0, stream, H, n, damp_mode, damp, lambda_out, status); }
-    { Launch l(K_DAMP_COPY, stream); launch_chained(damp_copy_kernel, dim3(cdiv(n, 1024), n), 256, 0, stream, H, R, V,
-                                                    n, lambda_out, bar); }
+    {
+        Launch l(K_LAMBDA, stream);
+        launch_chained(lambda_kernel, 1, 256, 0, stream, H, n, damp_mode, damp, lambda_out, status);
+    }
+    {
+        Launch l(K_DAMP_COPY, stream);
+        launch_chained(damp_copy_kernel, dim3(cdiv(n, 1024), n), 256, 0, stream, H, R, V, n, lambda_out, bar);
+    }
     // W = U^-T comes out of the factorisation sweep itself (V must start as zero)
     int st = cholesky_inverse_upper(R, n, V, Dbuf, bar, pws, status, stream);
     if (st) return st;
@@ -407,8 +416,10 @@ int ptq_minmax_grid(const float* W, int rows, int cols, int64_t ldw, int bits, f
     cudaStream_t stream = static_cast<cudaStream_t>(stream_);
     if (!W || !scale || !zero || rows < 1 || cols < 1 || ldw < cols || bits < 2 || bits > 8)
         return PTQ_ERR_INVALID_ARG;
-    { Launch l(K_MINMAX_GRID, stream); launch_chained(minmax_grid_kernel, rows, 256, 0, stream, W, rows, cols, ldw, bits,
-                                                      scale, zero, status); }
+    {
+        Launch l(K_MINMAX_GRID, stream);
+        launch_chained(minmax_grid_kernel, rows, 256, 0, stream, W, rows, cols, ldw, bits, scale, zero, status);
+    }
     return launch_status();
 }
 
@@ -495,20 +506,21 @@ int ptq_quantize_layer_dynamic(const float* W, int rows, int cols, int64_t ldw, 
         if (mode != PTQ_SCORE_NONE) {
             Launch l(K_SCORE_PARTIAL, stream);
             if (Wcur)
-                launch_chained(score_partial_kernel<double>, dim3(cdiv(m, kScoreCols), chunks), 256, 0, stream, Wcur, rows,
-                               m, ldc, scale,
-                                                                                                zero, bits, mode, partial);
+                launch_chained(score_partial_kernel<double>, dim3(cdiv(m, kScoreCols), chunks), 256, 0, stream, Wcur, rows, m,
+                               ldc, scale, zero, bits, mode, partial);
             else
                 launch_chained(score_partial_kernel<float>, dim3(cdiv(m, kScoreCols), chunks), 256, 0, stream, W, rows, m,
-                               ldw, scale,
-                                                                                               zero, bits, mode, partial);
+                               ldw, scale, zero, bits, mode, partial);
         }
         {
             Launch l(K_SCORE_FINAL, stream);
-            launch_chained(score_final_kernel, cdiv(m, 128), 128, 0, stream, partial, chunks, m, Acur, lda + 1, mode, S, status);
+            launch_chained(score_final_kernel, cdiv(m, 128), 128, 0, stream, partial, chunks, m, Acur, lda + 1, mode, S,
+                           status);
         }
-        { Launch l(K_RANK_SORT, stream); launch_chained(rank_sort_kernel, cdiv(m, kRankCols), 256, 0, stream, S, m,
-                                                        ascending, ordr, ocur); }
+        {
+            Launch l(K_RANK_SORT, stream);
+            launch_chained(rank_sort_kernel, cdiv(m, kRankCols), 256, 0, stream, S, m, ascending, ordr, ocur);
+        }
         double* An = Abuf[cur];
         double* Wn = Wbuf[cur];
         int32_t* onew = obuf[cur ^ 1];
@@ -517,11 +529,11 @@ int ptq_quantize_layer_dynamic(const float* W, int rows, int cols, int64_t ldw, 
             const dim3 grid(grid_x_for(m, 256), m + rows < 8192 ? m + rows : 8192);
             const int n_flags = cdiv(rows, kSweepRows) + 1;
             if (Wcur)
-                launch_chained(round_gather_kernel<double>, grid, 256, 0, stream, Acur, lda, Wcur, ldc, rows, ordr, ocur, m, b, An, Wn, E,
-                               onew, order_out + done, bar, sweep_flags, n_flags);
+                launch_chained(round_gather_kernel<double>, grid, 256, 0, stream, Acur, lda, Wcur, ldc, rows, ordr, ocur, m,
+                               b, An, Wn, E, onew, order_out + done, bar, sweep_flags, n_flags);
             else
-                launch_chained(round_gather_kernel<float>, grid, 256, 0, stream, Acur, lda, W, ldw, rows, ordr, ocur, m, b, An, Wn, E,
-                               onew, order_out + done, bar, sweep_flags, n_flags);
+                launch_chained(round_gather_kernel<float>, grid, 256, 0, stream, Acur, lda, W, ldw, rows, ordr, ocur, m, b,
+                               An, Wn, E, onew, order_out + done, bar, sweep_flags, n_flags);
         }
         int st = PTQ_OK;
         const CholRange range = {0, b < m ? b / kNB : cdiv(m, kNB), cdiv(m, kNB)};
@@ -550,9 +562,7 @@ int ptq_quantize_layer_dynamic(const float* W, int rows, int cols, int64_t ldw, 
             Launch l(K_DYN_AUX, stream);
             const int gr = rows < 4096 ? rows : 4096;
             launch_chained(emit_block_kernel, dim3(grid_x_for(b, 256), gr), 256, 0, stream, codes_p, m, onew, b, W, rows,
-                           cols, ldw,
-                                                                            scale, zero, codes, What,
-                                                                            want_loss ? dW : nullptr);
+                           cols, ldw, scale, zero, codes, What, want_loss ? dW : nullptr);
         }
         Acur = An + (size_t)b * m + b; lda = m;
         Wcur = Wn + b; ldc = m;
@@ -573,8 +583,10 @@ int ptq_quantize_layer_dynamic(const float* W, int rows, int cols, int64_t ldw, 
         dim3 grid;
         const int st = launch_dgemm(K_DGEMM_LOSS, g, 1, stream, 64, &grid);
         if (st) return st;
-        { Launch l(K_SUM_PARTIALS, stream); launch_chained(sum_partials_kernel, 1, 256, 0, stream, partials,
-                                                           (int)(grid.x * grid.y * grid.z), 0.5, loss_out); }
+        {
+            Launch l(K_SUM_PARTIALS, stream);
+            launch_chained(sum_partials_kernel, 1, 256, 0, stream, partials, (int)(grid.x * grid.y * grid.z), 0.5, loss_out);
+        }
     }
     return launch_status();
 }
@@ -607,8 +619,8 @@ int ptq_quantize_layer_per_row(const float* W, int rows, int cols, int64_t ldw, 
     {
         Launch l(K_PER_ROW, stream);
         launch_chained(per_row_kernel, rows, kPerRowThreads, per_row_smem_bytes(cols), stream, W, rows, cols, ldw, Hinv,
-                       scale, zero, bits, mode, ascending, codes, What, perm_rows,
-            want_loss ? H_undamped : nullptr, want_loss ? row_loss : nullptr, status);
+                       scale, zero, bits, mode, ascending, codes, What, perm_rows, want_loss ? H_undamped : nullptr,
+                       want_loss ? row_loss : nullptr, status);
     }
     if (want_loss) {
         Launch l(K_SUM_PARTIALS, stream);
@@ -636,8 +648,10 @@ int ptq_gemm_nt_sliced(double* C, int64_t ldc, const double* A, int64_t lda, con
 int ptq_sort_scores(const double* S, int cols, int ascending, int32_t* perm, void* stream_) {
     cudaStream_t stream = static_cast<cudaStream_t>(stream_);
     if (!S || !perm || cols < 1) return PTQ_ERR_INVALID_ARG;
-    { Launch l(K_RANK_SORT, stream); launch_chained(rank_sort_kernel, cdiv(cols, kRankCols), 256, 0, stream, S, cols,
-                                                    ascending ? 1 : 0, perm, nullptr); }
+    {
+        Launch l(K_RANK_SORT, stream);
+        launch_chained(rank_sort_kernel, cdiv(cols, kRankCols), 256, 0, stream, S, cols, ascending ? 1 : 0, perm, nullptr);
+    }
     return launch_status();
 }
 
@@ -761,16 +775,18 @@ int ptq_quantize_layer(const float* W, int rows, int cols, int64_t ldw, const do
     });
     if (st) return st;
     const int n_flags = cdiv(rows, kSweepRows) + 1;
-    { Launch l(K_PERM_CHECK, stream); launch_chained(perm_check_kernel, cdiv(n, 256), 256, 0, stream, perm, n, invperm, bar,
-                                                     sweep_flags, n_flags, status); }
+    {
+        Launch l(K_PERM_CHECK, stream);
+        launch_chained(perm_check_kernel, cdiv(n, 256), 256, 0, stream, perm, n, invperm, bar, sweep_flags, n_flags, status);
+    }
     {
         Launch l(K_SWEEP_GATHER, stream);
         if (n <= kGatherMaxCols)
-            launch_chained(sweep_gather_kernel<true>, n + rows, kGatherThreads, (size_t)n * sizeof(double), stream, Hinv, W, rows, n, ldw,
-                           perm, invperm, U, Wp, E, status);
+            launch_chained(sweep_gather_kernel<true>, n + rows, kGatherThreads, (size_t)n * sizeof(double), stream, Hinv, W,
+                           rows, n, ldw, perm, invperm, U, Wp, E, status);
         else
-            launch_chained(sweep_gather_kernel<false>, n + rows, kGatherThreads, 0, stream, Hinv, W, rows, n, ldw, perm, invperm, U, Wp, E,
-                           status);
+            launch_chained(sweep_gather_kernel<false>, n + rows, kGatherThreads, 0, stream, Hinv, W, rows, n, ldw, perm,
+                           invperm, U, Wp, E, status);
     }
     // Blocked Eq. 12 and the sweep: of everything at once, or, on wide layers, panel by panel (cholpanel.cuh).  There the part of
     // Eq. 11 that a panel's columns owe to all later ones, W[:, later] -= E[:, panel] U[panel, later], is one large product on
@@ -812,9 +828,8 @@ int ptq_quantize_layer(const float* W, int rows, int cols, int64_t ldw, const do
     int8_t* kexp = sliced ? reinterpret_cast<int8_t*>(Dbuf) : nullptr;      // the factorisation is done with Dbuf
     {
         Launch l(K_FINALIZE, stream);
-        launch_chained(finalize_kernel, dim3(cdiv(n, 1024), rows), 256, 0, stream, codes_p, invperm, W, rows, n, ldw,
-                       scale,
-                                                                           zero, codes, What, dW, H_undamped, kexp);
+        launch_chained(finalize_kernel, dim3(cdiv(n, 1024), rows), 256, 0, stream, codes_p, invperm, W, rows, n, ldw, scale,
+                       zero, codes, What, dW, H_undamped, kexp);
     }
     if (sliced) {
         // 1/2 sum_ij dW_ij (dW H)_ij on the int8 tensor path.  H is symmetric: per 64-column block j the column blocks
@@ -833,8 +848,10 @@ int ptq_quantize_layer(const float* W, int rows, int cols, int64_t ldw, const do
         prm.k_mode = X_K_OWN_J; prm.alpha = 0.5; prm.partials = partials + tiles;
         st = x_product(a, b, prm, stream);
         if (st) return st;
-        { Launch l(K_SUM_PARTIALS, stream); launch_chained(sum_partials_kernel, 1, 256, 0, stream, partials, 2 * tiles, 1.0,
-                                                           loss_out); }
+        {
+            Launch l(K_SUM_PARTIALS, stream);
+            launch_chained(sum_partials_kernel, 1, 256, 0, stream, partials, 2 * tiles, 1.0, loss_out);
+        }
     } else if (want_loss) {
         // sum_ic dW_ic (dW H)_ic; H is symmetric, so for the 64-column block of c only k up to the end of that block is
         // summed and the blocks before it are doubled
@@ -848,8 +865,10 @@ int ptq_quantize_layer(const float* W, int rows, int cols, int64_t ldw, const do
         dim3 grid;
         st = launch_dgemm(K_DGEMM_LOSS, g, 1, stream, 64, &grid);
         if (st) return st;
-        { Launch l(K_SUM_PARTIALS, stream); launch_chained(sum_partials_kernel, 1, 256, 0, stream, partials,
-                                                           (int)(grid.x * grid.y * grid.z), 0.5, loss_out); }
+        {
+            Launch l(K_SUM_PARTIALS, stream);
+            launch_chained(sum_partials_kernel, 1, 256, 0, stream, partials, (int)(grid.x * grid.y * grid.z), 0.5, loss_out);
+        }
     }
     return launch_status();
 }

@@ -709,13 +709,11 @@ inline int gram_accumulate(double* H, GramSource src, int cols, int n, void* ws,
             if (src.conv) {
                 src.col0 = c0;
                 launch_chained(gram_split_conv_kernel, cols_pad, 256, 0, stream, src, cols, nc, cols_pad, n_pad, Q, shifts,
-                               status,
-                                                                     clr, n_clr);
+                               status, clr, n_clr);
             } else {
                 const int vec_ok = (aligned16(src.base) && (src.ldx & 3) == 0) ? 1 : 0;
-                launch_chained(gram_split_kernel, cols_pad, 256, 0, stream, src.base + c0, cols, nc, src.ldx, cols_pad,
-                               n_pad, vec_ok,
-                                                                Q, shifts, status, clr, n_clr);
+                launch_chained(gram_split_kernel, cols_pad, 256, 0, stream, src.base + c0, cols, nc, src.ldx, cols_pad, n_pad,
+                               vec_ok, Q, shifts, status, clr, n_clr);
             }
         }
         CUtensorMap mapA, mapB;
@@ -728,12 +726,12 @@ inline int gram_accumulate(double* H, GramSource src, int cols, int n, void* ws,
         {
             Launch l(K_GRAM_I8, stream);
             launch_chained(gram_i8_kernel, grid, kGramThreads, kGramSmemBytes, stream, mapA, mapB, H, cols, n_pad, shifts,
-                                                                         num_tiles, nbj, status, n_full, ksplit, iacc);
+                           num_tiles, nbj, status, n_full, ksplit, iacc);
         }
         if (sliced > 0) {
             Launch l(K_GRAM_FINISH, stream);
-            launch_chained(gram_finish_kernel, dim3(sliced, kGramTN / kGramFinishCols), kGramTM, 0, stream, iacc, H, cols, n_full, nbj,
-                           shifts);
+            launch_chained(gram_finish_kernel, dim3(sliced, kGramTN / kGramFinishCols), kGramTM, 0, stream, iacc, H, cols,
+                           n_full, nbj, shifts);
         }
         if (cudaGetLastError() != cudaSuccess) return PTQ_ERR_CUDA;
     }
