@@ -206,3 +206,37 @@ def test_largest_scaling_shape_4096x11008_all_bit_widths():
         dWg = dW[torch.from_numpy(rows).cuda()]
         assert abs(0.5 * float(((dWg @ Hd) * dWg).sum()) - loss_rows) <= LOSS_RTOL * loss_rows
         del dW, dWg
+
+
+@pytest.mark.parametrize("cols", [25600, 25601])
+def test_rows_wider_than_the_shared_memory_of_the_gather(cols):
+    """Up to 25600 columns a row of the inverse Hessian is staged in shared memory while it is permuted, wider ones are read in
+    place.  The inverse Hessian couples the columns 2 k and 2 k + 1 only, so that the sweep has a closed form: the column of a
+    pair that comes second in the order takes up c / [Hinv]_jj of the first one's rounding error."""
+    rows, c = 3, 0.5
+    g = torch.Generator(device="cuda").manual_seed(cols)
+    W = torch.randn((rows, cols), device="cuda", generator=g)
+    perm = torch.randperm(cols, device="cuda", generator=g).to(torch.int32)
+    d = 1.0 + torch.rand(cols, dtype=torch.float64, device="cuda", generator=g)
+    Hinv = torch.diag(d)
+    left = torch.arange(0, cols - 1, 2, device="cuda")
+    Hinv[left, left + 1] = Hinv[left + 1, left] = c
+    scale, zero = torch.full((rows,), 0.25, device="cuda"), torch.full((rows,), 8.0, device="cuda")
+    codes = torch.empty((rows, cols), dtype=torch.uint8, device="cuda")
+    st, ws = ptq.new_status(), ptq.Workspace()
+    ptq.quantize_layer(W, Hinv, perm, scale, zero, 4, codes, None, None, None, ws, st)
+    torch.cuda.synchronize()
+    ptq.check_status(st)
+    del Hinv, ws
+    w = W.double()
+
+    def code(x):
+        return (torch.round(x / 0.25) + 8.0).clamp(0.0, 15.0)
+    want = code(w)
+    position = torch.empty(cols, dtype=torch.int64, device="cuda")
+    position[perm.long()] = torch.arange(cols, device="cuda")
+    swap = position[left] > position[left + 1]
+    first, second = left + swap.long(), left + 1 - swap.long()
+    e = (w[:, first] - 0.25 * (want[:, first] - 8.0)) / d[first]
+    want[:, second] = code(w[:, second] - c * e)
+    assert torch.equal(codes.double(), want)
