@@ -710,6 +710,9 @@ inline int sweep_launch(double* Wp, const double* U, double* E, uint8_t* codes_p
 // Behind one another they take the longer of the two; a tenth is asked of them to be worth it.  Measured, one after the
 // other -> one launch: 64 x 128 50 -> 36 us, 128 x 576 175 -> 115, 128 x 1152 334 -> 220, 1000 x 1152 372 -> 260, 256 x 2304
 // 742 -> 568, 1000 x 2048 811 -> 711, 1000 x 2900 1490 -> 1441, 2000 x 1152 478 -> 402; not taken: 2000 x 2048 1107 -> 1318.
+// The panels of wider layers were no part of the fit, but the choice holds for them.  Both factorisations and the sweep of all
+// panels, never in one launch -> as chosen, in ms: 16 x 3072 1.72 -> 1.45, 1000 x 3072 1.85 -> 1.61, 2047 x 3200 2.18 -> 2.03, 64 x
+// 4608 3.16 -> 2.71, 2000 x 4608 3.60 -> 3.43, 512 x 8192 8.43 -> 7.75, 1500 x 8192 (five of eight panels) 9.06 -> 8.60.
 inline int sweep_ctas_behind(int rows, int sweep_n, int n, const CholRange& range, int budget) {
     const int groups = cdiv(rows, kSweepRows), nb = cdiv(n, kNB);
     if (groups >= budget) return 0;
