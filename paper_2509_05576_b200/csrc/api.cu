@@ -55,7 +55,7 @@ bool sliced_loss(int rows, int cols) {
 }
 // Digits of E and U in the deferred part of Eq. 11 of layers that are swept panel by panel.  With eight the product is more
 // exact than the float64 MMA steps of the sweep for every kind of input measured, with seven it is less exact where the input
-// channels differ in scale (i8gemm.cuh).  Layers this tall and wide have never had float64 steps and keep seven: eight
+// channels differ in scale (i8gemm.cuh).  Layers this tall and wide had no float64 steps to match and keep seven: eight
 // would take 7.19 -> 7.32 ms at 4096 x 4096 and 53.6 -> 54.8 at 4096 x 11008.  Below, seven -> eight: 512 x 4608 6.18 -> 6.22 ms,
 // 2000 x 4608 7.63 -> 7.73, 512 x 8192 19.2 -> 19.3, 2000 x 8000 21.7 -> 22.1.
 inline int deferred_digits(int rows, int cols) { return rows >= 2048 && cols >= 4096 ? kXSlices : kXMoreSlices; }

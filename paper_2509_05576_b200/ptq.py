@@ -466,7 +466,7 @@ class LayerSet:
     """Independent layers (a network's layers, each with its own calibration input) quantized side by side on several
     streams of one GPU.  Layers up to a few thousand columns are bound by dependency chains (the pivots of the
     factorisations, the columns of the sweep), not by the number of SMs, so several of them fit on the GPU at once --
-    provided the two persistent cooperative kernels, which otherwise take one CTA per SM each, are held to a share of the
+    provided the persistent cooperative kernels, which otherwise take one CTA per SM each, are held to a share of the
     SMs (``ptq_set_cta_limit``).  ``cta_limit`` None: a quarter of the SMs for layers below 3072 columns, half for wider
     ones; 0: no limit.  The layers are dealt longest first (a rough estimate from the shapes) onto the stream with the
     least work so far.  Every stream has its own workspace, every layer its own LayerBuffers, kept in ``self.bufs`` in
