@@ -41,11 +41,12 @@ INT8_OVER_BF16 = 2.0                                   # nominal dense 4.5 / 2.2
 # profiles/, on the bench workload (Gram: scaled from the 16384-column capture by the calibration columns processed).
 # Each entry names the kernel sources it was taken with; when they have changed since, the traffic is reported as null.
 NCU_TRAFFIC = {
-    "chol_coop": {"bytes_per_launch": (45.38e6 + 5.53e6 + 21.63e6 + 0.19e6) / 2, "sources": ["chol.cuh", "dgemm.cuh"],
-                  "sha256_16": "e59387afe85874df"},
-    "sweep_coop": {"bytes_per_launch": 28.71e6 + 0.02e6, "sources": ["colloop.cuh"], "sha256_16": "712ec88ea0625c06"},
-    "gram_i8_tcgen05": {"bytes_per_launch": (507.5e6 + 27.5e6) * 4096 / 16384, "sources": ["gram.cuh"],
-                        "sha256_16": "fcdf7052c8ea150e"},
+    "chol_coop": {"bytes_per_launch": 45.36e6 + 4.63e6, "sources": ["chol.cuh", "dgemm.cuh"],
+                  "sha256_16": "23eb2eb884b9efbf"},
+    "factor_sweep": {"bytes_per_launch": 26.56e6 + 1.62e6, "sources": ["colloop.cuh", "chol.cuh", "dgemm.cuh"],
+                     "sha256_16": "b70811cac9ff8d49"},
+    "gram_i8_tcgen05": {"bytes_per_launch": (508.0e6 + 32.7e6) * 4096 / 16384, "sources": ["gram.cuh"],
+                        "sha256_16": "b90fa1b4cf5a41fb"},
 }
 
 
