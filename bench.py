@@ -72,7 +72,9 @@ def load_peaks():
 
 
 class ClockSampler:
-    """Samples SM clocks and throttle reasons with nvidia-smi while the timed region runs."""
+    """Samples SM clocks and throttle reasons with nvidia-smi while the timed region runs.  nvidia-smi may need longer than a short
+    region takes to print its first line, so ``start`` waits for that (before the warm-up) and ``mark`` says where the region
+    begins; a region shorter than the interval between two samples gets the last one before its end."""
 
     Q = ("index,clocks.sm,clocks.max.sm,power.draw,clocks_event_reasons.active,clocks_event_reasons.hw_slowdown,"
          "clocks_event_reasons.hw_thermal_slowdown,clocks_event_reasons.sw_thermal_slowdown,"
@@ -80,33 +82,44 @@ class ClockSampler:
 
     def __init__(self, gpu_index):
         self.gpu = str(gpu_index)
-        self.lines = []
+        self.lines = []                                    # (time, line)
         self.proc = None
+        self.first = threading.Event()
+        self.begin = 0.0
 
     def start(self):
         try:
             self.proc = subprocess.Popen(["nvidia-smi", "-i", self.gpu, f"--query-gpu={self.Q}",
-                                          "--format=csv,noheader,nounits", "-lms", "50"],
+                                          "--format=csv,noheader,nounits", "-lms", "25"],
                                          stdout=subprocess.PIPE, stderr=subprocess.DEVNULL, text=True)
             self.thread = threading.Thread(target=self._read, daemon=True)
             self.thread.start()
+            self.first.wait(timeout=10)
         except Exception:
             self.proc = None
 
+    def mark(self):
+        self.begin = time.monotonic()
+
     def _read(self):
         for line in self.proc.stdout:
-            self.lines.append(line.strip())
+            self.lines.append((time.monotonic(), line.strip()))
+            self.first.set()
 
     def stop(self):
         if self.proc is None:
             return {"sm_mhz": None, "sm_max_mhz": None, "reasons": ["nvidia-smi unavailable"]}
+        end = time.monotonic()
         self.proc.terminate()
         try:
             self.proc.wait(timeout=5)
         except Exception:
             self.proc.kill()
+        self.thread.join(timeout=5)
+        taken = [x for x in self.lines if x[0] <= end]
+        lines = [ln for t, ln in taken if t >= self.begin] or [ln for _, ln in taken[-1:]]
         sm, mx, reasons = [], [], set()
-        for ln in self.lines:
+        for ln in lines:
             f = [x.strip() for x in ln.split(",")]
             if len(f) < 9:
                 continue
@@ -345,6 +358,8 @@ def run_ours(args):
     def step(events=None):
         ptq.quantize_layer_full(Wd, Xd, spec.bits, spec.damp, bufs=bufs, ws=ws, stream=stream, events=events)
 
+    sampler = ClockSampler(os.environ.get("CUDA_VISIBLE_DEVICES", str(local)).split(",")[0] if world == 1 else local)
+    sampler.start()
     for _ in range(max(args.warmup, 3)):
         flush.fill_(1)
         step()
@@ -352,12 +367,11 @@ def run_ours(args):
     ptq.check_status(bufs.status, "warm-up")
 
     # ---- timed region: K steps, device time by CUDA events on the launching stream, L2 flushed between steps
-    sampler = ClockSampler(os.environ.get("CUDA_VISIBLE_DEVICES", str(local)).split(",")[0] if world == 1 else local)
     starts = [torch.cuda.Event(enable_timing=True) for _ in range(args.steps)]
     ends = [torch.cuda.Event(enable_timing=True) for _ in range(args.steps)]
     launches0 = ptq.launch_count()
     barrier()
-    sampler.start()
+    sampler.mark()
     for k in range(args.steps):
         flush.fill_(k & 0xFF)
         starts[k].record(stream)

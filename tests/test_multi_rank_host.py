@@ -3,7 +3,9 @@ path): per-rank seeds, max-over-ranks timing and whole-job throughput, run as tw
 import os
 import socket
 import sys
+import time
 
+import pytest
 import torch
 import torch.distributed as dist
 import torch.multiprocessing as mp
@@ -98,3 +100,22 @@ def test_the_bench_line_keeps_its_keys_and_stays_short():
     assert "layer_sets_ms" in got and "per_kernel" not in got["roofline"]
     report["roofline"]["peak_source"] = "p" * 500
     assert len(bench.bench_line(report)) <= bench.LINE_LIMIT
+
+
+@pytest.mark.parametrize("region", [0.3, 0.0])
+def test_clocks_are_sampled_however_late_the_first_line_and_however_short_the_region(tmp_path, monkeypatch, region):
+    """A stand-in for nvidia-smi that prints its first line after 0.4 s and another one every 50 ms, idle clocks first."""
+    tool = tmp_path / "nvidia-smi"
+    tool.write_text("#!/bin/bash\nsleep 0.4\nmhz=345\nwhile true; do\n"
+                    "echo \"0, $mhz, 1965, 100.0, 0x0, Not Active, Not Active, Not Active, Active\"\nsleep 0.05; mhz=1900\ndone\n")
+    tool.chmod(0o755)
+    monkeypatch.setenv("PATH", f"{tmp_path}:{os.environ['PATH']}")
+    import bench
+    sampler = bench.ClockSampler(0)
+    sampler.start()
+    time.sleep(0.3)                     # the warm-up
+    sampler.mark()
+    time.sleep(region)
+    out = sampler.stop()
+    assert out["samples"] >= 1 and out["sm_mhz"] == 1900.0 and out["sm_max_mhz"] == 1965.0
+    assert out["reasons"] == ["sw_power_cap"]
