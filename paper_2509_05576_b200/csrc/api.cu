@@ -285,9 +285,11 @@ size_t ptq_workspace_bytes(int call_id, int rows, int cols, int n) {
             add(2 * sizeof(unsigned));                      // grid barrier of the factorisation kernel
             add(((size_t)cdiv(rows, kSweepRows) + 1) * sizeof(unsigned));   // per-row-group progress counters of the sweep
             add(chol_scratch_doubles(cols) * sizeof(double));
-            if (cols >= kPanelMinCols) {                    // slices of U[panel, later] and of E[:, panel]
-                add(x_operand_bytes(cols, kPanelBlocks * kNB, deferred_digits(rows, cols)));
-                add(x_operand_bytes(rows, kPanelBlocks * kNB, deferred_digits(rows, cols)));
+            if (cols >= kPanelMinCols) {
+                // slices of U[panel, later] and of E[:, panel]; always for the most digits, so that what suffices for one
+                // layer suffices for every smaller one
+                add(x_operand_bytes(cols, kPanelBlocks * kNB, kXMoreSlices));
+                add(x_operand_bytes(rows, kPanelBlocks * kNB, kXMoreSlices));
             }
             break;
         case PTQ_CALL_QUANTIZE_LAYER_PER_ROW:

@@ -51,6 +51,18 @@ def test_workspace_sizes(lib):
     assert total < 8 * 2 ** 30
 
 
+@pytest.mark.parametrize("call", range(7))
+def test_a_workspace_for_one_layer_suffices_for_every_smaller_one(lib, call):
+    from paper_2509_05576_b200 import ptq
+    sizes = (1, 128, 2047, 2048, 4096)
+    for cols in (64, 128, 3071, 3072, 4095, 4096, 4608, 11008):
+        need = [ptq.workspace_bytes(call, rows, cols, 4096) for rows in sizes]
+        assert need == sorted(need)
+    for rows in sizes:
+        need = [ptq.workspace_bytes(call, rows, cols, 4096) for cols in (64, 128, 3071, 3072, 4095, 4096, 4608, 11008)]
+        assert need == sorted(need)
+
+
 def test_bad_arguments_are_rejected_on_the_host(lib):
     from paper_2509_05576_b200 import ptq
     vp = ctypes.c_void_p
